@@ -1,8 +1,10 @@
-"""Thin ctypes binding of ``libm2rnn.so`` (declared in ``include/m2rnn.h``).
+"""Thin binding of ``libm2rnn.so`` (declared in ``include/m2rnn.h``).
 
 Argument marshalling only: every step of the scan runs in the library's CUDA kernels.
 torch supplies device memory and the current stream; there is no CPU or eager fallback --
-a missing or stale library raises.
+a missing or stale library raises.  The calls of the scan and of the paths around it are marshalled
+in C++ (``csrc/py_native.cpp``, built as ``_native.so``): a decoded token takes a few microseconds on
+the GPU, so its host path is what counts.  The size queries and self-tests go through ctypes.
 
     y, hT, ckpt = m2rnn_fwd(q, k, v, gate, W, h0, save_ckpt=True)
     grads       = m2rnn_bwd(q, k, v, gate, W, h0, dy, ckpt=ckpt)
@@ -33,7 +35,7 @@ STATUS = {0: "M2RNN_OK", -1: "M2RNN_ERR_NULL", -2: "M2RNN_ERR_SHAPE", -3: "M2RNN
 class M2RNNError(RuntimeError):
     def __init__(self, status: int, where: str):
         self.status = status
-        msg = _lib().m2rnn_status_string(status).decode() if _LIB is not None else ""
+        msg = _lib().m2rnn_status_string(status).decode()
         super().__init__(f"{where}: {STATUS.get(status, status)} ({msg})")
 
 
@@ -92,6 +94,21 @@ def _lib() -> ctypes.CDLL:
     return _LIB
 
 
+class _NotLoaded:
+    """Stands for the native half until its first use: loads it and takes its own place."""
+
+    def __getattr__(self, name):
+        global _native
+        _lib()
+        from . import _native as mod
+        mod.set_error_class(M2RNNError)
+        _native = mod
+        return getattr(mod, name)
+
+
+_native = _NotLoaded()
+
+
 def _ptr(t):
     return None if t is None else ctypes.c_void_p(t.data_ptr())
 
@@ -122,15 +139,10 @@ def _chk(t, name, shape, dtype, strided_tokens=False):
         raise ValueError(f"{name} must be contiguous")
 
 
-_status_words: dict[int, torch.Tensor] = {}
-
-
 def device_status_word(device=None) -> torch.Tensor:
     """The int32 word kernels raise when a bounded wait runs out (one per device, zero = fine)."""
     idx = torch.cuda.current_device() if device is None else torch.device(device).index
-    if idx not in _status_words:
-        _status_words[idx] = torch.zeros(1, dtype=torch.int32, device=f"cuda:{idx}")
-    return _status_words[idx]
+    return _native.status_word(idx)
 
 
 def check_device_status(device=None) -> None:
@@ -226,35 +238,9 @@ def m2rnn_fwd(q, k, v, gate, W, h0=None, *, gate_kind=GATE_LOGIT, alpha=None, be
     q, k, v may be strided views along the token axis (e.g. slices of one fused projection output).
     With ``cu_seqlens`` (int32 [B+1], CUDA) and ``max_seqlen`` the batch is packed: q [tokens,Nq,K],
     k, v, gate [tokens,N], y [tokens,N,V]; states stay [B,N,K,V]."""
-    p = _params(q, k, v, W, gate_kind, ckpt_interval, cu_seqlens=cu_seqlens, max_seqlen=max_seqlen)
-    B, T, N, K, V, io = p.B, p.T, p.N, p.K, p.V, q.dtype
-    lead = (B, T) if cu_seqlens is None else (q.shape[0],)
-    _chk(q, "q", (*lead, p.Nq, K), io, True); _chk(k, "k", (*lead, p.Nk, K), io, True); _chk(v, "v", (*lead, N, V), io, True)
-    _chk(gate, "gate", (*lead, N), torch.float32); _chk(W, "W", (N, V, V), io)
-    _chk(h0, "h0", (B, N, K, V), torch.float32); _chk(w_r, "w_r", (N, V), io)
-    _chk(alpha, "alpha", (N,), torch.float32); _chk(beta, "beta", (N,), torch.float32)
-    out = out or {}
-    y = out.get("y")
-    if y is None:
-        y = torch.empty((*lead, N, V), dtype=io, device=q.device)
-    hT = out.get("hT")
-    if hT is None and want_hT:
-        hT = torch.empty((B, N, K, V), dtype=torch.float32, device=q.device)
-    ckpt = out.get("ckpt")
-    if ckpt is None and save_ckpt:
-        C = m2rnn_ckpt_interval(p)
-        ckpt = torch.empty((B, N, (T + C - 1) // C, K, V), dtype=torch.float32, device=q.device)
-    _chk(y, "y", (*lead, N, V), io); _chk(hT, "hT", (B, N, K, V), torch.float32)
-    need = m2rnn_fwd_workspace_bytes(p)
-    if workspace is None and need > 0:
-        workspace = torch.empty(need, dtype=torch.uint8, device=q.device)
-    rc = _lib().m2rnn_fwd(ctypes.byref(p), _ptr(q), _ptr(k), _ptr(v), _ptr(gate), _ptr(W), _ptr(h0),
-                          _ptr(alpha), _ptr(beta), _ptr(w_r), _ptr(y), _ptr(hT), _ptr(ckpt),
-                          _ptr(workspace), 0 if workspace is None else workspace.numel(),
-                          _ptr(device_status_word(q.device)), _stream(stream))
-    if rc != 0:
-        raise M2RNNError(rc, "m2rnn_fwd")
-    return y, hT, ckpt
+    y, hT, ckpt = (out.get("y"), out.get("hT"), out.get("ckpt")) if out else (None, None, None)
+    return _native.fwd(q, k, v, gate, W, h0, gate_kind, alpha, beta, w_r, save_ckpt, ckpt_interval, want_hT, y, hT, ckpt,
+                       workspace, stream, cu_seqlens, max_seqlen)
 
 
 def m2rnn_bwd(q, k, v, gate, W, h0, dy, d_hT=None, *, ckpt=None, gate_kind=GATE_LOGIT, alpha=None,
@@ -262,40 +248,9 @@ def m2rnn_bwd(q, k, v, gate, W, h0, dy, d_hT=None, *, ckpt=None, gate_kind=GATE_
               out=None, stream=None, cu_seqlens=None, max_seqlen=None):
     """Backward through time.  Returns dict(dq, dk, dv, dgate, dW, dh0) (dense, whatever the strides
     of q, k, v).  ``cu_seqlens`` / ``max_seqlen``: packed batch, as in ``m2rnn_fwd``."""
-    p = _params(q, k, v, W, gate_kind, ckpt_interval, dh_clip, cu_seqlens=cu_seqlens, max_seqlen=max_seqlen)
-    B, T, N, K, V, io = p.B, p.T, p.N, p.K, p.V, q.dtype
-    lead = (B, T) if cu_seqlens is None else (q.shape[0],)
-    _chk(q, "q", (*lead, p.Nq, K), io, True); _chk(k, "k", (*lead, p.Nk, K), io, True); _chk(v, "v", (*lead, N, V), io, True)
-    _chk(gate, "gate", (*lead, N), torch.float32); _chk(W, "W", (N, V, V), io)
-    _chk(h0, "h0", (B, N, K, V), torch.float32); _chk(w_r, "w_r", (N, V), io)
-    _chk(alpha, "alpha", (N,), torch.float32); _chk(beta, "beta", (N,), torch.float32)
-    _chk(dy, "dy", (*lead, N, V), io); _chk(d_hT, "d_hT", (B, N, K, V), torch.float32)
-    if ckpt is not None and T > 0:
-        C = m2rnn_ckpt_interval(p)
-        _chk(ckpt, "ckpt", (B, N, (T + C - 1) // C, K, V), torch.float32)
-    dev = q.device
-    out = out or {}
-    g = dict(dq=out.get("dq"), dk=out.get("dk"), dv=out.get("dv"), dgate=out.get("dgate"),
-             dW=out.get("dW"), dh0=out.get("dh0"))
-    if g["dq"] is None: g["dq"] = torch.empty(q.shape, dtype=io, device=dev)
-    if g["dk"] is None: g["dk"] = torch.empty(k.shape, dtype=io, device=dev)
-    if g["dv"] is None: g["dv"] = torch.empty(v.shape, dtype=io, device=dev)
-    if g["dgate"] is None: g["dgate"] = torch.empty_like(gate)
-    if g["dW"] is None: g["dW"] = torch.empty((N, V, V), dtype=torch.float32, device=dev)
-    if g["dh0"] is None and want_dh0: g["dh0"] = torch.empty((B, N, K, V), dtype=torch.float32, device=dev)
-    for x in ("dq", "dk", "dv"):
-        _chk(g[x], x, {"dq": q, "dk": k, "dv": v}[x].shape, io)
-    need = m2rnn_bwd_workspace_bytes(p, ckpt is not None)
-    if workspace is None:
-        workspace = torch.empty(max(need, 1), dtype=torch.uint8, device=dev)
-    rc = _lib().m2rnn_bwd(ctypes.byref(p), _ptr(q), _ptr(k), _ptr(v), _ptr(gate), _ptr(W), _ptr(h0),
-                          _ptr(alpha), _ptr(beta), _ptr(w_r), _ptr(ckpt), _ptr(dy), _ptr(d_hT),
-                          _ptr(g["dq"]), _ptr(g["dk"]), _ptr(g["dv"]), _ptr(g["dgate"]), _ptr(g["dW"]),
-                          _ptr(g["dh0"]), _ptr(workspace), workspace.numel(),
-                          _ptr(device_status_word(dev)), _stream(stream))
-    if rc != 0:
-        raise M2RNNError(rc, "m2rnn_bwd")
-    return g
+    dq, dk, dv, dgate, dW, dh0 = map(out.get, ("dq", "dk", "dv", "dgate", "dW", "dh0")) if out else (None,) * 6
+    return _native.bwd(q, k, v, gate, W, h0, dy, d_hT, ckpt, gate_kind, alpha, beta, w_r, ckpt_interval, dh_clip, want_dh0,
+                       workspace, dq, dk, dv, dgate, dW, dh0, stream, cu_seqlens, max_seqlen)
 
 
 def m2rnn_bwd_static_scratch(q, k, v, gate, W, h0, dy, d_hT=None, *, out, ckpt=None, gate_kind=GATE_LOGIT,
@@ -330,49 +285,13 @@ def m2rnn_bwd_static_scratch(q, k, v, gate, W, h0, dy, d_hT=None, *, out, ckpt=N
 def m2rnn_decode_step(q, k, v, gate, W, state, *, gate_kind=GATE_LOGIT, alpha=None, beta=None,
                       w_r=None, y=None, stream=None):
     """One decoding step; ``state`` [B,N,K,V] fp32 is updated in place.  Returns y [B,N,V]."""
-    p = _params(q, k, v, W, gate_kind, decode=True)
-    B, N, K, V, io = p.B, p.N, p.K, p.V, q.dtype
-    _chk(q, "q", (B, p.Nq, K), io); _chk(k, "k", (B, p.Nk, K), io); _chk(v, "v", (B, N, V), io)
-    _chk(gate, "gate", (B, N), torch.float32); _chk(W, "W", (N, V, V), io)
-    _chk(state, "state", (B, N, K, V), torch.float32); _chk(w_r, "w_r", (N, V), io)
-    _chk(alpha, "alpha", (N,), torch.float32); _chk(beta, "beta", (N,), torch.float32)
-    if y is None:
-        y = torch.empty((B, N, V), dtype=io, device=q.device)
-    _chk(y, "y", (B, N, V), io)
-    rc = _lib().m2rnn_decode_step(ctypes.byref(p), _ptr(q), _ptr(k), _ptr(v), _ptr(gate), _ptr(W),
-                                  _ptr(alpha), _ptr(beta), _ptr(w_r), _ptr(state), _ptr(y),
-                                  _ptr(device_status_word(q.device)), _stream(stream))
-    if rc != 0:
-        raise M2RNNError(rc, "m2rnn_decode_step")
-    return y
-
-
-def _norm_dims(y):
-    if y.dim() < 2:
-        raise ValueError("y needs at least the two trailing axes [N, V]")
-    d = y.shape[-2] * y.shape[-1]
-    tokens = y.numel() // d if d else 0
-    return tokens, d
+    return _native.decode_step(q, k, v, gate, W, state, gate_kind, alpha, beta, w_r, y, stream)
 
 
 def m2rnn_gated_norm_fwd(y, g_in, w, *, eps=0.0, silu=True, out=None, rstd=None, stream=None):
     """out = RMSNorm(y * SiLU(g_in)) over the head-concatenated features: y, g_in [..., N, V],
     w [N*V] (or [N, V]).  Returns (out like y, rstd [...] fp32)."""
-    tokens, d = _norm_dims(y)
-    io = y.dtype
-    _chk(g_in, "g_in", tuple(y.shape), io); _chk(w, "w", tuple(w.shape), io)
-    if w.numel() != d:
-        raise ValueError(f"w has {w.numel()} entries, the rows have {d}")
-    if out is None:
-        out = torch.empty_like(y)
-    if rstd is None:
-        rstd = torch.empty(tuple(y.shape[:-2]), dtype=torch.float32, device=y.device)
-    _chk(out, "out", tuple(y.shape), io); _chk(rstd, "rstd", tuple(y.shape[:-2]), torch.float32)
-    rc = _lib().m2rnn_gated_norm_fwd(tokens, d, _io_code(io), _ptr(y), _ptr(g_in), _ptr(w), float(eps), int(bool(silu)),
-                                     _ptr(out), _ptr(rstd), _stream(stream))
-    if rc != 0:
-        raise M2RNNError(rc, "m2rnn_gated_norm_fwd")
-    return out, rstd
+    return _native.gated_norm_fwd(y, g_in, w, eps, silu, out, rstd, stream)
 
 
 def m2rnn_gated_norm_bwd_workspace_bytes(tokens: int, d: int) -> int:
@@ -381,71 +300,21 @@ def m2rnn_gated_norm_bwd_workspace_bytes(tokens: int, d: int) -> int:
 
 def m2rnn_gated_norm_bwd(y, g_in, w, rstd, dout, *, silu=True, workspace=None, out=None, stream=None):
     """Backward of m2rnn_gated_norm_fwd -> dict(dy, dg, dw [N*V] fp32)."""
-    tokens, d = _norm_dims(y)
-    io = y.dtype
-    _chk(g_in, "g_in", tuple(y.shape), io); _chk(dout, "dout", tuple(y.shape), io); _chk(w, "w", tuple(w.shape), io)
-    _chk(rstd, "rstd", tuple(y.shape[:-2]), torch.float32)
-    out = out or {}
-    dy = out.get("dy", None); dg = out.get("dg", None); dw = out.get("dw", None)
-    dy = torch.empty_like(y) if dy is None else dy
-    dg = torch.empty_like(y) if dg is None else dg
-    dw = torch.empty((d,), dtype=torch.float32, device=y.device) if dw is None else dw
-    _chk(dy, "dy", tuple(y.shape), io); _chk(dg, "dg", tuple(y.shape), io); _chk(dw, "dw", (d,), torch.float32)
-    need = m2rnn_gated_norm_bwd_workspace_bytes(tokens, d)
-    if workspace is None:
-        workspace = torch.empty(max(need, 1), dtype=torch.uint8, device=y.device)
-    rc = _lib().m2rnn_gated_norm_bwd(tokens, d, _io_code(io), _ptr(y), _ptr(g_in), _ptr(w), _ptr(rstd), int(bool(silu)),
-                                     _ptr(dout), _ptr(dy), _ptr(dg), _ptr(dw), _ptr(workspace), workspace.numel(),
-                                     _stream(stream))
-    if rc != 0:
-        raise M2RNNError(rc, "m2rnn_gated_norm_bwd")
-    return dict(dy=dy, dg=dg, dw=dw)
-
-
-def _rows(t, name):
-    """[B,T,C] with contiguous channels and a regular token axis -> token stride in elements."""
-    if t.dim() == 3 and t.numel() == 0:
-        return t.shape[2]
-    if t.dim() != 3 or t.stride(2) != 1 or (t.shape[0] > 1 and t.stride(0) != t.shape[1] * t.stride(1)):
-        raise ValueError(f"{name}: expected [B,T,C] with contiguous channels and batch entries one after the other")
-    return t.stride(1)
+    dy, dg, dw = (out.get("dy"), out.get("dg"), out.get("dw")) if out else (None, None, None)
+    return _native.gated_norm_bwd(y, g_in, w, rstd, dout, silu, workspace, dy, dg, dw, stream)
 
 
 def m2rnn_conv_silu_fwd(x, w, bias=None, prev=None, *, out=None, stream=None):
     """SiLU(depthwise causal conv1d of width 4 along time) of x [B,T,C] (a view into a wider tensor is
     fine); w [C,4], bias [C], prev [B,3,C] (the three inputs before t = 0).  Returns out [B,T,C]."""
-    B, T, C = x.shape
-    io = x.dtype
-    _chk(w, "w", (C, 4), io); _chk(bias, "bias", (C,), io); _chk(prev, "prev", (B, 3, C), io)
-    if out is None:
-        out = torch.empty((B, T, C), dtype=io, device=x.device)
-    _chk(out, "out", (B, T, C), io, True)
-    rc = _lib().m2rnn_conv_silu_fwd(B, T, C, _io_code(io), _ptr(x), _rows(x, "x"), _ptr(w), _ptr(bias), _ptr(prev),
-                                    _ptr(out), _rows(out, "out"), _stream(stream))
-    if rc != 0:
-        raise M2RNNError(rc, "m2rnn_conv_silu_fwd")
-    return out
+    return _native.conv_silu_fwd(x, w, bias, prev, out, stream)
 
 
 def m2rnn_conv_silu_bwd(x, w, dout, bias=None, prev=None, *, out=None, workspace=None, stream=None):
     """Backward of ``m2rnn_conv_silu_fwd`` -> dict(dx [B,T,C], dw [C,4] fp32, dbias [C] fp32, dprev [B,3,C])."""
-    B, T, C = x.shape
-    io, dev = x.dtype, x.device
-    _chk(w, "w", (C, 4), io); _chk(bias, "bias", (C,), io); _chk(prev, "prev", (B, 3, C), io)
-    _chk(dout, "dout", (B, T, C), io, True)
-    out = dict(out or {})
-    if out.get("dx") is None: out["dx"] = torch.empty((B, T, C), dtype=io, device=dev)
-    if out.get("dw") is None: out["dw"] = torch.empty((C, 4), dtype=torch.float32, device=dev)
-    if out.get("dbias") is None: out["dbias"] = torch.empty((C,), dtype=torch.float32, device=dev)
-    if out.get("dprev") is None and prev is not None: out["dprev"] = torch.empty((B, 3, C), dtype=io, device=dev)
-    _chk(out["dx"], "dx", (B, T, C), io, True); _chk(out["dw"], "dw", (C, 4), torch.float32)
-    need = _lib().m2rnn_conv_silu_bwd_workspace_bytes(B, T, C)
-    if workspace is None:
-        workspace = torch.empty(max(need, 1), dtype=torch.uint8, device=dev)
-    rc = _lib().m2rnn_conv_silu_bwd(B, T, C, _io_code(io), _ptr(x), _rows(x, "x"), _ptr(w), _ptr(bias), _ptr(prev), _ptr(dout),
-                                    _rows(dout, "dout"), _ptr(out["dx"]), _rows(out["dx"], "dx"), _ptr(out["dw"]),
-                                    _ptr(out.get("dbias")), _ptr(out.get("dprev")), _ptr(workspace), workspace.numel(),
-                                    _stream(stream))
-    if rc != 0:
-        raise M2RNNError(rc, "m2rnn_conv_silu_bwd")
-    return out
+    res = dict(out) if out else {}
+    res["dx"], res["dw"], res["dbias"], dprev = _native.conv_silu_bwd(
+        x, w, dout, bias, prev, workspace, res.get("dx"), res.get("dw"), res.get("dbias"), res.get("dprev"), stream)
+    if dprev is not None:
+        res["dprev"] = dprev
+    return res

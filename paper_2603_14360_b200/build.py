@@ -1,4 +1,5 @@
-"""Builds ``libm2rnn.so`` in-tree with nvcc for sm_100a (cross-compiles without a GPU).
+"""Builds ``libm2rnn.so`` in-tree with nvcc for sm_100a (cross-compiles without a GPU) and the Python
+extension ``_native.so`` that calls it with g++ against torch's headers.
 
     python -m paper_2603_14360_b200.build [--force] [--verbose]
 """
@@ -14,6 +15,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libm2rnn.so")
+NATIVE = os.path.join(HERE, "_native.so")   # Python extension module: the binding's native half
 
 SOURCES = ["api.cu", "reduce.cu", "scan_f32.cu", "scan_fwd_bf16.cu", "scan_fwd_bf16_cs.cu", "scan_fwd_tc.cu", "scan_bwd_bf16.cu", "scan_bwd_tc.cu", "decode_bf16.cu", "decode_tc_bf16.cu",
            "bwd_static_scratch.cu", "gated_norm.cu", "conv_silu.cu", "selftest.cu"]
@@ -45,6 +47,28 @@ def _compile(src: str, force: bool, verbose: bool) -> str:
     return obj
 
 
+def _build_native(force: bool, verbose: bool) -> None:
+    src = os.path.join(CSRC, "py_native.cpp")
+    newest = max(os.path.getmtime(src), os.path.getmtime(os.path.join(ROOT, "include", "m2rnn.h")))
+    if not force and os.path.exists(NATIVE) and os.path.getmtime(NATIVE) >= newest:
+        return
+    import sysconfig
+    import torch
+    from torch.utils.cpp_extension import include_paths, library_paths
+    inc = [*include_paths("cuda"), sysconfig.get_paths()["include"], os.path.join(ROOT, "include")]
+    lib = library_paths("cuda")
+    tmp = f"{NATIVE}.{os.getpid()}.tmp"
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           *(f"-I{d}" for d in inc), src, "-o", tmp, f"-L{HERE}", "-l:libm2rnn.so", "-Wl,-rpath,$ORIGIN",
+           *(f"-L{d}" for d in lib), "-ltorch_python", "-ltorch", "-ltorch_cuda", "-ltorch_cpu", "-lc10_cuda", "-lc10"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if verbose or r.returncode:
+        sys.stderr.write(f"$ {' '.join(cmd)}\n{r.stdout}{r.stderr}")
+    if r.returncode:
+        raise RuntimeError("g++ failed on py_native.cpp")
+    os.replace(tmp, NATIVE)
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     os.makedirs(OBJ, exist_ok=True)
     with concurrent.futures.ThreadPoolExecutor(max_workers=os.cpu_count() or 4) as ex:
@@ -54,6 +78,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         subprocess.check_call(["nvcc", "-shared", "-gencode", "arch=compute_100a,code=sm_100a",
                                "-o", tmp, *objs])
         os.replace(tmp, LIB)
+    _build_native(force, verbose)
     return LIB
 
 

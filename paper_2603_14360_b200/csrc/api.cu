@@ -2,6 +2,7 @@
 // No allocation, no synchronisation, no state kept between calls.
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cstdlib>
 #include <cstring>
 
@@ -10,16 +11,58 @@
 
 namespace m2rnn {
 
+namespace {
+constexpr int kMaxDevices = 64;
+int current_device() {
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess) { (void)cudaGetLastError(); return -1; }
+  return dev;
+}
+}  // namespace
+
 // SMs of the current device (the plans size their grids by it); 148, a B200's count, when no device
 // can be asked -- the size queries of the ABI also run on hosts without a GPU.
 int sm_count() {
-  int dev = -1, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) {
+  static std::atomic<int> known[kMaxDevices];   // a constant of the device: asked for once
+  const int dev = current_device();
+  if (dev < 0) return 148;
+  if (dev < kMaxDevices)
+    if (const int n = known[dev].load(std::memory_order_relaxed)) return n;
+  int sms = 0;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) {
     (void)cudaGetLastError();
     return 148;
   }
+  if (dev < kMaxDevices) known[dev].store(sms, std::memory_order_relaxed);
   return sms;
+}
+
+// Lets `kernel` be launched with `bytes` of dynamic shared memory on the current device.  The
+// attribute stays with the loaded kernel, so it is set when a launch first needs more than any
+// before it (setting it on every launch cost a small call a tenth of its host time).
+cudaError_t allow_smem(const void *kernel, size_t bytes) {
+  constexpr int kSlots = 1024;   // (kernel, device) pairs: far more than the library has kernels
+  struct Entry { std::atomic<uintptr_t> key; std::atomic<int> bytes; };
+  static Entry table[kSlots];
+  if (bytes <= 48 * 1024) return cudaSuccess;   // what every kernel may use without asking
+  const int dev = current_device();
+  Entry *e = nullptr;
+  if (dev >= 0 && dev < kMaxDevices) {
+    const uintptr_t key = reinterpret_cast<uintptr_t>(kernel) * kMaxDevices + (uintptr_t)dev + 1;
+    size_t h = (size_t)((key * 0x9e3779b97f4a7c15ull) >> 54);
+    for (int probe = 0; probe < 64 && !e; ++probe, h = (h + 1) % kSlots) {
+      uintptr_t seen = table[h].key.load(std::memory_order_acquire);
+      if (seen == 0 && table[h].key.compare_exchange_strong(seen, key, std::memory_order_acq_rel)) seen = key;
+      if (seen == key) e = &table[h];
+    }
+  }
+  if (e && e->bytes.load(std::memory_order_acquire) >= (int)bytes) return cudaSuccess;
+  const cudaError_t rc = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (rc == cudaSuccess && e) {
+    int old = e->bytes.load(std::memory_order_relaxed);
+    while (old < (int)bytes && !e->bytes.compare_exchange_weak(old, (int)bytes, std::memory_order_release)) {}
+  }
+  return rc;
 }
 
 bool bwd_use_tc(int B, int N, int K, int V, int io_dtype) {

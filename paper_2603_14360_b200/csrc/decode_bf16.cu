@@ -198,12 +198,11 @@ cudaError_t launch_decode_v(const ScanArgs &a, cudaStream_t s) {
   const int GPI = WPU >= 8 ? 1 : 8 / WPU;   // units taken by a CTA at a time
   const int tasks_per_head = (a.B + GPI - 1) / GPI;
   const long ntasks = (long)a.N * tasks_per_head;
-  int dev = 0, sms = 148;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int sms = sm_count();
   const int grid = (int)(ntasks < sms ? ntasks : sms);
   const size_t smem = 16 + (size_t)(V / 16) * (V / 8) * 32 * 8 + sizeof(float) * 2 * GPI * WPU * V   // barriers, W, y partials
                       + sizeof(float) * 2 * (size_t)GPI * a.K * V;                                   // two stages of states
-  cudaError_t e = cudaFuncSetAttribute(decode_bf16_kernel<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(decode_bf16_kernel<V>, smem);
   if (e != cudaSuccess) return e;
   decode_bf16_kernel<V><<<grid, 256, smem, s>>>(a, WPU, GPI, tasks_per_head);
   return cudaGetLastError();

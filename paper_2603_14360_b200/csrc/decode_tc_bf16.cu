@@ -440,11 +440,10 @@ cudaError_t launch_tc(const ScanArgs &a, cudaStream_t s) {
   const int GPI = kM / a.K;
   const int tasks_per_head = (a.B + GPI - 1) / GPI;
   const long ntasks = (long)a.N * tasks_per_head;
-  int dev = 0, sms = 148;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int sms = sm_count();
   const int grid = (int)(ntasks < sms ? ntasks : sms);
   const size_t smem = TcSmem<V>::total;
-  cudaError_t e = cudaFuncSetAttribute(decode_tc_kernel<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(decode_tc_kernel<V>, smem);
   if (e != cudaSuccess) return e;
   decode_tc_kernel<V><<<grid, kThreads, smem, s>>>(a, GPI, tasks_per_head, map);
   return cudaGetLastError();

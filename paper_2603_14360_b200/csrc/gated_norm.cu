@@ -393,7 +393,7 @@ template <typename T, int kWarps>
 cudaError_t launch_bwd_w(long tokens, int d, const void *y, const void *g, const void *w, const float *rstd, int silu_on,
                          const void *dout, void *dy, void *dg, float *dw_part, cudaStream_t s) {
   const size_t smem = (size_t)kWarps * d * sizeof(float);
-  cudaError_t e = cudaFuncSetAttribute(gated_norm_bwd_kernel<T, kWarps>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(gated_norm_bwd_kernel<T, kWarps>, smem);
   if (e != cudaSuccess) return e;
   gated_norm_bwd_kernel<T, kWarps><<<grid_for(tokens, kWarps), kWarps * 32, smem, s>>>(
       tokens, d, static_cast<const T *>(y), static_cast<const T *>(g), static_cast<const T *>(w), rstd, silu_on,
@@ -414,7 +414,7 @@ cudaError_t launch_bwd_reg(long tokens, const void *y, const void *g, const void
                            const void *dout, void *dy, void *dg, float *dw_part, cudaStream_t s) {
   // the warps' dw sums, then (bf16) the warps' two-slot rings of three rows each
   const size_t smem = (size_t)kRegWarps * 256 * CPL * sizeof(float) + (sizeof(T) == 2 ? (size_t)kRegWarps * 2 * 3 * 256 * CPL * sizeof(T) : 0);
-  cudaError_t e = cudaFuncSetAttribute(gated_norm_bwd_reg_kernel<T, CPL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(gated_norm_bwd_reg_kernel<T, CPL>, smem);
   if (e != cudaSuccess) return e;
   gated_norm_bwd_reg_kernel<T, CPL><<<reg_grid(tokens, CPL), kRegWarps * 32, smem, s>>>(
       tokens, static_cast<const T *>(y), static_cast<const T *>(g), static_cast<const T *>(w), rstd, silu_on,

@@ -67,6 +67,10 @@ struct BwdPlan {
   int C_max;  // largest supported checkpoint interval
 };
 int sm_count();   // SMs of the current device (148 when there is none to ask)
+cudaError_t allow_smem(const void *kernel, size_t bytes);   // dynamic shared memory a launch may use
+template <typename... A> cudaError_t allow_smem(void (*kernel)(A...), size_t bytes) {
+  return allow_smem(reinterpret_cast<const void *>(kernel), bytes);
+}
 BwdPlan plan_bwd(int B, int N, int K, int V, int io_dtype);
 int plan_fwd_rows(int B, int N, int K, int V, int io_dtype);   // state rows per CTA of the forward kernel
 // Which bf16 forward kernel takes a problem: the tcgen05 kernel (scan_fwd_tc.cu) or the mma.sync

@@ -861,7 +861,7 @@ __global__ void __launch_bounds__(bwd_threads<V, NWC>(), V == 16 ? (NWC == 2 ? 3
 template <int V, int NWC>
 cudaError_t launch_bwd_t(const ScanArgs &a, cudaStream_t s) {
   const BwdLayout L = bwd_layout<V>(16 * NWC, a.C, V > 64);
-  cudaError_t e = cudaFuncSetAttribute(bwd_bf16_kernel<V, NWC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total);
+  cudaError_t e = allow_smem(bwd_bf16_kernel<V, NWC>, L.total);
   if (e != cudaSuccess) return e;
   const int RS = a.K / (16 * NWC);
   bwd_bf16_kernel<V, NWC><<<a.B * a.N * RS, bwd_threads<V, NWC>(), L.total, s>>>(a);

@@ -579,7 +579,7 @@ int bwd_tc_chunk() { return kCTc; }
 cudaError_t launch_bwd_bf16_tc(const ScanArgs &a, cudaStream_t s) {
   if (a.V != kV || a.KC != kNR || a.C < 1 || a.C > kCTc) return cudaErrorInvalidValue;
   const size_t smem = TcBwdSmem::total;
-  cudaError_t e = cudaFuncSetAttribute(bwd_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(bwd_tc_kernel, smem);
   if (e != cudaSuccess) return e;
   bwd_tc_kernel<<<a.B * a.N * (a.K / kNR), kThreads, smem, s>>>(a);
   return cudaGetLastError();

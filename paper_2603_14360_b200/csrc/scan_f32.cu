@@ -341,7 +341,7 @@ cudaError_t launch_fwd_f32(const ScanArgs &a, cudaStream_t s) {
   const int TPR = pick_tpr(a.K, a.V), nthreads = a.K * TPR, nj4 = a.V / TPR / 4, HP = a.V + kPad;
   const size_t smem = sizeof(float) * ((size_t)a.V * HP + (size_t)a.K * HP + 2 * (nthreads / 32) * a.V);
   auto kern = nj4 == 1 ? fwd_f32_kernel<1> : nj4 == 2 ? fwd_f32_kernel<2> : fwd_f32_kernel<4>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(kern, smem);
   if (e != cudaSuccess) return e;
   kern<<<a.B * a.N, nthreads, smem, s>>>(a, TPR);
   return cudaGetLastError();
@@ -352,7 +352,7 @@ cudaError_t launch_bwd_f32(const ScanArgs &a, cudaStream_t s) {
   const int nwarps = nthreads / 32;
   const size_t smem = sizeof(float) * ((size_t)a.V * HP + 2 * (size_t)a.K * HP + (size_t)nwarps * a.V + nwarps);
   auto kern = nj4 == 1 ? bwd_f32_kernel<1> : nj4 == 2 ? bwd_f32_kernel<2> : bwd_f32_kernel<4>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(kern, smem);
   if (e != cudaSuccess) return e;
   kern<<<a.B * a.N, nthreads, smem, s>>>(a, TPR);
   return cudaGetLastError();

@@ -456,13 +456,13 @@ cudaError_t launch_vwco(const ScanArgs &a, cudaStream_t s) {
   const unsigned grid = a.B * a.N * (a.K / a.KCf), threads = (a.KCf / 16 + 1) * 32;
   if constexpr (V == 16 && MAXW == 4) {
     if (a.KCf == 64) {   // the paper's layer shape (K = 64, V = 16): slab count known at compile time
-      cudaError_t e = cudaFuncSetAttribute(fwd_bf16_kernel<V, MAXW, CKPT, OCC, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      cudaError_t e = allow_smem(fwd_bf16_kernel<V, MAXW, CKPT, OCC, 4>, smem);
       if (e != cudaSuccess) return e;
       fwd_bf16_kernel<V, MAXW, CKPT, OCC, 4><<<grid, threads, smem, s>>>(a);
       return cudaGetLastError();
     }
   }
-  cudaError_t e = cudaFuncSetAttribute(fwd_bf16_kernel<V, MAXW, CKPT, OCC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(fwd_bf16_kernel<V, MAXW, CKPT, OCC>, smem);
   if (e != cudaSuccess) return e;
   fwd_bf16_kernel<V, MAXW, CKPT, OCC><<<grid, threads, smem, s>>>(a);
   return cudaGetLastError();

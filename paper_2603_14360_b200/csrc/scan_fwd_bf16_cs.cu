@@ -460,7 +460,7 @@ __global__ void __launch_bounds__((SP * NW + cs_service_warps(SP * NW)) * 32, OC
 template <int V, int SP, int NW, bool CKPT, int OCC>
 cudaError_t launch_cs(const ScanArgs &a, cudaStream_t s) {
   const size_t smem = CsSmem<V>::bytes(16 * NW);
-  cudaError_t e = cudaFuncSetAttribute(fwd_bf16_cs_kernel<V, SP, NW, CKPT, OCC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(fwd_bf16_cs_kernel<V, SP, NW, CKPT, OCC>, smem);
   if (e != cudaSuccess) return e;
   fwd_bf16_cs_kernel<V, SP, NW, CKPT, OCC><<<a.B * a.N * (a.K / (16 * NW)), (SP * NW + cs_service_warps(SP * NW)) * 32, smem, s>>>(a);
   return cudaGetLastError();

@@ -347,7 +347,7 @@ template <int V, int NR, bool CKPT>
 cudaError_t launch_tc_fwd(const ScanArgs &a, cudaStream_t s) {
   constexpr int HS = 128 / V, kRowsCta = kGroups * NR;
   const size_t smem = TcFwdSmem<V, NR>::total;
-  cudaError_t e = cudaFuncSetAttribute(fwd_tc_kernel<V, NR, CKPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(fwd_tc_kernel<V, NR, CKPT>, smem);
   if (e != cudaSuccess) return e;
   const int NG = (a.N + HS - 1) / HS, RS = (a.K + kRowsCta - 1) / kRowsCta;
   fwd_tc_kernel<V, NR, CKPT><<<a.B * NG * RS, kThreadsTc, smem, s>>>(a);
