@@ -73,10 +73,10 @@ bool bwd_use_tc(int B, int N, int K, int V, int io_dtype) {
   return true;
 }
 
-BwdPlan plan_bwd(int B, int N, int K, int V, int io_dtype) {
+BwdPlan plan_bwd(int B, int N, int K, int V, int io_dtype, size_t tokens) {
   BwdPlan pl{};
-  if (io_dtype == M2RNN_F32) {  // recomputed states live in global scratch
-    pl.KC = K; pl.C = 16; pl.C_max = 64;
+  if (io_dtype == M2RNN_F32) {
+    pl.KC = bwd_f32_rows(B, N, K, V, tokens * N * V * sizeof(float)); pl.C = bwd_f32_piece(); pl.C_max = 64;
     return pl;
   }
   if (bwd_use_tc(B, N, K, V, io_dtype)) {   // 32-row CTAs, chunks of four steps
@@ -130,8 +130,8 @@ bool fwd_use_tc(int B, int N, int K, int V, int io_dtype) {
   return V == 128 && K % 64 == 0 && 4L * (B > 0 ? B : 1) * N * (K / 64) >= 3L * sm_count();
 }
 
-int plan_fwd_rows(int B, int N, int K, int V, int io_dtype) {
-  if (io_dtype == M2RNN_F32) return K;
+int plan_fwd_rows(int B, int N, int K, int V, int io_dtype, size_t tokens) {
+  if (io_dtype == M2RNN_F32) return fwd_f32_rows(B, N, K, V, tokens * N * V * sizeof(float));
   if (fwd_use_tc(B, N, K, V, io_dtype)) return fwd_tc_rows_per_cta(B, N, K, V);
   // The smallest slab (a multiple of 16 rows that divides K) that still gives every CTA an SM of
   // its own; with more units than SMs the whole state stays in one CTA.  V = 128 keeps the slab
@@ -202,7 +202,7 @@ Workspace layout(const m2rnn_params *p, bool have_ckpt) {
   size_t off = 0;
   w.ckpt = off;
   if (!have_ckpt) off += align_up(BN * nch * KV * sizeof(float));
-  const int RS = p->K / plan_bwd(p->B, p->N, p->K, p->V, p->io_dtype).KC;   // row slabs per state (1 on the fp32 path)
+  const int RS = p->K / plan_bwd(p->B, p->N, p->K, p->V, p->io_dtype, tokens_of(p)).KC;   // row slabs per state
   w.dW_part = off;
   off += align_up(BN * RS * p->V * p->V * sizeof(float));
   const size_t TT = tokens_of(p);
@@ -211,7 +211,7 @@ Workspace layout(const m2rnn_params *p, bool have_ckpt) {
   w.dk_part = off;
   if (p->Nk < p->N) off += align_up(TT * p->N * p->K * sizeof(float));
   w.chunk_states = off;
-  if (p->io_dtype == M2RNN_F32) off += align_up(BN * C * KV * sizeof(float));
+  if (p->io_dtype == M2RNN_F32 && C > bwd_f32_piece()) off += align_up(BN * ((C + bwd_f32_piece() - 1) / bwd_f32_piece()) * KV * sizeof(float));
   w.dv_part = off;
   if (RS > 1) off += align_up((size_t)RS * TT * p->N * p->V * sizeof(float));
   w.dgate_part = off;
@@ -224,8 +224,8 @@ ScanArgs base_args(const m2rnn_params *p) {
   ScanArgs a{};
   a.B = p->B; a.T = p->T; a.N = p->N; a.Nq = p->Nq; a.Nk = p->Nk; a.K = p->K; a.V = p->V;
   a.gate_kind = p->gate_kind;
-  a.KC = plan_bwd(p->B, p->N, p->K, p->V, p->io_dtype).KC;
-  a.KCf = plan_fwd_rows(p->B, p->N, p->K, p->V, p->io_dtype);
+  a.KC = plan_bwd(p->B, p->N, p->K, p->V, p->io_dtype, tokens_of(p)).KC;
+  a.KCf = plan_fwd_rows(p->B, p->N, p->K, p->V, p->io_dtype, tokens_of(p));
   a.C = interval_of(p);
   a.nchunks = p->T > 0 ? (p->T + a.C - 1) / a.C : 0;
   a.dh_clip = p->dh_clip;
@@ -269,7 +269,7 @@ int m2rnn_ckpt_interval(const m2rnn_params *params) {
 int m2rnn_bwd_row_slab(const m2rnn_params *params) {
   int rc = check_params(params, false);
   if (rc != M2RNN_OK) return rc;
-  return plan_bwd(params->B, params->N, params->K, params->V, params->io_dtype).KC;
+  return plan_bwd(params->B, params->N, params->K, params->V, params->io_dtype, params->T > 0 ? tokens_of(params) : 0).KC;
 }
 
 size_t m2rnn_ckpt_bytes(const m2rnn_params *params) {
@@ -280,7 +280,7 @@ size_t m2rnn_ckpt_bytes(const m2rnn_params *params) {
 
 size_t m2rnn_fwd_workspace_bytes(const m2rnn_params *params) {
   if (check_params(params, true) != M2RNN_OK) return 0;
-  const int kcf = plan_fwd_rows(params->B, params->N, params->K, params->V, params->io_dtype);
+  const int kcf = plan_fwd_rows(params->B, params->N, params->K, params->V, params->io_dtype, tokens_of(params));
   const int RS = (params->K + kcf - 1) / kcf;
   if (RS <= 1) return 0;
   return align_up((size_t)RS * tokens_of(params) * params->N * params->V * sizeof(float));
@@ -419,9 +419,8 @@ int m2rnn_decode_step(const m2rnn_params *params, const void *q, const void *k, 
   a.beta = params->gate_kind == M2RNN_GATE_PSI ? beta : nullptr;
   a.h0 = state; a.hT = state; a.y = y; a.ckpt = nullptr; a.dev_status = dev_status;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  // one step of Eq. 1-3: a T=1 scan whose initial and final state share storage (each CTA reads
-  // its own slice of the state completely before it writes it back)
-  cudaError_t e = params->io_dtype == M2RNN_F32 ? launch_fwd_f32(a, s) : launch_decode_bf16(a, s);
+  // one step of Eq. 1-3, the state read and written in place
+  cudaError_t e = params->io_dtype == M2RNN_F32 ? launch_decode_f32(a, s) : launch_decode_bf16(a, s);
   return e == cudaSuccess ? M2RNN_OK : cuda_failed();
 }
 

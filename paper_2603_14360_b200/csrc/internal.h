@@ -13,15 +13,15 @@ namespace m2rnn {
 struct ScanArgs {
   int B, T, N, Nq, Nk, K, V;
   int gate_kind;
-  int KC;         // bf16 backward: state rows per CTA (a divisor of K)
-  int KCf;        // bf16 forward: state rows per CTA (a divisor of K)
+  int KC;         // backward: state rows per CTA (a divisor of K)
+  int KCf;        // forward: state rows per CTA (a divisor of K)
   int C;          // checkpoint interval (steps)
   int nchunks;    // ceil(T / C)
   float dh_clip;
   const void *q, *k, *v, *W, *w_r;
   const float *gate, *h0, *alpha, *beta;
   void *y;
-  float *y_part;  // bf16 forward, K/KCf > 1: [K/KCf][B,T,N,V] fp32 per-row-slab y, else null
+  float *y_part;  // forward, K/KCf > 1: [K/KCf][B,T,N,V] fp32 per-row-slab y, else null
   float *hT;
   float *ckpt;    // fwd: written (may be null); bwd: read
   // backward only
@@ -34,7 +34,7 @@ struct ScanArgs {
   float *dgate_part;   // [K/KC][B,T,N] fp32 per-row-slab dgate when K/KC > 1, else null
   float *dq_part;      // [B,T,N,K] fp32 per-head dq when Nq < N, else null
   float *dk_part;      // [B,T,N,K] fp32 per-head dk when Nk < N, else null
-  float *chunk_states; // fp32 path: [B*N, C, K, V] scratch for the recomputed states
+  float *chunk_states; // fp32 path, C > 16: [B*N, ceil(C/16), K, V] states between the pieces of a chunk
   int32_t *dev_status;
   // token addressing: elements between consecutive tokens of q, k, v (dense: Nq K, Nk K, N V; larger
   // when they alias one fused projection output), the tokens in the batch (B T, or the packed total)
@@ -62,7 +62,7 @@ inline size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 // How the backward pass splits a problem: state rows per CTA and the checkpoint interval (bounded
 // by shared memory in the bf16 backward kernel, which keeps two chunks of recomputed states on chip).
 struct BwdPlan {
-  int KC;     // rows per CTA (== K on the fp32 path)
+  int KC;     // rows per CTA (fp32 path: 8, or K for one launch per group of eight)
   int C;      // default checkpoint interval
   int C_max;  // largest supported checkpoint interval
 };
@@ -71,8 +71,9 @@ cudaError_t allow_smem(const void *kernel, size_t bytes);   // dynamic shared me
 template <typename... A> cudaError_t allow_smem(void (*kernel)(A...), size_t bytes) {
   return allow_smem(reinterpret_cast<const void *>(kernel), bytes);
 }
-BwdPlan plan_bwd(int B, int N, int K, int V, int io_dtype);
-int plan_fwd_rows(int B, int N, int K, int V, int io_dtype);   // state rows per CTA of the forward kernel
+// (tokens: of the batch; they only decide where an fp32 problem is too large for per-slab shares)
+BwdPlan plan_bwd(int B, int N, int K, int V, int io_dtype, size_t tokens = 0);
+int plan_fwd_rows(int B, int N, int K, int V, int io_dtype, size_t tokens = 0);   // state rows per CTA of the forward kernel
 // Which bf16 forward kernel takes a problem: the tcgen05 kernel (scan_fwd_tc.cu) or the mma.sync
 // kernels (scan_fwd_bf16*.cu).  The environment variable M2RNN_FWD_VARIANT = tc | mma | wide
 // overrides the choice (benchmarking only).
@@ -83,7 +84,11 @@ size_t bwd_bf16_smem_bytes(int KC, int V, int C);  // scan_bwd_bf16.cu
 
 // fp32 FMA path (scan_f32.cu)
 cudaError_t launch_fwd_f32(const ScanArgs &a, cudaStream_t s);
-cudaError_t launch_bwd_f32(const ScanArgs &a, cudaStream_t s);
+cudaError_t launch_bwd_f32(const ScanArgs &a, cudaStream_t s);      // KC = 8: every group of eight rows at once, KC = K: one after the other
+cudaError_t launch_decode_f32(const ScanArgs &a, cudaStream_t s);
+int fwd_f32_rows(int B, int N, int K, int V, size_t share_bytes);
+int bwd_f32_rows(int B, int N, int K, int V, size_t share_bytes);
+int bwd_f32_piece();   // steps whose states the backward kernel keeps on chip
 
 // bf16 tensor-core path
 cudaError_t launch_fwd_bf16(const ScanArgs &a, cudaStream_t s);     // scan_fwd_bf16.cu: picks a variant

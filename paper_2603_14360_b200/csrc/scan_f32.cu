@@ -1,361 +1,665 @@
-// fp32 FMA path of the M2RNN scan (forward, decode step, backward through time).
+// fp32 FMA path of the M2RNN scan (forward, decoding step, backward through time): the accuracy path
+// (<= 1e-4).  Everything is fp32 FMA with tanhf / expf.
 //
-// One CTA per (b,n).  The K x V state is spread over K*TPR threads: thread (i,c) owns row i
-// and the columns {(jj*TPR + c)*4 + e}; a row's TPR threads sit in one warp, so the
-// row-by-W product (Eq. 1) only needs warp-level synchronisation through shared memory.
-// Everything is plain fp32 FMA with tanhf/expf: this is the accuracy path (<= 1e-4).
+// The rows of a state are independent recurrences, so the unit of work is a group of eight rows, and
+// the product of a step, [8 x V] times the V x V transition matrix, is laid out to keep the matrix in
+// registers: lane (p, cg) of warp w holds the V/8 rows l of W that belong to part p for the two columns
+// 8w + 2cg, +1.  Per state row it reads its V/8 entries of the row from shared memory (the four lanes of
+// a part share them: one wavefront for a warp), multiplies, and leaves a partial sum per row and column;
+// three rounds of recursive halving over p then leave every lane with the finished sums of ONE row, p,
+// for its two columns -- the elements it owns for the element-wise part of the step.  One CTA barrier a
+// step makes the new rows visible.  Sums over l pair even and odd entries (packed fp32x2 FMA).
+// (Until then a CTA held a whole state and read W from shared memory for every product: 1 MB of
+// shared-memory traffic a step and a sixteenth of the SMs at 16 units.  K = V = 64, 16 units, T = 512:
+// forward 3.19 -> 0.39 ms, backward 18.6 -> 0.72 ms.)
 #include "device_common.cuh"
 #include "internal.h"
 
 namespace m2rnn {
 namespace {
 
-constexpr int kPad = 4;  // row pitch V+4 floats: rows land on different banks
+constexpr int kRows = 8;      // rows of a group
+constexpr int kSteps = 16;    // steps staged at a time, and steps of state the backward kernel keeps on chip
 
-__device__ __forceinline__ int col_of(int jj, int c, int TPR) { return (jj * TPR + c) * 4; }
+template <int V>
+struct Geom {
+  static constexpr int NW = V / 8;             // warps of a CTA
+  static constexpr int kThreads = 32 * NW;
+  static constexpr int HP = V + 8;             // row pitch: the eight rows of a group start 32 bytes apart
+                                               // in the banks, so their 32-byte pieces are conflict-free
+  static constexpr int NP = V / 16;            // pairs of l per thread
+  static constexpr int kTile = kRows * HP;     // floats of a group of rows
+};
 
-// Z row-segment = tanh( sum_l H[i][l] W[l][cols] + k_i v[cols] )   (Eq. 1)
-template <int NJ4>
-__device__ __forceinline__ void transition(const float *__restrict__ Hrow, const float *__restrict__ Ws,
-                                           int V, int HP, int c, int TPR, float k_i,
-                                           const float4 (&v4)[NJ4], float (&z)[NJ4 * 4]) {
-  float acc[NJ4 * 4];
+// first l of pair i of part p: parts interleave in 16-byte (V = 16: 8-byte) pieces
+template <int V>
+__device__ __forceinline__ int pair_l(int i, int p) {
+  return V == 16 ? 2 * p : 32 * (i >> 1) + 4 * p + 2 * (i & 1);
+}
+
+// this thread's part of W for the product rows x W: columns c0, c0 + 1
+template <int V>
+__device__ __forceinline__ void load_w(const float *__restrict__ W, int p, int c0, float2 (&w)[Geom<V>::NP][2]) {
 #pragma unroll
-  for (int jj = 0; jj < NJ4; ++jj) {
-    acc[jj * 4 + 0] = k_i * v4[jj].x;
-    acc[jj * 4 + 1] = k_i * v4[jj].y;
-    acc[jj * 4 + 2] = k_i * v4[jj].z;
-    acc[jj * 4 + 3] = k_i * v4[jj].w;
+  for (int i = 0; i < Geom<V>::NP; ++i) {
+    const int l = pair_l<V>(i, p);
+    const float2 a = *reinterpret_cast<const float2 *>(W + (size_t)l * V + c0), b = *reinterpret_cast<const float2 *>(W + (size_t)(l + 1) * V + c0);
+    w[i][0] = make_float2(a.x, b.x);
+    w[i][1] = make_float2(a.y, b.y);
   }
-  for (int l = 0; l < V; l += 4) {
-    const float4 h4 = *reinterpret_cast<const float4 *>(Hrow + l);
-    const float hv[4] = {h4.x, h4.y, h4.z, h4.w};
+}
+// ... for rows x W^T
+template <int V>
+__device__ __forceinline__ void load_wt(const float *__restrict__ W, int p, int c0, float2 (&w)[Geom<V>::NP][2]) {
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
+  for (int i = 0; i < Geom<V>::NP; ++i) {
+    const int j = pair_l<V>(i, p);
+    w[i][0] = *reinterpret_cast<const float2 *>(W + (size_t)c0 * V + j);
+    w[i][1] = *reinterpret_cast<const float2 *>(W + (size_t)(c0 + 1) * V + j);
+  }
+}
+
+// rows (8 of pitch HP, shared memory) times the matrix held in w -> row p, columns c0, c0 + 1
+template <int V>
+__device__ __forceinline__ float2 product(const float *rows, const float2 (&w)[Geom<V>::NP][2], int p, int lane) {
+  using G = Geom<V>;
+  float s[kRows][2];
 #pragma unroll
-      for (int jj = 0; jj < NJ4; ++jj) {
-        const float4 w4 = *reinterpret_cast<const float4 *>(Ws + (l + u) * HP + col_of(jj, c, TPR));
-        acc[jj * 4 + 0] = fmaf(hv[u], w4.x, acc[jj * 4 + 0]);
-        acc[jj * 4 + 1] = fmaf(hv[u], w4.y, acc[jj * 4 + 1]);
-        acc[jj * 4 + 2] = fmaf(hv[u], w4.z, acc[jj * 4 + 2]);
-        acc[jj * 4 + 3] = fmaf(hv[u], w4.w, acc[jj * 4 + 3]);
+  for (int r = 0; r < kRows; ++r) {
+    float2 a0 = make_float2(0.f, 0.f), a1 = a0;
+    const float *row = rows + r * G::HP;
+    if constexpr (V == 16) {
+      const float2 h = *reinterpret_cast<const float2 *>(row + 2 * p);
+      a0 = __fmul2_rn(h, w[0][0]);
+      a1 = __fmul2_rn(h, w[0][1]);
+    } else {
+#pragma unroll
+      for (int i = 0; i < V / 32; ++i) {
+        const float4 h = *reinterpret_cast<const float4 *>(row + 32 * i + 4 * p);
+        a0 = __ffma2_rn(make_float2(h.x, h.y), w[2 * i][0], a0);
+        a1 = __ffma2_rn(make_float2(h.x, h.y), w[2 * i][1], a1);
+        a0 = __ffma2_rn(make_float2(h.z, h.w), w[2 * i + 1][0], a0);
+        a1 = __ffma2_rn(make_float2(h.z, h.w), w[2 * i + 1][1], a1);
       }
     }
+    s[r][0] = a0.x + a0.y;
+    s[r][1] = a1.x + a1.y;
   }
+  // recursive halving over the parts (lane bits 4, 3, 2): part p ends with row p
 #pragma unroll
-  for (int x = 0; x < NJ4 * 4; ++x) z[x] = tanhf(acc[x]);
+  for (int m = 4; m >= 1; m >>= 1) {
+    const bool up = lane & (4 * m);
+#pragma unroll
+    for (int r = 0; r < m; ++r)
+#pragma unroll
+      for (int x = 0; x < 2; ++x) {
+        const float send = up ? s[r][x] : s[r + m][x], keep = up ? s[r + m][x] : s[r][x];
+        s[r][x] = keep + __shfl_xor_sync(0xffffffffu, send, 4 * m);
+      }
+  }
+  return make_float2(s[0][0], s[0][1]);
 }
 
-template <int NJ4>
-__device__ __forceinline__ void load_cols(const float *__restrict__ base, int c, int TPR, float4 (&out)[NJ4]) {
-#pragma unroll
-  for (int jj = 0; jj < NJ4; ++jj) out[jj] = *reinterpret_cast<const float4 *>(base + col_of(jj, c, TPR));
+__device__ __forceinline__ void cp16(float *dst, const float *src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp4(float *dst, const float *src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// [len][width] floats (width a multiple of 4) from rows `stride` apart, into dense rows, by the CTA
+__device__ __forceinline__ void stage_rows(float *dst, const float *src, long long stride, int len, int width, int tid, int nthreads) {
+  const int w4 = width >> 2;
+  for (int x = tid; x < len * w4; x += nthreads) {
+    const int t = x / w4, j = (x - t * w4) * 4;
+    cp16(dst + t * width + j, src + t * stride + j);
+  }
 }
 
-template <int NJ4>
-__device__ __forceinline__ void store_cols(float *__restrict__ base, int c, int TPR, const float (&h)[NJ4 * 4]) {
-#pragma unroll
-  for (int jj = 0; jj < NJ4; ++jj)
-    *reinterpret_cast<float4 *>(base + col_of(jj, c, TPR)) =
-        make_float4(h[jj * 4], h[jj * 4 + 1], h[jj * 4 + 2], h[jj * 4 + 3]);
+// sum over the eight rows p of q_p h_p for the thread's two columns: lanes p < 4 end with column c0,
+// lanes p >= 4 with column c0 + 1
+__device__ __forceinline__ float readout(float q, float2 h, int lane) {
+  const bool up = lane & 16;
+  const float2 v = make_float2(__fmul_rn(q, h.x), __fmul_rn(q, h.y));
+  float t = (up ? v.y : v.x) + __shfl_xor_sync(0xffffffffu, up ? v.x : v.y, 16);
+  t += __shfl_xor_sync(0xffffffffu, t, 8);
+  return t + __shfl_xor_sync(0xffffffffu, t, 4);
+}
+
+// Eq. 1 and 2 for the thread's two elements of a row (roundings spelled out: a decoding step repeats a
+// step of the scan bit for bit)
+__device__ __forceinline__ float2 update(float2 o, float k, float2 v, float f, float2 h, float2 &z) {
+  z = make_float2(tanhf(fmaf(k, v.x, o.x)), tanhf(fmaf(k, v.y, o.y)));
+  return make_float2(fmaf(1.f - f, z.x, __fmul_rn(f, h.x)), fmaf(1.f - f, z.y, __fmul_rn(f, h.y)));
 }
 
 // ------------------------------------------------------------------ forward (Algorithm 1)
-template <int NJ4>
-__global__ void __launch_bounds__(1024) fwd_f32_kernel(ScanArgs a, int TPR) {
+// One CTA per (b, n, slab of R = 8 ng rows); the groups of a slab take turns inside a step.
+template <int V>
+__host__ __device__ constexpr int fwd_stage_floats(int R) { return kSteps * (2 * R + V + 1); }
+template <int V>
+__host__ size_t fwd_f32_smem(int R) { return sizeof(float) * (2 * (size_t)R * Geom<V>::HP + 2 * (size_t)fwd_stage_floats<V>(R) + 2 * kSteps); }
+
+template <int V>
+__global__ void __launch_bounds__(Geom<V>::kThreads) fwd_f32_kernel(ScanArgs a) {
+  using G = Geom<V>;
   extern __shared__ __align__(16) float smem[];
-  const int K = a.K, V = a.V, N = a.N, HP = V + kPad;
-  const int tid = threadIdx.x, nthreads = blockDim.x, lane = tid & 31, warp = tid >> 5;
-  const int nwarps = nthreads >> 5;
-  const int i = tid / TPR, c = tid % TPR;
-  const int bn = blockIdx.x, b = bn / N, n = bn % N;
+  const int K = a.K, N = a.N, R = a.KCf, RS = K / R, ng = R / kRows;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, p = lane >> 2, c0 = 8 * warp + 2 * (lane & 3);
+  const int bn = blockIdx.x / RS, rs = blockIdx.x % RS, b = bn / N, n = bn % N, rbase = rs * R;
   const UnitSpan span = unit_span(a, b);   // this batch entry's tokens (a slice of a packed batch, or b T ..)
   const int T = span.T;
-  const size_t tok0 = span.tok0;
+  const size_t tok0 = span.tok0, KV = (size_t)K * V;
   const int hq = n / (N / a.Nq), hk = n / (N / a.Nk);
 
-  float *Ws = smem;                    // [V][HP]
-  float *Hs = Ws + V * HP;             // [K][HP]
-  float *ypart = Hs + K * HP;          // [2][nwarps][V]
+  float *H0 = smem, *H1 = H0 + R * G::HP;                    // the state before and after a step
+  float *stages = H1 + R * G::HP;                             // two stages: q, k [16][R], v [16][V], gate [16]
+  float *fS = stages + 2 * fwd_stage_floats<V>(R);            // [2][16] evaluated gates
 
-  const float *Wg = static_cast<const float *>(a.W) + (size_t)n * V * V;
-  for (int x = tid; x < V * V; x += nthreads) Ws[(x / V) * HP + (x % V)] = Wg[x];
-
-  const size_t KV = (size_t)K * V;
-  float h[NJ4 * 4];
-  if (a.h0) {
-    float4 t4[NJ4];
-    load_cols<NJ4>(a.h0 + bn * KV + (size_t)i * V, c, TPR, t4);
-#pragma unroll
-    for (int jj = 0; jj < NJ4; ++jj) { h[jj * 4] = t4[jj].x; h[jj * 4 + 1] = t4[jj].y; h[jj * 4 + 2] = t4[jj].z; h[jj * 4 + 3] = t4[jj].w; }
-  } else {
-#pragma unroll
-    for (int x = 0; x < NJ4 * 4; ++x) h[x] = 0.f;
+  float2 w[G::NP][2];
+  load_w<V>(static_cast<const float *>(a.W) + (size_t)n * V * V, p, c0, w);
+  for (int g = 0; g < ng; ++g) {
+    const int row = kRows * g + p;
+    *reinterpret_cast<float2 *>(H0 + row * G::HP + c0) =
+        a.h0 ? *reinterpret_cast<const float2 *>(a.h0 + bn * KV + (size_t)(rbase + row) * V + c0) : make_float2(0.f, 0.f);
   }
   const float al = a.alpha ? a.alpha[n] : 1.f, be = a.beta ? a.beta[n] : 0.f;
   const float *qg = static_cast<const float *>(a.q), *kg = static_cast<const float *>(a.k);
   const float *vg = static_cast<const float *>(a.v), *wr = static_cast<const float *>(a.w_r);
-  float *yg = static_cast<float *>(a.y);
+  const bool want_y = a.y != nullptr;
+  float *yg = a.y_part ? a.y_part + (size_t)rs * a.TT * N * V : static_cast<float *>(a.y);
+  const float2 wr2 = wr && rs == 0 ? *reinterpret_cast<const float2 *>(wr + (size_t)n * V + c0) : make_float2(0.f, 0.f);
+  const float wre = lane & 16 ? wr2.y : wr2.x;
+
+  auto stage = [&](int x) { return stages + (x & 1) * fwd_stage_floats<V>(R); };
+  auto fetch = [&](int ch) {
+    float *st = stage(ch);
+    const int t0 = ch * kSteps, len = min(kSteps, T - t0);
+    const size_t bt = tok0 + t0;
+    if (want_y) stage_rows(st, qg + bt * a.qs + hq * K + rbase, a.qs, len, R, tid, G::kThreads);
+    stage_rows(st + kSteps * R, kg + bt * a.ks + hk * K + rbase, a.ks, len, R, tid, G::kThreads);
+    stage_rows(st + 2 * kSteps * R, vg + bt * a.vs + n * V, a.vs, len, V, tid, G::kThreads);
+    if (tid < len) cp4(st + kSteps * (2 * R + V) + tid, a.gate + (bt + tid) * N + n);
+    cp_commit();
+  };
+  auto gates = [&](int ch) {   // the thread that copied a gate evaluates it
+    if (tid < min(kSteps, T - ch * kSteps)) fS[(ch & 1) * kSteps + tid] = gate_value(a.gate_kind, stage(ch)[kSteps * (2 * R + V) + tid], al, be, nullptr);
+  };
+  const int nst = (T + kSteps - 1) / kSteps;
+  if (nst > 0) {
+    fetch(0);
+    cp_wait<0>();
+    gates(0);
+  }
   __syncthreads();
-
-  for (int t = 0; t < T; ++t) {
-    const size_t bt = tok0 + t;
-    if (a.ckpt && (t % a.C) == 0)
-      store_cols<NJ4>(a.ckpt + ((size_t)bn * a.nchunks + t / a.C) * KV + (size_t)i * V, c, TPR, h);
-    const float k_i = kg[bt * a.ks + hk * K + i];
-    const float q_i = qg[bt * a.qs + hq * K + i];
-    const float f = gate_value(a.gate_kind, a.gate[bt * N + n], al, be, nullptr);
-    float4 v4[NJ4];
-    load_cols<NJ4>(vg + bt * a.vs + n * V, c, TPR, v4);
-
-    store_cols<NJ4>(Hs + i * HP, c, TPR, h);
-    __syncwarp();
-    float z[NJ4 * 4];
-    transition<NJ4>(Hs + i * HP, Ws, V, HP, c, TPR, k_i, v4, z);
-    __syncwarp();
-#pragma unroll
-    for (int x = 0; x < NJ4 * 4; ++x) h[x] = f * h[x] + (1.f - f) * z[x];  // Eq. 2
-    if (!yg) continue;  // checkpoint-only pass (first pass of the backward call)
-    // readout partial q_i * H_t[i][cols] summed over the warp's rows (Eq. 3)
-    float *yp = ypart + ((t & 1) * nwarps + warp) * V;
-#pragma unroll
-    for (int x = 0; x < NJ4 * 4; ++x) {
-      float yv = q_i * h[x];
-      for (int off = TPR; off < 32; off <<= 1) yv += __shfl_xor_sync(0xffffffffu, yv, off);
-      if (lane < TPR) yp[col_of(x >> 2, c, TPR) + (x & 3)] = yv;
+  int ck_left = 0, ck_idx = 0;
+  for (int ch = 0; ch < nst; ++ch) {
+    if (ch + 1 < nst) fetch(ch + 1);
+    const float *qS = stage(ch), *kS = qS + kSteps * R, *vS = kS + kSteps * R, *fs = fS + (ch & 1) * kSteps;
+    const int len = min(kSteps, T - ch * kSteps);
+    for (int s = 0; s < len; ++s) {
+      if (a.ckpt) {
+        if (ck_left == 0) {
+          float *dst = a.ckpt + ((size_t)bn * a.nchunks + ck_idx) * KV + (size_t)rbase * V;
+          for (int g = 0; g < ng; ++g)
+            *reinterpret_cast<float2 *>(dst + (size_t)(kRows * g + p) * V + c0) = *reinterpret_cast<const float2 *>(H0 + (kRows * g + p) * G::HP + c0);
+          ++ck_idx;
+          ck_left = a.C;
+        }
+        --ck_left;
+      }
+      const float f = fs[s];
+      const float2 v2 = *reinterpret_cast<const float2 *>(vS + s * V + c0);
+      float y = 0.f;     // Eq. 3, group by group (the order in which the shares of single groups are added too)
+      for (int g = 0; g < ng; ++g) {
+        const float2 o = product<V>(H0 + g * G::kTile, w, p, lane);
+        const int row = kRows * g + p;
+        float2 z;
+        const float2 h = update(o, kS[s * R + row], v2, f, *reinterpret_cast<const float2 *>(H0 + row * G::HP + c0), z);
+        *reinterpret_cast<float2 *>(H1 + row * G::HP + c0) = h;
+        if (want_y) {
+          const float share = readout(qS[s * R + row], h, lane);
+          y = g == 0 ? fmaf(wre, lane & 16 ? v2.y : v2.x, share) : y + share;
+        }
+      }
+      __syncthreads();   // H_t is complete, H_{t-1} is free
+      if (want_y && (p & 3) == 0) yg[((tok0 + ch * kSteps + s) * N + n) * V + c0 + (p >> 2)] = y;
+      float *t = H0; H0 = H1; H1 = t;
     }
-    __syncthreads();
-    if (tid < V) {
-      float s = 0.f;
-      for (int w = 0; w < nwarps; ++w) s += ypart[((t & 1) * nwarps + w) * V + tid];
-      if (wr) s += wr[(size_t)n * V + tid] * vg[bt * a.vs + n * V + tid];
-      yg[(bt * N + n) * V + tid] = s;
+    if (ch + 1 < nst) {
+      cp_wait<0>();
+      gates(ch + 1);
+      __syncthreads();
     }
   }
-  if (a.hT) store_cols<NJ4>(a.hT + bn * KV + (size_t)i * V, c, TPR, h);
+  if (a.hT)
+    for (int g = 0; g < ng; ++g)
+      *reinterpret_cast<float2 *>(a.hT + bn * KV + (size_t)(rbase + kRows * g + p) * V + c0) = *reinterpret_cast<const float2 *>(H0 + (kRows * g + p) * G::HP + c0);
 }
 
 // ------------------------------------------------------------------ backward (Algorithm 2)
-template <int NJ4>
-__global__ void __launch_bounds__(1024) bwd_f32_kernel(ScanArgs a, int TPR) {
+// One CTA per (b, n, group of eight rows).  Time goes backwards in pieces of up to 16 steps; of a piece
+// the CTA (A) redoes the forward steps, keeping H_{t-1} and Z_t of every step in shared memory,
+// (B) walks them backwards -- G = C + q dy^T, dX, C <- f G + dX W^T, dX in Z's place --, and (C) takes
+// everything that is a sum over steps or rows from those two arrays at once: dW += H_{t-1}^T dX as a
+// register-tiled product over the piece's 8 x 16 rows, dq, dk, dv, dgate.  Only (A) and (B) are serial,
+// with one barrier a step.  A checkpoint interval above 16 first walks the chunk forward once and
+// leaves the states between pieces in the scratch tensor.
+// slab0 / nslab: the groups of rows this launch takes.  All of them (nslab = K/8), each leaving its
+// shares of dv, dgate and dW as partials; or one after the other (nslab = 1), the later ones
+// adding to what the earlier ones wrote.
+template <int V>
+struct BwdGeom {
+  using G = Geom<V>;
+  static constexpr int kStage = kSteps * (2 * kRows + 2 * V + 1);     // q, k [16][8], v, dy [16][V], gate [16]
+  // dW tiles: 4 x JT elements per thread; with fewer tiles than threads, SP threads share a tile and
+  // take every SP-th step
+  static constexpr int JT = V == 128 ? 8 : 4;
+  static constexpr int kTiles = (V / 4) * (V / JT), SP = G::kThreads / kTiles;
+  static constexpr int kFloats = (2 * kSteps + 1) * G::kTile + 2 * kStage + 4 * kSteps + kSteps * G::kThreads;
+  // W and W^T both stay in registers where they fit beside the dW tile; at V = 128 (32 + 32 + 32 of 128
+  // registers) each phase reloads its own from L2 once per piece
+  static constexpr bool kReload = V == 128;
+};
+
+template <int V>
+__global__ void __launch_bounds__(Geom<V>::kThreads) bwd_f32_kernel(ScanArgs a, int slab0, int nslab) {
+  using G = Geom<V>;
+  using BG = BwdGeom<V>;
   extern __shared__ __align__(16) float smem[];
-  const int K = a.K, V = a.V, N = a.N, HP = V + kPad;
-  const int tid = threadIdx.x, nthreads = blockDim.x, lane = tid & 31, warp = tid >> 5;
-  const int nwarps = nthreads >> 5;
-  const int i = tid / TPR, c = tid % TPR;
-  const int bn = blockIdx.x, b = bn / N, n = bn % N;
-  const UnitSpan span = unit_span(a, b);   // this batch entry's tokens (a slice of a packed batch, or b T ..)
+  const int K = a.K, N = a.N;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, p = lane >> 2, c0 = 8 * warp + 2 * (lane & 3);
+  const int bn = blockIdx.x / nslab, rs = slab0 + blockIdx.x % nslab, b = bn / N, n = bn % N, rbase = rs * kRows;
+  const bool add = nslab == 1 && rs > 0;   // earlier launches have written dv, dgate and dW
+  const UnitSpan span = unit_span(a, b);
   const int T = span.T;
-  const size_t tok0 = span.tok0;
+  const size_t tok0 = span.tok0, KV = (size_t)K * V;
   const int hq = n / (N / a.Nq), hk = n / (N / a.Nk);
 
-  float *Ws = smem;                 // [V][HP]
-  float *Hs = Ws + V * HP;          // [K][HP]  H_{t-1}
-  float *Xs = Hs + K * HP;          // [K][HP]  dX_t
-  float *dvpart = Xs + K * HP;      // [nwarps][V]
-  float *red = dvpart + nwarps * V; // [nwarps]
+  float *Hc = smem;                               // [17][8][HP]: H before step s of the piece; [len] the last H_t
+  float *Xc = Hc + (kSteps + 1) * G::kTile;       // [16][8][HP]: Z_t, then dX_t
+  float *stages = Xc + kSteps * G::kTile;
+  float *fS = stages + 2 * BG::kStage, *dfS = fS + 2 * kSteps;   // [2][16] gates and their slopes
+  float *dfp = dfS + 2 * kSteps;                  // [16][threads] shares of df
 
-  const float *Wg = static_cast<const float *>(a.W) + (size_t)n * V * V;
-  for (int x = tid; x < V * V; x += nthreads) Ws[(x / V) * HP + (x % V)] = Wg[x];
-
-  const size_t KV = (size_t)K * V;
+  const float *Wn = static_cast<const float *>(a.W) + (size_t)n * V * V;
+  float2 w[G::NP][2], wt[BG::kReload ? 1 : G::NP][2];
+  if constexpr (!BG::kReload) {
+    load_w<V>(Wn, p, c0, w);
+    load_wt<V>(Wn, p, c0, wt);
+  }
   const float al = a.alpha ? a.alpha[n] : 1.f, be = a.beta ? a.beta[n] : 0.f;
   const float *qg = static_cast<const float *>(a.q), *kg = static_cast<const float *>(a.k);
   const float *vg = static_cast<const float *>(a.v), *wr = static_cast<const float *>(a.w_r);
   const float *dyg = static_cast<const float *>(a.dy);
-  float *scratch = a.chunk_states + (size_t)bn * a.C * KV;
+  const int own = p * G::HP + c0;                 // this thread's two elements inside a group of rows
+  const size_t own_g = (size_t)(rbase + p) * V + c0;   // ... inside a state in memory
 
-  float Cg[NJ4 * 4];  // carried dL/dH_t, this thread's segment
-  if (a.d_hT) {
-    float4 t4[NJ4];
-    load_cols<NJ4>(a.d_hT + bn * KV + (size_t)i * V, c, TPR, t4);
-#pragma unroll
-    for (int jj = 0; jj < NJ4; ++jj) { Cg[jj * 4] = t4[jj].x; Cg[jj * 4 + 1] = t4[jj].y; Cg[jj * 4 + 2] = t4[jj].z; Cg[jj * 4 + 3] = t4[jj].w; }
-  } else {
-#pragma unroll
-    for (int x = 0; x < NJ4 * 4; ++x) Cg[x] = 0.f;
-  }
-  // dW[l][j4..j4+3] accumulators: float4 slot d = l*(V/4) + j4/4, strided over the CTA
-  constexpr int kMaxDW = 8;
-  float4 dWacc[kMaxDW];
-#pragma unroll
-  for (int x = 0; x < kMaxDW; ++x) dWacc[x] = make_float4(0.f, 0.f, 0.f, 0.f);
-  const int ndw = V * V / 4;
-  __syncthreads();
+  // pieces: chunk ch (the checkpoint interval) holds ceil(len / 16) of them
+  const int ppc = (a.C + kSteps - 1) / kSteps, nch = (T + a.C - 1) / a.C;
+  struct Piece { int t0, len; };
+  auto piece = [&](int ch, int i) {
+    const int t0 = ch * a.C + i * kSteps;
+    return Piece{t0, max(0, min(min(kSteps, a.C - i * kSteps), T - t0))};
+  };
+  auto stage = [&](int x) { return stages + (x & 1) * BG::kStage; };
+  constexpr int oK = kSteps * kRows, oV = 2 * oK, oDY = oV + kSteps * V, oG = oDY + kSteps * V;
+  auto fetch = [&](int x, Piece pc) {
+    float *st = stage(x);
+    const size_t bt = tok0 + pc.t0;
+    stage_rows(st, qg + bt * a.qs + hq * K + rbase, a.qs, pc.len, kRows, tid, G::kThreads);
+    stage_rows(st + oK, kg + bt * a.ks + hk * K + rbase, a.ks, pc.len, kRows, tid, G::kThreads);
+    stage_rows(st + oV, vg + bt * a.vs + n * V, a.vs, pc.len, V, tid, G::kThreads);
+    stage_rows(st + oDY, dyg + (bt * N + n) * V, (long long)N * V, pc.len, V, tid, G::kThreads);
+    if (tid < pc.len) cp4(st + oG + tid, a.gate + (bt + tid) * N + n);
+    cp_commit();
+  };
+  auto gates = [&](int x, Piece pc) {
+    if (tid < pc.len) fS[(x & 1) * kSteps + tid] = gate_value(a.gate_kind, stage(x)[oG + tid], al, be, &dfS[(x & 1) * kSteps + tid]);
+  };
+  float *scratch = a.chunk_states + (size_t)bn * ppc * KV;   // states at the start of a chunk's pieces
 
-  for (int ch = (T + a.C - 1) / a.C - 1; ch >= 0; --ch) {   // this unit's chunks; a.nchunks is the checkpoint tensor's extent
-    const int t0 = ch * a.C, len = min(a.C, T - t0);
-    // pass 1 for this chunk: states H_{t0} .. H_{t0+len-1}, each the H_{t-1} of one step
-    float h[NJ4 * 4];
-    {
-      float4 t4[NJ4];
-      load_cols<NJ4>(a.ckpt + ((size_t)bn * a.nchunks + ch) * KV + (size_t)i * V, c, TPR, t4);
+  float2 C = a.d_hT ? *reinterpret_cast<const float2 *>(a.d_hT + (size_t)bn * KV + own_g) : make_float2(0.f, 0.f);   // carried dL/dH_t
+  float2 dW[4][BG::JT / 2];
 #pragma unroll
-      for (int jj = 0; jj < NJ4; ++jj) { h[jj * 4] = t4[jj].x; h[jj * 4 + 1] = t4[jj].y; h[jj * 4 + 2] = t4[jj].z; h[jj * 4 + 3] = t4[jj].w; }
-    }
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < BG::JT / 2; ++j) dW[i][j] = make_float2(0.f, 0.f);
+  // (a warp's tiles are four by eight, so that its loads of H and dX are one wavefront each)
+  constexpr int WJ = V >= 64 ? 2 : 1;
+  const int tile = tid % BG::kTiles, tsp = tid / BG::kTiles, tw = tile >> 5;
+  const int tl = 4 * (V == 16 ? (tile >> 2) : 4 * (tw / WJ) + (lane >> 3)), tj = 4 * (V == 16 ? (tile & 3) : 8 * (tw % WJ) + (lane & 7));
+
+  // forward steps of a piece from the state in Hc[0]
+  auto forward = [&](int x, int len) {
+    const float *st = stage(x), *fs = fS + (x & 1) * kSteps;
     for (int s = 0; s < len; ++s) {
-      store_cols<NJ4>(scratch + (size_t)s * KV + (size_t)i * V, c, TPR, h);
-      if (s == len - 1) break;
-      const size_t bt = tok0 + t0 + s;
-      const float k_i = kg[bt * a.ks + hk * K + i];
-      const float f = gate_value(a.gate_kind, a.gate[bt * N + n], al, be, nullptr);
-      float4 v4[NJ4];
-      load_cols<NJ4>(vg + bt * a.vs + n * V, c, TPR, v4);
-      store_cols<NJ4>(Hs + i * HP, c, TPR, h);
-      __syncwarp();
-      float z[NJ4 * 4];
-      transition<NJ4>(Hs + i * HP, Ws, V, HP, c, TPR, k_i, v4, z);
-      __syncwarp();
-#pragma unroll
-      for (int x = 0; x < NJ4 * 4; ++x) h[x] = f * h[x] + (1.f - f) * z[x];
+      float *hs = Hc + s * G::kTile;
+      const float2 o = product<V>(hs, w, p, lane);
+      float2 z;
+      const float2 h = update(o, st[oK + s * kRows + p], *reinterpret_cast<const float2 *>(st + oV + s * V + c0), fs[s], *reinterpret_cast<const float2 *>(hs + own), z);
+      *reinterpret_cast<float2 *>(hs + G::kTile + own) = h;
+      *reinterpret_cast<float2 *>(Xc + s * G::kTile + own) = z;
+      __syncthreads();
     }
-    __syncthreads();
-    // pass 2: reverse sweep over the chunk
-    for (int s = len - 1; s >= 0; --s) {
-      const size_t bt = tok0 + t0 + s;
-      const float k_i = kg[bt * a.ks + hk * K + i];
-      const float q_i = qg[bt * a.qs + hq * K + i];
-      float dfdx;
-      const float f = gate_value(a.gate_kind, a.gate[bt * N + n], al, be, &dfdx);
-      float4 v4[NJ4], dy4[NJ4], hp4[NJ4];
-      load_cols<NJ4>(vg + bt * a.vs + n * V, c, TPR, v4);
-      load_cols<NJ4>(dyg + (bt * N + n) * V, c, TPR, dy4);
-      load_cols<NJ4>(scratch + (size_t)s * KV + (size_t)i * V, c, TPR, hp4);
-      float hp[NJ4 * 4], vv[NJ4 * 4], dyv[NJ4 * 4];
-#pragma unroll
-      for (int jj = 0; jj < NJ4; ++jj) {
-        hp[jj * 4] = hp4[jj].x; hp[jj * 4 + 1] = hp4[jj].y; hp[jj * 4 + 2] = hp4[jj].z; hp[jj * 4 + 3] = hp4[jj].w;
-        vv[jj * 4] = v4[jj].x; vv[jj * 4 + 1] = v4[jj].y; vv[jj * 4 + 2] = v4[jj].z; vv[jj * 4 + 3] = v4[jj].w;
-        dyv[jj * 4] = dy4[jj].x; dyv[jj * 4 + 1] = dy4[jj].y; dyv[jj * 4 + 2] = dy4[jj].z; dyv[jj * 4 + 3] = dy4[jj].w;
-      }
-      store_cols<NJ4>(Hs + i * HP, c, TPR, hp);
-      __syncwarp();
-      float z[NJ4 * 4];
-      transition<NJ4>(Hs + i * HP, Ws, V, HP, c, TPR, k_i, v4, z);
+  };
 
-      float G[NJ4 * 4], dX[NJ4 * 4];
-      float dq_i = 0.f, dk_i = 0.f, df = 0.f;
-#pragma unroll
-      for (int x = 0; x < NJ4 * 4; ++x) {
-        const float ht = f * hp[x] + (1.f - f) * z[x];   // H_t
-        G[x] = Cg[x] + q_i * dyv[x];                     // G = C + q dy^T
-        dq_i = fmaf(ht, dyv[x], dq_i);                   // dq = H_t dy
-        df = fmaf(G[x], hp[x] - z[x], df);               // df = sum G (.) (H_{t-1} - Z)
-        dX[x] = (1.f - f) * G[x] * (1.f - z[x] * z[x]);  // through the gate and tanh
-        dk_i = fmaf(dX[x], vv[x], dk_i);                 // dk = dX v
+  int x = 0;   // piece counter: picks the stage
+  bool fetched = false;
+  for (int ch = nch - 1; ch >= 0; --ch) {
+    int np = (min(a.C, T - ch * a.C) + kSteps - 1) / kSteps;
+    const float *ck = a.ckpt + ((size_t)bn * a.nchunks + ch) * KV + own_g;
+    if (np > 1) {   // walk the chunk forward once, leaving the states between its pieces
+      if constexpr (BG::kReload) load_w<V>(Wn, p, c0, w);
+      __syncthreads();   // the piece before is done with every array
+      float2 h = *reinterpret_cast<const float2 *>(ck);
+      for (int i = 0; i + 1 < np; ++i, ++x) {
+        const Piece pc = piece(ch, i);
+        *reinterpret_cast<float2 *>(Hc + own) = h;
+        fetch(x, pc);
+        cp_wait<0>();
+        gates(x, pc);
+        __syncthreads();
+        forward(x, pc.len);
+        h = *reinterpret_cast<const float2 *>(Hc + pc.len * G::kTile + own);
+        *reinterpret_cast<float2 *>(scratch + (size_t)(i + 1) * KV + own_g) = h;
+        __syncthreads();
       }
-      store_cols<NJ4>(Xs + i * HP, c, TPR, dX);
-      for (int off = 1; off < TPR; off <<= 1) {
-        dq_i += __shfl_xor_sync(0xffffffffu, dq_i, off);
-        dk_i += __shfl_xor_sync(0xffffffffu, dk_i, off);
+      fetched = false;
+    }
+    for (int i = np - 1; i >= 0; --i, ++x) {
+      const Piece pc = piece(ch, i);
+      if (!fetched) fetch(x, pc);
+      const float2 h0 = i > 0 ? *reinterpret_cast<const float2 *>(scratch + (size_t)i * KV + own_g) : *reinterpret_cast<const float2 *>(ck);
+      if constexpr (BG::kReload) load_w<V>(Wn, p, c0, w);
+      cp_wait<0>();
+      gates(x, pc);
+      __syncthreads();   // inputs are in; the piece before is done with every array
+      *reinterpret_cast<float2 *>(Hc + own) = h0;
+      __syncthreads();
+      // the next piece's inputs, unless a pass over its chunk comes first
+      fetched = i > 0 || (ch > 0 && a.C <= kSteps);
+      if (fetched) fetch(x + 1, i > 0 ? piece(ch, i - 1) : piece(ch - 1, 0));
+      // (A)
+      forward(x, pc.len);
+      // (B)
+      const float *st = stage(x), *fs = fS + (x & 1) * kSteps;
+      if constexpr (BG::kReload) load_wt<V>(Wn, p, c0, w);
+      for (int s = pc.len - 1; s >= 0; --s) {
+        const float f = fs[s], q = st[s * kRows + p];
+        const float2 dy = *reinterpret_cast<const float2 *>(st + oDY + s * V + c0);
+        const float2 hp = *reinterpret_cast<const float2 *>(Hc + s * G::kTile + own);
+        float *xs = Xc + s * G::kTile;
+        const float2 z = *reinterpret_cast<const float2 *>(xs + own);
+        const float2 Gv = make_float2(fmaf(q, dy.x, C.x), fmaf(q, dy.y, C.y));                    // G = C + q dy^T
+        dfp[s * G::kThreads + tid] = fmaf(Gv.x, hp.x - z.x, Gv.y * (hp.y - z.y));               // df = sum G (.) (H_{t-1} - Z)
+        *reinterpret_cast<float2 *>(xs + own) =
+            make_float2((1.f - f) * Gv.x * (1.f - z.x * z.x), (1.f - f) * Gv.y * (1.f - z.y * z.y));   // dX: through the gate and tanh
+        __syncthreads();
+        float2 o;                                                                                // C_{t-1} = f G + dX W^T
+        if constexpr (BG::kReload) o = product<V>(xs, w, p, lane);
+        else o = product<V>(xs, wt, p, lane);
+        C = make_float2(fmaf(f, Gv.x, o.x), fmaf(f, Gv.y, o.y));
+        if (a.dh_clip > 0.f) C = make_float2(fminf(fmaxf(C.x, -a.dh_clip), a.dh_clip), fminf(fmaxf(C.y, -a.dh_clip), a.dh_clip));
       }
-      for (int off = 1; off < 32; off <<= 1) df += __shfl_xor_sync(0xffffffffu, df, off);
-      if (c == 0) {
-        if (a.dq_part) a.dq_part[(bt * N + n) * K + i] = dq_i;
-        else static_cast<float *>(a.dq)[(bt * a.Nq + hq) * K + i] = dq_i;
-        if (a.dk_part) a.dk_part[(bt * N + n) * K + i] = dk_i;
-        else static_cast<float *>(a.dk)[(bt * a.Nk + hk) * K + i] = dk_i;
-      }
-      if (lane == 0) red[warp] = df;
-      // dv partial: sum over the warp's rows of dX[i][col] * k_i
+      // (C) dW += H_{t-1}^T dX over the piece's steps and rows
+      for (int s = tsp; s < pc.len; s += BG::SP) {
+        const float *hs = Hc + s * G::kTile + tl, *xs = Xc + s * G::kTile + tj;
 #pragma unroll
-      for (int x = 0; x < NJ4 * 4; ++x) {
-        float dvv = dX[x] * k_i;
-        for (int off = TPR; off < 32; off <<= 1) dvv += __shfl_xor_sync(0xffffffffu, dvv, off);
-        if (lane < TPR) dvpart[warp * V + col_of(x >> 2, c, TPR) + (x & 3)] = dvv;
-      }
-      __syncthreads();  // Hs, Xs, dvpart, red complete for every row
-
-      // C_{t-1}[i][l] = f G[i][l] + sum_j dX[i][j] W[l][j]
-      float Cn[NJ4 * 4];
+        for (int r = 0; r < kRows; ++r) {
+          const float4 h4 = *reinterpret_cast<const float4 *>(hs + r * G::HP);
+          const float hv[4] = {h4.x, h4.y, h4.z, h4.w};
 #pragma unroll
-      for (int x = 0; x < NJ4 * 4; ++x) Cn[x] = f * G[x];
-      for (int j = 0; j < V; j += 4) {
-        const float4 x4 = *reinterpret_cast<const float4 *>(Xs + i * HP + j);
+          for (int jj = 0; jj < BG::JT / 4; ++jj) {
+            const float4 x4 = *reinterpret_cast<const float4 *>(xs + r * G::HP + jj * (V / 2));
 #pragma unroll
-        for (int x = 0; x < NJ4 * 4; ++x) {
-          const int l = col_of(x >> 2, c, TPR) + (x & 3);
-          const float4 w4 = *reinterpret_cast<const float4 *>(Ws + l * HP + j);
-          Cn[x] = fmaf(x4.x, w4.x, Cn[x]);
-          Cn[x] = fmaf(x4.y, w4.y, Cn[x]);
-          Cn[x] = fmaf(x4.z, w4.z, Cn[x]);
-          Cn[x] = fmaf(x4.w, w4.w, Cn[x]);
-        }
-      }
-#pragma unroll
-      for (int x = 0; x < NJ4 * 4; ++x) {
-        float cv = Cn[x];
-        if (a.dh_clip > 0.f) cv = fminf(fmaxf(cv, -a.dh_clip), a.dh_clip);
-        Cg[x] = cv;
-      }
-      // dW += H_{t-1}^T dX
-#pragma unroll
-      for (int x = 0; x < kMaxDW; ++x) {
-        const int d = tid + x * nthreads;
-        if (d < ndw) {
-          const int l = d / (V / 4), j = (d % (V / 4)) * 4;
-          float4 acc = dWacc[x];
-          for (int r = 0; r < K; ++r) {
-            const float hv = Hs[r * HP + l];
-            const float4 x4 = *reinterpret_cast<const float4 *>(Xs + r * HP + j);
-            acc.x = fmaf(hv, x4.x, acc.x);
-            acc.y = fmaf(hv, x4.y, acc.y);
-            acc.z = fmaf(hv, x4.z, acc.z);
-            acc.w = fmaf(hv, x4.w, acc.w);
+            for (int e = 0; e < 4; ++e) {
+              dW[e][2 * jj] = __ffma2_rn(make_float2(hv[e], hv[e]), make_float2(x4.x, x4.y), dW[e][2 * jj]);
+              dW[e][2 * jj + 1] = __ffma2_rn(make_float2(hv[e], hv[e]), make_float2(x4.z, x4.w), dW[e][2 * jj + 1]);
+            }
           }
-          dWacc[x] = acc;
         }
       }
-      if (tid < V) {
-        float sdv = 0.f;
-        for (int w = 0; w < nwarps; ++w) sdv += dvpart[w * V + tid];
-        if (wr) sdv += wr[(size_t)n * V + tid] * dyg[(bt * N + n) * V + tid];
-        static_cast<float *>(a.dv)[(bt * N + n) * V + tid] = sdv;
+      // dq = H_t dy, dk = dX v: eight lanes per (step, row)
+      const size_t bt0 = tok0 + pc.t0;
+      for (int it = tid >> 3; it < pc.len * kRows; it += G::kThreads / 8) {
+        const int s = it >> 3, r = it & 7, e = tid & 7;
+        const float *hs = Hc + (s + 1) * G::kTile + r * G::HP, *xs = Xc + s * G::kTile + r * G::HP;
+        const float *dys = st + oDY + s * V, *vs = st + oV + s * V;
+        float dq = 0.f, dk = 0.f;
+#pragma unroll
+        for (int j = 0; j < V / 16; ++j) {
+          const int c = 16 * j + 2 * e;
+          const float2 h2 = *reinterpret_cast<const float2 *>(hs + c), d2 = *reinterpret_cast<const float2 *>(dys + c);
+          const float2 x2 = *reinterpret_cast<const float2 *>(xs + c), v2 = *reinterpret_cast<const float2 *>(vs + c);
+          dq = fmaf(h2.x, d2.x, fmaf(h2.y, d2.y, dq));
+          dk = fmaf(x2.x, v2.x, fmaf(x2.y, v2.y, dk));
+        }
+        // (all lanes of a warp take the same number of turns: len x 8 items are whole groups of four)
+#pragma unroll
+        for (int off = 1; off < 8; off <<= 1) { dq += __shfl_xor_sync(0xffffffffu, dq, off); dk += __shfl_xor_sync(0xffffffffu, dk, off); }
+        if (e == 0) {
+          const size_t bt = bt0 + s;
+          if (a.dq_part) a.dq_part[(bt * N + n) * K + rbase + r] = dq;
+          else static_cast<float *>(a.dq)[(bt * a.Nq + hq) * K + rbase + r] = dq;
+          if (a.dk_part) a.dk_part[(bt * N + n) * K + rbase + r] = dk;
+          else static_cast<float *>(a.dk)[(bt * a.Nk + hk) * K + rbase + r] = dk;
+        }
       }
-      if (tid == 0) {
-        float sdf = 0.f;
-        for (int w = 0; w < nwarps; ++w) sdf += red[w];
-        a.dgate[bt * N + n] = sdf * dfdx;
+      // dv = dX^T k over these rows (+ w_r (.) dy from Eq. 3, added with the first group)
+      for (int it = tid; it < pc.len * (V / 4); it += G::kThreads) {
+        const int s = it / (V / 4), j = 4 * (it % (V / 4));
+        float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int r = 0; r < kRows; ++r) {
+          const float k = st[oK + s * kRows + r];
+          const float4 x4 = *reinterpret_cast<const float4 *>(Xc + s * G::kTile + r * G::HP + j);
+          o.x = fmaf(k, x4.x, o.x); o.y = fmaf(k, x4.y, o.y); o.z = fmaf(k, x4.z, o.z); o.w = fmaf(k, x4.w, o.w);
+        }
+        if (wr && rs == 0) {
+          const float4 w4 = *reinterpret_cast<const float4 *>(wr + (size_t)n * V + j), d4 = *reinterpret_cast<const float4 *>(st + oDY + s * V + j);
+          o.x = fmaf(w4.x, d4.x, o.x); o.y = fmaf(w4.y, d4.y, o.y); o.z = fmaf(w4.z, d4.z, o.z); o.w = fmaf(w4.w, d4.w, o.w);
+        }
+        const size_t at = ((bt0 + s) * N + n) * V + j;
+        float4 *dst = reinterpret_cast<float4 *>((a.dv_part ? a.dv_part + (size_t)rs * a.TT * N * V : static_cast<float *>(a.dv)) + at);
+        if (add) { const float4 old = *dst; o.x += old.x; o.y += old.y; o.z += old.z; o.w += old.w; }
+        *dst = o;
       }
-      __syncthreads();  // before Hs / Xs / dvpart / red are overwritten
+      // dgate: a warp sums the threads' shares of a step, then the gate's slope
+      for (int s = warp; s < pc.len; s += G::NW) {
+        float df = 0.f;
+#pragma unroll
+        for (int i2 = 0; i2 < G::NW; ++i2) df += dfp[s * G::kThreads + 32 * i2 + lane];
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) df += __shfl_xor_sync(0xffffffffu, df, off);
+        if (lane == 0) {
+          float *dst = (a.dgate_part ? a.dgate_part + (size_t)rs * a.TT * N : a.dgate) + (bt0 + s) * N + n;
+          df *= dfS[(x & 1) * kSteps + s];
+          *dst = add ? *dst + df : df;
+        }
+      }
     }
   }
-  if (a.dh0) store_cols<NJ4>(a.dh0 + bn * KV + (size_t)i * V, c, TPR, Cg);
-  float *dWp = a.dW_part + (size_t)bn * V * V;
+  if (a.dh0) *reinterpret_cast<float2 *>(a.dh0 + (size_t)bn * KV + own_g) = C;
+  // dW: the threads that share a tile are added in a fixed order
+  float *dWp = a.dW_part + (nslab == 1 ? (size_t)bn : ((size_t)b * nslab + rs) * N + n) * V * V;
+  if constexpr (BG::SP > 1) {
+    float *sh = Hc;   // [SP - 1][tiles][16]
+    __syncthreads();
+    if (tsp > 0)
 #pragma unroll
-  for (int x = 0; x < kMaxDW; ++x) {
-    const int d = tid + x * nthreads;
-    if (d < ndw) *reinterpret_cast<float4 *>(dWp + (size_t)d * 4) = dWacc[x];
+      for (int e = 0; e < 4; ++e)
+        *reinterpret_cast<float4 *>(sh + ((size_t)(tsp - 1) * BG::kTiles + tile) * 16 + 4 * e) = make_float4(dW[e][0].x, dW[e][0].y, dW[e][1].x, dW[e][1].y);
+    __syncthreads();
+    if (tsp > 0) return;
+    for (int k = 0; k < BG::SP - 1; ++k)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float4 o = *reinterpret_cast<const float4 *>(sh + ((size_t)k * BG::kTiles + tile) * 16 + 4 * e);
+        dW[e][0].x += o.x; dW[e][0].y += o.y; dW[e][1].x += o.z; dW[e][1].y += o.w;
+      }
   }
+#pragma unroll
+  for (int e = 0; e < 4; ++e)
+#pragma unroll
+    for (int jj = 0; jj < BG::JT / 4; ++jj) {
+      float4 *dst = reinterpret_cast<float4 *>(dWp + (size_t)(tl + e) * V + tj + jj * (V / 2));
+      float4 o = make_float4(dW[e][2 * jj].x, dW[e][2 * jj].y, dW[e][2 * jj + 1].x, dW[e][2 * jj + 1].y);
+      if (add) { const float4 old = *dst; o.x += old.x; o.y += old.y; o.z += old.z; o.w += old.w; }
+      *dst = o;
+    }
 }
 
-int pick_tpr(int K, int V) {
-  int tpr = 32;
-  while (tpr > V / 4 || tpr * K > 1024) tpr >>= 1;
-  return tpr;
+// ------------------------------------------------------------------ decoding step (Eq. 1-3 once)
+// Persistent CTAs over (head, batch entry) in head-major order, W reloaded only when the head changes;
+// the groups of eight rows of a state stream through a ring of kRing stages (cp.async), are
+// multiplied, updated and written back in place.  The readout is complete inside the CTA.
+// Bound by FMA at V >= 64 (V/8 FMA per byte of state against 6 at the chip's rates), by HBM below.
+constexpr int kRing = 4;
+
+template <int V>
+struct DecGeom {
+  static constexpr int kOcc = V == 128 ? 1 : 768 / Geom<V>::kThreads;   // CTAs per SM: 24 warps (V = 128: 16) at 85 registers or more
+  static constexpr int kStage = Geom<V>::kTile + 2 * kRows + V;   // rows, then k [8], q [8], v [V]
+};
+
+template <int V>
+__global__ void __launch_bounds__(Geom<V>::kThreads, DecGeom<V>::kOcc) decode_f32_kernel(ScanArgs a) {
+  using G = Geom<V>;
+  constexpr int kStage = DecGeom<V>::kStage;
+  extern __shared__ __align__(16) float smem[];
+  const int K = a.K, N = a.N, B = a.B, ng = K / kRows;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, p = lane >> 2, c0 = 8 * warp + 2 * (lane & 3);
+  const size_t KV = (size_t)K * V;
+  const float *qg = static_cast<const float *>(a.q), *kg = static_cast<const float *>(a.k);
+  const float *vg = static_cast<const float *>(a.v), *wr = static_cast<const float *>(a.w_r);
+  float *state = a.hT, *yg = static_cast<float *>(a.y);   // state == a.h0: updated in place
+  const long units = (long)N * B, u0 = units * blockIdx.x / gridDim.x, u1 = units * (blockIdx.x + 1) / gridDim.x;
+
+  long uf = u0;   // next group to fetch: unit and group
+  int gf = 0;
+  auto fetch = [&](int slot) {   // always one commit group, possibly empty
+    if (uf < u1) {
+      const int n = (int)(uf / B), b = (int)(uf % B), r0 = gf * kRows;
+      const size_t bn = (size_t)b * N + n;
+      float *st = smem + slot * kStage;
+      const float *src = state + bn * KV + (size_t)r0 * V;
+      for (int i = tid; i < kRows * (V / 4); i += G::kThreads) cp16(st + (i / (V / 4)) * G::HP + 4 * (i % (V / 4)), src + 4 * i);
+      if (tid < 2) cp16(st + G::kTile + 4 * tid, kg + ((size_t)b * a.Nk + n / (N / a.Nk)) * K + r0 + 4 * tid);
+      else if (tid < 4) cp16(st + G::kTile + 4 * tid, qg + ((size_t)b * a.Nq + n / (N / a.Nq)) * K + r0 + 4 * (tid - 2));
+      else if (tid < 4 + V / 4) cp16(st + G::kTile + 4 * tid, vg + bn * V + 4 * (tid - 4));
+      if (++gf == ng) { gf = 0; ++uf; }
+    }
+    cp_commit();
+  };
+#pragma unroll
+  for (int i = 0; i < kRing - 1; ++i) fetch(i);
+  float2 w[G::NP][2];
+  int head = -1, slot = 0;
+  for (long u = u0; u < u1; ++u) {
+    const int n = (int)(u / B), b = (int)(u % B);
+    const size_t bn = (size_t)b * N + n;
+    const float graw = a.gate[bn];
+    if (n != head) { load_w<V>(static_cast<const float *>(a.W) + (size_t)n * V * V, p, c0, w); head = n; }
+    const float f = gate_value(a.gate_kind, graw, a.alpha ? a.alpha[n] : 1.f, a.beta ? a.beta[n] : 0.f, nullptr);
+    float y = 0.f, wrv = 0.f;
+    if (wr) wrv = wr[(size_t)n * V + c0 + (p >> 2)];
+    for (int g = 0; g < ng; ++g) {
+      cp_wait<kRing - 2>();
+      __syncthreads();                                   // this group is in for everybody; the one before is used up
+      const float *st = smem + slot * kStage, *vec = st + G::kTile;
+      fetch(slot == 0 ? kRing - 1 : slot - 1);           // into the slot just freed
+      const float2 o = product<V>(st, w, p, lane);
+      float2 z;
+      const float2 v2 = *reinterpret_cast<const float2 *>(vec + 2 * kRows + c0);
+      const float2 h = update(o, vec[p], v2, f, *reinterpret_cast<const float2 *>(st + p * G::HP + c0), z);
+      *reinterpret_cast<float2 *>(state + bn * KV + (size_t)(g * kRows + p) * V + c0) = h;
+      const float share = readout(vec[kRows + p], h, lane);
+      y = g == 0 ? fmaf(wrv, lane & 16 ? v2.y : v2.x, share) : y + share;
+      slot = slot + 1 == kRing ? 0 : slot + 1;
+    }
+    if ((p & 3) == 0) yg[bn * V + c0 + (p >> 2)] = y;
+  }
+  cp_wait<0>();
+}
+
+template <int V>
+cudaError_t launch_fwd_v(const ScanArgs &a, cudaStream_t s) {
+  const size_t smem = fwd_f32_smem<V>(a.KCf);
+  const cudaError_t e = allow_smem(fwd_f32_kernel<V>, smem);
+  if (e != cudaSuccess) return e;
+  fwd_f32_kernel<V><<<a.B * a.N * (a.K / a.KCf), Geom<V>::kThreads, smem, s>>>(a);
+  return cudaGetLastError();
+}
+
+template <int V>
+cudaError_t launch_bwd_v(const ScanArgs &a, cudaStream_t s) {
+  const size_t smem = sizeof(float) * (size_t)BwdGeom<V>::kFloats;
+  cudaError_t e = allow_smem(bwd_f32_kernel<V>, smem);
+  const int slabs = a.K / kRows, nslab = a.KC == kRows ? slabs : 1;
+  for (int s0 = 0; s0 < slabs && e == cudaSuccess; s0 += nslab) {
+    bwd_f32_kernel<V><<<a.B * a.N * nslab, Geom<V>::kThreads, smem, s>>>(a, s0, nslab);
+    e = cudaGetLastError();
+  }
+  return e;
+}
+
+template <int V>
+cudaError_t launch_decode_v(const ScanArgs &a, cudaStream_t s) {
+  const size_t smem = sizeof(float) * (size_t)kRing * DecGeom<V>::kStage;
+  const cudaError_t e = allow_smem(decode_f32_kernel<V>, smem);
+  if (e != cudaSuccess) return e;
+  const long units = (long)a.B * a.N, room = (long)sm_count() * DecGeom<V>::kOcc;
+  decode_f32_kernel<V><<<(unsigned)(units < room ? units : room), Geom<V>::kThreads, smem, s>>>(a);
+  return cudaGetLastError();
 }
 
 }  // namespace
 
-cudaError_t launch_fwd_f32(const ScanArgs &a, cudaStream_t s) {
-  const int TPR = pick_tpr(a.K, a.V), nthreads = a.K * TPR, nj4 = a.V / TPR / 4, HP = a.V + kPad;
-  const size_t smem = sizeof(float) * ((size_t)a.V * HP + (size_t)a.K * HP + 2 * (nthreads / 32) * a.V);
-  auto kern = nj4 == 1 ? fwd_f32_kernel<1> : nj4 == 2 ? fwd_f32_kernel<2> : fwd_f32_kernel<4>;
-  cudaError_t e = allow_smem(kern, smem);
-  if (e != cudaSuccess) return e;
-  kern<<<a.B * a.N, nthreads, smem, s>>>(a, TPR);
-  return cudaGetLastError();
+// Rows per CTA of the forward kernel: whole states where that gives every SM 16 warps (half of what it
+// holds) -- the groups take turns behind one barrier a step and y needs no shares in memory --, else
+// eight rows.  `share_bytes`: one slab's share of y; whole states too where the shares of all groups
+// would exceed kMaxShares.
+constexpr size_t kMaxShares = (size_t)4 << 30;
+int fwd_f32_rows(int B, int N, int K, int V, size_t share_bytes) {
+  const long units = (long)(B > 0 ? B : 1) * N;
+  return units * (V / 8) >= 16L * sm_count() || share_bytes * (K / kRows) > kMaxShares ? K : kRows;
 }
 
+// Rows per CTA of the backward kernel: eight, all groups at once (partials of dv, dgate and dW per
+// group); K stands for one launch per group, each adding to the results of the one before, where the
+// units alone give every SM 64 warps or the shares of dv would exceed kMaxShares.
+int bwd_f32_rows(int B, int N, int K, int V, size_t share_bytes) {
+  const long units = (long)(B > 0 ? B : 1) * N;
+  return units * (V / 8) >= 64L * sm_count() || share_bytes * (K / kRows) > kMaxShares ? K : kRows;
+}
+int bwd_f32_piece() { return kSteps; }
+
+cudaError_t launch_fwd_f32(const ScanArgs &a, cudaStream_t s) {
+  switch (a.V) {
+    case 16: return launch_fwd_v<16>(a, s);
+    case 32: return launch_fwd_v<32>(a, s);
+    case 64: return launch_fwd_v<64>(a, s);
+    default: return launch_fwd_v<128>(a, s);
+  }
+}
 cudaError_t launch_bwd_f32(const ScanArgs &a, cudaStream_t s) {
-  const int TPR = pick_tpr(a.K, a.V), nthreads = a.K * TPR, nj4 = a.V / TPR / 4, HP = a.V + kPad;
-  const int nwarps = nthreads / 32;
-  const size_t smem = sizeof(float) * ((size_t)a.V * HP + 2 * (size_t)a.K * HP + (size_t)nwarps * a.V + nwarps);
-  auto kern = nj4 == 1 ? bwd_f32_kernel<1> : nj4 == 2 ? bwd_f32_kernel<2> : bwd_f32_kernel<4>;
-  cudaError_t e = allow_smem(kern, smem);
-  if (e != cudaSuccess) return e;
-  kern<<<a.B * a.N, nthreads, smem, s>>>(a, TPR);
-  return cudaGetLastError();
+  switch (a.V) {
+    case 16: return launch_bwd_v<16>(a, s);
+    case 32: return launch_bwd_v<32>(a, s);
+    case 64: return launch_bwd_v<64>(a, s);
+    default: return launch_bwd_v<128>(a, s);
+  }
+}
+cudaError_t launch_decode_f32(const ScanArgs &a, cudaStream_t s) {
+  switch (a.V) {
+    case 16: return launch_decode_v<16>(a, s);
+    case 32: return launch_decode_v<32>(a, s);
+    case 64: return launch_decode_v<64>(a, s);
+    default: return launch_decode_v<128>(a, s);
+  }
 }
 
 }  // namespace m2rnn

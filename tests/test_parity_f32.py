@@ -102,3 +102,22 @@ def test_backward_repeats_bit_for_bit(oracle):
     b = parity.gpu_bwd(cfg, g)
     for name in a:
         assert torch.equal(a[name], b[name]), name
+
+
+# the two slab plans of each direction and the edges of a 16-step piece: whole states (forward: V/8 units
+# >= 16 an SM; backward: >= 64, one launch per group of rows), a checkpoint interval longer than a piece
+@pytest.mark.parametrize("B,T,N,K,V,ckpt", [(4, 17, 37, 32, 128, 0), (37, 3, 16, 16, 128, 0), (1, 16, 1, 16, 32, 0), (2, 70, 2, 32, 64, 40),
+                                            (1, 47, 3, 16, 16, 64), (300, 5, 4, 32, 16, 0), (1, 50, 1, 48, 128, 33)])
+def test_slab_plans_and_pieces(oracle, B, T, N, K, V, ckpt):
+    cfg = ScanConfig("plan", B=B, T=T, N=N, K=K, V=V, dtype="f32", w_scale=0.7, seed=900 + T)
+    d = inputs.make_inputs(cfg, backward=True, residual=True, d_hT=True)
+    g = parity.to_dev(d)
+    y, hT, ck = parity.gpu_fwd(cfg, g, save_ckpt=True, ckpt_interval=ckpt)
+    y_ref, hT_ref = parity.oracle_fwd(oracle, cfg, d)
+    assert parity.rel_err(y, y_ref) < 1e-4 and parity.rel_err(hT, hT_ref) < 1e-4
+    out, ref = parity.gpu_bwd(cfg, g, ckpt=ck, ckpt_interval=ckpt), parity.oracle_bwd(oracle, cfg, d)
+    assert max(parity.rel_err(out[name], ref[name]) for name in ref) < 1e-4
+    state = g["h0"].clone()
+    first = {x: g[x][:, 0].contiguous() for x in ("q", "k", "v", "gate")}
+    y1 = binding.m2rnn_decode_step(first["q"], first["k"], first["v"], first["gate"], g["W"], state, w_r=g["w_r"])
+    assert torch.equal(y1, y[:, 0])
