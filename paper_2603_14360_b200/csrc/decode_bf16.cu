@@ -1,18 +1,18 @@
-// bf16 decoding step (Eq. 1-3 once on a cached fp32 state) for sm_100a.
+// bf16 decoding step (Eq. 1-3 once on a cached fp32 state) for sm_100a, V <= 64.
 //
-// The step streams the whole state through the chip once (read + write, fp32), so the kernel is
-// laid out around HBM: persistent CTAs walk a contiguous range of (head, batch) units in
-// head-major order, keep the head's transition matrix as MMA fragments in shared memory (re-read
-// only when the head changes), and prefetch the states of the next units with the bulk async-copy
-// engine (cp.async.bulk into a two-stage shared-memory buffer, completion on an mbarrier) while
-// the current ones are computed.  Every warp takes 16 state rows from the staged copy into
-// accumulator-layout registers, runs the state x W product
-// on tensor cores (mma.sync, bf16 operands, fp32 accumulate), applies the outer product, tanh
-// and the gate in registers, writes the rows back in place and leaves its share of the readout
-// in shared memory, where the unit's warps are summed.
-#include <cstdlib>
-#include <cstring>
-
+// The step streams every state through the chip once (fp32, read and write), so the kernel is laid out
+// around HBM: warps that need nothing from one another.  A warp takes a contiguous range of (head,
+// batch) units in head-major order, keeps the head's transition matrix as MMA fragments in registers,
+// and walks its units in slabs of 16 rows (16 V contiguous floats).  Slabs are copied (cp.async) several
+// ahead into a ring in shared memory whose every 16 bytes are read by the lane that copied them: no
+// barrier of any kind.  A slab goes through mma.sync (bf16 operands, fp32 accumulate), outer product,
+// tanh and gate in registers and is stored straight back.  The readout is summed over a unit's slabs
+// in registers.
+// The code a warp runs once is kept short: the first pass through an instruction comes from the L2
+// (the slab loop unrolled by four cost a small batch 4 us, 64-bit divisions another 1.5).
+// A CTA that takes eight slabs at a time behind barriers, two stages ahead, spends 1.9 us of latency on
+// them whatever their size.  The paper's layer (N = 84, K = 64, V = 16) at batch 48: 25.6 -> 6.3 us, at
+// batch 400: 200 -> 50 us (5.5 TB/s).
 #include "device_common.cuh"
 #include "internal.h"
 #include "mma_tile.cuh"
@@ -21,206 +21,232 @@
 namespace m2rnn {
 namespace {
 
+template <int V>
+struct DecCfg {
+  static constexpr int kWarps = V == 64 ? 8 : (V == 32 ? 16 : 32);  // one CTA per SM (its warps share nothing but the launch)
+  static constexpr int kStages = V == 64 ? 6 : (V == 32 ? 5 : 4);   // slabs on their way per warp: 6 x 4, 5 x 2, 4 x 1 KB
+  static constexpr bool kSplit = V >= 64;   // the state enters the product as the sum of two bf16 operands
+  static constexpr int kSlabBytes = 16 * V * 4;
+  static constexpr int kSmem = kWarps * kStages * kSlabBytes;
+};
+
 // Memory column of MMA column m = 8nt + 2c + e: a thread's registers of the tile pair
 // (2x, 2x+1) are the four adjacent columns 16x + 4c .. 16x + 4c + 3, so the four lanes of a row
-// group read 64 contiguous bytes of a row per load.
-template <int V>
-__host__ __device__ constexpr int dec_col(int m) {
-  return V == 16 ? 4 * ((m & 7) >> 1) + 2 * (m >> 3) + (m & 1)
-                 : 16 * (m >> 4) + 4 * ((m & 7) >> 1) + 2 * ((m >> 3) & 1) + (m & 1);
+// group touch 64 contiguous bytes of a row.
+__host__ __device__ constexpr int dec_col(int m) { return 16 * (m >> 4) + 4 * ((m & 7) >> 1) + 2 * ((m >> 3) & 1) + (m & 1); }
+
+__device__ __forceinline__ uint32_t movmatrix_trans(uint32_t a) {
+  uint32_t d;
+  asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(d) : "r"(a));
+  return d;
+}
+// A operand of k-tile kt from the state in accumulator layout: the bf16 rounding, and what it leaves out
+// as a second operand (used where kSplit: the product then sees the state with 16 bits of mantissa)
+template <int NT>
+__device__ __forceinline__ void a_fragment(const float (&H)[NT][4], int kt, uint32_t (&hi)[4], uint32_t (&lo)[4]) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const float x = H[2 * kt + (i >> 1)][2 * (i & 1)], y = H[2 * kt + (i >> 1)][2 * (i & 1) + 1];
+    hi[i] = pack_bf16(x, y);
+    lo[i] = pack_bf16(x - __uint_as_float(hi[i] << 16), y - __uint_as_float(hi[i] & 0xffff0000u));
+  }
+}
+
+__device__ __forceinline__ void cp16(uint32_t dst_sa, const float *src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst_sa), "l"(src) : "memory");
 }
 
 template <int V>
-__device__ __forceinline__ uint2 dec_w_fragment(const uint16_t *__restrict__ w, int kt, int nt, int lane) {
-  const int g = lane >> 2, c = lane & 3;
-  const int col = dec_col<V>(8 * nt + g);
-  const int r0 = dec_col<V>(16 * kt + 2 * c), r1 = dec_col<V>(16 * kt + 2 * c + 1);
-  const int r2 = dec_col<V>(16 * kt + 8 + 2 * c), r3 = dec_col<V>(16 * kt + 8 + 2 * c + 1);
-  return make_uint2((uint32_t)w[r0 * V + col] | ((uint32_t)w[r1 * V + col] << 16),
-                    (uint32_t)w[r2 * V + col] | ((uint32_t)w[r3 * V + col] << 16));
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, uint32_t bytes) {
-  asm volatile("{\n .reg .b64 st;\n mbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n}" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
-// global -> shared bulk copy (no multicast); both addresses 16-byte aligned, size a multiple of 16
-__device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t bytes, uint64_t *bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-               ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
-}
-
-template <int V>
-__global__ void __launch_bounds__(256, 1) decode_bf16_kernel(ScanArgs a, int WPU, int GPI, int tasks_per_head) {
-  constexpr int NT = V / 8, KT = V / 16, SEG = V / 4, NX = V == 16 ? 1 : V / 16;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  uint64_t *full = reinterpret_cast<uint64_t *>(smem_raw);                // [2] stage landed
-  uint2 *Wf = reinterpret_cast<uint2 *>(smem_raw + 16);                   // [KT][NT][32]
-  float *ypart = reinterpret_cast<float *>(smem_raw + 16 + KT * NT * 32 * 8);  // [2][GPI][WPU][V]
-
-  const int K = a.K, N = a.N, B = a.B;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, c = lane & 3;
-  const int grp = warp / WPU, wu = warp % WPU;      // unit slot of this warp, its 16-row slab
-  const bool active_warp = grp < GPI;
+__global__ void __launch_bounds__(32 * DecCfg<V>::kWarps, 1) decode_bf16_kernel(ScanArgs a, int per, int extra) {
+  using Cfg = DecCfg<V>;
+  constexpr int NT = V / 8, KT = V / 16, SEG = V / 4, NX = V / 16, kStages = Cfg::kStages, kWarps = Cfg::kWarps;
+  extern __shared__ __align__(128) unsigned char smem[];
+  const int K = a.K, N = a.N, B = a.B, slabs = K / 16;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31, g = lane >> 2, c = lane & 3;
+  const int dq = N / a.Nq, dk = N / a.Nk;
   const size_t KV = (size_t)K * V;
-  const __nv_bfloat16 *qg = static_cast<const __nv_bfloat16 *>(a.q), *kg = static_cast<const __nv_bfloat16 *>(a.k);
+  const uint16_t *qg = static_cast<const uint16_t *>(a.q), *kg = static_cast<const uint16_t *>(a.k), *Wg = static_cast<const uint16_t *>(a.W);
   const __nv_bfloat16 *vg = static_cast<const __nv_bfloat16 *>(a.v), *wr = static_cast<const __nv_bfloat16 *>(a.w_r);
   __nv_bfloat16 *yg = static_cast<__nv_bfloat16 *>(a.y);
   float *state = a.hT;   // == a.h0: updated in place
 
-  const size_t unit_floats = KV;                                          // one unit's state
-  float *stage = ypart + 2 * GPI * WPU * V;                               // [2][GPI][K][V] fp32
-  if (tid == 0) {
-    mbar_init(&full[0], 1);
-    mbar_init(&full[1], 1);
-    fence_mbar_init();
-  }
-  __syncthreads();
+  // this warp's units (the first `extra` warps take per + 1); neighbouring ranges go to different SMs
+  const int wid = warp * (int)gridDim.x + (int)blockIdx.x;
+  int left = per + (wid < extra);           // units to go, and to request
+  if (left == 0) return;
+  const unsigned u0 = (unsigned)wid * per + min(wid, extra);
 
-  const long ntasks = (long)N * tasks_per_head;
-  const long t_begin = ntasks * blockIdx.x / gridDim.x, t_end = ntasks * (blockIdx.x + 1) / gridDim.x;
-  // one thread streams the states of a task's units into a stage, 16 KB per copy
-  auto prefetch = [&](long task, int st) {
-    const int n = (int)(task / tasks_per_head), b0 = (int)(task % tasks_per_head) * GPI;
-    const int units = min(GPI, B - b0);
-    const uint32_t bytes = (uint32_t)(unit_floats * 4);
-    mbar_expect_tx(&full[st], bytes * units);
-    for (int u = 0; u < units; ++u) {
-      const char *src = reinterpret_cast<const char *>(state + ((size_t)(b0 + u) * N + n) * unit_floats);
-      char *dst = reinterpret_cast<char *>(stage + ((size_t)st * GPI + u) * unit_floats);
-      for (uint32_t off = 0; off < bytes; off += 16384u) bulk_g2s(dst + off, src + off, min(16384u, bytes - off), &full[st]);
-    }
-  };
-  if (tid == 0 && t_begin < t_end) prefetch(t_begin, 0);
-  int cur_head = -1;
-  int it = 0;
-  for (long task = t_begin; task < t_end; ++task, ++it) {
-    const int n = (int)(task / tasks_per_head);
-    const int b = (int)(task % tasks_per_head) * GPI + grp;
-    // the other stage was last read before the barrier that closed the previous iteration
-    if (tid == 0 && task + 1 < t_end) prefetch(task + 1, (it + 1) & 1);
-    if (n != cur_head) {
-      __syncthreads();   // everyone is done with the previous head's fragments
-      const uint16_t *w = reinterpret_cast<const uint16_t *>(a.W) + (size_t)n * V * V;
-      for (int x = tid; x < KT * NT * 32; x += blockDim.x) Wf[x] = dec_w_fragment<V>(w, x / (NT * 32), (x / 32) % NT, x & 31);
-      cur_head = n;
-      __syncthreads();
-    }
-    const bool live = active_warp && b < B;
-    if (!mbar_wait(&full[it & 1], (it >> 1) & 1)) { report_timeout(a.dev_status); return; }
-    float *yp = ypart + (size_t)(((it & 1) * GPI + (active_warp ? grp : 0)) * WPU + wu) * V;
-    if (live) {
-      const size_t bn = (size_t)b * N + n;
-      const int hq = n / (N / a.Nq), hk = n / (N / a.Nk);
-      const int r0 = 16 * wu + g;
-      // state rows r0 and r0+8 in accumulator layout
-      float H[NT][4];
-      float *hrow0 = state + bn * KV + (size_t)r0 * V, *hrow1 = hrow0 + 8 * V;
-      const float *srow0 = stage + ((size_t)(it & 1) * GPI + grp) * unit_floats + (size_t)r0 * V, *srow1 = srow0 + 8 * V;
+  // a stage of the ring: [2 V/16 chunks][32 lanes] x 16 bytes
+  const uint32_t ring_sa = smem_u32(smem) + (uint32_t)warp * kStages * Cfg::kSlabBytes + 16u * lane;
+  const int lane_off = g * V + 4 * c;   // this lane's first element of a slab
+
+  int n = (int)(u0 / (unsigned)B), b = (int)(u0 - (unsigned)n * B);
+  // the next slab to request
+  const size_t unit_step = (size_t)N * KV;
+  const float *pf = state + ((size_t)b * N + n) * KV + lane_off;
+  int nf = n, bf = b, sf = 0;
+  int todo = left;
+  auto request = [&](int st) {   // always one group, possibly empty
+    if (todo > 0) {
+      const uint32_t dst = ring_sa + (uint32_t)st * Cfg::kSlabBytes;
 #pragma unroll
       for (int x = 0; x < NX; ++x) {
-        const float4 t0 = *reinterpret_cast<const float4 *>(srow0 + 16 * x + 4 * c);
-        const float4 t1 = *reinterpret_cast<const float4 *>(srow1 + 16 * x + 4 * c);
+        cp16(dst + 1024u * x, pf + 16 * x);
+        cp16(dst + 1024u * x + 512u, pf + 16 * x + 8 * V);
+      }
+      pf += 16 * V;
+      if (++sf == slabs) {
+        sf = 0; --todo; ++bf;
+        pf += unit_step - KV;
+        if (bf == B) { bf = 0; ++nf; pf = state + (size_t)nf * KV + lane_off; }
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+#pragma unroll
+  for (int s = 0; s < kStages; ++s) request(s);
+
+  // A unit's vectors, fetched one unit ahead.  k and q: lane (g, c) holds the entries of rows g and g + 8 of
+  // slabs c and c + 4 as one word each; slab s takes its pair from lane (g, s % 4).
+  struct Vecs { uint32_t k[2], q[2]; uint2 v[NX]; float gate; };
+  auto fetch = [&](int n, int b, int hk, int hq, Vecs &o) {
+    const uint16_t *kp = kg + ((size_t)b * a.Nk + hk) * K, *qp = qg + ((size_t)b * a.Nq + hq) * K;
+    const size_t bn = (size_t)b * N + n;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      o.k[h] = o.q[h] = 0u;
+      if (c + 4 * h < slabs) {
+        const int r = 16 * (c + 4 * h) + g;
+        o.k[h] = (uint32_t)kp[r] | ((uint32_t)kp[r + 8] << 16);
+        o.q[h] = (uint32_t)qp[r] | ((uint32_t)qp[r + 8] << 16);
+      }
+    }
+#pragma unroll
+    for (int x = 0; x < NX; ++x) o.v[x] = *reinterpret_cast<const uint2 *>(vg + bn * V + 16 * x + 4 * c);
+    o.gate = a.gate[bn];
+  };
+  Vecs next;
+  int hk = n / dk, hq = n / dq;
+  fetch(n, b, hk, hq, next);
+
+  uint32_t W[KT][NT][2];
+  int head = -1, st = 0;
+  for (; left > 0; --left) {
+    const Vecs cur = next;
+    const size_t bn = (size_t)b * N + n;
+    int n1 = n, b1 = b + 1;
+    if (b1 == B) { b1 = 0; ++n1; hk = n1 / dk; hq = n1 / dq; }
+    if (left > 1) fetch(n1, b1, hk, hq, next);
+    if (n != head) {
+      // B fragments: a word of W holds two adjacent columns of a row, the fragment wants two adjacent rows
+      // of a column: one 8 x 8 transpose per register
+      const uint16_t *w = Wg + (size_t)n * V * V;
+#pragma unroll
+      for (int kt = 0; kt < KT; ++kt)
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+            W[kt][nt][h] = movmatrix_trans(*reinterpret_cast<const uint32_t *>(w + dec_col(16 * kt + 8 * h + g) * V + dec_col(8 * nt + 2 * c)));
+      head = n;
+    }
+    const float f = gate_value(a.gate_kind, cur.gate, a.alpha ? a.alpha[n] : 1.f, a.beta ? a.beta[n] : 0.f, nullptr);
+    float part[SEG];
+#pragma unroll
+    for (int e = 0; e < SEG; ++e) part[e] = 0.f;
+#pragma unroll 1
+    for (int s = 0; s < slabs; ++s) {
+      const uint32_t kk = __shfl_sync(0xffffffffu, s < 4 ? cur.k[0] : cur.k[1], 4 * g + (s & 3));
+      const uint32_t qq = __shfl_sync(0xffffffffu, s < 4 ? cur.q[0] : cur.q[1], 4 * g + (s & 3));
+      const float k0 = __uint_as_float(kk << 16), k1 = __uint_as_float(kk & 0xffff0000u);
+      const float q0 = __uint_as_float(qq << 16), q1 = __uint_as_float(qq & 0xffff0000u);
+      asm volatile("cp.async.wait_group %0;" ::"n"(kStages - 1) : "memory");
+      // rows g and g + 8 of the slab in accumulator layout
+      float H[NT][4];
+      const uint32_t src = ring_sa + (uint32_t)st * Cfg::kSlabBytes;
+#pragma unroll
+      for (int x = 0; x < NX; ++x) {
+        const float4 t0 = lds128(src + 1024u * x), t1 = lds128(src + 1024u * x + 512u);
         H[2 * x][0] = t0.x; H[2 * x][1] = t0.y; H[2 * x + 1][0] = t0.z; H[2 * x + 1][1] = t0.w;
         H[2 * x][2] = t1.x; H[2 * x][3] = t1.y; H[2 * x + 1][2] = t1.z; H[2 * x + 1][3] = t1.w;
       }
-      const float k0 = __bfloat162float(kg[((size_t)b * a.Nk + hk) * K + r0]), k1 = __bfloat162float(kg[((size_t)b * a.Nk + hk) * K + r0 + 8]);
-      const float q0 = __bfloat162float(qg[((size_t)b * a.Nq + hq) * K + r0]), q1 = __bfloat162float(qg[((size_t)b * a.Nq + hq) * K + r0 + 8]);
-      const float f = gate_value(a.gate_kind, a.gate[bn], a.alpha ? a.alpha[n] : 1.f, a.beta ? a.beta[n] : 0.f, nullptr);
-      // P = k v^T + H W
+      request(st);   // the stage is read (by this lane, which alone uses its part of it)
+      if (++st == kStages) st = 0;
+      // P = k v^T + H W   (Eq. 1 before the non-linearity)
       float P[NT][4];
 #pragma unroll
       for (int x = 0; x < NX; ++x) {
-        const uint2 vr = *reinterpret_cast<const uint2 *>(vg + bn * V + 16 * x + 4 * c);
-        const float v0 = __uint_as_float(vr.x << 16), v1 = __uint_as_float(vr.x & 0xffff0000u);
-        const float v2 = __uint_as_float(vr.y << 16), v3 = __uint_as_float(vr.y & 0xffff0000u);
-        P[2 * x][0] = k0 * v0; P[2 * x][1] = k0 * v1; P[2 * x][2] = k1 * v0; P[2 * x][3] = k1 * v1;
-        P[2 * x + 1][0] = k0 * v2; P[2 * x + 1][1] = k0 * v3; P[2 * x + 1][2] = k1 * v2; P[2 * x + 1][3] = k1 * v3;
+        const float2 va = make_float2(__uint_as_float(cur.v[x].x << 16), __uint_as_float(cur.v[x].x & 0xffff0000u));
+        const float2 vb = make_float2(__uint_as_float(cur.v[x].y << 16), __uint_as_float(cur.v[x].y & 0xffff0000u));
+        P[2 * x][0] = k0 * va.x; P[2 * x][1] = k0 * va.y; P[2 * x][2] = k1 * va.x; P[2 * x][3] = k1 * va.y;
+        P[2 * x + 1][0] = k0 * vb.x; P[2 * x + 1][1] = k0 * vb.y; P[2 * x + 1][2] = k1 * vb.x; P[2 * x + 1][3] = k1 * vb.y;
       }
 #pragma unroll
       for (int kt = 0; kt < KT; ++kt) {
-        const uint32_t Ak[4] = {pack_bf16(H[2 * kt][0], H[2 * kt][1]), pack_bf16(H[2 * kt][2], H[2 * kt][3]),
-                                pack_bf16(H[2 * kt + 1][0], H[2 * kt + 1][1]), pack_bf16(H[2 * kt + 1][2], H[2 * kt + 1][3])};
+        uint32_t hi[4], lo[4];
+        a_fragment<NT>(H, kt, hi, lo);
 #pragma unroll
         for (int nt = 0; nt < NT; ++nt) {
-          const uint2 wv = Wf[(kt * NT + nt) * 32 + lane];
-          mma_bf16_16816(P[nt], Ak, wv.x, wv.y);
+          mma_bf16_16816(P[nt], hi, W[kt][nt][0], W[kt][nt][1]);
+          if constexpr (Cfg::kSplit) mma_bf16_16816(P[nt], lo, W[kt][nt][0], W[kt][nt][1]);
         }
       }
-      float part[SEG];
-#pragma unroll
-      for (int nt = 0; nt < NT; ++nt) {
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          const float z = tanh_approx(P[nt][r]);        // Eq. 1
-          H[nt][r] = fmaf(f, H[nt][r] - z, z);          // Eq. 2
-        }
-        part[2 * nt] = fmaf(q1, H[nt][2], q0 * H[nt][0]);       // Eq. 3, this thread's two rows
-        part[2 * nt + 1] = fmaf(q1, H[nt][3], q0 * H[nt][1]);
-      }
+      float *dst = state + bn * KV + (size_t)(16 * s + g) * V + 4 * c;
 #pragma unroll
       for (int x = 0; x < NX; ++x) {
-        *reinterpret_cast<float4 *>(hrow0 + 16 * x + 4 * c) = make_float4(H[2 * x][0], H[2 * x][1], H[2 * x + 1][0], H[2 * x + 1][1]);
-        *reinterpret_cast<float4 *>(hrow1 + 16 * x + 4 * c) = make_float4(H[2 * x][2], H[2 * x][3], H[2 * x + 1][2], H[2 * x + 1][3]);
-      }
-      // column sums over the warp's 16 rows; idx = 2nt+e of a thread <-> memory column 16(idx>>2)+4c+(idx&3)
-      reduce_over_rows<SEG>(part, lane);
-      using RO = RowReduceOut<V>;
-      if (RO::owner(lane)) {
-        const int idx0 = (g >> (3 - RO::R)) * RO::CNT;
 #pragma unroll
-        for (int j = 0; j < RO::CNT; ++j) {
-          const int idx = idx0 + j;
-          const int col = V == 16 ? 4 * c + idx : 16 * (idx >> 2) + 4 * c + (idx & 3);
-          yp[col] = part[j];
-        }
+        for (int nt = 2 * x; nt < 2 * x + 2; ++nt)
+#pragma unroll
+          for (int r = 0; r < 4; ++r) {
+            const float z = tanh_approx(P[nt][r]);        // Eq. 1
+            H[nt][r] = fmaf(f, H[nt][r] - z, z);          // Eq. 2
+          }
+        *reinterpret_cast<float4 *>(dst + 16 * x) = make_float4(H[2 * x][0], H[2 * x][1], H[2 * x + 1][0], H[2 * x + 1][1]);
+        *reinterpret_cast<float4 *>(dst + 16 * x + 8 * V) = make_float4(H[2 * x][2], H[2 * x][3], H[2 * x + 1][2], H[2 * x + 1][3]);
+#pragma unroll
+        for (int nt = 2 * x; nt < 2 * x + 2; ++nt)
+#pragma unroll
+          for (int e = 0; e < 2; ++e) part[2 * nt + e] = fmaf(q0, H[nt][e], fmaf(q1, H[nt][2 + e], part[2 * nt + e]));   // Eq. 3, this thread's two rows
       }
     }
-    __syncthreads();
-    // y = sum over the unit's warps (+ w_r (.) v)
-    for (int x = tid; x < GPI * V; x += blockDim.x) {
-      const int gi = x / V, j = x % V;
-      const int bb = (int)(task % tasks_per_head) * GPI + gi;
-      if (bb < B) {
-        const float *p = ypart + (size_t)(((it & 1) * GPI + gi) * WPU) * V + j;
-        float s = 0.f;
-        for (int w = 0; w < WPU; ++w) s += p[(size_t)w * V];
-        const size_t bn = (size_t)bb * N + n;
-        if (wr) s = fmaf(__bfloat162float(wr[(size_t)n * V + j]), __bfloat162float(vg[bn * V + j]), s);
-        yg[bn * V + j] = __float2bfloat16_rn(s);
+    // column sums over the unit's rows; idx = 2nt+e of a thread <-> memory column 16(idx>>2)+4c+(idx&3)
+    reduce_over_rows<SEG>(part, lane);
+    using RO = RowReduceOut<V>;
+    if (RO::owner(lane)) {
+      const int idx0 = (g >> (3 - RO::R)) * RO::CNT, col = 16 * (idx0 >> 2) + 4 * c + (idx0 & 3);
+      if (wr) {
+#pragma unroll
+        for (int j = 0; j < RO::CNT; ++j)
+          part[j] = fmaf(__bfloat162float(wr[(size_t)n * V + col + j]), __bfloat162float(vg[bn * V + col + j]), part[j]);
       }
+      if constexpr (RO::CNT == 2) *reinterpret_cast<uint32_t *>(yg + bn * V + col) = pack_bf16(part[0], part[1]);
+      else yg[bn * V + col] = __float2bfloat16_rn(part[0]);
     }
+    n = n1; b = b1;
   }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
 
 template <int V>
 cudaError_t launch_decode_v(const ScanArgs &a, cudaStream_t s) {
-  const int WPU = a.K / 16;
-  const int GPI = WPU >= 8 ? 1 : 8 / WPU;   // units taken by a CTA at a time
-  const int tasks_per_head = (a.B + GPI - 1) / GPI;
-  const long ntasks = (long)a.N * tasks_per_head;
-  const int sms = sm_count();
-  const int grid = (int)(ntasks < sms ? ntasks : sms);
-  const size_t smem = 16 + (size_t)(V / 16) * (V / 8) * 32 * 8 + sizeof(float) * 2 * GPI * WPU * V   // barriers, W, y partials
-                      + sizeof(float) * 2 * (size_t)GPI * a.K * V;                                   // two stages of states
-  cudaError_t e = allow_smem(decode_bf16_kernel<V>, smem);
+  const cudaError_t e = allow_smem(decode_bf16_kernel<V>, DecCfg<V>::kSmem);
   if (e != cudaSuccess) return e;
-  decode_bf16_kernel<V><<<grid, 256, smem, s>>>(a, WPU, GPI, tasks_per_head);
+  const long units = (long)a.B * a.N, room = sm_count(), grid = units < room ? units : room, warps = grid * DecCfg<V>::kWarps;
+  decode_bf16_kernel<V><<<(unsigned)grid, 32 * DecCfg<V>::kWarps, DecCfg<V>::kSmem, s>>>(a, (int)(units / warps), (int)(units % warps));
   return cudaGetLastError();
 }
 
 }  // namespace
 
-// The tcgen05 kernel takes the shapes whose states stack into a 128-row tile; the mma.sync kernel
-// above covers the rest.  M2RNN_DECODE_VARIANT=legacy forces the latter (benchmarking only).
+// V = 128 goes to the tcgen05 kernel: there a slab's 256 mma.sync take longer than its bytes need (2.1 GB of
+// state: 622 us with W shared through shared memory, 395 there).  At V = 64 they do not (210 MB: 44 us
+// here, 61 there).
 cudaError_t launch_decode_bf16(const ScanArgs &a, cudaStream_t s) {
-  const char *variant = getenv("M2RNN_DECODE_VARIANT");
-  if (decode_tc_supported(a) && !(variant && !strcmp(variant, "legacy"))) return launch_decode_tc_bf16(a, s);
   switch (a.V) {
     case 16: return launch_decode_v<16>(a, s);
     case 32: return launch_decode_v<32>(a, s);
     case 64: return launch_decode_v<64>(a, s);
-    case 128: return launch_decode_v<128>(a, s);
-    default: return cudaErrorInvalidValue;
+    default: return launch_decode_tc_bf16(a, s);
   }
 }
 

@@ -1,4 +1,4 @@
-// bf16 decoding step (Eq. 1-3 once on a cached fp32 state) on the 5th-generation tensor cores.
+// bf16 decoding step (Eq. 1-3 once on a cached fp32 state) on the 5th-generation tensor cores, V = 128.
 //
 // At decode time the K rows of every (b,n) state are independent rows of one product per head:
 // [B*K, V] x [V, V].  A CTA stacks the states of 128/K units of one head into an M = 128 tile and
@@ -9,13 +9,18 @@
 //   - the staged fp32 tile is already the canonical K-major 128-byte-swizzled layout of a 32-bit
 //     operand, so it is the A operand as it stands (the tensor core reads it as tf32, which keeps
 //     three more mantissa bits of the state than a bf16 copy would, and no conversion pass runs);
-//   - one thread issues the V/8 MMAs and commits them to an mbarrier;
-//   - every thread then owns one state row and half of its columns: tcgen05.ld, + k_i v^T, tanh,
-//     gate against the staged fp32 row, write H_t back in place (global) and into the stage;
+//   - a warp of its own issues the V/8 MMAs as soon as a tile has landed, into one of two accumulators;
+//   - each of 512 compute threads then owns one state row and a quarter of its columns: tcgen05.ld,
+//     + k_i v^T, tanh, gate against the staged fp32 row, H_t back into the stage, from where TMA
+//     stores it in place;
 //   - the readout y = H_t^T q is a column sum over the stage.
 // Persistent CTAs walk (head, batch) tasks in head-major order; W_n^T is rebuilt in shared memory
 // (K-major B tile) only when the head changes.  Every wait is bounded; a wait that runs out ends
 // the CTA through the common exit, which frees the tensor memory.
+// What bounds it: HBM with many tasks per SM (512 x 32 states of 64 KB, read and written: 352 us, 6.1 TB/s);
+// with few, a task's chain of barriers.  With eight compute warps, the MMAs issued by one of them
+// (which waited for the next tile before its own readout) and divisions in the vectors' addresses a
+// task took 6 300 cycles whatever its bytes: 397 us there, 64 us for 1 800 states of 48 KB (now 42).
 #include <cuda.h>
 
 #include "device_common.cuh"
@@ -96,15 +101,15 @@ struct TcSmem {
   // offsets from the 1024-byte aligned base
   static constexpr uint32_t oB = 0, oStage = oB + b_bytes, oVec = oStage + 2 * stage_bytes;
   // vectors (two buffers, the next task's are fetched a task ahead): k [128], q [128], f [128] per
-  // row, v [128/K <= 8][V]; then the warps' readout partials [8][V]
+  // row, v [128/K <= 8][V]; then (two buffers) the readout's partials per 16 rows [8][V]
   static constexpr uint32_t vec_floats = 3 * kM + 8 * V;
-  static constexpr uint32_t vec_bytes = (2 * vec_floats + 8 * V) * 4;
-  static constexpr uint32_t oBar = oVec + vec_bytes;          // 8 mbarriers, tmem slot, flag
+  static constexpr uint32_t vec_bytes = 2 * (vec_floats + 8 * V) * 4;
+  static constexpr uint32_t oBar = oVec + vec_bytes;          // 9 mbarriers, tmem slot
   static constexpr uint32_t total = oBar + 128 + 1024;         // + slack for the alignment of the base
 };
 
-constexpr int kComputeThreads = 256;            // 8 compute warps ...
-constexpr int kThreads = kComputeThreads + 32;   // ... and one warp that moves the states
+constexpr int kComputeThreads = 512;            // 16 compute warps,
+constexpr int kThreads = kComputeThreads + 64;   // one warp that moves the states and one that issues the MMAs
 
 // Barrier 1: the compute warps only (the mover never joins it), plain or with an AND over a
 // per-thread predicate.
@@ -120,35 +125,35 @@ template <int V>
 __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(ScanArgs a, int GPI, int tasks_per_head,
                                                                 const __grid_constant__ CUtensorMap state_map) {
   using S = TcSmem<V>;
-  constexpr int HC = V / 2;             // columns per thread in the epilogue
+  static_assert(V == 128, "an epilogue warp takes 32 of 128 columns");
+  constexpr int kCW = kComputeThreads / 32;
   extern __shared__ unsigned char smem_dyn[];
   // the swizzled tiles want a 1024-byte aligned base
   const uint32_t base_sa = (smem_u32(smem_dyn) + 1023u) & ~1023u;
   unsigned char *base = smem_dyn + (base_sa - smem_u32(smem_dyn));
   float *stage = reinterpret_cast<float *>(base + S::oStage);
   float *vecs = reinterpret_cast<float *>(base + S::oVec);
-  float *ypart = vecs + 2 * S::vec_floats;                  // [8 warps][V]
+  float *ypart = vecs + 2 * S::vec_floats;                  // [2][8][V]
   uint64_t *full = reinterpret_cast<uint64_t *>(base + S::oBar);   // [2] a task's states have landed in the stage
   uint64_t *mma_done = full + 2;                                    // [2] one per accumulator
-  uint64_t *epi_done = mma_done + 2;                                // [2] H_t of the task is in the stage (8 warps arrive)
-  uint64_t *stage_free = epi_done + 2;                              // [2] no compute warp reads the stage any more (8 arrive)
-  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(stage_free + 2);
-  volatile uint32_t *early_flag = tmem_slot + 1;   // the next task's MMAs are already in flight
+  uint64_t *epi_done = mma_done + 2;                                // [2] H_t of the task is in the stage (the compute warps arrive)
+  uint64_t *stage_free = epi_done + 2;                              // [2] no compute warp reads the stage any more (likewise)
+  uint64_t *b_ready = stage_free + 2;                               // the B tile holds the next head's W (likewise)
+  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(b_ready + 1);
 
   const int K = a.K, N = a.N, B = a.B;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const __nv_bfloat16 *qg = static_cast<const __nv_bfloat16 *>(a.q), *kg = static_cast<const __nv_bfloat16 *>(a.k);
-  const __nv_bfloat16 *vg = static_cast<const __nv_bfloat16 *>(a.v), *wr = static_cast<const __nv_bfloat16 *>(a.w_r);
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+  const __nv_bfloat16 *wr = static_cast<const __nv_bfloat16 *>(a.w_r);
   __nv_bfloat16 *yg = static_cast<__nv_bfloat16 *>(a.y);
 
   if (tid == 0) {
     for (int s = 0; s < 2; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&mma_done[s], 1);
-      mbar_init(&epi_done[s], kComputeThreads / 32);
-      mbar_init(&stage_free[s], kComputeThreads / 32);
+      mbar_init(&epi_done[s], kCW);
+      mbar_init(&stage_free[s], kCW);
     }
-    *early_flag = 0u;
+    mbar_init(b_ready, kCW);
     fence_mbar_init();
   }
   if (warp == 0) {   // 2 x V columns of tensor memory: two accumulators, used by alternate tasks
@@ -161,14 +166,14 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(ScanArgs a, int 
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem_base = *tmem_slot;
 
-  // Persistent CTA: tasks [t_begin, t_end) in head-major order; task -> (head n, batch group tb),
-  // stepped without divisions
-  const long ntasks = (long)N * tasks_per_head;
-  const long t_begin = ntasks * blockIdx.x / gridDim.x, t_end = ntasks * (blockIdx.x + 1) / gridDim.x;
-  const int n0 = (int)(t_begin / tasks_per_head), tb0 = (int)(t_begin % tasks_per_head);
+  // Persistent CTA: tasks in head-major order; task -> (head n, batch group tb), stepped without divisions
+  const unsigned ntasks = (unsigned)N * tasks_per_head, per = ntasks / gridDim.x, extra = ntasks % gridDim.x;
+  const int count = (int)(per + (blockIdx.x < extra));
+  const unsigned t_begin = blockIdx.x * per + min(blockIdx.x, extra);
+  const int n0 = (int)(t_begin / (unsigned)tasks_per_head), tb0 = (int)(t_begin - (unsigned)n0 * tasks_per_head);
   auto advance = [&](int &n, int &tb) { if (++tb == tasks_per_head) { tb = 0; ++n; } };
 
-  if (warp == kComputeThreads / 32) {
+  if (warp == kCW) {
     // ================================================================ the warp that moves states
     // Per task and 32-column block one box of [K rows][32 columns] per unit of the state viewed as
     // a [B*N*K, V] matrix.  Loads run two tasks ahead, into the stage whose store has drained.
@@ -192,18 +197,17 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(ScanArgs a, int 
       asm volatile("cp.async.bulk.commit_group;" ::: "memory");
     };
     int nl = n0, tbl = tb0, ns = n0, tbs = tb0;   // next task to load / to store
-    long loaded = t_begin;
-    for (int st = 0; st < 2 && loaded < t_end; ++st, ++loaded) { load_task(nl, tbl, st); advance(nl, tbl); }
+    int loaded = 0;
+    for (int st = 0; st < 2 && loaded < count; ++st, ++loaded) { load_task(nl, tbl, st); advance(nl, tbl); }
     bool ok = true;
-    int it = 0;
-    for (long task = t_begin; task < t_end; ++task, ++it) {
+    for (int it = 0; it < count; ++it) {
       const int st = it & 1;
       const uint32_t par = (uint32_t)(it >> 1) & 1u;
       // H_t is in the stage (written through the generic proxy, fenced by its writers): store it
       if (!mbar_wait(&epi_done[st], par)) { ok = false; break; }
       store_task(ns, tbs, st);
       advance(ns, tbs);
-      if (loaded < t_end) {
+      if (loaded < count) {
         // the stage is free for the task after next once the readout no longer reads it and the
         // store has read it
         if (!mbar_wait(&stage_free[st], par)) { ok = false; break; }
@@ -216,133 +220,160 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(ScanArgs a, int 
     }
     asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");   // the last stores
     if (!ok) report_timeout(a.dev_status);
+  } else if (warp == kCW + 1) {
+    // ================================================================ the warp that issues the MMAs
+    // A task's product starts as soon as its states have landed, whatever the compute warps are at: its
+    // accumulator is free by then (the stage was reloaded after the epilogue two tasks ago).  A
+    // change of head waits for the B tile.
+    constexpr uint32_t idesc = umma_idesc_tf32(kM, V);
+    int n = n0, tb = tb0, head = -1;
+    uint32_t b_par = 0;
+    bool ok = true;
+    for (int it = 0; it < count; ++it) {
+      const int st = it & 1;
+      if (n != head) {
+        if (!mbar_wait(b_ready, b_par)) { ok = false; break; }
+        b_par ^= 1u;
+        head = n;
+      }
+      if (!mbar_wait(&full[st], (uint32_t)(it >> 1) & 1u)) { ok = false; break; }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      if (lane == 0) {
+        const uint32_t a_sa = base_sa + S::oStage + (uint32_t)st * S::stage_bytes;
+#pragma unroll
+        for (int ks = 0; ks < V / 8; ++ks) {
+          // 8 elements (32 bytes) per step inside a 128-byte block, then the next block
+          const uint32_t koff = (uint32_t)(ks / 4) * 128u * kM + (uint32_t)(ks % 4) * 32u;
+          const uint32_t koffb = (uint32_t)(ks / 4) * 128u * V + (uint32_t)(ks % 4) * 32u;
+          umma_tf32(tmem_base + (uint32_t)st * V, umma_desc_sw128(a_sa + koff), umma_desc_sw128(base_sa + S::oB + koffb), idesc, ks > 0);
+        }
+        umma_commit(&mma_done[st]);
+      }
+      __syncwarp();
+      advance(n, tb);
+    }
+    if (!ok) report_timeout(a.dev_status);
   } else {
     // ================================================================ compute warps
-    // Per-row scalars (threads 0..127: k_i, q_i, f of the row's unit) and the units' v vectors
-    // (threads 128..255) of a task, fetched into registers a task ahead and parked in shared
-    // memory when the current task no longer reads that buffer.
-    constexpr int kVPer = 8 * V / 128;   // v entries per thread at most (8 units)
+    // Per-row scalars (threads 0..127: k_i, q_i, f of the row's unit) and the units' v vectors (the
+    // other threads) of a task, fetched into registers at the start of the task before and parked
+    // in shared memory before that task's last barrier.
+    constexpr int kVThreads = kComputeThreads - kM, kVPer = (8 * V + kVThreads - 1) / kVThreads;
     const int dq = N / a.Nq, dk = N / a.Nk;
     const int my_u = (tid & (kM - 1)) / K, my_r = (tid & (kM - 1)) % K;
+    const uint16_t *qg = static_cast<const uint16_t *>(a.q), *kg = static_cast<const uint16_t *>(a.k), *vg = static_cast<const uint16_t *>(a.v);
     // raw values only: nothing may depend on a load before the task that issued it is over
-    struct VecRegs { uint16_t k, q; float gate; uint16_t v[kVPer]; int n; };
-    auto fetch_vecs = [&](int n, int tb, VecRegs &o) {
+    struct VecRegs { uint16_t k, q; float gate; uint16_t v[kVPer]; };
+    auto fetch_vecs = [&](int n, int tb, int hk, int hq, VecRegs &o) {
       const int b0 = tb * GPI;
-      o.n = n;
       o.k = o.q = 0; o.gate = 0.f;
       if (tid < kM) {
         const int bb = b0 + my_u;
         if (my_u < GPI && bb < B) {
-          o.k = reinterpret_cast<const uint16_t *>(kg)[((size_t)bb * a.Nk + n / dk) * K + my_r];
-          o.q = reinterpret_cast<const uint16_t *>(qg)[((size_t)bb * a.Nq + n / dq) * K + my_r];
+          o.k = kg[((size_t)bb * a.Nk + hk) * K + my_r];
+          o.q = qg[((size_t)bb * a.Nq + hq) * K + my_r];
           o.gate = a.gate[(size_t)bb * N + n];
         }
       } else {
 #pragma unroll
         for (int m = 0; m < kVPer; ++m) {
-          const int x = tid - kM + m * kM, u = x / V, bb = b0 + u;
-          o.v[m] = (x < GPI * V && bb < B) ? reinterpret_cast<const uint16_t *>(vg)[((size_t)bb * N + n) * V + (x % V)] : (uint16_t)0;
+          const int x = tid - kM + m * kVThreads, bb = b0 + x / V;
+          o.v[m] = (x < GPI * V && bb < B) ? vg[((size_t)bb * N + n) * V + (x % V)] : (uint16_t)0;
         }
       }
     };
-    const float *alpha = a.alpha, *beta = a.beta;
-    auto park_vecs = [&](int buf, const VecRegs &o) {
+    auto park_vecs = [&](int buf, int n, const VecRegs &o) {
       float *vb = vecs + (size_t)buf * S::vec_floats;
       if (tid < kM) {
         vb[tid] = __uint_as_float((uint32_t)o.k << 16);
         vb[kM + tid] = __uint_as_float((uint32_t)o.q << 16);
         // rows of absent units carry gate 0 -> some f; their results are never used
-        vb[2 * kM + tid] = gate_value(a.gate_kind, o.gate, alpha ? alpha[o.n] : 1.f, beta ? beta[o.n] : 0.f, nullptr);
+        vb[2 * kM + tid] = gate_value(a.gate_kind, o.gate, a.alpha ? a.alpha[n] : 1.f, a.beta ? a.beta[n] : 0.f, nullptr);
       } else {
 #pragma unroll
         for (int m = 0; m < kVPer; ++m) {
-          const int x = tid - kM + m * kM;
+          const int x = tid - kM + m * kVThreads;
           if (x < GPI * V) vb[3 * kM + x] = __uint_as_float((uint32_t)o.v[m] << 16);
         }
       }
     };
-    if (t_begin < t_end) {
-      VecRegs first;
-      fetch_vecs(n0, tb0, first);
-      park_vecs(0, first);
-    }
-
-    constexpr uint32_t idesc = umma_idesc_tf32(kM, V);
-    // the V/8 MMAs of the task whose states sit in stage st, into accumulator st (one thread)
-    auto issue_mmas = [&](int st) {
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t a_sa = base_sa + S::oStage + (uint32_t)st * S::stage_bytes;
+    // B tile = W_n^T widened to fp32, K-major: row j holds W[:, j]; element (j, l) sits in block l/32 at
+    // row j, 16-byte chunk ((l%32)/4) ^ (j%8), like the rows of a stage.  A thread takes V V / 4096 pieces
+    // of eight adjacent columns of a row of W, a warp's lanes 32 adjacent rows (each of its stores
+    // then covers all banks).  The pieces of the next head are loaded at the start of the last task of
+    // the head before and stored after that task's product, so that a change of head costs the stores
+    // only (loading two bytes at a time where they were needed cost 3 us).
+    constexpr int kWPer = V * V / 8 / kComputeThreads;
+    uint4 wreg[kWPer];
+    auto load_w = [&](int n) {
+      const uint16_t *w = static_cast<const uint16_t *>(a.W) + (size_t)n * V * V;
 #pragma unroll
-      for (int ks = 0; ks < V / 8; ++ks) {
-        // 8 elements (32 bytes) per step inside a 128-byte block, then the next block
-        const uint32_t koff = (uint32_t)(ks / 4) * 128u * kM + (uint32_t)(ks % 4) * 32u;
-        const uint32_t koffb = (uint32_t)(ks / 4) * 128u * V + (uint32_t)(ks % 4) * 32u;
-        umma_tf32(tmem_base + (uint32_t)st * V, umma_desc_sw128(a_sa + koff), umma_desc_sw128(base_sa + S::oB + koffb), idesc, ks > 0);
+      for (int i = 0; i < kWPer; ++i) {
+        const int x = tid + i * kComputeThreads, l = x % V, j0 = (x / V) * 8;
+        wreg[i] = *reinterpret_cast<const uint4 *>(w + l * V + j0);
       }
-      umma_commit(&mma_done[st]);
     };
-    int cur_head = -1, it = 0, n = n0, tb = tb0;
+    auto store_w = [&]() {
+#pragma unroll
+      for (int i = 0; i < kWPer; ++i) {
+        const int x = tid + i * kComputeThreads, l = x % V, j0 = (x / V) * 8;
+        const uint32_t u[4] = {wreg[i].x, wreg[i].y, wreg[i].z, wreg[i].w};
+        unsigned char *dst = base + S::oB + (uint32_t)(l / 32) * (V * 128) + (uint32_t)j0 * 128 + 4u * (l & 3);
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+          *reinterpret_cast<uint32_t *>(dst + e * 128 + ((((l % 32) / 4) ^ e) << 4)) = (e & 1) ? (u[e >> 1] & 0xffff0000u) : (u[e >> 1] << 16);
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy writes -> visible to the tensor core
+      __syncwarp();
+      if (lane == 0) mbar_arrive(b_ready);
+    };
+    int n = n0, tb = tb0, hk = n / dk, hq = n / dq;
+    load_w(n);
+    VecRegs next;
+    fetch_vecs(n, tb, hk, hq, next);
+    store_w();
+    park_vecs(0, n, next);
+    compute_sync();
+
+    const int i = 32 * (warp & 3) + lane, quarter = warp >> 2, u_i = i / K, spu = K / 16;
     bool failed = false;
-    bool early = false;   // this task's MMAs were issued during the previous one
-    for (long task = t_begin; task < t_end; ++task, ++it) {
+    for (int it = 0; it < count; ++it) {
       const int st = it & 1;
       const uint32_t par = (uint32_t)(it >> 1) & 1u;
       const int b0 = tb * GPI;
       const int rows = min(GPI, B - b0) * K;     // live rows of the tile
-      const bool has_next = task + 1 < t_end;
+      const bool has_next = it + 1 < count;
       int n1 = n, tb1 = tb;
       advance(n1, tb1);
-      VecRegs next;
-      if (has_next) fetch_vecs(n1, tb1, next);   // lands while this task is computed
-      if (n != cur_head) {
-        // B tile = W_n^T widened to fp32, K-major: row j holds W[:, j]; element (j, l) sits in block
-        // l/32 at row j, 16-byte chunk ((l%32)/4) ^ (j%8), like the rows of a stage
-        const uint16_t *w = reinterpret_cast<const uint16_t *>(a.W) + (size_t)n * V * V;
-        for (int x = tid; x < V * V / 4; x += kComputeThreads) {
-          const int j = x % V, l0 = (x / V) * 4;
-          uint32_t p[4];
-#pragma unroll
-          for (int e = 0; e < 4; ++e) p[e] = (uint32_t)w[(l0 + e) * V + j] << 16;
-          const uint32_t off = S::oB + (uint32_t)(l0 / 32) * (V * 128) + (uint32_t)j * 128 + ((((l0 % 32) / 4) ^ (j & 7)) << 4);
-          *reinterpret_cast<uint4 *>(base + off) = make_uint4(p[0], p[1], p[2], p[3]);
-        }
-        cur_head = n;
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy writes -> visible to the tensor core
-      }
+      const bool new_head = has_next && n1 != n;
+      if (n1 != n) { hk = n1 / dk; hq = n1 / dq; }
+      if (has_next) fetch_vecs(n1, tb1, hk, hq, next);   // lands while this task is computed
+      if (new_head) load_w(n1);
       const float *kvec = vecs + (size_t)st * S::vec_floats, *qvec = kvec + kM, *fvec = qvec + kM, *vvec = fvec + kM;
-      // the task's states have landed (this barrier also orders the B tile's writes before the MMAs)
-      if (!compute_sync_and(mbar_wait(&full[st], par))) { failed = true; break; }
-      float *sg = stage + (size_t)st * (kM * V);
-      if (tid == 0 && !early) issue_mmas(st);
-      if (!compute_sync_and(mbar_wait(&mma_done[st], par))) { failed = true; break; }
+      float *sg = stage + (size_t)st * (kM * V), *yp = ypart + st * 8 * V;
+      const bool ok = mbar_wait(&mma_done[st], par);
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-
-      // epilogue: thread = (row i, column half)
-      {
-        const int i = 32 * (warp & 3) + lane, half = warp >> 2;
-        const int u = i / K;
+      // epilogue: thread = (row i, 32 columns)
+      if (ok) {
         const bool live = i < rows;
         const float ki = kvec[i], f = fvec[i];
-        const float *vrow = vvec + (size_t)(live ? u : 0) * V + half * HC;
+        const float *vrow = vvec + (size_t)(live ? u_i : 0) * V + 32 * quarter;
+        float P[32];
+        tmem_ld32(tmem_base + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(st * V + 32 * quarter), P);
+        if (live) {
 #pragma unroll
-        for (int cb = 0; cb < HC / 32; ++cb) {
-          float P[32];
-          tmem_ld32(tmem_base + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(st * V + half * HC + 32 * cb), P);
-          if (live) {
+          for (int x = 0; x < 8; ++x) {
+            float4 *sp = reinterpret_cast<float4 *>(sg + stage_off<V>(i, 32 * quarter + 4 * x));
+            const float4 h4 = *sp;
+            const float4 v4 = *reinterpret_cast<const float4 *>(vrow + 4 * x);
+            float hn[4];
+            const float hv[4] = {h4.x, h4.y, h4.z, h4.w}, vv[4] = {v4.x, v4.y, v4.z, v4.w};
 #pragma unroll
-            for (int x = 0; x < 8; ++x) {
-              float4 *sp = reinterpret_cast<float4 *>(sg + stage_off<V>(i, half * HC + 32 * cb + 4 * x));
-              const float4 h4 = *sp;
-              const float4 v4 = *reinterpret_cast<const float4 *>(vrow + 32 * cb + 4 * x);
-              float hn[4];
-              const float hv[4] = {h4.x, h4.y, h4.z, h4.w}, vv[4] = {v4.x, v4.y, v4.z, v4.w};
-#pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                const float z = tanh_approx(fmaf(ki, vv[e], P[4 * x + e]));   // Eq. 1
-                hn[e] = fmaf(f, hv[e] - z, z);                               // Eq. 2
-              }
-              *sp = make_float4(hn[0], hn[1], hn[2], hn[3]);
+            for (int e = 0; e < 4; ++e) {
+              const float z = tanh_approx(fmaf(ki, vv[e], P[4 * x + e]));   // Eq. 1
+              hn[e] = fmaf(f, hv[e] - z, z);                               // Eq. 2
             }
+            *sp = make_float4(hn[0], hn[1], hn[2], hn[3]);
           }
         }
       }
@@ -350,52 +381,35 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(ScanArgs a, int 
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // H_t in the stage -> visible to the TMA store
       __syncwarp();
       if (lane == 0) mbar_arrive(&epi_done[st]);
-      compute_sync();
-      if (warp == 0) {
-        // The next task's product does not depend on this one: start it now, into the other
-        // accumulator, so that the tensor core works while the readout runs (unless the head
-        // changes, which rebuilds the B tile first).  The outcome reaches every thread through
-        // shared memory at the next barrier.
-        bool go = has_next && n1 == n;
-        if (go) go = mbar_wait(&full[st ^ 1], (uint32_t)((it + 1) >> 1) & 1u);
-        if (go && lane == 0) issue_mmas(st ^ 1);
-        if (lane == 0) *early_flag = go ? 1u : 0u;
-      }
-      // readout (Eq. 3): y[u][j] = sum over the unit's rows of q_i H_t[i][j].  Each warp sums 16 rows
-      // (all of one unit, K >= 16); then the warps of a unit are added.
+      if (new_head) store_w();   // (the product of this task, the last of its head, is complete)
+      if (!compute_sync_and(ok)) { failed = true; break; }
+      // readout (Eq. 3): y[u][j] = sum over the unit's rows of q_i H_t[i][j].  A warp sums 16 rows (all of
+      // one unit, K >= 16) of 64 columns; then the 16-row sums of a unit are added.
       {
-        // lane = (row group, 32-column block, 16-byte chunk): one 128-byte row of a block per 8 lanes
-        constexpr int NB = V / 32, RG = 4 / NB;
-        const int c8 = lane & 7, m = (lane >> 3) % NB, rg = lane / (8 * NB);
+        const int c8 = lane & 7, m = 2 * (warp & 1) + ((lane >> 3) & 1), r0 = 16 * (warp >> 1) + 8 * (lane >> 4);
         float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-        for (int rr = 0; rr < 16 / RG; ++rr) {
-          const int i = 16 * warp + rg * (16 / RG) + rr;
-          const float qi = qvec[i];
-          const float4 h4 = *reinterpret_cast<const float4 *>(sg + (uint32_t)m * (kM * 32) + (uint32_t)i * 32 + (uint32_t)((c8 ^ (i & 7)) << 2));
+        for (int rr = 0; rr < 8; ++rr) {
+          const float qi = qvec[r0 + rr];
+          const float4 h4 = *reinterpret_cast<const float4 *>(sg + (uint32_t)m * (kM * 32) + (uint32_t)(r0 + rr) * 32 + (uint32_t)((c8 ^ rr) << 2));
           acc.x = fmaf(qi, h4.x, acc.x); acc.y = fmaf(qi, h4.y, acc.y); acc.z = fmaf(qi, h4.z, acc.z); acc.w = fmaf(qi, h4.w, acc.w);
         }
-        if constexpr (RG == 2) {
-          acc.x += __shfl_xor_sync(0xffffffffu, acc.x, 16); acc.y += __shfl_xor_sync(0xffffffffu, acc.y, 16);
-          acc.z += __shfl_xor_sync(0xffffffffu, acc.z, 16); acc.w += __shfl_xor_sync(0xffffffffu, acc.w, 16);
-        }
-        if (rg == 0) *reinterpret_cast<float4 *>(ypart + warp * V + 32 * m + 4 * c8) = acc;
+        acc.x += __shfl_xor_sync(0xffffffffu, acc.x, 16); acc.y += __shfl_xor_sync(0xffffffffu, acc.y, 16);
+        acc.z += __shfl_xor_sync(0xffffffffu, acc.z, 16); acc.w += __shfl_xor_sync(0xffffffffu, acc.w, 16);
+        if (lane < 16) *reinterpret_cast<float4 *>(yp + (warp >> 1) * V + 32 * m + 4 * c8) = acc;
       }
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&stage_free[st]);   // this warp has read the stage for the last time
+      if (lane == 0) mbar_arrive(&stage_free[st]);   // (after the shuffles: this warp has read the stage for the last time)
+      if (has_next) park_vecs(st ^ 1, n1, next);     // last read by the task before, two barriers ago
       compute_sync();
       for (int x = tid; x < GPI * V; x += kComputeThreads) {
         const int u = x / V, j = x % V, bb = b0 + u;
         if (bb < B) {
-          float s = 0.f;
-          for (int w = u * K / 16; w < (u + 1) * K / 16; ++w) s += ypart[w * V + j];
-          if (wr) s = fmaf(__bfloat162float(wr[(size_t)n * V + j]), vvec[x], s);
-          yg[((size_t)bb * N + n) * V + j] = __float2bfloat16_rn(s);
+          float y = 0.f;
+          for (int w = u * spu; w < (u + 1) * spu; ++w) y += yp[w * V + j];
+          if (wr) y = fmaf(__bfloat162float(wr[(size_t)n * V + j]), vvec[x], y);
+          yg[((size_t)bb * N + n) * V + j] = __float2bfloat16_rn(y);
         }
       }
-      if (has_next) park_vecs(st ^ 1, next);
-      early = *early_flag != 0u;   // written before the barrier in front of the final sum
-      compute_sync();   // vectors and partial sums are free again
       n = n1; tb = tb1;
     }
     if (failed) report_timeout(a.dev_status);
@@ -451,12 +465,6 @@ cudaError_t launch_tc(const ScanArgs &a, cudaStream_t s) {
 
 }  // namespace
 
-bool decode_tc_supported(const ScanArgs &a) {
-  return (a.V == 64 || a.V == 128) && (a.K == 16 || a.K == 32 || a.K == 64 || a.K == 128);
-}
-
-cudaError_t launch_decode_tc_bf16(const ScanArgs &a, cudaStream_t s) {
-  return a.V == 64 ? launch_tc<64>(a, s) : launch_tc<128>(a, s);
-}
+cudaError_t launch_decode_tc_bf16(const ScanArgs &a, cudaStream_t s) { return launch_tc<128>(a, s); }
 
 }  // namespace m2rnn

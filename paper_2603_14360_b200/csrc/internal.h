@@ -102,7 +102,6 @@ int bwd_tc_rows_per_cta();
 int bwd_tc_chunk();
 cudaError_t launch_bwd_bf16_tc(const ScanArgs &a, cudaStream_t s);  // scan_bwd_tc.cu
 cudaError_t launch_decode_bf16(const ScanArgs &a, cudaStream_t s);  // decode_bf16.cu: picks a kernel
-bool decode_tc_supported(const ScanArgs &a);                         // decode_tc_bf16.cu
 cudaError_t launch_decode_tc_bf16(const ScanArgs &a, cudaStream_t s);  // decode_tc_bf16.cu: tcgen05 path
 
 // reductions shared by both paths (reduce.cu)

@@ -56,3 +56,20 @@ def test_decode_chain_tracks_the_scan():
     yd = torch.stack(ys, dim=1)
     assert parity.rel_err(yd, y.double().cpu().numpy()) < 1e-2
     assert parity.rel_err(state, hT.double().cpu().numpy()) < 1e-3
+
+
+# where the kernels' splits change: several units per warp with a change of head inside a warp (V <= 64), rings
+# that wrap inside a unit, rows that do not fill the 128-row tile and a head per task (V = 128)
+@pytest.mark.parametrize("shape", [(70, 70, 16, 16), (1, 200, 128, 16), (50, 60, 16, 32), (3, 60, 112, 32), (130, 10, 80, 64), (2, 160, 48, 128),
+                                   (3, 55, 80, 128), (1, 150, 112, 128), (65, 3, 32, 128)], ids=lambda s: "x".join(map(str, s)))
+def test_decode_splits(oracle, shape):
+    B, N, K, V = shape
+    cfg = ScanConfig("split", B=B, T=1, N=N, K=K, V=V, Nq=1, Nk=1, gate_mean=1.0, seed=600 + B)
+    d = inputs.make_inputs(cfg, residual=True)
+    g, f = parity.to_dev(d), inputs.to_f64
+    state = g["h0"].clone()
+    first = lambda t, x: t[x][:, 0]
+    y_ref, s_ref = oracle.decode_step(*(f(first(d, x)) for x in ("q", "k", "v", "gate")), f(d["W"]), f(d["h0"]), w_r=f(d["w_r"]))
+    y = binding.m2rnn_decode_step(*(first(g, x).contiguous() for x in ("q", "k", "v", "gate")), g["W"], state, w_r=g["w_r"])
+    binding.check_device_status()
+    assert parity.rel_err(y, y_ref) < 1e-2 and parity.rel_err(state, s_ref) < 5e-3
