@@ -44,7 +44,7 @@ cudaError_t allow_smem(const void *kernel, size_t bytes) {
   constexpr int kSlots = 1024;   // (kernel, device) pairs: far more than the library has kernels
   struct Entry { std::atomic<uintptr_t> key; std::atomic<int> bytes; };
   static Entry table[kSlots];
-  if (bytes <= 48 * 1024) return cudaSuccess;   // what every kernel may use without asking
+  if (bytes <= 40 * 1024) return cudaSuccess;   // with up to 8 KB of static shared memory: what every kernel may use unasked
   const int dev = current_device();
   Entry *e = nullptr;
   if (dev >= 0 && dev < kMaxDevices) {

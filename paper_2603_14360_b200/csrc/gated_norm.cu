@@ -5,17 +5,18 @@
 //     x = y (.) g,   s = 1 / sqrt(mean x^2 + eps),   out = w (.) x s            (s is cached)
 //     p = w (.) dout, r = sum p x, dx = s p - r s^3 x / d, dy = dx (.) g, dg = dx (.) y (SiLU'),
 //     dw = sum over tokens of dout (.) x s.
-// HBM-bound.  One warp per token (tokens are plentiful and a row is 2-16 KB), 16-byte loads and
-// stores.  Forward: for the common row lengths (d = 256 x 1, 2, 4, 8) a lane keeps its share of the
-// product in registers between the reduction and the scaling; other lengths walk the row twice
-// and the second walk is served by the L1.  No shared memory limits the resident warps there.
-// (A variant that streamed blocks of rows through a shared-memory ring with bulk copies and eight
-// compute warps per SM was slower: the sigmoid makes the row work latency-bound and needs the
-// warps.)  dw: per-warp accumulators in shared memory, one partial per CTA, then a fixed-order
-// second stage.
+// HBM-bound.  One to eight warps share a row so that a lane holds at most three chunks of eight features:
+// that keeps its share of the row, its columns' dw sums and the next row on the way (16-byte cp.async
+// into a ring) within two (backward) to four CTAs per SM, whatever the row length.  One partial of dw per
+// persistent CTA, added by a fixed-order second stage.  16 384 rows: of 1 344 features (84 heads x 16)
+// forward 26 us (5.1 TB/s), backward 39 us (5.6 TB/s); of 1 888, 42 and 69 us (6.0 TB/s).  (A warp per row,
+// rows of other lengths than 256 times a power of two walked twice: 31 and 80, 64 and 141 us.  A CTA
+// per row or four rows at a time, a chunk per thread: 31-42 and 60 us, the barriers show.)
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
+
+#include <type_traits>
 
 #include "internal.h"
 #include "m2rnn.h"
@@ -23,22 +24,10 @@
 namespace m2rnn {
 namespace {
 
-constexpr int kFwdWarps = 8;
-constexpr int kMaxCtas = 592;   // 4 per SM on 148 SMs: also the number of dw partials at most
+constexpr int kMaxCtas = 592;   // 4 per SM on 148 SMs: the number of dw partials at most
 constexpr int kMaxD = 8192;
-constexpr int kBwdSmemBudget = 48 * 1024;   // per-warp dw accumulators of a CTA
+constexpr int kThreads = 256, kWarps = kThreads / 32;
 
-// 8 consecutive elements as floats
-__device__ __forceinline__ void load8(const __nv_bfloat16 *p, float (&f)[8]) {
-  const uint4 r = *reinterpret_cast<const uint4 *>(p);
-  const uint32_t u[4] = {r.x, r.y, r.z, r.w};
-#pragma unroll
-  for (int i = 0; i < 4; ++i) { f[2 * i] = __uint_as_float(u[i] << 16); f[2 * i + 1] = __uint_as_float(u[i] & 0xffff0000u); }
-}
-__device__ __forceinline__ void load8(const float *p, float (&f)[8]) {
-  const float4 a = *reinterpret_cast<const float4 *>(p), b = *reinterpret_cast<const float4 *>(p + 4);
-  f[0] = a.x; f[1] = a.y; f[2] = a.z; f[3] = a.w; f[4] = b.x; f[5] = b.y; f[6] = b.z; f[7] = b.w;
-}
 __device__ __forceinline__ uint32_t pack2(float lo, float hi) {
   const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<const uint32_t *>(&v);
@@ -55,312 +44,307 @@ __device__ __forceinline__ float warp_sum(float v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
-// SiLU and its derivative.  fp32 I/O: sigmoid through ex2.approx + rcp.approx (~1e-6 relative);
-// bf16 I/O: through one tanh.approx (~2^-11, below the rounding of the bf16 result) -- the kernels
-// are bound by the special-function unit as much as by HBM, and this halves its work
+// Sigmoid of a pair.  fp32 I/O: through ex2.approx + rcp.approx (~1e-6 relative); bf16 I/O: through
+// tanh.approx (~2^-11, below the rounding of the bf16 result), half the work of the special-function unit.
+// The arithmetic below is in packed fp32 pairs: the backward kernel is bound by instruction issue as
+// much as by HBM.
 template <typename T>
-__device__ __forceinline__ float silu_t(float x, float *dx) {
-  float sg;
+__device__ __forceinline__ float2 sigmoid2(float2 x) {
   if constexpr (sizeof(T) == 2) {
-    float th;
-    asm("tanh.approx.f32 %0, %1;" : "=f"(th) : "f"(0.5f * x));
-    sg = fmaf(0.5f, th, 0.5f);
+    const float2 h = __fmul2_rn(x, make_float2(0.5f, 0.5f));
+    float2 th;
+    asm("tanh.approx.f32 %0, %1;" : "=f"(th.x) : "f"(h.x));
+    asm("tanh.approx.f32 %0, %1;" : "=f"(th.y) : "f"(h.y));
+    return __ffma2_rn(th, make_float2(0.5f, 0.5f), make_float2(0.5f, 0.5f));
   } else {
-    sg = __fdividef(1.f, 1.f + __expf(-x));
+    return make_float2(__fdividef(1.f, 1.f + __expf(-x.x)), __fdividef(1.f, 1.f + __expf(-x.y)));
   }
-  if (dx) *dx = sg * (1.f + x * (1.f - sg));
-  return x * sg;
 }
 
-// CPL > 0: d = 256 CPL, every lane owns CPL chunks and keeps their products in registers.
-// CPL = 0: any d, the row is read twice.
-template <typename T, int CPL>
-__global__ void __launch_bounds__(kFwdWarps * 32) gated_norm_fwd_kernel(long tokens, int d, const T *__restrict__ y,
-                                                                          const T *__restrict__ g_in, const T *__restrict__ w,
-                                                                          float eps, int use_silu, T *__restrict__ out,
-                                                                          float *__restrict__ rstd) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int chunks = d >> 3;
-  for (long t = (long)blockIdx.x * kFwdWarps + warp; t < tokens; t += (long)gridDim.x * kFwdWarps) {
-    const T *yt = y + t * d, *gt = g_in + t * d;
-    float ss = 0.f;
-    if constexpr (CPL > 0) {
-      float x[CPL][8];
-      {
-        float a[CPL][8], b[CPL][8];
+// eight elements of a row: one (bf16) or two (fp32) pieces of 16 bytes
+template <typename T> struct Raw8 { static constexpr int kPieces = sizeof(T) / 2; uint4 v[kPieces]; };
+__device__ __forceinline__ float2 pair_of(const Raw8<__nv_bfloat16> &r, int i) {
+  const uint32_t u[4] = {r.v[0].x, r.v[0].y, r.v[0].z, r.v[0].w};
+  return make_float2(__uint_as_float(u[i] << 16), __uint_as_float(u[i] & 0xffff0000u));
+}
+__device__ __forceinline__ float2 pair_of(const Raw8<float> &r, int i) {
+  const uint4 q = r.v[i >> 1];
+  return (i & 1) ? make_float2(__uint_as_float(q.z), __uint_as_float(q.w)) : make_float2(__uint_as_float(q.x), __uint_as_float(q.y));
+}
+template <typename T>
+__device__ __forceinline__ Raw8<T> load_raw(const T *p) {
+  Raw8<T> r;
 #pragma unroll
-        for (int j = 0; j < CPL; ++j) { load8(yt + 8 * (lane + 32 * j), a[j]); load8(gt + 8 * (lane + 32 * j), b[j]); }
+  for (int i = 0; i < Raw8<T>::kPieces; ++i) r.v[i] = reinterpret_cast<const uint4 *>(p)[i];
+  return r;
+}
+
+// Whether rows go through the ring (below) or straight to registers: bf16 only.  (fp32 moves twice the bytes
+// per lane, its ring leaves room for one CTA per SM: 4 096 x 1 344 forward 22 us with it, 16 without.)
+__host__ __device__ constexpr bool uses_ring(int elem) { return elem == 2; }
+// CTAs per SM a variant is compiled for and launched with: what its registers and its ring allow.
+// chunks: of a lane at a time (CPL R)
+__host__ __device__ constexpr int resident(bool bwd, int elem, int chunks) {
+  return bwd ? (elem == 4 && chunks > 3 ? 1 : 2) : (chunks <= 2 ? 4 : 3);
+}
+
+// The way of a CTA's warps over the rows.  G warps share a row, a lane takes CPL chunks of eight features of it;
+// the CTA holds 8/G such groups, each with R rows at a time (short rows only).  Rows travel through a
+// ring of two stages in shared memory of which a lane copies (cp.async) and reads its own 16-byte
+// pieces only: the next rows are on their way while these are worked on, a second pass over a row
+// reads them again, and no barrier is needed.
+template <typename T, int CPL, int R, int G, int NTENS>
+struct Walk {
+  static constexpr int NP = Raw8<T>::kPieces, kGroups = kWarps / G;
+  static constexpr bool kRing = uses_ring(sizeof(T));
+  static constexpr int kSmem = kRing ? 2 * NTENS * R * CPL * NP * kThreads * 16 : 0;
+  uint4 *ring;
+  int lane, group, gw;               // gw: warp of the group
+  long t, step, tokens;
+  int d, col;                        // the lane's first column; chunk j is 256 G columns further
+  __device__ __forceinline__ Walk(unsigned char *smem, long tokens_, int d_) {
+    const int tid = threadIdx.x, warp = tid >> 5;
+    lane = tid & 31;
+    group = warp / G; gw = warp % G;
+    ring = reinterpret_cast<uint4 *>(smem) + tid;
+    tokens = tokens_; d = d_;
+    t = ((long)blockIdx.x * kGroups + group) * R;
+    step = (long)gridDim.x * kGroups * R;
+    col = 8 * (32 * gw + lane);
+  }
+  __device__ __forceinline__ bool on(int j) const { return col + 256 * G * j < d; }
+  __device__ __forceinline__ uint4 *piece(int stage, int x, int r, int j, int p) const {
+    return ring + ((((stage * NTENS + x) * R + r) * CPL + j) * NP + p) * kThreads;
+  }
+  __device__ __forceinline__ void fetch(int stage, long t0, const T *const (&src)[NTENS]) const {   // always one group, possibly empty
+    if constexpr (!kRing) return;
 #pragma unroll
-        for (int j = 0; j < CPL; ++j)
+    for (int r = 0; r < R; ++r)
+      if (t0 + r < tokens) {
 #pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            x[j][e] = a[j][e] * (use_silu ? silu_t<T>(b[j][e], nullptr) : b[j][e]);
-            ss = fmaf(x[j][e], x[j][e], ss);
-          }
-      }
-      ss = warp_sum(ss);
-      const float s = 1.f / sqrtf(ss / (float)d + eps);
+        for (int x = 0; x < NTENS; ++x) {
+          const T *p = src[x] + (t0 + r) * d + col;
 #pragma unroll
-      for (int j = 0; j < CPL; ++j) {
-        float wv[8], o[8];
-        load8(w + 8 * (lane + 32 * j), wv);
+          for (int j = 0; j < CPL; ++j)
+            if (on(j))
 #pragma unroll
-        for (int e = 0; e < 8; ++e) o[e] = wv[e] * x[j][e] * s;
-        store8(out + t * d + 8 * (lane + 32 * j), o);
-      }
-      if (rstd && lane == 0) rstd[t] = s;
-    } else {
-#pragma unroll 4
-      for (int c = lane; c < chunks; c += 32) {
-        float a[8], b[8];
-        load8(yt + 8 * c, a);
-        load8(gt + 8 * c, b);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          const float x = a[e] * (use_silu ? silu_t<T>(b[e], nullptr) : b[e]);
-          ss = fmaf(x, x, ss);
+              for (int q = 0; q < NP; ++q)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(piece(stage, x, r, j, q))),
+                             "l"(reinterpret_cast<const uint4 *>(p + 256 * G * j) + q) : "memory");
         }
       }
-      ss = warp_sum(ss);
-      const float s = 1.f / sqrtf(ss / (float)d + eps);
-#pragma unroll 4
-      for (int c = lane; c < chunks; c += 32) {   // the same lane reads the same bytes again: L1 hits
-        float a[8], b[8], wv[8], o[8];
-        load8(yt + 8 * c, a);
-        load8(gt + 8 * c, b);
-        load8(w + 8 * c, wv);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) o[e] = wv[e] * (a[e] * (use_silu ? silu_t<T>(b[e], nullptr) : b[e])) * s;
-        store8(out + t * d + 8 * c, o);
-      }
-      if (rstd && lane == 0) rstd[t] = s;
-    }
-  }
-}
-
-template <typename T, int kWarps>
-__global__ void __launch_bounds__(kWarps * 32) gated_norm_bwd_kernel(long tokens, int d, const T *__restrict__ y,
-                                                                       const T *__restrict__ g_in, const T *__restrict__ w,
-                                                                       const float *__restrict__ rstd, int use_silu,
-                                                                       const T *__restrict__ dout, T *__restrict__ dy,
-                                                                       T *__restrict__ dg_in, float *__restrict__ dw_part) {
-  extern __shared__ __align__(16) float acc_all[];   // [kWarps][d] partial sums of dw
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float *acc = acc_all + (size_t)warp * d;
-  const int chunks = d >> 3;
-  for (int c = lane; c < chunks; c += 32) {
-    *reinterpret_cast<float4 *>(acc + 8 * c) = make_float4(0.f, 0.f, 0.f, 0.f);
-    *reinterpret_cast<float4 *>(acc + 8 * c + 4) = make_float4(0.f, 0.f, 0.f, 0.f);
-  }
-  for (long t = (long)blockIdx.x * kWarps + warp; t < tokens; t += (long)gridDim.x * kWarps) {
-    const T *yt = y + t * d, *gt = g_in + t * d, *dot = dout + t * d;
-    const float s = rstd[t];
-    // r = sum_j w_j dout_j x_j
-    float r = 0.f;
-#pragma unroll 2
-    for (int c = lane; c < chunks; c += 32) {
-      float a[8], b[8], wv[8], dv[8];
-      load8(yt + 8 * c, a);
-      load8(gt + 8 * c, b);
-      load8(w + 8 * c, wv);
-      load8(dot + 8 * c, dv);
-#pragma unroll
-      for (int e = 0; e < 8; ++e) r = fmaf(wv[e] * dv[e], a[e] * (use_silu ? silu_t<T>(b[e], nullptr) : b[e]), r);
-    }
-    r = warp_sum(r);
-    const float k3 = r * s * s * s / (float)d;
-    // second pass over the same row (served by the L1): the gradients
-#pragma unroll 2
-    for (int c = lane; c < chunks; c += 32) {
-      float a[8], b[8], wv[8], dv[8], o1[8], o2[8];
-      load8(yt + 8 * c, a);
-      load8(gt + 8 * c, b);
-      load8(w + 8 * c, wv);
-      load8(dot + 8 * c, dv);
-      float4 w0 = *reinterpret_cast<const float4 *>(acc + 8 * c), w1 = *reinterpret_cast<const float4 *>(acc + 8 * c + 4);
-      float aw[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        float dsl = 1.f;
-        const float g = use_silu ? silu_t<T>(b[e], &dsl) : b[e];
-        const float x = a[e] * g;
-        const float dx = s * wv[e] * dv[e] - k3 * x;
-        o1[e] = dx * g;
-        o2[e] = dx * a[e] * dsl;
-        aw[e] = fmaf(dv[e] * x, s, aw[e]);
-      }
-      store8(dy + t * d + 8 * c, o1);
-      store8(dg_in + t * d + 8 * c, o2);
-      *reinterpret_cast<float4 *>(acc + 8 * c) = make_float4(aw[0], aw[1], aw[2], aw[3]);
-      *reinterpret_cast<float4 *>(acc + 8 * c + 4) = make_float4(aw[4], aw[5], aw[6], aw[7]);
-    }
-  }
-  __syncthreads();
-  // this CTA's partial of dw: the warps' sums in a fixed order
-  for (int j = threadIdx.x; j < d; j += blockDim.x) {
-    float v = 0.f;
-#pragma unroll
-    for (int wi = 0; wi < kWarps; ++wi) v += acc_all[(size_t)wi * d + j];
-    dw_part[(size_t)blockIdx.x * d + j] = v;
-  }
-}
-
-// The same for d = 256 CPL (CPL = 1, 2, 4): a lane owns CPL fixed chunks of every row, keeps the
-// row's inputs in registers as loaded (16 bytes per chunk and tensor for bf16) between the
-// reduction and the gradients, and sums its columns of dw in registers over all its tokens.
-template <typename T> struct Raw8;
-template <> struct Raw8<__nv_bfloat16> {
-  uint4 v;
-  __device__ __forceinline__ void load(const __nv_bfloat16 *p) { v = *reinterpret_cast<const uint4 *>(p); }
-  __device__ __forceinline__ void get(float (&f)[8]) const {
-    const uint32_t u[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) { f[2 * i] = __uint_as_float(u[i] << 16); f[2 * i + 1] = __uint_as_float(u[i] & 0xffff0000u); }
-  }
-};
-template <> struct Raw8<float> {
-  float4 lo, hi;
-  __device__ __forceinline__ void load(const float *p) { lo = *reinterpret_cast<const float4 *>(p); hi = *reinterpret_cast<const float4 *>(p + 4); }
-  __device__ __forceinline__ void get(float (&f)[8]) const {
-    f[0] = lo.x; f[1] = lo.y; f[2] = lo.z; f[3] = lo.w; f[4] = hi.x; f[5] = hi.y; f[6] = hi.z; f[7] = hi.w;
-  }
-};
-
-constexpr int kRegWarps = 8;
-
-template <typename T, int CPL>
-__global__ void __launch_bounds__(kRegWarps * 32) gated_norm_bwd_reg_kernel(long tokens, const T *__restrict__ y,
-                                                                              const T *__restrict__ g_in, const T *__restrict__ w,
-                                                                              const float *__restrict__ rstd, int use_silu,
-                                                                              const T *__restrict__ dout, T *__restrict__ dy,
-                                                                              T *__restrict__ dg_in, float *__restrict__ dw_part) {
-  constexpr int d = 256 * CPL;
-  extern __shared__ __align__(16) float acc_all[];   // [kRegWarps][d]: the warps' sums at the end
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  Raw8<T> wr[CPL];
-  float acc[CPL][8];
-#pragma unroll
-  for (int j = 0; j < CPL; ++j) {
-    wr[j].load(w + 8 * (lane + 32 * j));
-#pragma unroll
-    for (int e = 0; e < 8; ++e) acc[j][e] = 0.f;
-  }
-  // bf16: the next token's three rows are on their way (cp.async into a two-slot ring of the warp, a
-  // lane copies and later reads its own chunks only) while this token is worked on; without that a
-  // warp's loads and its arithmetic took turns and the kernel ran at half of the HBM bandwidth
-  constexpr bool kRing = sizeof(T) == 2;
-  const long t_first = (long)blockIdx.x * kRegWarps + warp, t_step = (long)gridDim.x * kRegWarps;
-  uint4 *ring = reinterpret_cast<uint4 *>(acc_all + (size_t)kRegWarps * d) + (size_t)warp * (2 * 3 * CPL * 32);
-  auto fetch = [&](long t, int slot) {   // always one group, possibly empty
-    if (t < tokens) {
-      const T *src[3] = {y + t * d, g_in + t * d, dout + t * d};
-#pragma unroll
-      for (int x = 0; x < 3; ++x)
-#pragma unroll
-        for (int j = 0; j < CPL; ++j) {
-          const uint32_t dst = (uint32_t)__cvta_generic_to_shared(ring + ((slot * 3 + x) * CPL + j) * 32 + lane);
-          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src[x] + 8 * (lane + 32 * j)) : "memory");
-        }
-    }
     asm volatile("cp.async.commit_group;" ::: "memory");
-  };
-  if constexpr (kRing) fetch(t_first, 0);
-  int slot = 0;
-  for (long t = t_first; t < tokens; t += t_step) {
-    const T *yt = y + t * d, *gt = g_in + t * d, *dot = dout + t * d;
-    Raw8<T> ar[CPL], br[CPL], dr[CPL];
-    if constexpr (kRing) {
-      fetch(t + t_step, slot ^ 1);
-      asm volatile("cp.async.wait_group 1;" ::: "memory");
+  }
+  __device__ __forceinline__ Raw8<T> get(const T *const (&src)[NTENS], int stage, int x, int r, int j) const {
+    Raw8<T> v;
+    if constexpr (!kRing) return t + r < tokens ? load_raw(src[x] + (t + r) * d + col + 256 * G * j) : Raw8<T>{};
 #pragma unroll
-      for (int j = 0; j < CPL; ++j) {
-        ar[j].v = ring[((slot * 3 + 0) * CPL + j) * 32 + lane];
-        br[j].v = ring[((slot * 3 + 1) * CPL + j) * 32 + lane];
-        dr[j].v = ring[((slot * 3 + 2) * CPL + j) * 32 + lane];
+    for (int q = 0; q < NP; ++q) v.v[q] = *piece(stage, x, r, j, q);
+    return v;
+  }
+  // v[r] summed over the group.  red: [2][kWarps][R] floats, used in turn so that one barrier a call is enough
+  __device__ __forceinline__ void row_sums(float (&v)[R], float *red, int buf) const {
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[r] = warp_sum(v[r]);
+    if constexpr (G > 1) {
+      red += (buf * kWarps + group * G) * R;
+      if (lane == 0) {
+#pragma unroll
+        for (int r = 0; r < R; ++r) red[gw * R + r] = v[r];
       }
-      slot ^= 1;
-    } else {
+      asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "n"(32 * G) : "memory");
 #pragma unroll
-      for (int j = 0; j < CPL; ++j) {
-        ar[j].load(yt + 8 * (lane + 32 * j));
-        br[j].load(gt + 8 * (lane + 32 * j));
-        dr[j].load(dot + 8 * (lane + 32 * j));
+      for (int r = 0; r < R; ++r) {
+        v[r] = red[r];
+#pragma unroll
+        for (int w = 1; w < G; ++w) v[r] += red[w * R + r];
       }
-    }
-    const float s = rstd[t];
-    float r = 0.f;   // r = sum_j w_j dout_j x_j
-#pragma unroll
-    for (int j = 0; j < CPL; ++j) {
-      float a[8], b[8], dv[8], wv[8];
-      ar[j].get(a); br[j].get(b); dr[j].get(dv); wr[j].get(wv);
-#pragma unroll
-      for (int e = 0; e < 8; ++e) r = fmaf(wv[e] * dv[e], a[e] * (use_silu ? silu_t<T>(b[e], nullptr) : b[e]), r);
-    }
-    r = warp_sum(r);
-    const float k3 = r * s * s * s / (float)d;
-#pragma unroll
-    for (int j = 0; j < CPL; ++j) {
-      float a[8], b[8], dv[8], wv[8], o1[8], o2[8];
-      ar[j].get(a); br[j].get(b); dr[j].get(dv); wr[j].get(wv);
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        float dsl = 1.f;
-        const float g = use_silu ? silu_t<T>(b[e], &dsl) : b[e];
-        const float x = a[e] * g;
-        const float dx = s * wv[e] * dv[e] - k3 * x;
-        o1[e] = dx * g;
-        o2[e] = dx * a[e] * dsl;
-        acc[j][e] = fmaf(dv[e] * x, s, acc[j][e]);
-      }
-      store8(dy + t * d + 8 * (lane + 32 * j), o1);
-      store8(dg_in + t * d + 8 * (lane + 32 * j), o2);
     }
   }
-  if constexpr (kRing) asm volatile("cp.async.wait_group 0;" ::: "memory");
+};
+
+template <typename T, int CPL, int R, int G>
+__global__ void __launch_bounds__(kThreads, resident(false, sizeof(T), CPL * R)) gated_norm_fwd_kernel(
+    long tokens, int d, const T *__restrict__ y, const T *__restrict__ g_in, const T *__restrict__ w, float eps, int use_silu,
+    T *__restrict__ out, float *__restrict__ rstd) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ float red[2 * kWarps * R];
+  Walk<T, CPL, R, G, 2> wk(smem, tokens, d);
+  const T *const src[2] = {y, g_in};
+  wk.fetch(0, wk.t, src);
+  const float inv_d = 1.f / (float)d;
+  int st = 0;
+  for (; wk.t < tokens; wk.t += wk.step, st ^= 1) {
+    wk.fetch(st ^ 1, wk.t + wk.step, src);
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    float2 x[R][CPL][4];
+    float ss[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      float2 s2 = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int j = 0; j < CPL; ++j)
+        if (wk.on(j)) {
+          const Raw8<T> a = wk.get(src, st, 0, r, j), b = wk.get(src, st, 1, r, j);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            float2 g = pair_of(b, i);
+            if (use_silu) g = __fmul2_rn(g, sigmoid2<T>(g));
+            x[r][j][i] = __fmul2_rn(pair_of(a, i), g);
+            s2 = __ffma2_rn(x[r][j][i], x[r][j][i], s2);
+          }
+        }
+      ss[r] = s2.x + s2.y;
+    }
+    wk.row_sums(ss, red, st);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      if (wk.t + r >= tokens) break;   // (a row past the end: arithmetic on stale shared memory, nothing stored)
+      const float s = 1.f / sqrtf(ss[r] * inv_d + eps);
+#pragma unroll
+      for (int j = 0; j < CPL; ++j)
+        if (wk.on(j)) {
+          const Raw8<T> wv = load_raw(w + wk.col + 256 * G * j);
+          float o[8];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float2 p = __fmul2_rn(__fmul2_rn(pair_of(wv, i), x[r][j][i]), make_float2(s, s));
+            o[2 * i] = p.x; o[2 * i + 1] = p.y;
+          }
+          store8(out + (wk.t + r) * d + wk.col + 256 * G * j, o);
+        }
+      if (rstd && wk.col == 0) rstd[wk.t + r] = s;
+    }
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+}
+
+template <typename T, int CPL, int R, int G>
+__global__ void __launch_bounds__(kThreads, resident(true, sizeof(T), CPL * R)) gated_norm_bwd_kernel(
+    long tokens, int d, const T *__restrict__ y, const T *__restrict__ g_in, const T *__restrict__ w, const float *__restrict__ rstd,
+    int use_silu, const T *__restrict__ dout, T *__restrict__ dy, T *__restrict__ dg_in, float *__restrict__ dw_part) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ float red[2 * kWarps * R];
+  Walk<T, CPL, R, G, 3> wk(smem, tokens, d);
+  const T *const src[3] = {y, g_in, dout};
+  wk.fetch(0, wk.t, src);
+  Raw8<T> wr[CPL];
+  float2 acc[CPL][4];
 #pragma unroll
   for (int j = 0; j < CPL; ++j) {
-    float *p = acc_all + (size_t)warp * d + 8 * (lane + 32 * j);
-    *reinterpret_cast<float4 *>(p) = make_float4(acc[j][0], acc[j][1], acc[j][2], acc[j][3]);
-    *reinterpret_cast<float4 *>(p + 4) = make_float4(acc[j][4], acc[j][5], acc[j][6], acc[j][7]);
+    if (wk.on(j)) wr[j] = load_raw(w + wk.col + 256 * G * j);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) acc[j][i] = make_float2(0.f, 0.f);
   }
+  const float inv_d = 1.f / (float)d;
+  const float2 one = make_float2(1.f, 1.f), mone = make_float2(-1.f, -1.f);
+  int st = 0;
+  for (; wk.t < tokens; wk.t += wk.step, st ^= 1) {
+    float s[R], rs[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) s[r] = wk.t + r < tokens ? rstd[wk.t + r] : 0.f;
+    wk.fetch(st ^ 1, wk.t + wk.step, src);
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    float2 sg[R][CPL][4];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {   // r = sum_j w_j dout_j x_j
+      float2 r2 = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int j = 0; j < CPL; ++j)
+        if (wk.on(j)) {
+          const Raw8<T> a = wk.get(src, st, 0, r, j), b = wk.get(src, st, 1, r, j), dv = wk.get(src, st, 2, r, j);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            float2 g = pair_of(b, i);
+            sg[r][j][i] = one;
+            if (use_silu) { sg[r][j][i] = sigmoid2<T>(g); g = __fmul2_rn(g, sg[r][j][i]); }
+            r2 = __ffma2_rn(__fmul2_rn(pair_of(wr[j], i), pair_of(dv, i)), __fmul2_rn(pair_of(a, i), g), r2);
+          }
+        }
+      rs[r] = r2.x + r2.y;
+    }
+    wk.row_sums(rs, red, st);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      if (wk.t + r >= tokens) break;
+      const float k3 = rs[r] * s[r] * s[r] * s[r] * inv_d;
+      const float2 mk = make_float2(-k3, -k3), s2 = make_float2(s[r], s[r]);
+#pragma unroll
+      for (int j = 0; j < CPL; ++j)
+        if (wk.on(j)) {
+          const Raw8<T> a = wk.get(src, st, 0, r, j), b = wk.get(src, st, 1, r, j), dv = wk.get(src, st, 2, r, j);
+          float o1[8], o2[8];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float2 av = pair_of(a, i), bv = pair_of(b, i), sd = __fmul2_rn(s2, pair_of(dv, i)), q = sg[r][j][i];
+            const float2 g = use_silu ? __fmul2_rn(bv, q) : bv;
+            const float2 x = __fmul2_rn(av, g);
+            const float2 dx = __ffma2_rn(pair_of(wr[j], i), sd, __fmul2_rn(mk, x));           // s w dout - k3 x
+            const float2 p1 = __fmul2_rn(dx, g);
+            float2 p2 = __fmul2_rn(dx, av);
+            if (use_silu) p2 = __fmul2_rn(p2, __ffma2_rn(g, __ffma2_rn(q, mone, one), q));      // SiLU' = sg + g (1 - sg)
+            acc[j][i] = __ffma2_rn(sd, x, acc[j][i]);
+            o1[2 * i] = p1.x; o1[2 * i + 1] = p1.y;
+            o2[2 * i] = p2.x; o2[2 * i + 1] = p2.y;
+          }
+          store8(dy + (wk.t + r) * d + wk.col + 256 * G * j, o1);
+          store8(dg_in + (wk.t + r) * d + wk.col + 256 * G * j, o2);
+        }
+    }
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  // this CTA's partial of dw: the groups' sums in a fixed order, through shared memory (kGroups x d floats)
+  float *sh = reinterpret_cast<float *>(smem);
   __syncthreads();
-  // this CTA's partial of dw: the warps' sums in a fixed order
-  for (int j = threadIdx.x; j < d; j += blockDim.x) {
+#pragma unroll
+  for (int j = 0; j < CPL; ++j)
+    if (wk.on(j))
+#pragma unroll
+      for (int i = 0; i < 4; ++i) *reinterpret_cast<float2 *>(sh + wk.group * d + wk.col + 256 * G * j + 2 * i) = acc[j][i];
+  __syncthreads();
+  for (int c = threadIdx.x; c < d; c += kThreads) {
     float v = 0.f;
 #pragma unroll
-    for (int wi = 0; wi < kRegWarps; ++wi) v += acc_all[(size_t)wi * d + j];
-    dw_part[(size_t)blockIdx.x * d + j] = v;
+    for (int k = 0; k < kWarps / G; ++k) v += sh[k * d + c];
+    dw_part[(size_t)blockIdx.x * d + c] = v;
   }
 }
 
-// dw[j] = sum over the R per-CTA partials, in a fixed order: eight interleaved running sums per
-// column (one per warp of the CTA), then their sum in warp order
-__global__ void __launch_bounds__(256) reduce_partials_kernel(const float *__restrict__ part, float *__restrict__ out, int R, int n) {
-  __shared__ float sm[8][32];
+// dw[j] = sum over the R per-CTA partials, in a fixed order: 32 interleaved running sums per column (one
+// per warp of the CTA), then their sum in warp order
+__global__ void __launch_bounds__(1024) reduce_partials_kernel(const float *__restrict__ part, float *__restrict__ out, int R, int n) {
+  __shared__ float sm[32][33];
   const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
   const int j = blockIdx.x * 32 + lane;
   float v = 0.f;
-  if (j < n)
-    for (int r = grp; r < R; r += 8) v += part[(size_t)r * n + j];
+  if (j < n) {
+#pragma unroll 4
+    for (int r = grp; r < R; r += 32) v += part[(size_t)r * n + j];
+  }
   sm[grp][lane] = v;
   __syncthreads();
-  if (grp == 0 && j < n) {
-    float t = 0.f;
-#pragma unroll
-    for (int g = 0; g < 8; ++g) t += sm[g][lane];
-    out[j] = t;
-  }
+  v = warp_sum(sm[lane][grp]);   // warp grp adds column grp's 32 sums
+  if (lane == 0 && blockIdx.x * 32 + grp < n) out[blockIdx.x * 32 + grp] = v;
 }
 
-// warps per CTA of the backward kernel: as many as the budget for their dw accumulators allows
-int bwd_warps(int d) {
-  if (d == 256 || d == 512 || d == 1024) return kRegWarps;   // the register variant
-  return d * 4 * 8 <= kBwdSmemBudget ? 8 : (d * 4 * 4 <= kBwdSmemBudget ? 4 : (d * 4 * 2 <= kBwdSmemBudget ? 2 : 1));
-}
-
-int grid_for(long tokens, int warps) {
-  const long need = (tokens + warps - 1) / warps;
-  return (int)(need < kMaxCtas ? need : kMaxCtas);
+// How a call is split: warps per row (a lane holds at most three chunks: with four the backward kernel spills at
+// two CTAs per SM; d > 6 144 has no choice), chunks per lane, rows at a time (short rows: as many
+// bytes on their way as four chunks) and persistent CTAs, as many as are resident.
+struct Split { int g, cpl, r, grid; };
+Split split_of(long tokens, int d, bool bwd, int io_dtype) {
+  Split s;
+  const int chunks = d / 8;
+  const int most = io_dtype == M2RNN_F32 ? 64 : 96;   // chunks of a warp
+  s.g = chunks <= most ? 1 : (chunks <= 2 * most ? 2 : (chunks <= 4 * most ? 4 : 8));
+  s.cpl = (chunks + 32 * s.g - 1) / (32 * s.g);
+  s.r = s.g > 1 || s.cpl > 2 ? 1 : (s.cpl == 1 ? 4 : 2);
+  const int sms = sm_count(), per = kWarps / s.g;
+  if (tokens < 8L * sms * per) s.r = 1;
+  const long need = (tokens + per * s.r - 1) / (per * s.r);
+  const long slots = (long)sms * resident(bwd, io_dtype == M2RNN_F32 ? 4 : 2, s.cpl * s.r);
+  s.grid = (int)(need < slots ? need : slots);
+  if (s.grid > kMaxCtas) s.grid = kMaxCtas;
+  return s;
 }
 
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -372,68 +356,47 @@ int check(long tokens, int d, int io_dtype) {
   return M2RNN_OK;
 }
 
+// f(CPL, R, G) as compile-time constants
+template <typename F>
+cudaError_t with_split(const Split &s, F f) {
+#define M2RNN_CASE(C, R_, G_) \
+  if (s.cpl == C && s.r == R_ && s.g == G_) \
+    return f(std::integral_constant<int, C>{}, std::integral_constant<int, R_>{}, std::integral_constant<int, G_>{})
+  M2RNN_CASE(1, 4, 1); M2RNN_CASE(1, 1, 1); M2RNN_CASE(2, 2, 1); M2RNN_CASE(2, 1, 1); M2RNN_CASE(3, 1, 1);
+  M2RNN_CASE(2, 1, 2); M2RNN_CASE(3, 1, 2); M2RNN_CASE(2, 1, 4); M2RNN_CASE(3, 1, 4); M2RNN_CASE(2, 1, 8); M2RNN_CASE(3, 1, 8); M2RNN_CASE(4, 1, 8);
+#undef M2RNN_CASE
+  return cudaErrorInvalidValue;
+}
+
 template <typename T>
 cudaError_t launch_fwd(long tokens, int d, const void *y, const void *g, const void *w, float eps, int silu_on, void *out,
                        float *rstd, cudaStream_t s) {
-  const long need = (tokens + kFwdWarps - 1) / kFwdWarps;
-  const int grid = (int)(need < 148 * 8 ? need : 148 * 8);
-  const T *yp = static_cast<const T *>(y), *gp = static_cast<const T *>(g), *wp = static_cast<const T *>(w);
-  T *op = static_cast<T *>(out);
-  switch (d) {
-    case 256: gated_norm_fwd_kernel<T, 1><<<grid, kFwdWarps * 32, 0, s>>>(tokens, d, yp, gp, wp, eps, silu_on, op, rstd); break;
-    case 512: gated_norm_fwd_kernel<T, 2><<<grid, kFwdWarps * 32, 0, s>>>(tokens, d, yp, gp, wp, eps, silu_on, op, rstd); break;
-    case 1024: gated_norm_fwd_kernel<T, 4><<<grid, kFwdWarps * 32, 0, s>>>(tokens, d, yp, gp, wp, eps, silu_on, op, rstd); break;
-    case 2048: gated_norm_fwd_kernel<T, 8><<<grid, kFwdWarps * 32, 0, s>>>(tokens, d, yp, gp, wp, eps, silu_on, op, rstd); break;
-    default: gated_norm_fwd_kernel<T, 0><<<grid, kFwdWarps * 32, 0, s>>>(tokens, d, yp, gp, wp, eps, silu_on, op, rstd); break;
-  }
-  return cudaGetLastError();
-}
-
-template <typename T, int kWarps>
-cudaError_t launch_bwd_w(long tokens, int d, const void *y, const void *g, const void *w, const float *rstd, int silu_on,
-                         const void *dout, void *dy, void *dg, float *dw_part, cudaStream_t s) {
-  const size_t smem = (size_t)kWarps * d * sizeof(float);
-  cudaError_t e = allow_smem(gated_norm_bwd_kernel<T, kWarps>, smem);
-  if (e != cudaSuccess) return e;
-  gated_norm_bwd_kernel<T, kWarps><<<grid_for(tokens, kWarps), kWarps * 32, smem, s>>>(
-      tokens, d, static_cast<const T *>(y), static_cast<const T *>(g), static_cast<const T *>(w), rstd, silu_on,
-      static_cast<const T *>(dout), static_cast<T *>(dy), static_cast<T *>(dg), dw_part);
-  return cudaGetLastError();
-}
-
-// persistent CTAs for the register variant: as many as are resident at once (its register need
-// grows with CPL), so that the per-CTA prologue and partial of dw are paid once per SM slot
-int reg_grid(long tokens, int cpl) {
-  const long need = (tokens + kRegWarps - 1) / kRegWarps;
-  const long slots = (long)sm_count() * (cpl >= 4 ? 1 : (cpl == 2 ? 2 : 4));
-  return (int)(need < slots ? need : slots);
-}
-
-template <typename T, int CPL>
-cudaError_t launch_bwd_reg(long tokens, const void *y, const void *g, const void *w, const float *rstd, int silu_on,
-                           const void *dout, void *dy, void *dg, float *dw_part, cudaStream_t s) {
-  // the warps' dw sums, then (bf16) the warps' two-slot rings of three rows each
-  const size_t smem = (size_t)kRegWarps * 256 * CPL * sizeof(float) + (sizeof(T) == 2 ? (size_t)kRegWarps * 2 * 3 * 256 * CPL * sizeof(T) : 0);
-  cudaError_t e = allow_smem(gated_norm_bwd_reg_kernel<T, CPL>, smem);
-  if (e != cudaSuccess) return e;
-  gated_norm_bwd_reg_kernel<T, CPL><<<reg_grid(tokens, CPL), kRegWarps * 32, smem, s>>>(
-      tokens, static_cast<const T *>(y), static_cast<const T *>(g), static_cast<const T *>(w), rstd, silu_on,
-      static_cast<const T *>(dout), static_cast<T *>(dy), static_cast<T *>(dg), dw_part);
-  return cudaGetLastError();
+  const Split sp = split_of(tokens, d, false, sizeof(T) == 2 ? M2RNN_BF16 : M2RNN_F32);
+  return with_split(sp, [&](auto C, auto R, auto G) {
+    auto kern = gated_norm_fwd_kernel<T, C(), R(), G()>;
+    constexpr int smem = Walk<T, C(), R(), G(), 2>::kSmem;
+    const cudaError_t e = allow_smem(kern, smem);
+    if (e != cudaSuccess) return e;
+    kern<<<sp.grid, kThreads, smem, s>>>(tokens, d, static_cast<const T *>(y), static_cast<const T *>(g), static_cast<const T *>(w), eps, silu_on,
+                                         static_cast<T *>(out), rstd);
+    return cudaGetLastError();
+  });
 }
 
 template <typename T>
 cudaError_t launch_bwd(long tokens, int d, const void *y, const void *g, const void *w, const float *rstd, int silu_on,
                        const void *dout, void *dy, void *dg, float *dw_part, cudaStream_t s) {
-  if (d == 256) return launch_bwd_reg<T, 1>(tokens, y, g, w, rstd, silu_on, dout, dy, dg, dw_part, s);
-  if (d == 512) return launch_bwd_reg<T, 2>(tokens, y, g, w, rstd, silu_on, dout, dy, dg, dw_part, s);
-  if (d == 1024) return launch_bwd_reg<T, 4>(tokens, y, g, w, rstd, silu_on, dout, dy, dg, dw_part, s);
-  switch (bwd_warps(d)) {
-    case 8: return launch_bwd_w<T, 8>(tokens, d, y, g, w, rstd, silu_on, dout, dy, dg, dw_part, s);
-    case 4: return launch_bwd_w<T, 4>(tokens, d, y, g, w, rstd, silu_on, dout, dy, dg, dw_part, s);
-    case 2: return launch_bwd_w<T, 2>(tokens, d, y, g, w, rstd, silu_on, dout, dy, dg, dw_part, s);
-    default: return launch_bwd_w<T, 1>(tokens, d, y, g, w, rstd, silu_on, dout, dy, dg, dw_part, s);
-  }
+  const Split sp = split_of(tokens, d, true, sizeof(T) == 2 ? M2RNN_BF16 : M2RNN_F32);
+  return with_split(sp, [&](auto C, auto R, auto G) {
+    auto kern = gated_norm_bwd_kernel<T, C(), R(), G()>;
+    constexpr int sums = 256 * C() * kWarps * 4;    // groups x the columns they can hold, at the end
+    constexpr int smem = Walk<T, C(), R(), G(), 3>::kSmem > sums ? Walk<T, C(), R(), G(), 3>::kSmem : sums;
+    const cudaError_t e = allow_smem(kern, smem);
+    if (e != cudaSuccess) return e;
+    kern<<<sp.grid, kThreads, smem, s>>>(tokens, d, static_cast<const T *>(y), static_cast<const T *>(g), static_cast<const T *>(w), rstd, silu_on,
+                                         static_cast<const T *>(dout), static_cast<T *>(dy), static_cast<T *>(dg), dw_part);
+    return cudaGetLastError();
+  });
 }
 
 }  // namespace
@@ -481,8 +444,7 @@ int m2rnn_gated_norm_bwd(int64_t tokens, int32_t d, int32_t io_dtype, const void
   cudaError_t e = io_dtype == M2RNN_BF16 ? launch_bwd<__nv_bfloat16>((long)tokens, d, y, g_in, w, rstd, silu_on, dout, dy, dg_in, part, s)
                                          : launch_bwd<float>((long)tokens, d, y, g_in, w, rstd, silu_on, dout, dy, dg_in, part, s);
   if (e != cudaSuccess) { (void)cudaGetLastError(); return M2RNN_ERR_CUDA; }
-  const int partials = (d == 256 || d == 512 || d == 1024) ? reg_grid((long)tokens, d / 256) : grid_for((long)tokens, bwd_warps(d));
-  reduce_partials_kernel<<<(d + 31) / 32, 256, 0, s>>>(part, dw, partials, d);
+  reduce_partials_kernel<<<(d + 31) / 32, 1024, 0, s>>>(part, dw, split_of((long)tokens, d, true, io_dtype).grid, d);
   return cudaGetLastError() == cudaSuccess ? M2RNN_OK : M2RNN_ERR_CUDA;
 }
 

@@ -78,3 +78,12 @@ def test_gated_norm_rejects_bad_arguments():
     d = parity.to_dev(inputs.make_gated_norm_inputs(1, 4, 3, 4, "bf16", seed=1))     # d = 12: not a multiple of 8
     with pytest.raises(binding.M2RNNError):
         binding.m2rnn_gated_norm_fwd(d["y"], d["g_in"], d["w"])
+
+
+# one to eight warps per row, rows one by one and four or two at a time, lengths on both sides of each edge
+@pytest.mark.parametrize("shape", [(1, 1, 96, 8), (3, 41, 12, 64), (2, 33, 97, 8), (1, 70, 24, 64), (1, 37, 193, 8), (1, 9, 96, 64), (1, 5, 128, 64),
+                                   (4, 2500, 3, 8), (2, 5000, 33, 8), (1, 1250, 50, 32)], ids=lambda s: "x".join(map(str, s)))
+@pytest.mark.parametrize("dtype,tol", [("bf16", 2e-2), ("f32", 1e-4)])
+def test_gated_norm_splits(oracle, shape, dtype, tol):
+    errs = _run(oracle, shape, dtype, True, 1e-6)
+    assert max(errs.values()) < tol, errs
