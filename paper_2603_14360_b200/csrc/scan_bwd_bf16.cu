@@ -153,8 +153,11 @@ __global__ void __launch_bounds__(bwd_threads<V, NWC>(), V == 16 ? (NWC == 2 ? 3
   // branches on it without a vote: 3 to 11 % faster across the shapes)
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const int g = lane >> 2, c = lane & 3;
-  const int unit = blockIdx.x / RS, rs = blockIdx.x % RS;
-  const int b = unit / N, n = unit % N;
+  const int place = blockIdx.x / RS, rs = blockIdx.x % RS;
+  // (V = 16 keeps the grid's order: what the compiler makes of its three-CTA variant is 9 % slower on dense
+  // batches with b from anywhere else, and its CTAs are small)
+  const int b = V == 16 ? place / N : batch_entry(a, place / N, smem), n = place % N;
+  const int unit = V == 16 ? place : b * N + n;
   const UnitSpan span = unit_span(a, b);   // this batch entry's tokens (a slice of a packed batch, or b T ..)
   const int T = span.T;
   const size_t tok0 = span.tok0;

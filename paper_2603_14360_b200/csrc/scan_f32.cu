@@ -148,7 +148,8 @@ __global__ void __launch_bounds__(Geom<V>::kThreads) fwd_f32_kernel(ScanArgs a) 
   extern __shared__ __align__(16) float smem[];
   const int K = a.K, N = a.N, R = a.KCf, RS = K / R, ng = R / kRows;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, p = lane >> 2, c0 = 8 * warp + 2 * (lane & 3);
-  const int bn = blockIdx.x / RS, rs = blockIdx.x % RS, b = bn / N, n = bn % N, rbase = rs * R;
+  const int place = blockIdx.x / RS, rs = blockIdx.x % RS, rbase = rs * R;
+  const int b = batch_entry(a, place / N, smem), n = place % N, bn = b * N + n;
   const UnitSpan span = unit_span(a, b);   // this batch entry's tokens (a slice of a packed batch, or b T ..)
   const int T = span.T;
   const size_t tok0 = span.tok0, KV = (size_t)K * V;
@@ -271,7 +272,8 @@ __global__ void __launch_bounds__(Geom<V>::kThreads) bwd_f32_kernel(ScanArgs a, 
   extern __shared__ __align__(16) float smem[];
   const int K = a.K, N = a.N;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, p = lane >> 2, c0 = 8 * warp + 2 * (lane & 3);
-  const int bn = blockIdx.x / nslab, rs = slab0 + blockIdx.x % nslab, b = bn / N, n = bn % N, rbase = rs * kRows;
+  const int place = blockIdx.x / nslab, rs = slab0 + blockIdx.x % nslab, rbase = rs * kRows;
+  const int b = batch_entry(a, place / N, smem), n = place % N, bn = b * N + n;
   const bool add = nslab == 1 && rs > 0;   // earlier launches have written dv, dgate and dW
   const UnitSpan span = unit_span(a, b);
   const int T = span.T;

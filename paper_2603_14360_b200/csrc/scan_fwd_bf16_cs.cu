@@ -70,7 +70,8 @@ __global__ void __launch_bounds__((SP * NW + cs_service_warps(SP * NW)) * 32, OC
   const int Kf = a.K, N = a.N;            // rows of the whole state
   const int RS = Kf / K;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int bn = blockIdx.x / RS, rs = blockIdx.x % RS, b = bn / N, n = bn % N;
+  const int place = blockIdx.x / RS, rs = blockIdx.x % RS;
+  const int b = batch_entry(a, place / N, smem_raw), n = place % N, bn = b * N + n;
   const UnitSpan span = unit_span(a, b);   // this batch entry's tokens (a slice of a packed batch, or b T ..)
   const int T = span.T;
   const size_t tok0 = span.tok0;

@@ -78,7 +78,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) fwd_tc_kernel(ScanArgs a) {
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const int NG = (N + HS - 1) / HS;               // head groups
   const int RS = (K + kRowsCta - 1) / kRowsCta;   // CTAs per (b, head group)
-  const int rs = blockIdx.x % RS, hg = (blockIdx.x / RS) % NG, b = blockIdx.x / (RS * NG);
+  const int rs = blockIdx.x % RS, hg = (blockIdx.x / RS) % NG, b = batch_entry(a, blockIdx.x / (RS * NG), smem_dyn);
   const int rbase = rs * kRowsCta;
   const UnitSpan span = unit_span(a, b);   // this batch entry's tokens (a slice of a packed batch, or b T ..)
   const int T = span.T;
