@@ -117,6 +117,7 @@ int bwd_f32_piece();   // steps whose states the backward kernel keeps on chip
 
 // bf16 tensor-core path
 cudaError_t launch_fwd_bf16(const ScanArgs &a, cudaStream_t s);     // scan_fwd_bf16.cu: picks a variant
+cudaError_t launch_fwd_v16(const ScanArgs &a, cudaStream_t s);      // scan_fwd_v16.cu: V = 16
 bool fwd_cs_supported(const ScanArgs &a);                            // scan_fwd_bf16_cs.cu
 cudaError_t launch_fwd_bf16_cs(const ScanArgs &a, cudaStream_t s);  // scan_fwd_bf16_cs.cu: two or four warps per 16-row slab
 cudaError_t launch_bwd_bf16(const ScanArgs &a, cudaStream_t s);     // scan_bwd_bf16.cu

@@ -47,9 +47,7 @@ struct FwdSmem {
 // OCC: CTAs per SM the kernel is compiled for.  With more (b,n) units than SMs, two co-resident
 // CTAs (two chain warps per scheduler) hide each other's latencies; the price is a smaller
 // register budget.
-// NWT: the slab count when it is known at compile time (0: read from the arguments); with it every
-// shared-memory offset of a step is an immediate.
-template <int V, int MAXW, bool CKPT, int OCC, int NWT = 0>
+template <int V, int MAXW, bool CKPT, int OCC>
 __global__ void __launch_bounds__((MAXW + 1) * 32, OCC) fwd_bf16_kernel(ScanArgs a) {
   using G = TileGeom<V>;
   constexpr int NT = G::NT, KT = G::KT, SEG = G::SEG;
@@ -62,9 +60,9 @@ __global__ void __launch_bounds__((MAXW + 1) * 32, OCC) fwd_bf16_kernel(ScanArgs
   extern __shared__ __align__(16) unsigned char smem_raw[];
 
   const int Kf = a.K, N = a.N;                       // rows of the whole state
-  const int K = NWT ? 16 * NWT : a.KCf;              // rows of this CTA's slab
+  const int K = a.KCf;                               // rows of this CTA's slab
   const int RS = Kf / K;
-  const int NW = NWT ? NWT : (K >> 4);
+  const int NW = K >> 4;
   constexpr bool kPacked = V <= 64;                  // packed fp32x2 arithmetic (spills at V = 128)
   constexpr int TC = FwdSmem<V>::tc(MAXW * 16);   // K > 64 <=> MAXW == 8
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;   // (through a shuffle: known to be warp-uniform)
@@ -455,14 +453,6 @@ template <int V, int MAXW, bool CKPT, int OCC>
 cudaError_t launch_vwco(const ScanArgs &a, cudaStream_t s) {
   const size_t smem = FwdSmem<V>::bytes(a.KCf);
   const unsigned grid = a.B * a.N * (a.K / a.KCf), threads = (a.KCf / 16 + 1) * 32;
-  if constexpr (V == 16 && MAXW == 4) {
-    if (a.KCf == 64) {   // the paper's layer shape (K = 64, V = 16): slab count known at compile time
-      cudaError_t e = allow_smem(fwd_bf16_kernel<V, MAXW, CKPT, OCC, 4>, smem);
-      if (e != cudaSuccess) return e;
-      fwd_bf16_kernel<V, MAXW, CKPT, OCC, 4><<<grid, threads, smem, s>>>(a);
-      return cudaGetLastError();
-    }
-  }
   cudaError_t e = allow_smem(fwd_bf16_kernel<V, MAXW, CKPT, OCC>, smem);
   if (e != cudaSuccess) return e;
   fwd_bf16_kernel<V, MAXW, CKPT, OCC><<<grid, threads, smem, s>>>(a);
@@ -474,11 +464,6 @@ cudaError_t launch_vwc(const ScanArgs &a, cudaStream_t s) {
   // two CTAs per SM where there are units to fill them and the slab count leaves the registers
   if constexpr (MAXW == 4 && V <= 64) {
     const long ctas = (long)a.B * a.N * (a.K / a.KCf);
-    // V = 16: the state is small enough for three CTAs per SM, which takes e.g. the 336 units of
-    // the paper's layer shape (84 heads x batch 4) in one wave instead of two
-    if constexpr (V == 16) {
-      if (ctas > 2 * sm_count()) return launch_vwco<V, MAXW, CKPT, 3>(a, s);
-    }
     if (ctas > sm_count()) return launch_vwco<V, MAXW, CKPT, 2>(a, s);
   }
   return launch_vwco<V, MAXW, CKPT, 1>(a, s);
@@ -501,10 +486,10 @@ cudaError_t launch_v(const ScanArgs &a, cudaStream_t s) {
 // (benchmarking only).
 cudaError_t launch_fwd_bf16(const ScanArgs &a, cudaStream_t s) {
   if (fwd_use_tc(a.B, a.N, a.K, a.V, M2RNN_BF16)) return launch_fwd_bf16_tc(a, s);
+  if (a.V == 16) return launch_fwd_v16(a, s);
   const char *variant = getenv("M2RNN_FWD_VARIANT");
   if (fwd_cs_supported(a) && !(variant && !strcmp(variant, "wide"))) return launch_fwd_bf16_cs(a, s);
   switch (a.V) {
-    case 16: return launch_v<16>(a, s);
     case 32: return launch_v<32>(a, s);
     case 64: return launch_v<64>(a, s);
     case 128: return launch_v<128>(a, s);
