@@ -127,7 +127,8 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_tc_kernel(ScanArgs a) {
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const int RS = K / kNR;
   const int place = blockIdx.x / RS, rs = blockIdx.x % RS;
-  const int b = batch_entry(a, place / N, smem_dyn), n = place % N, unit = b * N + n;
+  const int n = place % N;
+  const int b = batch_entry(a, place / N, smem_dyn), unit = b * N + n;
   const int rbase = rs * kNR;
   const UnitSpan span = unit_span(a, b);
   const int T = span.T;
