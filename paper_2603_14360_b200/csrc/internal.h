@@ -89,7 +89,7 @@ inline size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 // How the backward pass splits a problem: state rows per CTA and the checkpoint interval (bounded
 // by shared memory in the bf16 backward kernel, which keeps two chunks of recomputed states on chip).
 struct BwdPlan {
-  int KC;     // rows per CTA (fp32 path: 8, or K for one launch per group of eight)
+  int KC;     // rows per CTA (fp32 path: 4 or 8, or K for one launch per group of eight)
   int C;      // default checkpoint interval
   int C_max;  // largest supported checkpoint interval
 };
@@ -111,7 +111,7 @@ size_t bwd_bf16_smem_bytes(int KC, int V, int C);  // scan_bwd_bf16.cu
 
 // fp32 FMA path (scan_f32.cu)
 cudaError_t launch_fwd_f32(const ScanArgs &a, cudaStream_t s);
-cudaError_t launch_bwd_f32(const ScanArgs &a, cudaStream_t s);      // KC = 8: every group of eight rows at once, KC = K: one after the other
+cudaError_t launch_bwd_f32(const ScanArgs &a, cudaStream_t s);      // KC = 4, 8: every group of that many rows at once, KC = K: groups of eight one after the other
 cudaError_t launch_decode_f32(const ScanArgs &a, cudaStream_t s);
 int fwd_f32_rows(int B, int N, int K, int V, size_t share_bytes);
 int bwd_f32_rows(int B, int N, int K, int V, size_t share_bytes);

@@ -11,14 +11,14 @@
 // step makes the new rows visible.  Sums over l pair even and odd entries (packed fp32x2 FMA).
 // (Until then a CTA held a whole state and read W from shared memory for every product: 1 MB of
 // shared-memory traffic a step and a sixteenth of the SMs at 16 units.  K = V = 64, 16 units, T = 512:
-// forward 3.19 -> 0.39 ms, backward 18.6 -> 0.72 ms.)
+// forward 3.19 -> 0.37 ms, backward 18.6 -> 0.63 ms.)
 #include "device_common.cuh"
 #include "internal.h"
 
 namespace m2rnn {
 namespace {
 
-constexpr int kRows = 8;      // rows of a group
+constexpr int kRows = 8;      // rows of a group (forward and backward: or four, see rows_per_group)
 constexpr int kSteps = 16;    // steps staged at a time, and steps of state the backward kernel keeps on chip
 
 template <int V>
@@ -28,7 +28,7 @@ struct Geom {
   static constexpr int HP = V + 8;             // row pitch: the eight rows of a group start 32 bytes apart
                                                // in the banks, so their 32-byte pieces are conflict-free
   static constexpr int NP = V / 16;            // pairs of l per thread
-  static constexpr int kTile = kRows * HP;     // floats of a group of rows
+  static constexpr int kTile = kRows * HP;     // floats of a group of eight rows
 };
 
 // first l of pair i of part p: parts interleave in 16-byte (V = 16: 8-byte) pieces
@@ -59,13 +59,35 @@ __device__ __forceinline__ void load_wt(const float *__restrict__ W, int p, int 
   }
 }
 
-// rows (8 of pitch HP, shared memory) times the matrix held in w -> row p, columns c0, c0 + 1
-template <int V>
-__device__ __forceinline__ float2 product(const float *rows, const float2 (&w)[Geom<V>::NP][2], int p, int lane) {
+// What a lane owns of a group of R rows: E = R/4 adjacent columns of one row -- of eight rows row p, both
+// columns; of four, row p/2, column p%2.
+template <int R>
+struct Own {
+  static constexpr int E = R / 4;
+  __device__ static int row(int p) { return R == 8 ? p : p >> 1; }
+  __device__ static int col(int p, int c0) { return R == 8 ? c0 : c0 + (p & 1); }
+};
+template <int E> struct Vec { float x[E]; };
+template <int E>
+__device__ __forceinline__ Vec<E> get(const float *p) {
+  Vec<E> v;
+  if constexpr (E == 2) { const float2 t = *reinterpret_cast<const float2 *>(p); v.x[0] = t.x; v.x[1] = t.y; }
+  else v.x[0] = *p;
+  return v;
+}
+template <int E>
+__device__ __forceinline__ void put(float *p, const Vec<E> &v) {
+  if constexpr (E == 2) *reinterpret_cast<float2 *>(p) = make_float2(v.x[0], v.x[1]);
+  else *p = v.x[0];
+}
+
+// R rows (pitch HP, shared memory) times the matrix held in w -> the lane's own elements
+template <int V, int R>
+__device__ __forceinline__ Vec<R / 4> product(const float *rows, const float2 (&w)[Geom<V>::NP][2], int p, int lane) {
   using G = Geom<V>;
-  float s[kRows][2];
+  float s[R][2];
 #pragma unroll
-  for (int r = 0; r < kRows; ++r) {
+  for (int r = 0; r < R; ++r) {
     float2 a0 = make_float2(0.f, 0.f), a1 = a0;
     const float *row = rows + r * G::HP;
     if constexpr (V == 16) {
@@ -85,19 +107,26 @@ __device__ __forceinline__ float2 product(const float *rows, const float2 (&w)[G
     s[r][0] = a0.x + a0.y;
     s[r][1] = a1.x + a1.y;
   }
-  // recursive halving over the parts (lane bits 4, 3, 2): part p ends with row p
+  // recursive halving over the parts (lane bits 4, 3, 2), rows first, then (four rows) columns
 #pragma unroll
-  for (int m = 4; m >= 1; m >>= 1) {
-    const bool up = lane & (4 * m);
+  for (int m = R / 2, bit = 16; m >= 1; m >>= 1, bit >>= 1) {
+    const bool up = lane & bit;
 #pragma unroll
     for (int r = 0; r < m; ++r)
 #pragma unroll
       for (int x = 0; x < 2; ++x) {
         const float send = up ? s[r][x] : s[r + m][x], keep = up ? s[r + m][x] : s[r][x];
-        s[r][x] = keep + __shfl_xor_sync(0xffffffffu, send, 4 * m);
+        s[r][x] = keep + __shfl_xor_sync(0xffffffffu, send, bit);
       }
   }
-  return make_float2(s[0][0], s[0][1]);
+  Vec<R / 4> o;
+  if constexpr (R == 8) {
+    o.x[0] = s[0][0]; o.x[1] = s[0][1];
+  } else {
+    const bool up = lane & 4;
+    o.x[0] = (up ? s[0][1] : s[0][0]) + __shfl_xor_sync(0xffffffffu, up ? s[0][0] : s[0][1], 4);
+  }
+  return o;
 }
 
 __device__ __forceinline__ void cp16(float *dst, const float *src) {
@@ -118,21 +147,40 @@ __device__ __forceinline__ void stage_rows(float *dst, const float *src, long lo
   }
 }
 
-// sum over the eight rows p of q_p h_p for the thread's two columns: lanes p < 4 end with column c0,
-// lanes p >= 4 with column c0 + 1
-__device__ __forceinline__ float readout(float q, float2 h, int lane) {
-  const bool up = lane & 16;
-  const float2 v = make_float2(__fmul_rn(q, h.x), __fmul_rn(q, h.y));
-  float t = (up ? v.y : v.x) + __shfl_xor_sync(0xffffffffu, up ? v.x : v.y, 16);
-  t += __shfl_xor_sync(0xffffffffu, t, 8);
-  return t + __shfl_xor_sync(0xffffffffu, t, 4);
+// The readout (Eq. 3) adds shares of four rows, in the order of the rows, whatever the group size: a scan in
+// groups of four, one in groups of eight and a decoding step agree bit for bit.  Column of y that a lane holds:
+template <int R> __device__ __forceinline__ int y_col(int lane, int c0) { return R == 8 ? c0 + ((lane >> 3) & 1) : c0 + ((lane >> 2) & 1); }
+template <int R> __device__ __forceinline__ bool y_owner(int lane) { return R == 8 ? (lane & 20) == 0 : (lane & 24) == 0; }
+// y (of this lane's column) plus the group's shares; first: y is wr v of that column, to be added to the first share
+template <int R>
+__device__ __forceinline__ float readout(float y, bool first, float wr, float v, float q, const Vec<R / 4> &h, int lane) {
+  float t;
+  if constexpr (R == 8) {   // rows p: bits 8 and 4 of the lane inside a half, bit 16 the half
+    const bool up = lane & 8;
+    const float a = __fmul_rn(q, h.x[0]), b = __fmul_rn(q, h.x[1]);
+    t = (up ? b : a) + __shfl_xor_sync(0xffffffffu, up ? a : b, 8);
+    t += __shfl_xor_sync(0xffffffffu, t, 4);
+  } else {                  // rows p / 2: bits 16 and 8
+    t = __fmul_rn(q, h.x[0]);
+    t += __shfl_xor_sync(0xffffffffu, t, 16);
+    t += __shfl_xor_sync(0xffffffffu, t, 8);
+  }
+  y = first ? fmaf(wr, v, t) : y + t;
+  if constexpr (R == 8) y += __shfl_xor_sync(0xffffffffu, t, 16);   // (lanes of the first half, which own y)
+  return y;
 }
 
-// Eq. 1 and 2 for the thread's two elements of a row (roundings spelled out: a decoding step repeats a
-// step of the scan bit for bit)
-__device__ __forceinline__ float2 update(float2 o, float k, float2 v, float f, float2 h, float2 &z) {
-  z = make_float2(tanhf(fmaf(k, v.x, o.x)), tanhf(fmaf(k, v.y, o.y)));
-  return make_float2(fmaf(1.f - f, z.x, __fmul_rn(f, h.x)), fmaf(1.f - f, z.y, __fmul_rn(f, h.y)));
+// Eq. 1 and 2 for the lane's elements of a row (roundings spelled out: a decoding step repeats a step of the
+// scan bit for bit)
+template <int E>
+__device__ __forceinline__ Vec<E> update(const Vec<E> &o, float k, const Vec<E> &v, float f, const Vec<E> &h, Vec<E> &z) {
+  Vec<E> r;
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    z.x[e] = tanhf(fmaf(k, v.x[e], o.x[e]));
+    r.x[e] = fmaf(1.f - f, z.x[e], __fmul_rn(f, h.x[e]));
+  }
+  return r;
 }
 
 // ------------------------------------------------------------------ forward (Algorithm 1)
@@ -142,12 +190,16 @@ __host__ __device__ constexpr int fwd_stage_floats(int R) { return kSteps * (2 *
 template <int V>
 __host__ size_t fwd_f32_smem(int R) { return sizeof(float) * (2 * (size_t)R * Geom<V>::HP + 2 * (size_t)fwd_stage_floats<V>(R) + 2 * kSteps); }
 
-template <int V>
+// GR: rows of a group
+template <int V, int GR>
 __global__ void __launch_bounds__(Geom<V>::kThreads) fwd_f32_kernel(ScanArgs a) {
   using G = Geom<V>;
+  constexpr int E = GR / 4;
+  constexpr int kTile = GR * G::HP;
   extern __shared__ __align__(16) float smem[];
-  const int K = a.K, N = a.N, R = a.KCf, RS = K / R, ng = R / kRows;
+  const int K = a.K, N = a.N, R = a.KCf, RS = K / R, ng = R / GR;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, p = lane >> 2, c0 = 8 * warp + 2 * (lane & 3);
+  const int orow = Own<GR>::row(p), ocol = Own<GR>::col(p, c0), ycol = y_col<GR>(lane, c0);
   const int place = blockIdx.x / RS, rs = blockIdx.x % RS, rbase = rs * R;
   const int b = batch_entry(a, place / N, smem), n = place % N, bn = b * N + n;
   const UnitSpan span = unit_span(a, b);   // this batch entry's tokens (a slice of a packed batch, or b T ..)
@@ -162,17 +214,15 @@ __global__ void __launch_bounds__(Geom<V>::kThreads) fwd_f32_kernel(ScanArgs a) 
   float2 w[G::NP][2];
   load_w<V>(static_cast<const float *>(a.W) + (size_t)n * V * V, p, c0, w);
   for (int g = 0; g < ng; ++g) {
-    const int row = kRows * g + p;
-    *reinterpret_cast<float2 *>(H0 + row * G::HP + c0) =
-        a.h0 ? *reinterpret_cast<const float2 *>(a.h0 + bn * KV + (size_t)(rbase + row) * V + c0) : make_float2(0.f, 0.f);
+    const int row = GR * g + orow;
+    put<E>(H0 + row * G::HP + ocol, a.h0 ? get<E>(a.h0 + bn * KV + (size_t)(rbase + row) * V + ocol) : Vec<E>{});
   }
   const float al = a.alpha ? a.alpha[n] : 1.f, be = a.beta ? a.beta[n] : 0.f;
   const float *qg = static_cast<const float *>(a.q), *kg = static_cast<const float *>(a.k);
   const float *vg = static_cast<const float *>(a.v), *wr = static_cast<const float *>(a.w_r);
   const bool want_y = a.y != nullptr;
   float *yg = a.y_part ? a.y_part + (size_t)rs * a.TT * N * V : static_cast<float *>(a.y);
-  const float2 wr2 = wr && rs == 0 ? *reinterpret_cast<const float2 *>(wr + (size_t)n * V + c0) : make_float2(0.f, 0.f);
-  const float wre = lane & 16 ? wr2.y : wr2.x;
+  const float wre = wr && rs == 0 ? wr[(size_t)n * V + ycol] : 0.f;
 
   auto stage = [&](int x) { return stages + (x & 1) * fwd_stage_floats<V>(R); };
   auto fetch = [&](int ch) {
@@ -205,28 +255,26 @@ __global__ void __launch_bounds__(Geom<V>::kThreads) fwd_f32_kernel(ScanArgs a) 
         if (ck_left == 0) {
           float *dst = a.ckpt + ((size_t)bn * a.nchunks + ck_idx) * KV + (size_t)rbase * V;
           for (int g = 0; g < ng; ++g)
-            *reinterpret_cast<float2 *>(dst + (size_t)(kRows * g + p) * V + c0) = *reinterpret_cast<const float2 *>(H0 + (kRows * g + p) * G::HP + c0);
+            put<E>(dst + (size_t)(GR * g + orow) * V + ocol, get<E>(H0 + (GR * g + orow) * G::HP + ocol));
           ++ck_idx;
           ck_left = a.C;
         }
         --ck_left;
       }
       const float f = fs[s];
-      const float2 v2 = *reinterpret_cast<const float2 *>(vS + s * V + c0);
+      const Vec<E> v = get<E>(vS + s * V + ocol);
+      const float vy = vS[s * V + ycol];
       float y = 0.f;     // Eq. 3, group by group (the order in which the shares of single groups are added too)
       for (int g = 0; g < ng; ++g) {
-        const float2 o = product<V>(H0 + g * G::kTile, w, p, lane);
-        const int row = kRows * g + p;
-        float2 z;
-        const float2 h = update(o, kS[s * R + row], v2, f, *reinterpret_cast<const float2 *>(H0 + row * G::HP + c0), z);
-        *reinterpret_cast<float2 *>(H1 + row * G::HP + c0) = h;
-        if (want_y) {
-          const float share = readout(qS[s * R + row], h, lane);
-          y = g == 0 ? fmaf(wre, lane & 16 ? v2.y : v2.x, share) : y + share;
-        }
+        const Vec<E> o = product<V, GR>(H0 + g * kTile, w, p, lane);
+        const int row = GR * g + orow;
+        Vec<E> z;
+        const Vec<E> h = update<E>(o, kS[s * R + row], v, f, get<E>(H0 + row * G::HP + ocol), z);
+        put<E>(H1 + row * G::HP + ocol, h);
+        if (want_y) y = readout<GR>(y, g == 0, wre, vy, qS[s * R + row], h, lane);
       }
       __syncthreads();   // H_t is complete, H_{t-1} is free
-      if (want_y && (p & 3) == 0) yg[((tok0 + ch * kSteps + s) * N + n) * V + c0 + (p >> 2)] = y;
+      if (want_y && y_owner<GR>(lane)) yg[((tok0 + ch * kSteps + s) * N + n) * V + ycol] = y;
       float *t = H0; H0 = H1; H1 = t;
     }
     if (ch + 1 < nst) {
@@ -237,7 +285,7 @@ __global__ void __launch_bounds__(Geom<V>::kThreads) fwd_f32_kernel(ScanArgs a) 
   }
   if (a.hT)
     for (int g = 0; g < ng; ++g)
-      *reinterpret_cast<float2 *>(a.hT + bn * KV + (size_t)(rbase + kRows * g + p) * V + c0) = *reinterpret_cast<const float2 *>(H0 + (kRows * g + p) * G::HP + c0);
+      put<E>(a.hT + bn * KV + (size_t)(rbase + GR * g + orow) * V + ocol, get<E>(H0 + (GR * g + orow) * G::HP + ocol));
 }
 
 // ------------------------------------------------------------------ backward (Algorithm 2)
@@ -251,28 +299,30 @@ __global__ void __launch_bounds__(Geom<V>::kThreads) fwd_f32_kernel(ScanArgs a) 
 // slab0 / nslab: the groups of rows this launch takes.  All of them (nslab = K/8), each leaving its
 // shares of dv, dgate and dW as partials; or one after the other (nslab = 1), the later ones
 // adding to what the earlier ones wrote.
-template <int V>
+template <int V, int GR>
 struct BwdGeom {
   using G = Geom<V>;
-  static constexpr int kStage = kSteps * (2 * kRows + 2 * V + 1);     // q, k [16][8], v, dy [16][V], gate [16]
+  static constexpr int kTile = GR * G::HP;
+  static constexpr int kStage = kSteps * (2 * GR + 2 * V + 1);        // q, k [16][GR], v, dy [16][V], gate [16]
   // dW tiles: 4 x JT elements per thread; with fewer tiles than threads, SP threads share a tile and
   // take every SP-th step
   static constexpr int JT = V == 128 ? 8 : 4;
   static constexpr int kTiles = (V / 4) * (V / JT), SP = G::kThreads / kTiles;
-  static constexpr int kFloats = (2 * kSteps + 1) * G::kTile + 2 * kStage + 4 * kSteps + kSteps * G::kThreads;
+  static constexpr int kFloats = (2 * kSteps + 1) * kTile + 2 * kStage + 4 * kSteps + kSteps * G::kThreads;
   // W and W^T both stay in registers where they fit beside the dW tile; at V = 128 (32 + 32 + 32 of 128
   // registers) each phase reloads its own from L2 once per piece
   static constexpr bool kReload = V == 128;
 };
 
-template <int V>
-__global__ void __launch_bounds__(Geom<V>::kThreads) bwd_f32_kernel(ScanArgs a, int slab0, int nslab) {
+template <int V, int GR>
+__global__ void __launch_bounds__(Geom<V>::kThreads, 512 / Geom<V>::kThreads) bwd_f32_kernel(ScanArgs a, int slab0, int nslab) {
   using G = Geom<V>;
-  using BG = BwdGeom<V>;
+  using BG = BwdGeom<V, GR>;
+  constexpr int E = GR / 4;
   extern __shared__ __align__(16) float smem[];
   const int K = a.K, N = a.N;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, p = lane >> 2, c0 = 8 * warp + 2 * (lane & 3);
-  const int place = blockIdx.x / nslab, rs = slab0 + blockIdx.x % nslab, rbase = rs * kRows;
+  const int place = blockIdx.x / nslab, rs = slab0 + blockIdx.x % nslab, rbase = rs * GR;
   const int b = batch_entry(a, place / N, smem), n = place % N, bn = b * N + n;
   const bool add = nslab == 1 && rs > 0;   // earlier launches have written dv, dgate and dW
   const UnitSpan span = unit_span(a, b);
@@ -280,9 +330,9 @@ __global__ void __launch_bounds__(Geom<V>::kThreads) bwd_f32_kernel(ScanArgs a, 
   const size_t tok0 = span.tok0, KV = (size_t)K * V;
   const int hq = n / (N / a.Nq), hk = n / (N / a.Nk);
 
-  float *Hc = smem;                               // [17][8][HP]: H before step s of the piece; [len] the last H_t
-  float *Xc = Hc + (kSteps + 1) * G::kTile;       // [16][8][HP]: Z_t, then dX_t
-  float *stages = Xc + kSteps * G::kTile;
+  float *Hc = smem;                               // [17][GR][HP]: H before step s of the piece; [len] the last H_t
+  float *Xc = Hc + (kSteps + 1) * BG::kTile;       // [16][GR][HP]: Z_t, then dX_t
+  float *stages = Xc + kSteps * BG::kTile;
   float *fS = stages + 2 * BG::kStage, *dfS = fS + 2 * kSteps;   // [2][16] gates and their slopes
   float *dfp = dfS + 2 * kSteps;                  // [16][threads] shares of df
 
@@ -296,8 +346,9 @@ __global__ void __launch_bounds__(Geom<V>::kThreads) bwd_f32_kernel(ScanArgs a, 
   const float *qg = static_cast<const float *>(a.q), *kg = static_cast<const float *>(a.k);
   const float *vg = static_cast<const float *>(a.v), *wr = static_cast<const float *>(a.w_r);
   const float *dyg = static_cast<const float *>(a.dy);
-  const int own = p * G::HP + c0;                 // this thread's two elements inside a group of rows
-  const size_t own_g = (size_t)(rbase + p) * V + c0;   // ... inside a state in memory
+  const int orow = Own<GR>::row(p), ocol = Own<GR>::col(p, c0);
+  const int own = orow * G::HP + ocol;            // this thread's elements inside a group of rows
+  const size_t own_g = (size_t)(rbase + orow) * V + ocol;   // ... inside a state in memory
 
   // pieces: chunk ch (the checkpoint interval) holds ceil(len / 16) of them
   const int ppc = (a.C + kSteps - 1) / kSteps, nch = (T + a.C - 1) / a.C;
@@ -307,12 +358,12 @@ __global__ void __launch_bounds__(Geom<V>::kThreads) bwd_f32_kernel(ScanArgs a, 
     return Piece{t0, max(0, min(min(kSteps, a.C - i * kSteps), T - t0))};
   };
   auto stage = [&](int x) { return stages + (x & 1) * BG::kStage; };
-  constexpr int oK = kSteps * kRows, oV = 2 * oK, oDY = oV + kSteps * V, oG = oDY + kSteps * V;
+  constexpr int oK = kSteps * GR, oV = 2 * oK, oDY = oV + kSteps * V, oG = oDY + kSteps * V;
   auto fetch = [&](int x, Piece pc) {
     float *st = stage(x);
     const size_t bt = tok0 + pc.t0;
-    stage_rows(st, qg + bt * a.qs + hq * K + rbase, a.qs, pc.len, kRows, tid, G::kThreads);
-    stage_rows(st + oK, kg + bt * a.ks + hk * K + rbase, a.ks, pc.len, kRows, tid, G::kThreads);
+    stage_rows(st, qg + bt * a.qs + hq * K + rbase, a.qs, pc.len, GR, tid, G::kThreads);
+    stage_rows(st + oK, kg + bt * a.ks + hk * K + rbase, a.ks, pc.len, GR, tid, G::kThreads);
     stage_rows(st + oV, vg + bt * a.vs + n * V, a.vs, pc.len, V, tid, G::kThreads);
     stage_rows(st + oDY, dyg + (bt * N + n) * V, (long long)N * V, pc.len, V, tid, G::kThreads);
     if (tid < pc.len) cp4(st + oG + tid, a.gate + (bt + tid) * N + n);
@@ -323,7 +374,7 @@ __global__ void __launch_bounds__(Geom<V>::kThreads) bwd_f32_kernel(ScanArgs a, 
   };
   float *scratch = a.chunk_states + (size_t)bn * ppc * KV;   // states at the start of a chunk's pieces
 
-  float2 C = a.d_hT ? *reinterpret_cast<const float2 *>(a.d_hT + (size_t)bn * KV + own_g) : make_float2(0.f, 0.f);   // carried dL/dH_t
+  Vec<E> C = a.d_hT ? get<E>(a.d_hT + (size_t)bn * KV + own_g) : Vec<E>{};   // carried dL/dH_t
   float2 dW[4][BG::JT / 2];
 #pragma unroll
   for (int i = 0; i < 4; ++i)
@@ -338,12 +389,12 @@ __global__ void __launch_bounds__(Geom<V>::kThreads) bwd_f32_kernel(ScanArgs a, 
   auto forward = [&](int x, int len) {
     const float *st = stage(x), *fs = fS + (x & 1) * kSteps;
     for (int s = 0; s < len; ++s) {
-      float *hs = Hc + s * G::kTile;
-      const float2 o = product<V>(hs, w, p, lane);
-      float2 z;
-      const float2 h = update(o, st[oK + s * kRows + p], *reinterpret_cast<const float2 *>(st + oV + s * V + c0), fs[s], *reinterpret_cast<const float2 *>(hs + own), z);
-      *reinterpret_cast<float2 *>(hs + G::kTile + own) = h;
-      *reinterpret_cast<float2 *>(Xc + s * G::kTile + own) = z;
+      float *hs = Hc + s * BG::kTile;
+      const Vec<E> o = product<V, GR>(hs, w, p, lane);
+      Vec<E> z;
+      const Vec<E> h = update<E>(o, st[oK + s * GR + orow], get<E>(st + oV + s * V + ocol), fs[s], get<E>(hs + own), z);
+      put<E>(hs + BG::kTile + own, h);
+      put<E>(Xc + s * BG::kTile + own, z);
       __syncthreads();
     }
   };
@@ -356,17 +407,17 @@ __global__ void __launch_bounds__(Geom<V>::kThreads) bwd_f32_kernel(ScanArgs a, 
     if (np > 1) {   // walk the chunk forward once, leaving the states between its pieces
       if constexpr (BG::kReload) load_w<V>(Wn, p, c0, w);
       __syncthreads();   // the piece before is done with every array
-      float2 h = *reinterpret_cast<const float2 *>(ck);
+      Vec<E> h = get<E>(ck);
       for (int i = 0; i + 1 < np; ++i, ++x) {
         const Piece pc = piece(ch, i);
-        *reinterpret_cast<float2 *>(Hc + own) = h;
+        put<E>(Hc + own, h);
         fetch(x, pc);
         cp_wait<0>();
         gates(x, pc);
         __syncthreads();
         forward(x, pc.len);
-        h = *reinterpret_cast<const float2 *>(Hc + pc.len * G::kTile + own);
-        *reinterpret_cast<float2 *>(scratch + (size_t)(i + 1) * KV + own_g) = h;
+        h = get<E>(Hc + pc.len * BG::kTile + own);
+        put<E>(scratch + (size_t)(i + 1) * KV + own_g, h);
         __syncthreads();
       }
       fetched = false;
@@ -374,12 +425,12 @@ __global__ void __launch_bounds__(Geom<V>::kThreads) bwd_f32_kernel(ScanArgs a, 
     for (int i = np - 1; i >= 0; --i, ++x) {
       const Piece pc = piece(ch, i);
       if (!fetched) fetch(x, pc);
-      const float2 h0 = i > 0 ? *reinterpret_cast<const float2 *>(scratch + (size_t)i * KV + own_g) : *reinterpret_cast<const float2 *>(ck);
+      const Vec<E> h0 = get<E>(i > 0 ? scratch + (size_t)i * KV + own_g : ck);
       if constexpr (BG::kReload) load_w<V>(Wn, p, c0, w);
       cp_wait<0>();
       gates(x, pc);
       __syncthreads();   // inputs are in; the piece before is done with every array
-      *reinterpret_cast<float2 *>(Hc + own) = h0;
+      put<E>(Hc + own, h0);
       __syncthreads();
       // the next piece's inputs, unless a pass over its chunk comes first
       fetched = i > 0 || (ch > 0 && a.C <= kSteps);
@@ -390,27 +441,35 @@ __global__ void __launch_bounds__(Geom<V>::kThreads) bwd_f32_kernel(ScanArgs a, 
       const float *st = stage(x), *fs = fS + (x & 1) * kSteps;
       if constexpr (BG::kReload) load_wt<V>(Wn, p, c0, w);
       for (int s = pc.len - 1; s >= 0; --s) {
-        const float f = fs[s], q = st[s * kRows + p];
-        const float2 dy = *reinterpret_cast<const float2 *>(st + oDY + s * V + c0);
-        const float2 hp = *reinterpret_cast<const float2 *>(Hc + s * G::kTile + own);
-        float *xs = Xc + s * G::kTile;
-        const float2 z = *reinterpret_cast<const float2 *>(xs + own);
-        const float2 Gv = make_float2(fmaf(q, dy.x, C.x), fmaf(q, dy.y, C.y));                    // G = C + q dy^T
-        dfp[s * G::kThreads + tid] = fmaf(Gv.x, hp.x - z.x, Gv.y * (hp.y - z.y));               // df = sum G (.) (H_{t-1} - Z)
-        *reinterpret_cast<float2 *>(xs + own) =
-            make_float2((1.f - f) * Gv.x * (1.f - z.x * z.x), (1.f - f) * Gv.y * (1.f - z.y * z.y));   // dX: through the gate and tanh
+        const float f = fs[s], q = st[s * GR + orow];
+        const Vec<E> dy = get<E>(st + oDY + s * V + ocol), hp = get<E>(Hc + s * BG::kTile + own);
+        float *xs = Xc + s * BG::kTile;
+        const Vec<E> z = get<E>(xs + own);
+        Vec<E> Gv, dX;
+        float df = 0.f;
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+          Gv.x[e] = fmaf(q, dy.x[e], C.x[e]);                        // G = C + q dy^T
+          df = fmaf(Gv.x[e], hp.x[e] - z.x[e], df);                  // df = sum G (.) (H_{t-1} - Z)
+          dX.x[e] = (1.f - f) * Gv.x[e] * (1.f - z.x[e] * z.x[e]);   // through the gate and tanh
+        }
+        dfp[s * G::kThreads + tid] = df;
+        put<E>(xs + own, dX);
         __syncthreads();
-        float2 o;                                                                                // C_{t-1} = f G + dX W^T
-        if constexpr (BG::kReload) o = product<V>(xs, w, p, lane);
-        else o = product<V>(xs, wt, p, lane);
-        C = make_float2(fmaf(f, Gv.x, o.x), fmaf(f, Gv.y, o.y));
-        if (a.dh_clip > 0.f) C = make_float2(fminf(fmaxf(C.x, -a.dh_clip), a.dh_clip), fminf(fmaxf(C.y, -a.dh_clip), a.dh_clip));
+        Vec<E> o;                                                    // C_{t-1} = f G + dX W^T
+        if constexpr (BG::kReload) o = product<V, GR>(xs, w, p, lane);
+        else o = product<V, GR>(xs, wt, p, lane);
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+          C.x[e] = fmaf(f, Gv.x[e], o.x[e]);
+          if (a.dh_clip > 0.f) C.x[e] = fminf(fmaxf(C.x[e], -a.dh_clip), a.dh_clip);
+        }
       }
       // (C) dW += H_{t-1}^T dX over the piece's steps and rows
       for (int s = tsp; s < pc.len; s += BG::SP) {
-        const float *hs = Hc + s * G::kTile + tl, *xs = Xc + s * G::kTile + tj;
+        const float *hs = Hc + s * BG::kTile + tl, *xs = Xc + s * BG::kTile + tj;
 #pragma unroll
-        for (int r = 0; r < kRows; ++r) {
+        for (int r = 0; r < GR; ++r) {
           const float4 h4 = *reinterpret_cast<const float4 *>(hs + r * G::HP);
           const float hv[4] = {h4.x, h4.y, h4.z, h4.w};
 #pragma unroll
@@ -426,9 +485,9 @@ __global__ void __launch_bounds__(Geom<V>::kThreads) bwd_f32_kernel(ScanArgs a, 
       }
       // dq = H_t dy, dk = dX v: eight lanes per (step, row)
       const size_t bt0 = tok0 + pc.t0;
-      for (int it = tid >> 3; it < pc.len * kRows; it += G::kThreads / 8) {
-        const int s = it >> 3, r = it & 7, e = tid & 7;
-        const float *hs = Hc + (s + 1) * G::kTile + r * G::HP, *xs = Xc + s * G::kTile + r * G::HP;
+      for (int it = tid >> 3; it < pc.len * GR; it += G::kThreads / 8) {
+        const int s = it / GR, r = it % GR, e = tid & 7;
+        const float *hs = Hc + (s + 1) * BG::kTile + r * G::HP, *xs = Xc + s * BG::kTile + r * G::HP;
         const float *dys = st + oDY + s * V, *vs = st + oV + s * V;
         float dq = 0.f, dk = 0.f;
 #pragma unroll
@@ -439,7 +498,7 @@ __global__ void __launch_bounds__(Geom<V>::kThreads) bwd_f32_kernel(ScanArgs a, 
           dq = fmaf(h2.x, d2.x, fmaf(h2.y, d2.y, dq));
           dk = fmaf(x2.x, v2.x, fmaf(x2.y, v2.y, dk));
         }
-        // (all lanes of a warp take the same number of turns: len x 8 items are whole groups of four)
+        // (all lanes of a warp take the same number of turns: len x GR items are whole groups of four)
 #pragma unroll
         for (int off = 1; off < 8; off <<= 1) { dq += __shfl_xor_sync(0xffffffffu, dq, off); dk += __shfl_xor_sync(0xffffffffu, dk, off); }
         if (e == 0) {
@@ -455,9 +514,9 @@ __global__ void __launch_bounds__(Geom<V>::kThreads) bwd_f32_kernel(ScanArgs a, 
         const int s = it / (V / 4), j = 4 * (it % (V / 4));
         float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-        for (int r = 0; r < kRows; ++r) {
-          const float k = st[oK + s * kRows + r];
-          const float4 x4 = *reinterpret_cast<const float4 *>(Xc + s * G::kTile + r * G::HP + j);
+        for (int r = 0; r < GR; ++r) {
+          const float k = st[oK + s * GR + r];
+          const float4 x4 = *reinterpret_cast<const float4 *>(Xc + s * BG::kTile + r * G::HP + j);
           o.x = fmaf(k, x4.x, o.x); o.y = fmaf(k, x4.y, o.y); o.z = fmaf(k, x4.z, o.z); o.w = fmaf(k, x4.w, o.w);
         }
         if (wr && rs == 0) {
@@ -484,7 +543,7 @@ __global__ void __launch_bounds__(Geom<V>::kThreads) bwd_f32_kernel(ScanArgs a, 
       }
     }
   }
-  if (a.dh0) *reinterpret_cast<float2 *>(a.dh0 + (size_t)bn * KV + own_g) = C;
+  if (a.dh0) put<E>(a.dh0 + (size_t)bn * KV + own_g, C);
   // dW: the threads that share a tile are added in a fixed order
   float *dWp = a.dW_part + (nslab == 1 ? (size_t)bn : ((size_t)b * nslab + rs) * N + n) * V * V;
   if constexpr (BG::SP > 1) {
@@ -533,7 +592,7 @@ __global__ void __launch_bounds__(Geom<V>::kThreads, DecGeom<V>::kOcc) decode_f3
   constexpr int kStage = DecGeom<V>::kStage;
   extern __shared__ __align__(16) float smem[];
   const int K = a.K, N = a.N, B = a.B, ng = K / kRows;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, p = lane >> 2, c0 = 8 * warp + 2 * (lane & 3);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, p = lane >> 2, c0 = 8 * warp + 2 * (lane & 3), ycol = y_col<kRows>(lane, c0);
   const size_t KV = (size_t)K * V;
   const float *qg = static_cast<const float *>(a.q), *kg = static_cast<const float *>(a.k);
   const float *vg = static_cast<const float *>(a.v), *wr = static_cast<const float *>(a.w_r);
@@ -566,46 +625,52 @@ __global__ void __launch_bounds__(Geom<V>::kThreads, DecGeom<V>::kOcc) decode_f3
     const float graw = a.gate[bn];
     if (n != head) { load_w<V>(static_cast<const float *>(a.W) + (size_t)n * V * V, p, c0, w); head = n; }
     const float f = gate_value(a.gate_kind, graw, a.alpha ? a.alpha[n] : 1.f, a.beta ? a.beta[n] : 0.f, nullptr);
-    float y = 0.f, wrv = 0.f;
-    if (wr) wrv = wr[(size_t)n * V + c0 + (p >> 2)];
+    float y = 0.f;
+    const float wrv = wr ? wr[(size_t)n * V + ycol] : 0.f;
     for (int g = 0; g < ng; ++g) {
       cp_wait<kRing - 2>();
       __syncthreads();                                   // this group is in for everybody; the one before is used up
       const float *st = smem + slot * kStage, *vec = st + G::kTile;
       fetch(slot == 0 ? kRing - 1 : slot - 1);           // into the slot just freed
-      const float2 o = product<V>(st, w, p, lane);
-      float2 z;
-      const float2 v2 = *reinterpret_cast<const float2 *>(vec + 2 * kRows + c0);
-      const float2 h = update(o, vec[p], v2, f, *reinterpret_cast<const float2 *>(st + p * G::HP + c0), z);
-      *reinterpret_cast<float2 *>(state + bn * KV + (size_t)(g * kRows + p) * V + c0) = h;
-      const float share = readout(vec[kRows + p], h, lane);
-      y = g == 0 ? fmaf(wrv, lane & 16 ? v2.y : v2.x, share) : y + share;
+      const Vec<2> o = product<V, kRows>(st, w, p, lane);
+      Vec<2> z;
+      const Vec<2> h = update<2>(o, vec[p], get<2>(vec + 2 * kRows + c0), f, get<2>(st + p * G::HP + c0), z);
+      put<2>(state + bn * KV + (size_t)(g * kRows + p) * V + c0, h);
+      y = readout<kRows>(y, g == 0, wrv, vec[2 * kRows + ycol], vec[kRows + p], h, lane);
       slot = slot + 1 == kRing ? 0 : slot + 1;
     }
-    if ((p & 3) == 0) yg[bn * V + c0 + (p >> 2)] = y;
+    if (y_owner<kRows>(lane)) yg[bn * V + ycol] = y;
   }
   cp_wait<0>();
 }
 
-template <int V>
-cudaError_t launch_fwd_v(const ScanArgs &a, cudaStream_t s) {
+template <int V, int GR>
+cudaError_t launch_fwd_g(const ScanArgs &a, cudaStream_t s) {
   const size_t smem = fwd_f32_smem<V>(a.KCf);
-  const cudaError_t e = allow_smem(fwd_f32_kernel<V>, smem);
+  const cudaError_t e = allow_smem(fwd_f32_kernel<V, GR>, smem);
   if (e != cudaSuccess) return e;
-  fwd_f32_kernel<V><<<a.B * a.N * (a.K / a.KCf), Geom<V>::kThreads, smem, s>>>(a);
+  fwd_f32_kernel<V, GR><<<a.B * a.N * (a.K / a.KCf), Geom<V>::kThreads, smem, s>>>(a);
   return cudaGetLastError();
 }
-
 template <int V>
-cudaError_t launch_bwd_v(const ScanArgs &a, cudaStream_t s) {
-  const size_t smem = sizeof(float) * (size_t)BwdGeom<V>::kFloats;
-  cudaError_t e = allow_smem(bwd_f32_kernel<V>, smem);
-  const int slabs = a.K / kRows, nslab = a.KC == kRows ? slabs : 1;
+cudaError_t launch_fwd_v(const ScanArgs &a, cudaStream_t s) {
+  return a.KCf == kRows / 2 ? launch_fwd_g<V, kRows / 2>(a, s) : launch_fwd_g<V, kRows>(a, s);
+}
+
+template <int V, int GR>
+cudaError_t launch_bwd_g(const ScanArgs &a, cudaStream_t s) {
+  const size_t smem = sizeof(float) * (size_t)BwdGeom<V, GR>::kFloats;
+  cudaError_t e = allow_smem(bwd_f32_kernel<V, GR>, smem);
+  const int slabs = a.K / GR, nslab = a.KC == GR ? slabs : 1;
   for (int s0 = 0; s0 < slabs && e == cudaSuccess; s0 += nslab) {
-    bwd_f32_kernel<V><<<a.B * a.N * nslab, Geom<V>::kThreads, smem, s>>>(a, s0, nslab);
+    bwd_f32_kernel<V, GR><<<a.B * a.N * nslab, Geom<V>::kThreads, smem, s>>>(a, s0, nslab);
     e = cudaGetLastError();
   }
   return e;
+}
+template <int V>
+cudaError_t launch_bwd_v(const ScanArgs &a, cudaStream_t s) {
+  return a.KC == kRows / 2 ? launch_bwd_g<V, kRows / 2>(a, s) : launch_bwd_g<V, kRows>(a, s);
 }
 
 template <int V>
@@ -620,22 +685,24 @@ cudaError_t launch_decode_v(const ScanArgs &a, cudaStream_t s) {
 
 }  // namespace
 
-// Rows per CTA of the forward kernel: whole states where that gives every SM 16 warps (half of what it
-// holds) -- the groups take turns behind one barrier a step and y needs no shares in memory --, else
-// eight rows.  `share_bytes`: one slab's share of y; whole states too where the shares of all groups
-// would exceed kMaxShares.
+// Rows per CTA.  The step of a warp is a chain of dependent instructions, so a small problem wants as many warps
+// as it can get: groups of four rows while groups of eight would leave an SM fewer than 16 warps (16 units, K = V
+// = 64, T = 512: forward 379 -> 366 us, backward 721 -> 629), else of eight, which need fewer instructions
+// in all.  Forward: whole states where that gives every SM 16 warps -- the groups take turns behind
+// one barrier a step and y needs no shares in memory.  Backward: K stands for one launch per group of
+// eight, each adding to the results of the one before, where the units alone give every SM 64 warps.
+// `share_bytes`: one group's share of y or dv; whole states (one group after the other) too where the
+// shares of all groups would exceed kMaxShares.
 constexpr size_t kMaxShares = (size_t)4 << 30;
 int fwd_f32_rows(int B, int N, int K, int V, size_t share_bytes) {
-  const long units = (long)(B > 0 ? B : 1) * N;
-  return units * (V / 8) >= 16L * sm_count() || share_bytes * (K / kRows) > kMaxShares ? K : kRows;
+  const long warps = (long)(B > 0 ? B : 1) * N * (V / 8), most = 16L * sm_count();   // of whole states
+  if (warps >= most || share_bytes * (K / kRows) > kMaxShares) return K;
+  return warps * (K / kRows) >= most ? kRows : kRows / 2;
 }
-
-// Rows per CTA of the backward kernel: eight, all groups at once (partials of dv, dgate and dW per
-// group); K stands for one launch per group, each adding to the results of the one before, where the
-// units alone give every SM 64 warps or the shares of dv would exceed kMaxShares.
 int bwd_f32_rows(int B, int N, int K, int V, size_t share_bytes) {
-  const long units = (long)(B > 0 ? B : 1) * N;
-  return units * (V / 8) >= 64L * sm_count() || share_bytes * (K / kRows) > kMaxShares ? K : kRows;
+  const long warps = (long)(B > 0 ? B : 1) * N * (V / 8), most = 16L * sm_count();
+  if (warps >= 4 * most || share_bytes * (K / kRows) > kMaxShares) return K;
+  return warps * (K / kRows) >= most ? kRows : kRows / 2;
 }
 int bwd_f32_piece() { return kSteps; }
 
