@@ -27,14 +27,10 @@ namespace {
 // A CTA is 32 channel chunks (one warp = 256 or 512 contiguous bytes of a token) x 4 time sub-tiles.
 constexpr int kLanes = 32, kSub = 4;
 constexpr int kConvThreads = kLanes * kSub;
-constexpr int kStepsFwd = 64;                    // time steps per thread of the forward kernel
-constexpr int kUFwd = 8, kGFwd = 3;              // ... fetched in batches of kUFwd steps, kGFwd batches ahead
+constexpr int kUFwd = 8, kGFwd = 3;              // forward: rows are fetched in batches of kUFwd steps, kGFwd batches ahead
 constexpr int kOccFwd = 6;
-constexpr int kTileFwd = kSub * kStepsFwd;       // ... per CTA
-constexpr int kStepsBwd = 64;                    // backward: longer runs, fewer halo steps
-constexpr int kUBwd = 4, kGBwd = 2;              // fetched in batches of kUBwd steps, kGBwd batches ahead
+constexpr int kUBwd = 4, kGBwd = 2;              // backward: in batches of kUBwd steps, kGBwd batches ahead
 constexpr int kOccBwd = 4;                       // CTAs per SM the backward kernel is compiled for
-constexpr int kTileBwd = kSub * kStepsBwd;       // one partial sum of dw and dbias per CTA
 
 template <typename T> struct Chunk;             // the channels of one thread
 template <> struct Chunk<float> {
@@ -61,7 +57,13 @@ template <> struct Chunk<__nv_bfloat16> {   // 8 bytes: four channels keep a thr
 // rounding of the result) on the bf16 path, through expf on the fp32 path
 template <typename T> __device__ __forceinline__ float sigmoid_of(float x);
 template <> __device__ __forceinline__ float sigmoid_of<float>(float x) {
-  return x >= 0.f ? 1.f / (1.f + expf(-x)) : expf(x) / (1.f + expf(x));
+  // No branch, one exponential, and the quotient of a number in [1, 2] by Newton's iteration: x -> x + x (1 - d x)
+  // squares the relative error of the starting value.  A divide's own path for extreme operands kept the
+  // channels of a thread from overlapping: 46 us, 0.7 of it per time step, however small the problem.
+  const float e = expf(-fabsf(x)), d = 1.f + e;
+  float r = __fdividef(1.f, d);
+  r = fmaf(r, fmaf(-d, r, 1.f), r);
+  return x >= 0.f ? r : e * r;
 }
 template <> __device__ __forceinline__ float sigmoid_of<__nv_bfloat16>(float x) { return fmaf(0.5f, tanh_approx(0.5f * x), 0.5f); }
 
@@ -98,15 +100,16 @@ __device__ __forceinline__ void load_row(const T *x, long long xs, const T *prev
   for (int e = 0; e < CH; ++e) v[e] = 0.f;
 }
 
-template <typename T>
+template <typename T, int STEPS>
 __global__ void __launch_bounds__(kConvThreads, kOccFwd) conv_silu_fwd_kernel(int B, int Tn, int C, const T *__restrict__ x, long long xs,
                                                                      const T *__restrict__ w, const T *__restrict__ bias,
                                                                      const T *__restrict__ prev, T *__restrict__ out, long long os) {
   constexpr int CH = Chunk<T>::CH;
   const int cc = blockIdx.x * kLanes + (threadIdx.x % kLanes), sub = threadIdx.x / kLanes;
   if (cc * CH >= C) return;
-  const int c0 = cc * CH, ntile = (Tn + kTileFwd - 1) / kTileFwd;
-  const int b = blockIdx.y / ntile, t0 = (blockIdx.y % ntile) * kTileFwd + sub * kStepsFwd, t1 = min(Tn, t0 + kStepsFwd);
+  constexpr int kTile = kSub * STEPS;
+  const int c0 = cc * CH, ntile = (Tn + kTile - 1) / kTile;
+  const int b = blockIdx.y / ntile, t0 = (blockIdx.y % ntile) * kTile + sub * STEPS, t1 = min(Tn, t0 + STEPS);
   if (t0 >= Tn) return;
   constexpr int CP = CH / 2;            // channel pairs
   float2 w2[4][CP], b2[CP];             // w2[s][p] = tap s of channels 2p, 2p+1
@@ -175,8 +178,8 @@ __global__ void __launch_bounds__(kConvThreads, kOccFwd) conv_silu_fwd_kernel(in
 }
 
 // partial sums of a tile: part[tile][5][C] = dw taps 0..3 and dbias
-template <typename T>
-__global__ void __launch_bounds__(kConvThreads, kOccBwd) conv_silu_bwd_kernel(int B, int Tn, int C, const T *__restrict__ x, long long xs,
+template <typename T, int STEPS>
+__global__ void __launch_bounds__(kConvThreads) conv_silu_bwd_kernel(int B, int Tn, int C, const T *__restrict__ x, long long xs,
                                                                      const T *__restrict__ w, const T *__restrict__ bias,
                                                                      const T *__restrict__ prev, const T *__restrict__ dout, long long ds,
                                                                      T *__restrict__ dx, long long dxs, T *__restrict__ dprev,
@@ -186,9 +189,10 @@ __global__ void __launch_bounds__(kConvThreads, kOccBwd) conv_silu_bwd_kernel(in
   const int lane = threadIdx.x % kLanes, sub = threadIdx.x / kLanes;
   const int cc = blockIdx.x * kLanes + lane;
   const bool live = cc * CH < C;
-  const int c0 = live ? cc * CH : 0, ntile = (Tn + kTileBwd - 1) / kTileBwd;
-  const int b = blockIdx.y / ntile, t0 = (blockIdx.y % ntile) * kTileBwd + sub * kStepsBwd;
-  const int t1 = max(t0, min(Tn, t0 + kStepsBwd));   // an empty run when the sequence ends before it
+  constexpr int kTile = kSub * STEPS;
+  const int c0 = live ? cc * CH : 0, ntile = (Tn + kTile - 1) / kTile;
+  const int b = blockIdx.y / ntile, t0 = (blockIdx.y % ntile) * kTile + sub * STEPS;
+  const int t1 = max(t0, min(Tn, t0 + STEPS));   // an empty run when the sequence ends before it
   constexpr int CP = CH / 2;            // channel pairs
   float2 w2[4][CP], b2[CP];
 #pragma unroll
@@ -353,6 +357,33 @@ __global__ void conv_silu_reduce_kernel(const float *__restrict__ part, int ntil
   else if (dbias) dbias[c] = acc;
 }
 
+int tiles(int T, int steps) { return (T + kSub * steps - 1) / (kSub * steps); }
+// Time steps per thread: 64, whose three-row halo and the partial sums of a run weigh least, where that makes
+// two CTAs per SM; 32 where it does not, and 16 where even those leave SMs without a CTA (a thread's run is a
+// chain: [1, 1001, 1472] bf16, 48 CTAs of 64 steps, forward 5.3 -> 3.9 us and backward 11.0 -> 8.3; 384 CTAs of
+// 64 steps lose 10 % as 768 of 32).
+int steps_per_thread(int B, int T, int C) {
+  const long sms = sm_count(), cols = (long)B * ((C / 4 + kLanes - 1) / kLanes);
+  if (cols * tiles(T, 64) >= 2 * sms) return 64;
+  return cols * tiles(T, 16) <= sms ? 16 : 32;
+}
+dim3 conv_grid(int B, int T, int C, int steps) { return dim3((C / 4 + kLanes - 1) / kLanes, (unsigned)(B * tiles(T, steps))); }
+
+template <typename T, int STEPS>
+void launch_fwd(int B, int Tn, int C, const void *x, long long xs, const void *w, const void *bias, const void *prev, void *out, long long os,
+                cudaStream_t s) {
+  conv_silu_fwd_kernel<T, STEPS><<<conv_grid(B, Tn, C, STEPS), kConvThreads, 0, s>>>(
+      B, Tn, C, static_cast<const T *>(x), xs, static_cast<const T *>(w), static_cast<const T *>(bias), static_cast<const T *>(prev),
+      static_cast<T *>(out), os);
+}
+template <typename T, int STEPS>
+void launch_bwd(int B, int Tn, int C, const void *x, const long long (&st)[3], const void *w, const void *bias, const void *prev,
+                const void *dout, void *dx, void *dprev, float *part, cudaStream_t s) {
+  conv_silu_bwd_kernel<T, STEPS><<<conv_grid(B, Tn, C, STEPS), kConvThreads, 0, s>>>(
+      B, Tn, C, static_cast<const T *>(x), st[0], static_cast<const T *>(w), static_cast<const T *>(bias), static_cast<const T *>(prev),
+      static_cast<const T *>(dout), st[1], static_cast<T *>(dx), st[2], static_cast<T *>(dprev), part);
+}
+
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 int check(int B, int T, int C, int io_dtype, long long strides[], int nstrides) {
@@ -381,23 +412,20 @@ extern "C" int m2rnn_conv_silu_fwd(int32_t B, int32_t T, int32_t C, int32_t io_d
   if (B == 0 || T == 0) return M2RNN_OK;
   if (!x || !w || !out) return M2RNN_ERR_NULL;
   if (!aligned16(x) || !aligned16(w) || !aligned16(bias) || !aligned16(prev) || !aligned16(out)) return M2RNN_ERR_ALIGN;
-  const int ch = 4, ntile = (T + kTileFwd - 1) / kTileFwd;   // channels per thread
-  const dim3 grid((C / ch + kLanes - 1) / kLanes, (unsigned)(B * ntile));
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (io_dtype == M2RNN_BF16)
-    conv_silu_fwd_kernel<__nv_bfloat16><<<grid, kConvThreads, 0, s>>>(
-        B, T, C, static_cast<const __nv_bfloat16 *>(x), st[0], static_cast<const __nv_bfloat16 *>(w),
-        static_cast<const __nv_bfloat16 *>(bias), static_cast<const __nv_bfloat16 *>(prev), static_cast<__nv_bfloat16 *>(out), st[1]);
-  else
-    conv_silu_fwd_kernel<float><<<grid, kConvThreads, 0, s>>>(B, T, C, static_cast<const float *>(x), st[0], static_cast<const float *>(w),
-                                                              static_cast<const float *>(bias), static_cast<const float *>(prev),
-                                                              static_cast<float *>(out), st[1]);
+  const auto launch = [&](auto kernel_of) { kernel_of(B, T, C, x, st[0], w, bias, prev, out, st[1], s); };
+  const bool bf = io_dtype == M2RNN_BF16;
+  switch (steps_per_thread(B, T, C)) {
+    case 16: launch(bf ? launch_fwd<__nv_bfloat16, 16> : launch_fwd<float, 16>); break;
+    case 32: launch(bf ? launch_fwd<__nv_bfloat16, 32> : launch_fwd<float, 32>); break;
+    default: launch(bf ? launch_fwd<__nv_bfloat16, 64> : launch_fwd<float, 64>);
+  }
   return cudaGetLastError() == cudaSuccess ? M2RNN_OK : M2RNN_ERR_CUDA;
 }
 
 extern "C" size_t m2rnn_conv_silu_bwd_workspace_bytes(int32_t B, int32_t T, int32_t C) {
   if (B <= 0 || T <= 0 || C <= 0) return 0;
-  return align_up((size_t)B * ((T + kTileBwd - 1) / kTileBwd) * 5 * C * sizeof(float));
+  return align_up((size_t)B * tiles(T, steps_per_thread(B, T, C)) * 5 * C * sizeof(float));
 }
 
 extern "C" int m2rnn_conv_silu_bwd(int32_t B, int32_t T, int32_t C, int32_t io_dtype, const void *x, int64_t x_stride,
@@ -423,20 +451,16 @@ extern "C" int m2rnn_conv_silu_bwd(int32_t B, int32_t T, int32_t C, int32_t io_d
   const size_t need = m2rnn_conv_silu_bwd_workspace_bytes(B, T, C);
   if (!workspace || workspace_bytes < need) return M2RNN_ERR_WORKSPACE;
   if (reinterpret_cast<uintptr_t>(workspace) % kAlign) return M2RNN_ERR_ALIGN;
-  const int ch = 4, ntile = (T + kTileBwd - 1) / kTileBwd;   // channels per thread
-  const dim3 grid((C / ch + kLanes - 1) / kLanes, (unsigned)(B * ntile));
   float *part = static_cast<float *>(workspace);
-  if (io_dtype == M2RNN_BF16)
-    conv_silu_bwd_kernel<__nv_bfloat16><<<grid, kConvThreads, 0, s>>>(
-        B, T, C, static_cast<const __nv_bfloat16 *>(x), st[0], static_cast<const __nv_bfloat16 *>(w),
-        static_cast<const __nv_bfloat16 *>(bias), static_cast<const __nv_bfloat16 *>(prev), static_cast<const __nv_bfloat16 *>(dout),
-        st[1], static_cast<__nv_bfloat16 *>(dx), st[2], static_cast<__nv_bfloat16 *>(dprev), part);
-  else
-    conv_silu_bwd_kernel<float><<<grid, kConvThreads, 0, s>>>(B, T, C, static_cast<const float *>(x), st[0], static_cast<const float *>(w),
-                                                              static_cast<const float *>(bias), static_cast<const float *>(prev),
-                                                              static_cast<const float *>(dout), st[1], static_cast<float *>(dx), st[2],
-                                                              static_cast<float *>(dprev), part);
+  const int steps = steps_per_thread(B, T, C);
+  const auto launch = [&](auto kernel_of) { kernel_of(B, T, C, x, st, w, bias, prev, dout, dx, dprev, part, s); };
+  const bool bf = io_dtype == M2RNN_BF16;
+  switch (steps) {
+    case 16: launch(bf ? launch_bwd<__nv_bfloat16, 16> : launch_bwd<float, 16>); break;
+    case 32: launch(bf ? launch_bwd<__nv_bfloat16, 32> : launch_bwd<float, 32>); break;
+    default: launch(bf ? launch_bwd<__nv_bfloat16, 64> : launch_bwd<float, 64>);
+  }
   if (cudaGetLastError() != cudaSuccess) return M2RNN_ERR_CUDA;
-  conv_silu_reduce_kernel<<<(8 * 5 * C + 255) / 256, 256, 0, s>>>(part, B * ntile, C, dw, dbias);
+  conv_silu_reduce_kernel<<<(8 * 5 * C + 255) / 256, 256, 0, s>>>(part, B * tiles(T, steps), C, dw, dbias);
   return cudaGetLastError() == cudaSuccess ? M2RNN_OK : M2RNN_ERR_CUDA;
 }

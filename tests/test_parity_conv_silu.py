@@ -33,6 +33,13 @@ def test_forward_backward(oracle, dtype, shape, with_prev):
     assert all(torch.equal(again[x], got[x]) for x in got if got[x] is not None)     # fixed-order sums
 
 
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("shape", [(9, 130, 520), (10, 193, 1032), (33, 1, 1032), (34, 257, 1032)], ids=lambda s: "x".join(map(str, s)))
+def test_steps_per_thread(oracle, dtype, shape):
+    """Problems on both sides of the lines between 16, 32 and 64 time steps per thread, with a ragged last tile."""
+    test_forward_backward(oracle, dtype, shape, True)
+
+
 def test_no_bias_and_empty(oracle):
     d = inputs.make_conv_inputs(2, 19, 32, "f32", seed=9, prev=False)
     g = {k: (None if v is None else v.cuda()) for k, v in d.items()}
