@@ -52,6 +52,16 @@ def test_more_units_than_sms(oracle, K, V):
     assert max(errs.values()) < 1.5e-2
 
 
+@pytest.mark.parametrize("N", [2, 149])
+@pytest.mark.parametrize("K,V,T", [(16, 32, 17), (48, 32, 49), (64, 32, 33), (64, 32, 16), (48, 64, 32), (64, 64, 9), (64, 64, 49),
+                                   (16, 128, 33), (32, 128, 25), (32, 128, 8)])
+def test_stage_ends(oracle, N, K, V, T):
+    """Lengths at and around whole stages of the column-split kernel (two and three stages of 8 and 16 steps),
+    with one slab per CTA and with the whole state, and the residual term."""
+    cfg = ScanConfig("ends", B=1, T=T, N=N, K=K, V=V, gate_mean=1.0, w_scale=0.5, seed=700 + T + V)
+    parity.check_fwd(oracle, cfg, residual=True)
+
+
 @pytest.mark.parametrize("K,V", [(16, 16), (64, 64), (128, 128)])
 def test_saturating_inputs(oracle, K, V):
     cfg = ScanConfig("sat", B=2, T=96, N=2, K=K, V=V, dist="saturating", gate_mean=0.0, seed=7)
