@@ -433,12 +433,13 @@ __global__ void __launch_bounds__((SP * NW + cs_service_warps(SP * NW)) * 32, 1)
   };
 
   float P0[NTH][4], P1[NTH][4];
-  int ck_left = 0, ck_idx = 0;
+  int ck_left = 0;   // steps until the next checkpoint
+  float *ck_ptr = CKPT ? a.ckpt + (size_t)bn * a.nchunks * KV : nullptr;
   auto maybe_checkpoint = [&](int steps) {   // called before an even-numbered step
     if constexpr (CKPT) {
       if (ck_left == 0) {
-        store_state(a.ckpt + ((size_t)bn * a.nchunks + ck_idx) * KV);
-        ++ck_idx;
+        store_state(ck_ptr);
+        ck_ptr += KV;
         ck_left = a.C;
       }
       ck_left -= steps;

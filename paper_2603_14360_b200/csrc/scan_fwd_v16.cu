@@ -263,12 +263,13 @@ __global__ void __launch_bounds__((NW + kSvc) * 32, OCC) fwd_v16_kernel(ScanArgs
   };
 
   float P0[2][4], P1[2][4];
-  int ck_left = 0, ck_idx = 0;
+  int ck_left = 0;   // steps until the next checkpoint
+  float *ck_ptr = CKPT ? a.ckpt + (size_t)bn * a.nchunks * KV : nullptr;
   auto maybe_checkpoint = [&](int steps) {   // called before an even-numbered step
     if constexpr (CKPT) {
       if (ck_left == 0) {
-        store_state(a.ckpt + ((size_t)bn * a.nchunks + ck_idx) * KV);
-        ++ck_idx;
+        store_state(ck_ptr);
+        ck_ptr += KV;
         ck_left = a.C;
       }
       ck_left -= steps;
