@@ -31,20 +31,22 @@ namespace m2rnn {
 namespace {
 
 constexpr int kBarrierBytes = 128;
-constexpr size_t kSmemMax = 227 * 1024;
 
 // Byte offsets inside a stage of TC steps: H_t fragments [TC][K/16][V/16][512], then k [TC][K], v [TC][V] and f [TC] as
 // fp32 and q [TC][K] as it is.
 // The hand-over of a stage costs the chain warps some 50 ns, so a stage is 16 steps where three of that size fit into
 // shared memory or else two do (their chain warps then look for the next stage only when they need its first
 // row, which leaves the service warps the time between), and three of 8 steps for the largest groups.
-template <int V, int K>
+template <int V, int K, int OCC>
 struct CsStage {
+  static constexpr size_t kSmemMax = (OCC == 1 ? 227 : 228 / OCC - 1) * 1024;
   static constexpr size_t total_of(int tc, int stages) {
     return kBarrierBytes + (size_t)stages * tc * (K * V * 2 + K * 4 + V * 4 + 4 + K * 2 + (K + V) * 2) + (size_t)tc * 2 * V * 4;
   }
-  static constexpr bool kThree = total_of(16, 3) <= kSmemMax, kTwo = total_of(16, 2) <= kSmemMax;
-  static constexpr int TC = kThree || kTwo ? 16 : 8, kStages = kThree || !kTwo ? 3 : 2;
+  static constexpr bool k16 = OCC == 1 || K <= 32;      // (two service warps stage no more than that)
+  static constexpr bool kThree = k16 && total_of(16, 3) <= kSmemMax, kTwo = k16 && total_of(16, 2) <= kSmemMax;
+  static constexpr int TC = kThree || kTwo ? 16 : 8, kStages = kThree || (!kTwo && total_of(8, 3) <= kSmemMax) ? 3 : 2;
+  static constexpr bool kFits = total_of(TC, kStages) <= kSmemMax;
   static constexpr bool kLate = kStages == 2 || V == 128;
   static constexpr uint32_t k = TC * K * V * 2;
   static constexpr uint32_t v = k + TC * K * 4;
@@ -56,7 +58,7 @@ struct CsStage {
   // both halves of the sums of a stage's y
   static constexpr uint32_t ybytes = TC * 2 * V * 4;
   static constexpr uint32_t total = kBarrierBytes + kStages * (bytes + raw) + ybytes;
-  static_assert(total == total_of(TC, kStages) && total <= kSmemMax, "a block's shared memory");
+  static_assert(total == total_of(TC, kStages), "a block's shared memory");
 };
 
 // Where lane (g, c) of a chain warp keeps the 16 bytes of an A fragment inside the fragment's 512: for the warps of the slab
@@ -72,8 +74,12 @@ template <int VP>
 __host__ __device__ constexpr int part_col(int m) { return (VP / 4) * ((m & 7) >> 1) + 2 * (m >> 3) + (m & 1); }
 
 // service warps of a CTA: one per scheduler that also hosts chain warps, so that their work does not
-// weigh on a single scheduler (the chain warps of a slab advance in lockstep with the slowest)
-__host__ __device__ constexpr int cs_service_warps(int chain_warps) { return chain_warps < 4 ? chain_warps : 4; }
+// weigh on a single scheduler (the chain warps of a slab advance in lockstep with the slowest); two where CTAs share
+// an SM
+__host__ __device__ constexpr int cs_service_warps(int chain_warps, int occ) { return occ > 1 ? 2 : chain_warps < 4 ? chain_warps : 4; }
+__host__ __device__ constexpr int cs_threads(int chain_warps, int occ) { return (chain_warps + cs_service_warps(chain_warps, occ)) * 32; }
+// registers a thread can have
+__host__ __device__ constexpr int cs_regs(int chain_warps, int occ) { return 65536 / (occ * cs_threads(chain_warps, occ)); }
 
 // asynchronous copy of 16 bytes from global to shared memory
 __device__ __forceinline__ void cp16(uint32_t dst_sa, const void *src) {
@@ -95,11 +101,11 @@ __device__ __forceinline__ void widen8(uint32_t src_sa, uint32_t dst_sa) {
 }
 __device__ __forceinline__ float2 widen(uint32_t x) { return make_float2(__uint_as_float(x << 16), __uint_as_float(x & 0xffff0000u)); }
 
-template <int V, int SP, int NW, bool CKPT>
-__global__ void __launch_bounds__((SP * NW + cs_service_warps(SP * NW)) * 32, 1) fwd_bf16_cs_kernel(ScanArgs a) {
+template <int V, int SP, int NW, bool CKPT, int OCC>
+__global__ void __launch_bounds__(cs_threads(SP * NW, OCC), OCC) fwd_bf16_cs_kernel(ScanArgs a) {
   constexpr int K = 16 * NW;         // rows of this CTA's slab group (NW slabs of 16 rows): a.KCf
-  using S = CsStage<V, K>;
-  constexpr int kSvc = cs_service_warps(SP * NW);
+  using S = CsStage<V, K, OCC>;
+  constexpr int kSvc = cs_service_warps(SP * NW, OCC);
   constexpr int VH = V / SP;         // columns of a part
   constexpr int NTH = VH / 8;        // accumulator tiles of a warp
   constexpr int KT = V / 16;         // k-tiles of the product
@@ -231,6 +237,8 @@ __global__ void __launch_bounds__((SP * NW + cs_service_warps(SP * NW)) * 32, 1)
 #pragma unroll 1
         for (int i = 0; i < kMine; i += kPair ? 2 : 1) {
           const int t = sw + kSvc * i;
+          // (past the end there are no fragments, and what stands in their place may be no number: zeros of B do not undo that)
+          const int t_of = w_of && st * TC + t + kSvc < T ? t + kSvc : t;
 #pragma unroll 1
           for (int kb = 0; kb < KT; kb += G) {   // k-tiles of y
             float Y[G][2][4];
@@ -249,7 +257,7 @@ __global__ void __launch_bounds__((SP * NW + cs_service_warps(SP * NW)) * 32, 1)
                 if (!(single && x)) asm volatile("ld.shared.v2.b32 {%0,%1}, [%2];" : "=r"(q0), "=r"(q1) : "r"(sa + S::q + 2u * (uint32_t)((kPair ? t + kSvc * x : t) * K + 16 * (kPair ? w : w + x) + 4 * c)));
                 b[x] = kPair && ((g >> 1) & 1) != x ? 0u : __byte_perm(q0, q1, qsel);
               }
-              const uint32_t fr = sa + (uint32_t)((kPair ? t + kSvc * w_of : t * NW + w + (single ? 0 : w_of)) * (KT * 512));
+              const uint32_t fr = sa + (uint32_t)((kPair ? t_of : t * NW + w + (single ? 0 : w_of)) * (KT * 512));
 #pragma unroll
               for (int kt = 0; kt < G; ++kt)
 #pragma unroll
@@ -510,18 +518,34 @@ __global__ void __launch_bounds__((SP * NW + cs_service_warps(SP * NW)) * 32, 1)
   if (a.hT) store_state(a.hT + bn * KV);
 }
 
-template <int V, int SP, int NW, bool CKPT>
+template <int V, int SP, int NW, bool CKPT, int OCC>
 cudaError_t launch_cs(const ScanArgs &a, cudaStream_t s) {
-  constexpr size_t smem = CsStage<V, 16 * NW>::total;
-  cudaError_t e = allow_smem(fwd_bf16_cs_kernel<V, SP, NW, CKPT>, smem);
+  constexpr size_t smem = CsStage<V, 16 * NW, OCC>::total;
+  static_assert(CsStage<V, 16 * NW, OCC>::kFits, "a block's shared memory");
+  cudaError_t e = allow_smem(fwd_bf16_cs_kernel<V, SP, NW, CKPT, OCC>, smem);
   if (e != cudaSuccess) return e;
-  fwd_bf16_cs_kernel<V, SP, NW, CKPT><<<a.B * a.N * (a.K / (16 * NW)), (SP * NW + cs_service_warps(SP * NW)) * 32, smem, s>>>(a);
+  fwd_bf16_cs_kernel<V, SP, NW, CKPT, OCC><<<a.B * a.N * (a.K / (16 * NW)), cs_threads(SP * NW, OCC), smem, s>>>(a);
   return cudaGetLastError();
+}
+
+template <int V, int SP, int NW, bool CKPT>
+cudaError_t launch_cs_o(const ScanArgs &a, cudaStream_t s) {
+  // With more CTAs than SMs two, or of the smaller groups three, share an SM, whose tensor pipe and tanh unit one
+  // CTA's chain leaves idle most of the time (1024 steps of 192 units, us: K = V = 32 258 -> 168, K = 48, V = 64
+  // 564 -> 481; of 440, three to an SM: K = V = 32 385 -> 223).  Where a round of pairs takes 1.8 times one of single CTAs,
+  // only if the rounds come out fewer for it; four slabs of V = 64 have no registers to share.
+  constexpr bool kHeavy = NW == 4;
+  const long ctas = (long)a.B * a.N * (a.K / (16 * NW)), sms = sm_count(), alone = (ctas + sms - 1) / sms, pairs = (ctas + 2 * sms - 1) / (2 * sms);
+  if constexpr (CsStage<V, 16 * NW, 3>::kFits && cs_regs(SP * NW, 3) >= 88)
+    if (ctas > 2 * sms) return launch_cs<V, SP, NW, CKPT, 3>(a, s);
+  if constexpr (CsStage<V, 16 * NW, 2>::kFits && cs_regs(SP * NW, 2) >= 88)
+    if (ctas > sms && (!kHeavy || 9 * pairs <= 5 * alone)) return launch_cs<V, SP, NW, CKPT, 2>(a, s);
+  return launch_cs<V, SP, NW, CKPT, 1>(a, s);
 }
 
 template <int V, int SP, int NW>
 cudaError_t launch_cs_v(const ScanArgs &a, cudaStream_t s) {
-  return a.ckpt ? launch_cs<V, SP, NW, true>(a, s) : launch_cs<V, SP, NW, false>(a, s);
+  return a.ckpt ? launch_cs_o<V, SP, NW, true>(a, s) : launch_cs_o<V, SP, NW, false>(a, s);
 }
 
 }  // namespace

@@ -52,12 +52,12 @@ def test_more_units_than_sms(oracle, K, V):
     assert max(errs.values()) < 1.5e-2
 
 
-@pytest.mark.parametrize("N", [2, 149])
-@pytest.mark.parametrize("K,V,T", [(16, 32, 17), (48, 32, 49), (64, 32, 33), (64, 32, 16), (48, 64, 32), (64, 64, 9), (64, 64, 49),
+@pytest.mark.parametrize("N", [2, 149, 297])
+@pytest.mark.parametrize("K,V,T", [(16, 64, 17), (32, 32, 33), (32, 64, 25), (16, 32, 17), (48, 32, 49), (64, 32, 33), (64, 32, 16), (48, 64, 32), (64, 64, 9), (64, 64, 49),
                                    (16, 128, 33), (32, 128, 25), (32, 128, 8)])
 def test_stage_ends(oracle, N, K, V, T):
     """Lengths at and around whole stages of the column-split kernel (two and three stages of 8 and 16 steps),
-    with one slab per CTA and with the whole state, and the residual term."""
+    with one slab per CTA, with the whole state, with two and three CTAs per SM, and the residual term."""
     cfg = ScanConfig("ends", B=1, T=T, N=N, K=K, V=V, gate_mean=1.0, w_scale=0.5, seed=700 + T + V)
     parity.check_fwd(oracle, cfg, residual=True)
 
