@@ -124,21 +124,28 @@ bool fwd_use_tc(int B, int N, int K, int V, int io_dtype) {
   // Measured (B200): the round trip of a tcgen05 step (operand store, proxy fence, barrier, eight
   // MMAs at ~30 cycles of issue each, commit, mbarrier, tcgen05.ld) is ~400 cycles before any
   // arithmetic, against ~30 for mma.sync on registers.  It pays only where the register kernels
-  // are bound by the legacy tensor path and there are rows to amortise it over: V = 128 with 64-row
-  // CTAs on at least three quarters of the SMs (the K = V = 128 point of the state-size sweep: 6.8
-  // against 7.8 ms).
-  return V == 128 && K % 64 == 0 && 4L * (B > 0 ? B : 1) * N * (K / 64) >= 3L * sm_count();
+  // are bound by the legacy tensor path and there are rows to amortise it over: V = 128, 64-row CTAs, and so many of
+  // them that 32-row CTAs no longer fit one to an SM (1024 steps of K = V = 128, us: 37 units 442 against 809, 40
+  // units 861 against 816; with checkpoints 995 against 926).
+  return V == 128 && K % 64 == 0 && (long)(B > 0 ? B : 1) * N * (K / 32) > sm_count();
 }
 
 int plan_fwd_rows(int B, int N, int K, int V, int io_dtype, size_t tokens) {
   if (io_dtype == M2RNN_F32) return fwd_f32_rows(B, N, K, V, tokens * N * V * sizeof(float));
   if (fwd_use_tc(B, N, K, V, io_dtype)) return fwd_tc_rows_per_cta(B, N, K, V);
-  // The smallest slab (a multiple of 16 rows that divides K) that still gives every CTA an SM of
-  // its own; with more units than SMs the whole state stays in one CTA.  V = 128 keeps the slab
-  // at 64 rows or fewer for the sake of registers.
+  // The smallest slab (a multiple of 16 rows that divides K) that still gives every CTA an SM of its own; with more
+  // units than SMs the largest that the column-split kernel has: 32 rows at V = 128 for the sake of
+  // registers, 64 below.  Up to 128 rows in one CTA of the one-warp-per-slab kernel only where a K that 48 and
+  // 64 do not divide would make V = 32 slabs of 16 rows (440 units, K = 112: 1029 against 1226 us for 1024 steps; K = 96,
+  // V = 64, 192 units: 1682 against 759), or the slabs' shares of y (fp32, added afterwards) take more than 4 GB.
   const int kSMs = sm_count();
   const long units = (long)(B > 0 ? B : 1) * N;
-  const int cap = V > 64 ? 32 : 128;
+  int cap = V > 64 ? 32 : 128;
+  if (V > 16 && V <= 64 && K > 64) {
+    int kc = 64;
+    while (K % kc) kc -= 16;
+    if ((V == 64 || kc > 16) && tokens * N * V * sizeof(float) * (K / kc) <= ((size_t)4 << 30)) cap = kc;
+  }
   int best = 0;
   for (int kc = 16; kc <= K && kc <= cap; kc += 16) {
     if (K % kc) continue;

@@ -365,8 +365,8 @@ cudaError_t launch_tc_v(const ScanArgs &a, cudaStream_t s) {
 
 }  // namespace
 
-// Rows per CTA of this kernel for a problem: two groups of 32 rows where that still spreads the
-// problem over the SMs (or fills them twice), else two groups of 16; K itself when it is smaller.
+// Rows per CTA of this kernel for a problem: two groups of 32 rows where two groups of 16 would not fit one CTA to an
+// SM, else those; K itself when it is smaller.
 int fwd_tc_rows_per_cta(int B, int N, int K, int V) {
   const char *rows = getenv("M2RNN_TC_ROWS");      // benchmarking only: 32 or 64
   int r;
@@ -375,7 +375,7 @@ int fwd_tc_rows_per_cta(int B, int N, int K, int V) {
   } else {
     const int HS = 128 / V;
     const long tiles = (long)(B > 0 ? B : 1) * ((N + HS - 1) / HS);
-    r = (K % 64 == 0 && 4 * tiles * (K / 64) >= 3L * sm_count()) ? 64 : 32;
+    r = (K % 64 == 0 && tiles * (K / 32) > sm_count()) ? 64 : 32;
   }
   if (r == 64 && K % 32) r = 32;
   return r;

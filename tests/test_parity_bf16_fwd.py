@@ -53,7 +53,7 @@ def test_more_units_than_sms(oracle, K, V):
 
 
 @pytest.mark.parametrize("N", [2, 149, 297])
-@pytest.mark.parametrize("K,V,T", [(16, 64, 17), (32, 32, 33), (32, 64, 25), (16, 32, 17), (48, 32, 49), (64, 32, 33), (64, 32, 16), (48, 64, 32), (64, 64, 9), (64, 64, 49),
+@pytest.mark.parametrize("K,V,T", [(16, 64, 17), (32, 32, 33), (32, 64, 25), (80, 64, 17), (112, 32, 17), (128, 64, 9), (16, 32, 17), (48, 32, 49), (64, 32, 33), (64, 32, 16), (48, 64, 32), (64, 64, 9), (64, 64, 49),
                                    (16, 128, 33), (32, 128, 25), (32, 128, 8)])
 def test_stage_ends(oracle, N, K, V, T):
     """Lengths at and around whole stages of the column-split kernel (two and three stages of 8 and 16 steps),
