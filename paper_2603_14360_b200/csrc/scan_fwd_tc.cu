@@ -6,9 +6,9 @@
 // with M = 128 lanes of tensor memory = state columns, N = 16 state rows per chain group and
 // K = 128.  W^T sits in tensor memory for the whole scan (the MMA's A operand: read from there, the
 // tensor core does not stream the 32 KB of W through shared memory every step, which cost ~90 cycles
-// per MMA when A was a shared-memory tile); the B operand is the bf16 copy of the 16 x 128 state
-// slab in shared memory, row-major (which is K-major for B), rewritten by the epilogue threads every
-// step.  For V < 128 the tile takes 128 / V heads at once: A is block diagonal (W_n^T per head), a
+// per MMA when A was a shared-memory tile); the B operand is the bf16 copy of the 16 x 128 or 32 x 128 state
+// slab in shared memory, rewritten by the epilogue threads every step: 32-row slabs column by column
+// (N-major for B: a thread's rows are two 16-byte stores), 16-row slabs row by row.  For V < 128 the tile takes 128 / V heads at once: A is block diagonal (W_n^T per head), a
 // tensor-memory lane is (head slot, column).  The wasted MMA work is free: the step is bound by the
 // tanh unit and by the latency of the round trip, not by the tensor pipe.
 //
@@ -17,7 +17,10 @@
 //     registers = rows; two warps share a lane quarter), so v_t[j] and f_t are per-thread scalars
 //     and k_t[i], q_t[i] are warp-uniform broadcasts;
 //   - the readout y_t[j] = sum_i q_t[i] H_t[i][j] is a sum over a thread's own registers: no shuffles;
-//   - the state stays in fp32 registers; one thread per group issues the 8 MMAs of the next step.
+//   - the state stays in fp32 registers; a warp of its own issues the 8 MMAs of the next step
+//     when the group's eight warps have arrived at an mbarrier: the issue stalls while the tensor core is busy,
+//     and a chain warp that issued behind a group-wide barrier held up the others (64 units of K = V = 128, 2048
+//     steps: 1625 -> 1134 us with the column-major slabs; 288 units with checkpoints 6353 -> 5040).
 // A CTA runs two independent chain groups of 8 warps (two 16-row slabs of the same unit group):
 // while one waits for its MMAs the other one's epilogue keeps the tanh unit busy.  Service warps
 // stage q, k, v and the gate (as in the other forward kernels) and write y.  Every wait is bounded.
@@ -35,9 +38,9 @@ namespace {
 constexpr int kStagesTc = 3;
 constexpr int kGroups = 2;            // chain groups per CTA
 constexpr int kWarpsG = 8;            // warps per group: lane quarter (warp % 4) x row half (warp / 4)
-constexpr int kSvcWarps = 4;
+constexpr int kSvcWarps = 3;          // (with the MMA warp 20 warps, five to a scheduler: a sixth would cost every warp registers)
 constexpr int kChainThreads = kGroups * kWarpsG * 32;
-constexpr int kThreadsTc = kChainThreads + kSvcWarps * 32;
+constexpr int kThreadsTc = kChainThreads + (kSvcWarps + 1) * 32;   // + the warp that issues the MMAs
 constexpr int kTmemCols = 128;        // 64 columns of W^T (128 K indices, two bf16 per column) + NR (<= 32) per group
 constexpr int kTmemD = 64;            // first accumulator column
 
@@ -61,6 +64,9 @@ __global__ void __launch_bounds__(kThreadsTc, 1) fwd_tc_kernel(ScanArgs a) {
   constexpr int HS = S::HS, TC = S::TC;
   constexpr int kRowsG = NR;            // state rows per group = N of the MMA
   constexpr int kRowsT = NR / 2;        // state rows per thread
+  // 32-row slabs lie column by column (64 bytes = a column's 32 rows, 64-byte swizzle, read N-major): a thread's 16 rows of
+  // its column are two 16-byte stores.  16-row slabs are row-major: eight 2-byte stores.
+  constexpr bool kColMajor = NR == 32;
   constexpr int kRowsCta = kGroups * NR;
   extern __shared__ unsigned char smem_dyn[];
   const uint32_t base_sa = (smem_u32(smem_dyn) + 1023u) & ~1023u;   // the swizzled tiles want 1024-byte alignment
@@ -68,7 +74,8 @@ __global__ void __launch_bounds__(kThreadsTc, 1) fwd_tc_kernel(ScanArgs a) {
   uint64_t *full = reinterpret_cast<uint64_t *>(base + S::oBar);    // [kStagesTc] a stage's inputs are staged
   uint64_t *done = full + kStagesTc;                                // [kStagesTc] the chain warps are through with it
   uint64_t *mma_done = done + kStagesTc;                            // [kGroups] the group's product has landed in tensor memory
-  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(mma_done + kGroups);
+  uint64_t *slab_full = mma_done + kGroups;                         // [kGroups] the group's bf16 slab is written
+  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(slab_full + kGroups);
   float *stages = reinterpret_cast<float *>(base + S::oStage);
 
   const int K = a.K, N = a.N;
@@ -92,7 +99,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) fwd_tc_kernel(ScanArgs a) {
       mbar_init(&full[s], kSvcWarps);
       mbar_init(&done[s], kWarpsG * groups_live);
     }
-    for (int g = 0; g < kGroups; ++g) mbar_init(&mma_done[g], 1);
+    for (int g = 0; g < kGroups; ++g) { mbar_init(&mma_done[g], 1); mbar_init(&slab_full[g], kWarpsG); }
     fence_mbar_init();
   }
   if (warp == 0) {
@@ -130,9 +137,33 @@ __global__ void __launch_bounds__(kThreadsTc, 1) fwd_tc_kernel(ScanArgs a) {
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 
-  if (warp >= kGroups * kWarpsG) {
+  if (warp == kGroups * kWarpsG + kSvcWarps) {
+    // ------------------------------------------------------------------ MMA warp
+    // One product per group and step, as soon as the group's eight warps have written the slab: 8 MMAs of 16 K indices,
+    // 8 columns of A each.
+    constexpr uint32_t idesc = idesc_bf16(128, kRowsG) | (kColMajor ? 1u << 16 : 0u);
+    for (int t = 0; t < T && !failed; ++t)
+      for (int g = 0; g < groups_live; ++g) {
+        if (!mbar_wait(&slab_full[g], t & 1)) { failed = true; break; }
+        if (elect_one()) {
+          const uint32_t b_sa = base_sa + S::oB + (uint32_t)g * S::b_bytes, d_tmem = tmem_base + (uint32_t)(kTmemD + kRowsG * g);
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+          for (int kk = 0; kk < 8; ++kk) {
+            if constexpr (kColMajor) {   // 16 columns of 64 bytes
+              umma_bf16_ts(d_tmem, tmem_base + 8u * kk, smem_desc_sw64(b_sa + 1024u * kk), idesc, kk > 0);
+            } else {                     // 32 bytes inside a 128-byte row of B (then the next 64-index block)
+              const uint32_t bo = (uint32_t)(kk >> 2) * (kRowsG * 128) + (uint32_t)(kk & 3) * 32u;
+              umma_bf16_ts(d_tmem, tmem_base + 8u * kk, smem_desc_sw128(b_sa + bo), idesc, kk > 0);
+            }
+          }
+          umma_commit_tc(&mma_done[g]);
+        }
+        __syncwarp();
+      }
+  } else if (warp >= kGroups * kWarpsG) {
     // ------------------------------------------------------------------ service warps
-    const int sl = tid - kChainThreads;          // 0 .. 127
+    const int sl = tid - kChainThreads;          // 0 .. 32 kSvcWarps - 1
     constexpr int kSvc = kSvcWarps * 32;
     const __nv_bfloat16 *qg = static_cast<const __nv_bfloat16 *>(a.q), *kg = static_cast<const __nv_bfloat16 *>(a.k);
     const __nv_bfloat16 *vg = static_cast<const __nv_bfloat16 *>(a.v), *wr = static_cast<const __nv_bfloat16 *>(a.w_r);
@@ -228,14 +259,19 @@ __global__ void __launch_bounds__(kThreadsTc, 1) fwd_tc_kernel(ScanArgs a) {
     const uint32_t b_sa = base_sa + S::oB + (uint32_t)g * S::b_bytes;
     // this thread's 2-byte slots in the B tile: row i = 8 half + x, K index L: block L / 64, 16-byte
     // chunk ((L % 64) / 8) ^ (i % 8) of the row
-    uint32_t b_addr[kRowsT];
+    uint32_t b_addr[kColMajor ? 2 : kRowsT];
+    if constexpr (kColMajor) {
+      // chunk c of column L at chunk c ^ ((L / 2) % 4)
 #pragma unroll
-    for (int x = 0; x < kRowsT; ++x) {
-      const int i = kRowsT * half + x;
-      b_addr[x] = b_sa + (uint32_t)(L >> 6) * (kRowsG * 128) + (uint32_t)i * 128u + ((((uint32_t)(L & 63) >> 3) ^ (uint32_t)(i & 7)) << 4) +
-                  (uint32_t)(L & 7) * 2u;
+      for (int x = 0; x < 2; ++x) b_addr[x] = b_sa + (uint32_t)L * 64u + (((uint32_t)(2 * half + x) ^ ((uint32_t)(L >> 1) & 3u)) << 4);
+    } else {
+#pragma unroll
+      for (int x = 0; x < kRowsT; ++x) {
+        const int i = kRowsT * half + x;
+        b_addr[x] = b_sa + (uint32_t)(L >> 6) * (kRowsG * 128) + (uint32_t)i * 128u + ((((uint32_t)(L & 63) >> 3) ^ (uint32_t)(i & 7)) << 4) +
+                    (uint32_t)(L & 7) * 2u;
+      }
     }
-    constexpr uint32_t idesc = idesc_bf16(128, kRowsG);
 
     float H[kRowsT];
     if (a.h0 && head_live) {
@@ -245,30 +281,27 @@ __global__ void __launch_bounds__(kThreadsTc, 1) fwd_tc_kernel(ScanArgs a) {
 #pragma unroll
       for (int i = 0; i < kRowsT; ++i) H[i] = 0.f;
     }
-    // bf16 copy of the slab -> B tile, then the 8 MMAs of the next step's product (one thread)
-    auto publish_and_issue = [&](bool issue) {
+    // bf16 copy of the slab -> B tile; the MMA warp issues the next step's product when all eight warps have done so
+    auto publish = [&]() {
+      if constexpr (kColMajor) {
 #pragma unroll
-      for (int i = 0; i < kRowsT; i += 2) {
-        const uint32_t pk = pack_bf16(H[i], H[i + 1]);
-        asm volatile("st.shared.b16 [%0], %1;" ::"r"(b_addr[i]), "h"((uint16_t)(pk & 0xffffu)) : "memory");
-        asm volatile("st.shared.b16 [%0], %1;" ::"r"(b_addr[i + 1]), "h"((uint16_t)(pk >> 16)) : "memory");
+        for (int x = 0; x < 2; ++x)
+          asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(b_addr[x]), "r"(pack_bf16(H[8 * x], H[8 * x + 1])), "r"(pack_bf16(H[8 * x + 2], H[8 * x + 3])),
+                       "r"(pack_bf16(H[8 * x + 4], H[8 * x + 5])), "r"(pack_bf16(H[8 * x + 6], H[8 * x + 7])) : "memory");
+      } else {
+#pragma unroll
+        for (int i = 0; i < kRowsT; i += 2) {
+          const uint32_t pk = pack_bf16(H[i], H[i + 1]);
+          asm volatile("st.shared.b16 [%0], %1;" ::"r"(b_addr[i]), "h"((uint16_t)(pk & 0xffffu)) : "memory");
+          asm volatile("st.shared.b16 [%0], %1;" ::"r"(b_addr[i + 1]), "h"((uint16_t)(pk >> 16)) : "memory");
+        }
       }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");     // generic-proxy writes -> visible to the tensor core
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      asm volatile("bar.sync %0, %1;" ::"r"(1 + g), "n"(kWarpsG * 32) : "memory");
-      if (issue && wg == 0 && elect_one()) {   // warp-uniform condition, then one elected lane
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-#pragma unroll
-        for (int kk = 0; kk < 8; ++kk) {
-          // 16 K indices per MMA: 8 columns of A, 32 bytes inside a 128-byte row of B (then the next
-          // 64-index block)
-          const uint32_t bo = (uint32_t)(kk >> 2) * (kRowsG * 128) + (uint32_t)(kk & 3) * 32u;
-          umma_bf16_ts(d_tmem, tmem_base + 8u * kk, smem_desc_sw128(b_sa + bo), idesc, kk > 0);
-        }
-        umma_commit_tc(&mma_done[g]);
-      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&slab_full[g]);
     };
-    publish_and_issue(T > 0);
+    if (T > 0) publish();
 
     uint32_t it = 0;           // products waited for so far
     // (the place of the next checkpoint walks: its 64-bit products, in every step of the loop, were 15 % of it:
@@ -323,8 +356,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) fwd_tc_kernel(ScanArgs a) {
           yacc = __ffma2_rn(make_float2(qq[i], qq[i + 1]), h, yacc);                      // Eq. 3, this thread's rows
         }
         if (want_y) *yp = yacc.x + yacc.y;
-        const bool last = ch == nchunks - 1 && tl == len - 1;
-        publish_and_issue(!last);
+        if (ch < nchunks - 1 || tl < len - 1) publish();
         kp += HS * kRowsCta; qp += HS * kRowsCta; vp += 128; fp += 8; yp += 2 * kGroups * 128;
       }
       __syncwarp();
