@@ -11,8 +11,8 @@
 // of several stages at a time, a lane each.  Stages are handed over by mbarriers; every wait is bounded and
 // reports through dev_status.
 // (With the readout in the chain warps, as eight movmatrix and four MMAs of a step, 128 units of K = V = 64 took 658 us for
-// 2048 steps, now 595; 64 units of K = V = 32 and 64 for 8192 steps 1036 and 1945, now 965 and 1726; 32 of
-// K = V = 128 for 4096 steps 1894, now 1726.  Tried and slower: H_t as row-major tiles, read back by ldmatrix, whose
+// 2048 steps, now 595; 64 units of K = V = 32 and 64 for 8192 steps 1036 and 1945, now 965 and 1726; 192
+// of K = 16, V = 128 for 1024 steps 586, now 529.  Tried and slower: H_t as row-major tiles, read back by ldmatrix, whose
 // stores are twice as many; k and v as bf16 up to the chain warps, which then widen them, 5 %.)
 // The slab count NW is a template parameter and four steps form one loop iteration, so that
 // every shared-memory offset of a step is an immediate.
@@ -552,7 +552,7 @@ cudaError_t launch_cs_v(const ScanArgs &a, cudaStream_t s) {
 
 // slabs per CTA this variant supports for a V: the register file holds (parts * slabs + 1) warps
 bool fwd_cs_supported(const ScanArgs &a) {
-  if (a.V == 128) return a.KCf <= 32;
+  if (a.V == 128) return a.KCf == 16;
   return (a.V == 32 || a.V == 64) && a.KCf <= 64;
 }
 
@@ -581,7 +581,6 @@ cudaError_t launch_fwd_bf16_cs(const ScanArgs &a, cudaStream_t s) {
     case 128:
       switch (nw) {
         case 1: return launch_cs_v<128, 4, 1>(a, s);
-        case 2: return launch_cs_v<128, 4, 2>(a, s);
       }
       break;
   }

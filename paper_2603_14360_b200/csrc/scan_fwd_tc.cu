@@ -7,8 +7,8 @@
 // K = 128.  W^T sits in tensor memory for the whole scan (the MMA's A operand: read from there, the
 // tensor core does not stream the 32 KB of W through shared memory every step, which cost ~90 cycles
 // per MMA when A was a shared-memory tile); the B operand is the bf16 copy of the 16 x 128 or 32 x 128 state
-// slab in shared memory, rewritten by the epilogue threads every step: 32-row slabs column by column
-// (N-major for B: a thread's rows are two 16-byte stores), 16-row slabs row by row.  For V < 128 the tile takes 128 / V heads at once: A is block diagonal (W_n^T per head), a
+// slab in shared memory, column by column (N-major for B: a thread's rows are one or two 16-byte stores),
+// rewritten by the epilogue threads every step.  For V < 128 the tile takes 128 / V heads at once: A is block diagonal (W_n^T per head), a
 // tensor-memory lane is (head slot, column).  The wasted MMA work is free: the step is bound by the
 // tanh unit and by the latency of the round trip, not by the tensor pipe.
 //
@@ -49,7 +49,7 @@ struct TcFwdSmem {
   static constexpr int kRowsG = NR, kRowsCta = kGroups * NR;
   static constexpr int HS = 128 / V;                         // heads per tile
   static constexpr int TC = HS * NR >= 64 ? 8 : 16;          // steps per stage
-  static constexpr uint32_t b_bytes = kRowsG * 128 * 2;      // B of one group: 2 blocks of [NR rows][128 bytes]
+  static constexpr uint32_t b_bytes = kRowsG * 128 * 2;      // B of one group: 128 columns of NR rows
   static constexpr uint32_t oB = 0, oBar = oB + kGroups * b_bytes, oStage = oBar + 128;
   // per stage (floats): k [TC][HS][rows of the CTA], q likewise, v [TC][128], f [TC][8],
   // y [TC][groups][row halves][128]
@@ -64,9 +64,9 @@ __global__ void __launch_bounds__(kThreadsTc, 1) fwd_tc_kernel(ScanArgs a) {
   constexpr int HS = S::HS, TC = S::TC;
   constexpr int kRowsG = NR;            // state rows per group = N of the MMA
   constexpr int kRowsT = NR / 2;        // state rows per thread
-  // 32-row slabs lie column by column (64 bytes = a column's 32 rows, 64-byte swizzle, read N-major): a thread's 16 rows of
-  // its column are two 16-byte stores.  16-row slabs are row-major: eight 2-byte stores.
-  constexpr bool kColMajor = NR == 32;
+  // A slab lies column by column (32 or 64 bytes = a column's rows, 32- or 64-byte swizzle, read N-major): a thread's 8 or 16
+  // rows of its column are one or two 16-byte stores.
+  constexpr int kChunks = kRowsT / 8;
   constexpr int kRowsCta = kGroups * NR;
   extern __shared__ unsigned char smem_dyn[];
   const uint32_t base_sa = (smem_u32(smem_dyn) + 1023u) & ~1023u;   // the swizzled tiles want 1024-byte alignment
@@ -141,7 +141,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) fwd_tc_kernel(ScanArgs a) {
     // ------------------------------------------------------------------ MMA warp
     // One product per group and step, as soon as the group's eight warps have written the slab: 8 MMAs of 16 K indices,
     // 8 columns of A each.
-    constexpr uint32_t idesc = idesc_bf16(128, kRowsG) | (kColMajor ? 1u << 16 : 0u);
+    constexpr uint32_t idesc = idesc_bf16(128, kRowsG) | (1u << 16);
     for (int t = 0; t < T && !failed; ++t)
       for (int g = 0; g < groups_live; ++g) {
         if (!mbar_wait(&slab_full[g], t & 1)) { failed = true; break; }
@@ -150,12 +150,8 @@ __global__ void __launch_bounds__(kThreadsTc, 1) fwd_tc_kernel(ScanArgs a) {
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
           for (int kk = 0; kk < 8; ++kk) {
-            if constexpr (kColMajor) {   // 16 columns of 64 bytes
-              umma_bf16_ts(d_tmem, tmem_base + 8u * kk, smem_desc_sw64(b_sa + 1024u * kk), idesc, kk > 0);
-            } else {                     // 32 bytes inside a 128-byte row of B (then the next 64-index block)
-              const uint32_t bo = (uint32_t)(kk >> 2) * (kRowsG * 128) + (uint32_t)(kk & 3) * 32u;
-              umma_bf16_ts(d_tmem, tmem_base + 8u * kk, smem_desc_sw128(b_sa + bo), idesc, kk > 0);
-            }
+            const uint32_t sa = b_sa + (uint32_t)(32 * kRowsG) * kk;   // 16 columns
+            umma_bf16_ts(d_tmem, tmem_base + 8u * kk, NR == 32 ? smem_desc_sw64(sa) : smem_desc_sw32(sa), idesc, kk > 0);
           }
           umma_commit_tc(&mma_done[g]);
         }
@@ -257,21 +253,11 @@ __global__ void __launch_bounds__(kThreadsTc, 1) fwd_tc_kernel(ScanArgs a) {
     const uint32_t d_tmem = tmem_base + (uint32_t)(kTmemD + kRowsG * g);
     const uint32_t taddr = d_tmem + ((uint32_t)(32 * quarter) << 16) + (uint32_t)(kRowsT * half);
     const uint32_t b_sa = base_sa + S::oB + (uint32_t)g * S::b_bytes;
-    // this thread's 2-byte slots in the B tile: row i = 8 half + x, K index L: block L / 64, 16-byte
-    // chunk ((L % 64) / 8) ^ (i % 8) of the row
-    uint32_t b_addr[kColMajor ? 2 : kRowsT];
-    if constexpr (kColMajor) {
-      // chunk c of column L at chunk c ^ ((L / 2) % 4)
+    // this thread's chunks of its column: chunk c of column L sits at c ^ ((L / 2) % 4), 32-byte columns c ^ ((L / 4) % 2)
+    uint32_t b_addr[kChunks];
 #pragma unroll
-      for (int x = 0; x < 2; ++x) b_addr[x] = b_sa + (uint32_t)L * 64u + (((uint32_t)(2 * half + x) ^ ((uint32_t)(L >> 1) & 3u)) << 4);
-    } else {
-#pragma unroll
-      for (int x = 0; x < kRowsT; ++x) {
-        const int i = kRowsT * half + x;
-        b_addr[x] = b_sa + (uint32_t)(L >> 6) * (kRowsG * 128) + (uint32_t)i * 128u + ((((uint32_t)(L & 63) >> 3) ^ (uint32_t)(i & 7)) << 4) +
-                    (uint32_t)(L & 7) * 2u;
-      }
-    }
+    for (int x = 0; x < kChunks; ++x)
+      b_addr[x] = b_sa + (uint32_t)(2 * kRowsG * L) + (((uint32_t)(kChunks * half + x) ^ (NR == 32 ? (uint32_t)(L >> 1) & 3u : (uint32_t)(L >> 2) & 1u)) << 4);
 
     float H[kRowsT];
     if (a.h0 && head_live) {
@@ -283,19 +269,10 @@ __global__ void __launch_bounds__(kThreadsTc, 1) fwd_tc_kernel(ScanArgs a) {
     }
     // bf16 copy of the slab -> B tile; the MMA warp issues the next step's product when all eight warps have done so
     auto publish = [&]() {
-      if constexpr (kColMajor) {
 #pragma unroll
-        for (int x = 0; x < 2; ++x)
-          asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(b_addr[x]), "r"(pack_bf16(H[8 * x], H[8 * x + 1])), "r"(pack_bf16(H[8 * x + 2], H[8 * x + 3])),
-                       "r"(pack_bf16(H[8 * x + 4], H[8 * x + 5])), "r"(pack_bf16(H[8 * x + 6], H[8 * x + 7])) : "memory");
-      } else {
-#pragma unroll
-        for (int i = 0; i < kRowsT; i += 2) {
-          const uint32_t pk = pack_bf16(H[i], H[i + 1]);
-          asm volatile("st.shared.b16 [%0], %1;" ::"r"(b_addr[i]), "h"((uint16_t)(pk & 0xffffu)) : "memory");
-          asm volatile("st.shared.b16 [%0], %1;" ::"r"(b_addr[i + 1]), "h"((uint16_t)(pk >> 16)) : "memory");
-        }
-      }
+      for (int x = 0; x < kChunks; ++x)
+        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(b_addr[x]), "r"(pack_bf16(H[8 * x], H[8 * x + 1])), "r"(pack_bf16(H[8 * x + 2], H[8 * x + 3])),
+                     "r"(pack_bf16(H[8 * x + 4], H[8 * x + 5])), "r"(pack_bf16(H[8 * x + 6], H[8 * x + 7])) : "memory");
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");     // generic-proxy writes -> visible to the tensor core
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();

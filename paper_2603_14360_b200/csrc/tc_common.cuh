@@ -8,22 +8,23 @@
 
 namespace m2rnn {
 
-// K-major, 128-byte-swizzled canonical layout (rows of 128 bytes = 64 bf16, groups of 8 rows 1024
-// bytes apart, the 16-byte chunks of a row XOR-ed with the row index modulo 8).
+// Shared-memory descriptors of bf16 tiles.
 //   bits  0-13 start address >> 4     bits 32-45 stride between 8-row groups >> 4
-//   bits 16-29 leading offset >> 4 (unused by swizzled K-major layouts)
-//   bits 46-47 descriptor version 1   bits 61-63 swizzle mode (2 = 128 bytes)
-__device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t sa) {
-  return (uint64_t)((sa & 0x3ffffu) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) | ((uint64_t)1 << 46) |
-         ((uint64_t)2 << 61);
-}
-// The same with 64-byte swizzling (mode 4): rows of 64 bytes = 32 bf16, groups of 8 rows 512 bytes
-// apart, the 16-byte chunks of a row XOR-ed with (row / 2) modulo 4.  Serves both readings of such a
-// tile: K-major (a row = one M/N index, 32 K indices) and MN-major (a row = one K index, 32 M/N
-// indices); the instruction descriptor's major bits say which.
+//   bits 16-29 leading offset >> 4 (unused here)
+//   bits 46-47 descriptor version 1   bits 61-63 swizzle mode
+// 64-byte swizzling (mode 4): rows of 64 bytes = 32 bf16, groups of 8 rows 512 bytes apart, the 16-byte
+// chunks of a row XOR-ed with (row / 2) modulo 4.  Serves both readings of such a tile: K-major (a row =
+// one M/N index, 32 K indices) and MN-major (a row = one K index, 32 M/N indices); the instruction
+// descriptor's major bits say which.
 __device__ __forceinline__ uint64_t smem_desc_sw64(uint32_t sa) {
   return (uint64_t)((sa & 0x3ffffu) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(512 >> 4) << 32) | ((uint64_t)1 << 46) |
          ((uint64_t)4 << 61);
+}
+// With 32-byte swizzling (mode 6): rows of 32 bytes = 16 bf16, groups of 8 rows 256 bytes apart, the two 16-byte chunks of a
+// row swapped in every other group of four rows.
+__device__ __forceinline__ uint64_t smem_desc_sw32(uint32_t sa) {
+  return (uint64_t)((sa & 0x3ffffu) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(256 >> 4) << 32) | ((uint64_t)1 << 46) |
+         ((uint64_t)6 << 61);
 }
 // Instruction descriptor of kind::f16 with bf16 operands: fp32 accumulator (bits 4-5 = 1), bf16 A
 // and B (bits 7-9 and 10-12 = 1), both K-major (bits 15, 16 = 0), N >> 3 in bits 17-22, M >> 4 in
@@ -67,15 +68,6 @@ __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&r)[8])
 }
 
 
-// Operands read "MN-major": a tile stored [k][m] with m contiguous (rows of 128 bytes = 64 elements
-// along M or N, eight rows = one 1024-byte swizzle atom along K).  Leading offset = distance between
-// the 64-element blocks along M/N, stride = distance between 8-row groups along K.
-__device__ __forceinline__ uint64_t smem_desc_mn_sw128(uint32_t sa, uint32_t lead_bytes) {
-  return (uint64_t)((sa & 0x3ffffu) >> 4) | ((uint64_t)((lead_bytes & 0x3ffffu) >> 4) << 16) | ((uint64_t)(1024 >> 4) << 32) |
-         ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
-}
-// kind::f16, bf16 operands, fp32 accumulator, A and B MN-major (bits 15 and 16)
-__host__ __device__ constexpr uint32_t idesc_bf16_mn(int M, int N) { return idesc_bf16(M, N) | (1u << 15) | (1u << 16); }
 // D[128 x N] (+)= A B^T with both operands from shared memory
 __device__ __forceinline__ void umma_bf16_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
   asm volatile(

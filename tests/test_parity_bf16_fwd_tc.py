@@ -82,6 +82,17 @@ def test_backward_from_this_kernels_checkpoints(oracle):
     parity.check_bwd(oracle, cfg, residual=True, d_hT=True)
 
 
+@pytest.mark.parametrize("B,N,K", [(1, 20, 128), (2, 13, 96), (1, 149, 32), (1, 38, 128)])
+def test_default_at_v128(oracle, monkeypatch, B, N, K):
+    """Without the override: 32-row CTAs, also more of them than SMs, and 64-row CTAs, forward and as the source of the
+    backward pass's checkpoints."""
+    monkeypatch.delenv("M2RNN_FWD_VARIANT", raising=False)
+    monkeypatch.delenv("M2RNN_TC_ROWS", raising=False)
+    cfg = ScanConfig("v128", B=B, T=21, N=N, K=K, V=128, gate_mean=1.0, w_scale=0.5, seed=500 + N)
+    parity.check_fwd(oracle, cfg, residual=True)
+    parity.check_bwd(oracle, cfg)
+
+
 def test_many_units(oracle):
     cfg = ScanConfig("many", B=20, T=37, N=8, K=64, V=64, gate_mean=1.0, seed=428)   # 160 CTAs
     parity.check_fwd(oracle, cfg)
