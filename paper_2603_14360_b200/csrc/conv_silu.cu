@@ -30,7 +30,7 @@ constexpr int kConvThreads = kLanes * kSub;
 constexpr int kUFwd = 8, kGFwd = 3;              // forward: rows are fetched in batches of kUFwd steps, kGFwd batches ahead
 constexpr int kOccFwd = 6;
 constexpr int kUBwd = 4, kGBwd = 2;              // backward: in batches of kUBwd steps, kGBwd batches ahead
-constexpr int kOccBwd = 4;                       // CTAs per SM the backward kernel is compiled for
+constexpr int kOccBwd = 4;                       // CTAs per SM the bf16 backward kernel is compiled for (fp32: as many as fit its registers)
 
 template <typename T> struct Chunk;             // the channels of one thread
 template <> struct Chunk<float> {
@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(kConvThreads, kOccFwd) conv_silu_fwd_kernel(in
 
 // partial sums of a tile: part[tile][5][C] = dw taps 0..3 and dbias
 template <typename T, int STEPS>
-__global__ void __launch_bounds__(kConvThreads) conv_silu_bwd_kernel(int B, int Tn, int C, const T *__restrict__ x, long long xs,
+__global__ void __launch_bounds__(kConvThreads, sizeof(T) == 2 ? kOccBwd : 1) conv_silu_bwd_kernel(int B, int Tn, int C, const T *__restrict__ x, long long xs,
                                                                      const T *__restrict__ w, const T *__restrict__ bias,
                                                                      const T *__restrict__ prev, const T *__restrict__ dout, long long ds,
                                                                      T *__restrict__ dx, long long dxs, T *__restrict__ dprev,
