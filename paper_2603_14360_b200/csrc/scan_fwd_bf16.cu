@@ -489,9 +489,10 @@ cudaError_t launch_fwd_bf16(const ScanArgs &a, cudaStream_t s) {
   if (fwd_use_tc(a.B, a.N, a.K, a.V, M2RNN_BF16)) return launch_fwd_bf16_tc(a, s);
   if (a.V == 16) return launch_fwd_v16(a, s);
   const char *variant = getenv("M2RNN_FWD_VARIANT");
-  // V = 128: with 32 rows per CTA a tcgen05 step takes what a column-split one did (32 units of K = V = 128, 4096 steps:
-  // 1715 against 1723 us, with checkpoints 1784 against 1995); with 16 rows mma.sync is far ahead (297 ns a step)
-  if (!variant && a.V == 128 && a.KCf == 32) return launch_fwd_bf16_tc(a, s);
+  // V = 128, 32 rows per CTA, checkpoints: the tcgen05 kernel's threads hold whole columns and store them with fewer
+  // instructions (32 units of K = V = 128, 4096 steps: 1995 -> 1784 us).  Without checkpoints the two take the same time
+  // (1723 and 1715) and the column-split kernel's sums keep the order they have with 16 rows, where it is far ahead.
+  if (!variant && a.V == 128 && a.KCf == 32 && a.ckpt) return launch_fwd_bf16_tc(a, s);
   if (fwd_cs_supported(a) && !(variant && !strcmp(variant, "wide"))) return launch_fwd_bf16_cs(a, s);
   switch (a.V) {
     case 32: return launch_v<32>(a, s);

@@ -552,7 +552,7 @@ cudaError_t launch_cs_v(const ScanArgs &a, cudaStream_t s) {
 
 // slabs per CTA this variant supports for a V: the register file holds (parts * slabs + 1) warps
 bool fwd_cs_supported(const ScanArgs &a) {
-  if (a.V == 128) return a.KCf == 16;
+  if (a.V == 128) return a.KCf <= 32;
   return (a.V == 32 || a.V == 64) && a.KCf <= 64;
 }
 
@@ -581,6 +581,7 @@ cudaError_t launch_fwd_bf16_cs(const ScanArgs &a, cudaStream_t s) {
     case 128:
       switch (nw) {
         case 1: return launch_cs_v<128, 4, 1>(a, s);
+        case 2: return launch_cs_v<128, 4, 2>(a, s);
       }
       break;
   }
