@@ -405,11 +405,11 @@ PyObject *py_gated_norm_fwd(PyObject *, PyObject *const *a, Py_ssize_t n) {
   int64_t tokens, d;
   norm_dims(y, tokens, d);
   const ScalarType io = y.scalar_type();
+  check(y, "y", y.sizes(), io);
   check(g, "g_in", y.sizes(), io);
   check(w, "w", w.sizes(), io);
   if (w.numel() != d) fail(PyExc_ValueError, "w has %lld entries, the rows have %lld", (long long)w.numel(), (long long)d);
   const at::IntArrayRef rows = y.sizes().slice(0, y.dim() - 2);
-  if (!y.is_cuda()) fail(PyExc_ValueError, "y must be a CUDA tensor");
   const Tensor out = given_or_empty(opt_tensor(a[5], "out"), y.sizes(), io, y.device());
   const Tensor rstd = given_or_empty(opt_tensor(a[6], "rstd"), rows, ScalarType::Float, y.device());
   check(out, "out", y.sizes(), io);
@@ -439,9 +439,11 @@ PyObject *py_gated_norm_bwd(PyObject *, PyObject *const *a, Py_ssize_t n) {
   int64_t tokens, d;
   norm_dims(y, tokens, d);
   const ScalarType io = y.scalar_type();
+  check(y, "y", y.sizes(), io);
   check(g, "g_in", y.sizes(), io);
   check(dout, "dout", y.sizes(), io);
   check(w, "w", w.sizes(), io);
+  if (w.numel() != d) fail(PyExc_ValueError, "w has %lld entries, the rows have %lld", (long long)w.numel(), (long long)d);
   check(rstd, "rstd", y.sizes().slice(0, y.dim() - 2), ScalarType::Float);
   const at::Device dev = g.device();
   const Tensor dy = given_or_empty(opt_tensor(a[7], "dy"), y.sizes(), io, dev);
@@ -485,10 +487,10 @@ PyObject *py_conv_silu_fwd(PyObject *, PyObject *const *a, Py_ssize_t n) {
   need_dims(x, "x", 3);
   const int64_t B = x.size(0), T = x.size(1), C = x.size(2);
   const ScalarType io = x.scalar_type();
+  check(x, "x", {B, T, C}, io, true);
   check(w, "w", {C, 4}, io);
   check(bias, "bias", {C}, io);
   check(prev, "prev", {B, 3, C}, io);
-  if (!x.is_cuda()) fail(PyExc_ValueError, "x must be a CUDA tensor");
   const Tensor out = given_or_empty(opt_tensor(a[4], "out"), {B, T, C}, io, x.device());
   check(out, "out", {B, T, C}, io, true);
   const int32_t code = io_code(x);
@@ -511,6 +513,7 @@ PyObject *py_conv_silu_bwd(PyObject *, PyObject *const *a, Py_ssize_t n) {
   need_dims(x, "x", 3);
   const int64_t B = x.size(0), T = x.size(1), C = x.size(2);
   const ScalarType io = x.scalar_type();
+  check(x, "x", {B, T, C}, io, true);
   check(w, "w", {C, 4}, io);
   check(bias, "bias", {C}, io);
   check(prev, "prev", {B, 3, C}, io);
