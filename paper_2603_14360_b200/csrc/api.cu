@@ -1,5 +1,7 @@
 // C ABI of the M2RNN scan library: argument checks, workspace layout, dispatch.
-// No allocation, no synchronisation, no state kept between calls.
+// No allocation, no synchronisation.  Kept between calls: constants of the device (its SM count) and which
+// kernels have had their limit of shared memory raised (smem_limit.h), both asked for once.
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <atomic>
@@ -8,6 +10,7 @@
 
 #include "internal.h"
 #include "m2rnn.h"
+#include "smem_limit.h"
 
 namespace m2rnn {
 
@@ -37,32 +40,45 @@ int sm_count() {
   return sms;
 }
 
-// Lets `kernel` be launched with `bytes` of dynamic shared memory on the current device.  The
-// attribute stays with the loaded kernel, so it is set when a launch first needs more than any
-// before it (setting it on every launch cost a small call a tenth of its host time).
+namespace {
+// cuCtxGetId through the runtime's driver entry point (no link against libcuda)
+struct CudaSmem {
+  bool context(uint64_t *id) const {
+    using GetId = CUresult (*)(CUcontext, unsigned long long *);
+    static const GetId get = [] {
+      void *p = nullptr;
+      cudaDriverEntryPointQueryResult q;
+      if (cudaGetDriverEntryPoint("cuCtxGetId", &p, cudaEnableDefault, &q) != cudaSuccess || q != cudaDriverEntryPointSuccess) {
+        (void)cudaGetLastError();
+        p = nullptr;
+      }
+      return reinterpret_cast<GetId>(p);
+    }();
+    unsigned long long n = 0;
+    if (!get || get(nullptr, &n) != CUDA_SUCCESS) return false;   // (null: the current context)
+    *id = n;
+    return true;
+  }
+  int most(const void *kernel, int *n) const {
+    int dev = 0, optin = 0;
+    cudaFuncAttributes at;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&at, kernel);
+    if (e == cudaSuccess) *n = optin - (int)at.sharedSizeBytes;
+    return e;
+  }
+  int set(const void *kernel, int n) const { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, n); }
+};
+}  // namespace
+
+// Lets `kernel` be launched with `bytes` of dynamic shared memory in the current context.  (Asking the runtime on
+// every launch cost a small call a tenth of its host time.)
 cudaError_t allow_smem(const void *kernel, size_t bytes) {
-  constexpr int kSlots = 1024;   // (kernel, device) pairs: far more than the library has kernels
-  struct Entry { std::atomic<uintptr_t> key; std::atomic<int> bytes; };
-  static Entry table[kSlots];
   if (bytes <= 40 * 1024) return cudaSuccess;   // with up to 8 KB of static shared memory: what every kernel may use unasked
-  const int dev = current_device();
-  Entry *e = nullptr;
-  if (dev >= 0 && dev < kMaxDevices) {
-    const uintptr_t key = reinterpret_cast<uintptr_t>(kernel) * kMaxDevices + (uintptr_t)dev + 1;
-    size_t h = (size_t)((key * 0x9e3779b97f4a7c15ull) >> 54);
-    for (int probe = 0; probe < 64 && !e; ++probe, h = (h + 1) % kSlots) {
-      uintptr_t seen = table[h].key.load(std::memory_order_acquire);
-      if (seen == 0 && table[h].key.compare_exchange_strong(seen, key, std::memory_order_acq_rel)) seen = key;
-      if (seen == key) e = &table[h];
-    }
-  }
-  if (e && e->bytes.load(std::memory_order_acquire) >= (int)bytes) return cudaSuccess;
-  const cudaError_t rc = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (rc == cudaSuccess && e) {
-    int old = e->bytes.load(std::memory_order_relaxed);
-    while (old < (int)bytes && !e->bytes.compare_exchange_weak(old, (int)bytes, std::memory_order_release)) {}
-  }
-  return rc;
+  static SmemLimits<CudaSmem> limits(cudaErrorInvalidValue);
+  CudaSmem api;
+  return static_cast<cudaError_t>(limits.allow(api, kernel, bytes));
 }
 
 bool bwd_use_tc(int B, int N, int K, int V, int io_dtype) {
