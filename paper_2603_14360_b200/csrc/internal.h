@@ -57,27 +57,41 @@ __device__ __forceinline__ UnitSpan unit_span(const ScanArgs &a, int b) {
 // The batch entry that the CTAs at place `pos` of the grid's order take.  Sequences of a packed batch are
 // taken longest first: CTAs are handed out in order, and a long one that starts last leaves the
 // other SMs idle (12 sequences of up to 4 000 tokens, K = V = 128, forward + backward: 20.4 -> 18.6 ms).
-// Every thread of the CTA calls it, before it uses `scratch` (shared memory) otherwise.
-// Above 1 024 sequences their order no longer matters and the search would cost.
+// Every thread of the CTA calls it, before it uses `scratch` (kRankWords words of shared memory) otherwise.
+// `pace`: the kernel's time per step, in 0.1 us.
 // (Not inlined: the kernels' inner loops are sensitive to what the compiler schedules around them.)
-static __device__ __noinline__ int longest_first(const int32_t *cu, int B, int pos, int *scratch);
-__device__ __forceinline__ int batch_entry(const ScanArgs &a, int pos, void *scratch) {
+constexpr int kRankBatch = 512, kRankWords = kRankBatch + 4;
+static __device__ __noinline__ int longest_first(const int32_t *cu, int B, float scan, int pos, int *scratch);
+__device__ __forceinline__ int batch_entry(const ScanArgs &a, int pos, void *scratch, int pace) {
   // (through a shuffle: known to be the same in all lanes, so that what derives from it stays in uniform
   // registers -- 5 to 9 % of a step in the tcgen05 kernel)
-  return __shfl_sync(0xffffffffu, a.cu && a.B > 1 && a.B <= 1024 ? longest_first(a.cu, a.B, pos, static_cast<int *>(scratch)) : pos, 0);
+  return __shfl_sync(0xffffffffu, a.cu && a.B > 1 && a.B <= kRankBatch ? longest_first(a.cu, a.B, 0.1f * pace * a.T, pos, static_cast<int *>(scratch)) : pos, 0);
 }
-static __device__ __noinline__ int longest_first(const int32_t *cu, int B, int pos, int *scratch) {
-  for (int b = threadIdx.x; b < B; b += blockDim.x) {
-    const int len = cu[b + 1] - cu[b];
-    int rank = 0;
-    for (int o = 0; o < B; ++o) {
-      const int other = cu[o + 1] - cu[o];
-      rank += other > len || (other == len && o < b);
-    }
-    if (rank == pos) *scratch = b;
+static __device__ __noinline__ int longest_first(const int32_t *cu, int B, float scan, int pos, int *scratch) {
+  // Every CTA ranks the batch for itself, some B^2 comparisons: 0.25 us, 1 us for 256 sequences.  Waves of CTAs times
+  // that has to stay below what the order can give, a part of the longest scan (`scan`, us), which counts once.
+  // Forward, K = V = 64, two heads, us in the grid's order / always ranked, from memory, length by length / now:
+  // 256 sequences of up to 256 tokens 164 / 136 / 127, 512 of 2048 2050 / 1809 / 1745, of 32 61 / 174 / 63, 1000 of 32 113 /
+  // 922 / 113; K = 64, V = 16, 16 heads, 256 of 2048 1491 / 1392 / 1340, of 256 201 / 277 / 202.
+  if ((float)gridDim.x * blockDim.x * ((float)B * B + 22000.f) > 1.75e9f * scan) return pos;
+  const int pad = (B + 3) & ~3;
+  for (int b = threadIdx.x; b < pad; b += blockDim.x) {   // keys: the length above the place in the batch, all different
+    const int len = b < B ? min(max(cu[b + 1] - cu[b], 0), (1 << 22) - 1) : 0;
+    scratch[b] = b < B ? len * kRankBatch + (kRankBatch - 1 - b) : -1;
   }
   __syncthreads();
-  const int b = *static_cast<volatile int *>(scratch);
+  for (int b = threadIdx.x; b < B; b += blockDim.x) {
+    const int key = scratch[b];
+    int rank = 0;
+#pragma unroll 4
+    for (int o = 0; o < pad; o += 4) {
+      const int4 k = *reinterpret_cast<const int4 *>(scratch + o);
+      rank += (k.x > key) + (k.y > key) + (k.z > key) + (k.w > key);
+    }
+    if (rank == pos) scratch[pad] = b;
+  }
+  __syncthreads();
+  const int b = *static_cast<volatile int *>(scratch + pad);
   __syncthreads();
   return b;
 }

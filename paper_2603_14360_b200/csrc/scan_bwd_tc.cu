@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_tc_kernel(ScanArgs a) {
   using S = TcBwdSmem;
   constexpr int V = kV;
   const int C = a.C;                 // steps per chunk (<= kCTc, which sizes the buffers)
-  extern __shared__ unsigned char smem_dyn[];
+  extern __shared__ __align__(16) unsigned char smem_dyn[];
   const uint32_t base_sa = (smem_u32(smem_dyn) + 1023u) & ~1023u;
   unsigned char *base = smem_dyn + (base_sa - smem_u32(smem_dyn));
   uint64_t *bars = reinterpret_cast<uint64_t *>(base + S::oBar);
@@ -128,7 +128,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_tc_kernel(ScanArgs a) {
   const int RS = K / kNR;
   const int place = blockIdx.x / RS, rs = blockIdx.x % RS;
   const int n = place % N;
-  const int b = batch_entry(a, place / N, smem_dyn), unit = b * N + n;
+  const int b = batch_entry(a, place / N, smem_dyn, 12), unit = b * N + n;
   const int rbase = rs * kNR;
   const UnitSpan span = unit_span(a, b);
   const int T = span.T;

@@ -201,7 +201,7 @@ __global__ void __launch_bounds__(Geom<V>::kThreads) fwd_f32_kernel(ScanArgs a) 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, p = lane >> 2, c0 = 8 * warp + 2 * (lane & 3);
   const int orow = Own<GR>::row(p), ocol = Own<GR>::col(p, c0), ycol = y_col<GR>(lane, c0);
   const int place = blockIdx.x / RS, rs = blockIdx.x % RS, rbase = rs * R;
-  const int b = batch_entry(a, place / N, smem), n = place % N, bn = b * N + n;
+  const int b = batch_entry(a, place / N, smem, 7), n = place % N, bn = b * N + n;
   const UnitSpan span = unit_span(a, b);   // this batch entry's tokens (a slice of a packed batch, or b T ..)
   const int T = span.T;
   const size_t tok0 = span.tok0, KV = (size_t)K * V;
@@ -323,7 +323,7 @@ __global__ void __launch_bounds__(Geom<V>::kThreads, 512 / Geom<V>::kThreads) bw
   const int K = a.K, N = a.N;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, p = lane >> 2, c0 = 8 * warp + 2 * (lane & 3);
   const int place = blockIdx.x / nslab, rs = slab0 + blockIdx.x % nslab, rbase = rs * GR;
-  const int b = batch_entry(a, place / N, smem), n = place % N, bn = b * N + n;
+  const int b = batch_entry(a, place / N, smem, 12), n = place % N, bn = b * N + n;
   const bool add = nslab == 1 && rs > 0;   // earlier launches have written dv, dgate and dW
   const UnitSpan span = unit_span(a, b);
   const int T = span.T;

@@ -68,7 +68,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) fwd_tc_kernel(ScanArgs a) {
   // rows of its column are one or two 16-byte stores.
   constexpr int kChunks = kRowsT / 8;
   constexpr int kRowsCta = kGroups * NR;
-  extern __shared__ unsigned char smem_dyn[];
+  extern __shared__ __align__(16) unsigned char smem_dyn[];
   const uint32_t base_sa = (smem_u32(smem_dyn) + 1023u) & ~1023u;   // the swizzled tiles want 1024-byte alignment
   unsigned char *base = smem_dyn + (base_sa - smem_u32(smem_dyn));
   uint64_t *full = reinterpret_cast<uint64_t *>(base + S::oBar);    // [kStagesTc] a stage's inputs are staged
@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) fwd_tc_kernel(ScanArgs a) {
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const int NG = (N + HS - 1) / HS;               // head groups
   const int RS = (K + kRowsCta - 1) / kRowsCta;   // CTAs per (b, head group)
-  const int rs = blockIdx.x % RS, hg = (blockIdx.x / RS) % NG, b = batch_entry(a, blockIdx.x / (RS * NG), smem_dyn);
+  const int rs = blockIdx.x % RS, hg = (blockIdx.x / RS) % NG, b = batch_entry(a, blockIdx.x / (RS * NG), smem_dyn, 4);
   const int rbase = rs * kRowsCta;
   const UnitSpan span = unit_span(a, b);   // this batch entry's tokens (a slice of a packed batch, or b T ..)
   const int T = span.T;

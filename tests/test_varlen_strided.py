@@ -115,6 +115,35 @@ def test_packed_batches(oracle, monkeypatch, case, variant):
             assert torch.equal(hT[b], g["h0"][b]) and torch.equal(out["dh0"][b], g["d_hT"][b])
 
 
+# batches on both sides of the sizes up to which the kernels take the longest sequences first, with ties, empty
+# sequences and one long one in the middle; two heads, so that each sequence has several CTAs
+@pytest.mark.gpu
+@pytest.mark.parametrize("B,T", [(2, 9), (33, 40), (131, 64), (300, 12), (300, 200), (512, 300), (513, 300)])
+@pytest.mark.parametrize("dtype,V", [("bf16", 16), ("bf16", 32), ("f32", 16)])
+def test_many_sequences(oracle, dtype, V, B, T):
+    rng = np.random.default_rng(B + T)
+    lengths = rng.integers(0, 7, B)
+    lengths[B // 2] = T
+    lengths[B // 3] = T - 1
+    cu = np.concatenate([[0], np.cumsum(lengths)]).astype(np.int32)
+    tokens, N = int(cu[-1]), 2
+    cfg = ScanConfig("many", B=1, T=tokens, N=N, K=16, V=V, dtype=dtype, gate_mean=1.0, w_scale=0.5, seed=B)
+    d = {x: (t[0] if x in ("q", "k", "v", "gate", "dy") else t) for x, t in inputs.make_inputs(cfg, backward=True).items()}
+    d["h0"] = d["h0"].repeat(B, 1, 1, 1) * torch.linspace(-1.0, 1.0, B).view(B, 1, 1, 1)     # every sequence its own state
+    args = [F(d[x]) for x in ("q", "k", "v", "gate", "W")]
+    y_ref, hT_ref = oracle.fwd_varlen(*args, cu, F(d["h0"]))
+    ref = oracle.bwd_varlen(*args, cu, F(d["h0"]), F(d["dy"]))
+    g = parity.to_dev(d)
+    kw = dict(cu_seqlens=torch.from_numpy(cu).cuda(), max_seqlen=T)
+    y, hT, ckpt = binding.m2rnn_fwd(g["q"], g["k"], g["v"], g["gate"], g["W"], g["h0"], save_ckpt=True, **kw)
+    out = binding.m2rnn_bwd(g["q"], g["k"], g["v"], g["gate"], g["W"], g["h0"], g["dy"], ckpt=ckpt, **kw)
+    binding.check_device_status()
+    tol = parity.TOL[dtype]
+    assert parity.rel_err(y, y_ref) <= tol and parity.rel_err(hT, hT_ref) <= tol
+    for x in ref:
+        assert parity.rel_err(out[x], ref[x]) <= tol, x
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("dtype,K,V,N,Nq", [("f32", 32, 32, 2, 2), ("bf16", 64, 64, 2, 2), ("bf16", 64, 16, 8, 1), ("bf16", 128, 128, 1, 1)])
 def test_views_into_a_fused_projection(oracle, dtype, K, V, N, Nq):
