@@ -5,7 +5,8 @@
 //     x = y (.) g,   s = 1 / sqrt(mean x^2 + eps),   out = w (.) x s            (s is cached)
 //     p = w (.) dout, r = sum p x, dx = s p - r s^3 x / d, dy = dx (.) g, dg = dx (.) y (SiLU'),
 //     dw = sum over tokens of dout (.) x s.
-// HBM-bound.  One to eight warps share a row so that a lane holds at most three chunks of eight features:
+// HBM-bound.  One to eight warps share a row so that a lane holds at most three chunks of eight features (four of a row
+// of 1 024, see split_of):
 // that keeps its share of the row, its columns' dw sums and the next row on the way (16-byte cp.async
 // into a ring) within two (backward) to four CTAs per SM, whatever the row length.  One partial of dw per
 // persistent CTA, added by a fixed-order second stage.  16 384 rows: of 1 344 features (84 heads x 16)
@@ -83,8 +84,9 @@ __device__ __forceinline__ Raw8<T> load_raw(const T *p) {
 // per lane, its ring leaves room for one CTA per SM: 4 096 x 1 344 forward 22 us with it, 16 without.)
 __host__ __device__ constexpr bool uses_ring(int elem) { return elem == 2; }
 // CTAs per SM a variant is compiled for and launched with: what its registers and its ring allow.
-// chunks: of a lane at a time (CPL R)
-__host__ __device__ constexpr int resident(bool bwd, int elem, int chunks) {
+// chunks: of a lane at a time (CPL R); full: see Walk
+__host__ __device__ constexpr int resident(bool bwd, int elem, int chunks, bool full) {
+  if (full) return bwd ? (chunks == 1 ? 3 : (chunks == 2 ? 2 : 1)) : (chunks == 1 ? 8 : (chunks == 2 && elem == 2 ? 5 : 3));
   return bwd ? (elem == 4 && chunks > 3 ? 1 : 2) : (chunks <= 2 ? 4 : 3);
 }
 
@@ -93,10 +95,12 @@ __host__ __device__ constexpr int resident(bool bwd, int elem, int chunks) {
 // ring of two stages in shared memory of which a lane copies (cp.async) and reads its own 16-byte
 // pieces only: the next rows are on their way while these are worked on, a second pass over a row
 // reads them again, and no barrier is needed.
-template <typename T, int CPL, int R, int G, int NTENS>
+// FULL: a row is exactly the lanes' chunks, which then are loaded without a look at the row's end, all of them
+// before the first is used, and need no ring.
+template <typename T, int CPL, int R, int G, int NTENS, bool FULL>
 struct Walk {
   static constexpr int NP = Raw8<T>::kPieces, kGroups = kWarps / G;
-  static constexpr bool kRing = uses_ring(sizeof(T));
+  static constexpr bool kRing = uses_ring(sizeof(T)) && !FULL;
   static constexpr int kSmem = kRing ? 2 * NTENS * R * CPL * NP * kThreads * 16 : 0;
   uint4 *ring;
   int lane, group, gw;               // gw: warp of the group
@@ -112,7 +116,7 @@ struct Walk {
     step = (long)gridDim.x * kGroups * R;
     col = 8 * (32 * gw + lane);
   }
-  __device__ __forceinline__ bool on(int j) const { return col + 256 * G * j < d; }
+  __device__ __forceinline__ bool on(int j) const { return FULL || col + 256 * G * j < d; }
   __device__ __forceinline__ uint4 *piece(int stage, int x, int r, int j, int p) const {
     return ring + ((((stage * NTENS + x) * R + r) * CPL + j) * NP + p) * kThreads;
   }
@@ -142,6 +146,14 @@ struct Walk {
     for (int q = 0; q < NP; ++q) v.v[q] = *piece(stage, x, r, j, q);
     return v;
   }
+  // the lane's chunks of this row (FULL)
+  template <int N> __device__ __forceinline__ void get_row(const T *const (&src)[NTENS], Raw8<T> (&row)[N][CPL]) const {
+    static_assert(FULL && R == 1 && N == NTENS);
+#pragma unroll
+    for (int j = 0; j < CPL; ++j)
+#pragma unroll
+      for (int x = 0; x < N; ++x) row[x][j] = load_raw(src[x] + t * d + col + 256 * G * j);
+  }
   // v[r] summed over the group.  red: [2][kWarps][R] floats, used in turn so that one barrier a call is enough
   __device__ __forceinline__ void row_sums(float (&v)[R], float *red, int buf) const {
 #pragma unroll
@@ -163,13 +175,13 @@ struct Walk {
   }
 };
 
-template <typename T, int CPL, int R, int G>
-__global__ void __launch_bounds__(kThreads, resident(false, sizeof(T), CPL * R)) gated_norm_fwd_kernel(
+template <typename T, int CPL, int R, int G, bool FULL>
+__global__ void __launch_bounds__(kThreads, resident(false, sizeof(T), CPL * R, FULL)) gated_norm_fwd_kernel(
     long tokens, int d, const T *__restrict__ y, const T *__restrict__ g_in, const T *__restrict__ w, float eps, int use_silu,
     T *__restrict__ out, float *__restrict__ rstd) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ float red[2 * kWarps * R];
-  Walk<T, CPL, R, G, 2> wk(smem, tokens, d);
+  Walk<T, CPL, R, G, 2, FULL> wk(smem, tokens, d);
   const T *const src[2] = {y, g_in};
   wk.fetch(0, wk.t, src);
   const float inv_d = 1.f / (float)d;
@@ -179,13 +191,15 @@ __global__ void __launch_bounds__(kThreads, resident(false, sizeof(T), CPL * R))
     asm volatile("cp.async.wait_group 1;" ::: "memory");
     float2 x[R][CPL][4];
     float ss[R];
+    Raw8<T> row[2][FULL ? CPL : 1];
+    if constexpr (FULL) wk.get_row(src, row);
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       float2 s2 = make_float2(0.f, 0.f);
 #pragma unroll
       for (int j = 0; j < CPL; ++j)
         if (wk.on(j)) {
-          const Raw8<T> a = wk.get(src, st, 0, r, j), b = wk.get(src, st, 1, r, j);
+          const Raw8<T> a = FULL ? row[0][FULL ? j : 0] : wk.get(src, st, 0, r, j), b = FULL ? row[1][FULL ? j : 0] : wk.get(src, st, 1, r, j);
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
             float2 g = pair_of(b, i);
@@ -219,13 +233,13 @@ __global__ void __launch_bounds__(kThreads, resident(false, sizeof(T), CPL * R))
   asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
 
-template <typename T, int CPL, int R, int G>
-__global__ void __launch_bounds__(kThreads, resident(true, sizeof(T), CPL * R)) gated_norm_bwd_kernel(
+template <typename T, int CPL, int R, int G, bool FULL>
+__global__ void __launch_bounds__(kThreads, resident(true, sizeof(T), CPL * R, FULL)) gated_norm_bwd_kernel(
     long tokens, int d, const T *__restrict__ y, const T *__restrict__ g_in, const T *__restrict__ w, const float *__restrict__ rstd,
     int use_silu, const T *__restrict__ dout, T *__restrict__ dy, T *__restrict__ dg_in, float *__restrict__ dw_part) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ float red[2 * kWarps * R];
-  Walk<T, CPL, R, G, 3> wk(smem, tokens, d);
+  Walk<T, CPL, R, G, 3, FULL> wk(smem, tokens, d);
   const T *const src[3] = {y, g_in, dout};
   wk.fetch(0, wk.t, src);
   Raw8<T> wr[CPL];
@@ -246,13 +260,16 @@ __global__ void __launch_bounds__(kThreads, resident(true, sizeof(T), CPL * R)) 
     wk.fetch(st ^ 1, wk.t + wk.step, src);
     asm volatile("cp.async.wait_group 1;" ::: "memory");
     float2 sg[R][CPL][4];
+    Raw8<T> row[3][FULL ? CPL : 1];
+    if constexpr (FULL) wk.get_row(src, row);
+    auto piece = [&](int x, int r, int j) { return FULL ? row[x][FULL ? j : 0] : wk.get(src, st, x, r, j); };
 #pragma unroll
     for (int r = 0; r < R; ++r) {   // r = sum_j w_j dout_j x_j
       float2 r2 = make_float2(0.f, 0.f);
 #pragma unroll
       for (int j = 0; j < CPL; ++j)
         if (wk.on(j)) {
-          const Raw8<T> a = wk.get(src, st, 0, r, j), b = wk.get(src, st, 1, r, j), dv = wk.get(src, st, 2, r, j);
+          const Raw8<T> a = piece(0, r, j), b = piece(1, r, j), dv = piece(2, r, j);
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
             float2 g = pair_of(b, i);
@@ -272,7 +289,7 @@ __global__ void __launch_bounds__(kThreads, resident(true, sizeof(T), CPL * R)) 
 #pragma unroll
       for (int j = 0; j < CPL; ++j)
         if (wk.on(j)) {
-          const Raw8<T> a = wk.get(src, st, 0, r, j), b = wk.get(src, st, 1, r, j), dv = wk.get(src, st, 2, r, j);
+          const Raw8<T> a = piece(0, r, j), b = piece(1, r, j), dv = piece(2, r, j);
           float o1[8], o2[8];
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
@@ -330,18 +347,33 @@ __global__ void __launch_bounds__(1024) reduce_partials_kernel(const float *__re
 // How a call is split: warps per row (a lane holds at most three chunks: with four the backward kernel spills at
 // two CTAs per SM; d > 6 144 has no choice), chunks per lane, rows at a time (short rows: as many
 // bytes on their way as four chunks) and persistent CTAs, as many as are resident.
-struct Split { int g, cpl, r, grid; };
+// Rows of exactly 256, 512 or 1 024 features: a warp each, its whole row loaded at once and without a ring, forward
+// in as many CTAs as there are rows for, up to eight an SM.  The general form costs such rows 2 to 35 % (16 384
+// rows, us: bf16 forward 7.7, 12.3, 19.7 -> 6.2, 10.3, 18.0; fp32 forward of 256 and 512 15.4, 22.9 -> 11.2, 18.4,
+// backward 27, 46, 65 -> 20, 33, 59).  Not where it is no better: the bf16 backward (14.4, 20.9, 31.3, ring) and the fp32 forward
+// of 1 024 (33.1, two warps a row; one 33 to 37).
+struct Split { int g, cpl, r, grid; bool full; };
 Split split_of(long tokens, int d, bool bwd, int io_dtype) {
   Split s;
   const int chunks = d / 8;
-  const int most = io_dtype == M2RNN_F32 ? 64 : 96;   // chunks of a warp
+  const int sms = sm_count();
+  const bool f32 = io_dtype == M2RNN_F32;
+  s.full = bwd ? f32 && (chunks == 32 || chunks == 64 || chunks == 128) : chunks == 32 || chunks == 64 || (chunks == 128 && !f32);
+  if (s.full) {
+    s.g = 1; s.cpl = chunks / 32; s.r = 1;
+    const long need = (tokens + kWarps - 1) / kWarps, slots = (long)sms * (bwd ? resident(true, 4, s.cpl, true) : 8);
+    s.grid = (int)(need < slots ? need : slots);
+    if (bwd && s.grid > kMaxCtas) s.grid = kMaxCtas;
+    return s;
+  }
+  const int most = f32 ? 64 : 96;   // chunks of a warp
   s.g = chunks <= most ? 1 : (chunks <= 2 * most ? 2 : (chunks <= 4 * most ? 4 : 8));
   s.cpl = (chunks + 32 * s.g - 1) / (32 * s.g);
   s.r = s.g > 1 || s.cpl > 2 ? 1 : (s.cpl == 1 ? 4 : 2);
-  const int sms = sm_count(), per = kWarps / s.g;
+  const int per = kWarps / s.g;
   if (tokens < 8L * sms * per) s.r = 1;
   const long need = (tokens + per * s.r - 1) / (per * s.r);
-  const long slots = (long)sms * resident(bwd, io_dtype == M2RNN_F32 ? 4 : 2, s.cpl * s.r);
+  const long slots = (long)sms * resident(bwd, f32 ? 4 : 2, s.cpl * s.r, false);
   s.grid = (int)(need < slots ? need : slots);
   if (s.grid > kMaxCtas) s.grid = kMaxCtas;
   return s;
@@ -356,12 +388,20 @@ int check(long tokens, int d, int io_dtype) {
   return M2RNN_OK;
 }
 
-// f(CPL, R, G) as compile-time constants
-template <typename F>
+// f(CPL, R, G, FULL) as compile-time constants; kFull: the most chunks a lane of a FULL form takes (0: there is none)
+template <int kFull, typename F>
 cudaError_t with_split(const Split &s, F f) {
+  using No = std::false_type;
+  using One = std::integral_constant<int, 1>;
+  if constexpr (kFull >= 2) {
+    if (s.full && s.cpl == 1) return f(One{}, One{}, One{}, std::true_type{});
+    if (s.full && s.cpl == 2) return f(std::integral_constant<int, 2>{}, One{}, One{}, std::true_type{});
+  }
+  if constexpr (kFull >= 4)
+    if (s.full && s.cpl == 4) return f(std::integral_constant<int, 4>{}, One{}, One{}, std::true_type{});
 #define M2RNN_CASE(C, R_, G_) \
   if (s.cpl == C && s.r == R_ && s.g == G_) \
-    return f(std::integral_constant<int, C>{}, std::integral_constant<int, R_>{}, std::integral_constant<int, G_>{})
+    return f(std::integral_constant<int, C>{}, std::integral_constant<int, R_>{}, std::integral_constant<int, G_>{}, No{})
   M2RNN_CASE(1, 4, 1); M2RNN_CASE(1, 1, 1); M2RNN_CASE(2, 2, 1); M2RNN_CASE(2, 1, 1); M2RNN_CASE(3, 1, 1);
   M2RNN_CASE(2, 1, 2); M2RNN_CASE(3, 1, 2); M2RNN_CASE(2, 1, 4); M2RNN_CASE(3, 1, 4); M2RNN_CASE(2, 1, 8); M2RNN_CASE(3, 1, 8); M2RNN_CASE(4, 1, 8);
 #undef M2RNN_CASE
@@ -372,9 +412,9 @@ template <typename T>
 cudaError_t launch_fwd(long tokens, int d, const void *y, const void *g, const void *w, float eps, int silu_on, void *out,
                        float *rstd, cudaStream_t s) {
   const Split sp = split_of(tokens, d, false, sizeof(T) == 2 ? M2RNN_BF16 : M2RNN_F32);
-  return with_split(sp, [&](auto C, auto R, auto G) {
-    auto kern = gated_norm_fwd_kernel<T, C(), R(), G()>;
-    constexpr int smem = Walk<T, C(), R(), G(), 2>::kSmem;
+  return with_split<sizeof(T) == 4 ? 2 : 4>(sp, [&](auto C, auto R, auto G, auto FULL) {
+    auto kern = gated_norm_fwd_kernel<T, C(), R(), G(), FULL()>;
+    constexpr int smem = Walk<T, C(), R(), G(), 2, FULL()>::kSmem;
     const cudaError_t e = allow_smem(kern, smem);
     if (e != cudaSuccess) return e;
     kern<<<sp.grid, kThreads, smem, s>>>(tokens, d, static_cast<const T *>(y), static_cast<const T *>(g), static_cast<const T *>(w), eps, silu_on,
@@ -387,10 +427,10 @@ template <typename T>
 cudaError_t launch_bwd(long tokens, int d, const void *y, const void *g, const void *w, const float *rstd, int silu_on,
                        const void *dout, void *dy, void *dg, float *dw_part, cudaStream_t s) {
   const Split sp = split_of(tokens, d, true, sizeof(T) == 2 ? M2RNN_BF16 : M2RNN_F32);
-  return with_split(sp, [&](auto C, auto R, auto G) {
-    auto kern = gated_norm_bwd_kernel<T, C(), R(), G()>;
+  return with_split<sizeof(T) == 4 ? 4 : 0>(sp, [&](auto C, auto R, auto G, auto FULL) {
+    auto kern = gated_norm_bwd_kernel<T, C(), R(), G(), FULL()>;
     constexpr int sums = 256 * C() * kWarps * 4;    // groups x the columns they can hold, at the end
-    constexpr int smem = Walk<T, C(), R(), G(), 3>::kSmem > sums ? Walk<T, C(), R(), G(), 3>::kSmem : sums;
+    constexpr int smem = Walk<T, C(), R(), G(), 3, FULL()>::kSmem > sums ? Walk<T, C(), R(), G(), 3, FULL()>::kSmem : sums;
     const cudaError_t e = allow_smem(kern, smem);
     if (e != cudaSuccess) return e;
     kern<<<sp.grid, kThreads, smem, s>>>(tokens, d, static_cast<const T *>(y), static_cast<const T *>(g), static_cast<const T *>(w), rstd, silu_on,

@@ -87,3 +87,11 @@ def test_gated_norm_rejects_bad_arguments():
 def test_gated_norm_splits(oracle, shape, dtype, tol):
     errs = _run(oracle, shape, dtype, True, 1e-6)
     assert max(errs.values()) < tol, errs
+
+
+# rows of exactly 256, 512 and 1024 features, one more than a pass of the forward grid takes (8 rows a CTA, 8 CTAs on each of 148 SMs)
+@pytest.mark.parametrize("shape", [(1, 9473, 4, 64), (1, 9473, 8, 64), (1, 9473, 16, 64)], ids=lambda s: "x".join(map(str, s)))
+@pytest.mark.parametrize("dtype,tol", [("bf16", 2e-2), ("f32", 1e-4)])
+def test_gated_norm_full_rows(oracle, shape, dtype, tol):
+    errs = _run(oracle, shape, dtype, True, 1e-6)
+    assert max(errs.values()) < tol, errs
