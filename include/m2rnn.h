@@ -169,9 +169,13 @@ int m2rnn_bwd(const m2rnn_params *params, const void *q, const void *k, const vo
  * array's memory is claimed at that moment: on a device that is already full the first call can
  * therefore fail with M2RNN_ERR_CUDA.  So make the first call on each device at start-up, while
  * memory is still to be had (any small problem will do), or run with CUDA_MODULE_LOADING=EAGER.
- *   - A problem whose m2rnn_bwd_workspace_bytes(params, ckpt != NULL) exceeds
- *     M2RNN_STATIC_SCRATCH_BYTES is refused with M2RNN_ERR_WORKSPACE before anything runs;
- *     passing the checkpoints written by m2rnn_fwd lowers the need.
+ *   - A problem whose scratch exceeds M2RNN_STATIC_SCRATCH_BYTES is refused with
+ *     M2RNN_ERR_WORKSPACE before anything runs; passing the checkpoints written by m2rnn_fwd lowers
+ *     the need.  The scratch is m2rnn_bwd_workspace_bytes(params, ckpt != NULL) at most: an M2RNN_F32
+ *     problem for which that is too much is taken one group of eight state rows after the other,
+ *     without the groups' shares of dv, dgate and dW.  It is slower then, and takes (floats, each
+ *     array rounded up to 256 bytes) B N V V, plus B T N K for each of q and k whose heads are shared, plus the
+ *     checkpoints if they are not passed, plus B N ceil(C/16) K V if the interval C is above 16.
  *   - The first call on each device looks up the array's device address (the device that is
  *     current at the call); that same start-up call must come before any stream capture.
  *   - All calls share the one array, which keeps whatever the last call left in it.  Nothing in

@@ -89,10 +89,10 @@ bool bwd_use_tc(int B, int N, int K, int V, int io_dtype) {
   return true;
 }
 
-BwdPlan plan_bwd(int B, int N, int K, int V, int io_dtype, size_t tokens) {
+BwdPlan plan_bwd(int B, int N, int K, int V, int io_dtype, size_t tokens, bool lean) {
   BwdPlan pl{};
   if (io_dtype == M2RNN_F32) {
-    pl.KC = bwd_f32_rows(B, N, K, V, tokens * N * V * sizeof(float)); pl.C = bwd_f32_piece(); pl.C_max = 64;
+    pl.KC = lean ? K : bwd_f32_rows(B, N, K, V, tokens * N * V * sizeof(float)); pl.C = bwd_f32_piece(); pl.C_max = 64;
     return pl;
   }
   if (bwd_use_tc(B, N, K, V, io_dtype)) {   // 32-row CTAs, chunks of four steps
@@ -217,7 +217,7 @@ struct Workspace {
   size_t ckpt, dW_part, dq_part, dk_part, chunk_states, dv_part, dgate_part, total;
 };
 
-Workspace layout(const m2rnn_params *p, bool have_ckpt) {
+Workspace layout(const m2rnn_params *p, bool have_ckpt, bool lean) {
   Workspace w{};
   const int C = interval_of(p);
   const size_t nch = p->T > 0 ? (size_t)(p->T + C - 1) / C : 0;
@@ -225,7 +225,7 @@ Workspace layout(const m2rnn_params *p, bool have_ckpt) {
   size_t off = 0;
   w.ckpt = off;
   if (!have_ckpt) off += align_up(BN * nch * KV * sizeof(float));
-  const int RS = p->K / plan_bwd(p->B, p->N, p->K, p->V, p->io_dtype, tokens_of(p)).KC;   // row slabs per state
+  const int RS = p->K / plan_bwd(p->B, p->N, p->K, p->V, p->io_dtype, tokens_of(p), lean).KC;   // row slabs per state
   w.dW_part = off;
   off += align_up(BN * RS * p->V * p->V * sizeof(float));
   const size_t TT = tokens_of(p);
@@ -243,11 +243,11 @@ Workspace layout(const m2rnn_params *p, bool have_ckpt) {
   return w;
 }
 
-ScanArgs base_args(const m2rnn_params *p) {
+ScanArgs base_args(const m2rnn_params *p, bool lean = false) {
   ScanArgs a{};
   a.B = p->B; a.T = p->T; a.N = p->N; a.Nq = p->Nq; a.Nk = p->Nk; a.K = p->K; a.V = p->V;
   a.gate_kind = p->gate_kind;
-  a.KC = plan_bwd(p->B, p->N, p->K, p->V, p->io_dtype, tokens_of(p)).KC;
+  a.KC = plan_bwd(p->B, p->N, p->K, p->V, p->io_dtype, tokens_of(p), lean).KC;
   a.KCf = plan_fwd_rows(p->B, p->N, p->K, p->V, p->io_dtype, tokens_of(p));
   a.C = interval_of(p);
   a.nchunks = p->T > 0 ? (p->T + a.C - 1) / a.C : 0;
@@ -261,6 +261,89 @@ ScanArgs base_args(const m2rnn_params *p) {
 }
 
 }  // namespace
+
+size_t bwd_workspace_bytes(const m2rnn_params *params, bool have_ckpt, bool lean) {
+  if (check_params(params, true) != M2RNN_OK) return 0;
+  return layout(params, have_ckpt, lean).total;
+}
+
+int bwd_call(const m2rnn_params *params, const void *q, const void *k, const void *v, const float *gate, const void *W,
+             const float *h0, const float *alpha, const float *beta, const void *w_r, const float *ckpt, const void *dy,
+             const float *d_hT, void *dq, void *dk, void *dv, float *dgate, float *dW, float *dh0, void *workspace,
+             size_t workspace_bytes, bool lean, int32_t *dev_status, void *stream) {
+  int rc = check_params(params, true);
+  if (rc != M2RNN_OK) return rc;
+  if (!dW) return M2RNN_ERR_NULL;
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  if (params->B == 0 || params->T == 0 || tokens_of(params) == 0) {
+    // empty scan: the only defined outputs are dW = 0 and dh0 = d_hT (or 0)
+    if (!aligned16(dW) || !aligned16(dh0) || !aligned16(d_hT)) return M2RNN_ERR_ALIGN;
+    cudaError_t e = cudaMemsetAsync(dW, 0, sizeof(float) * params->N * params->V * params->V, s);
+    if (e == cudaSuccess && dh0 && params->B > 0) {
+      const size_t bytes = sizeof(float) * (size_t)params->B * params->N * params->K * params->V;
+      e = d_hT ? cudaMemcpyAsync(dh0, d_hT, bytes, cudaMemcpyDeviceToDevice, s) : cudaMemsetAsync(dh0, 0, bytes, s);
+    }
+    return e == cudaSuccess ? M2RNN_OK : cuda_failed();
+  }
+  if (!q || !k || !v || !gate || !W || !dy || !dq || !dk || !dv || !dgate) return M2RNN_ERR_NULL;
+  if (params->gate_kind == M2RNN_GATE_PSI && (!alpha || !beta)) return M2RNN_ERR_NULL;
+  const void *ptrs[] = {q, k, v, gate, W, h0, w_r, ckpt, dy, d_hT, dq, dk, dv, dgate, dW, dh0};
+  for (const void *p : ptrs)
+    if (!aligned16(p)) return M2RNN_ERR_ALIGN;
+  const Workspace w = layout(params, ckpt != nullptr, lean);
+  if (w.total > 0 && (!workspace || workspace_bytes < w.total)) return M2RNN_ERR_WORKSPACE;
+  if (reinterpret_cast<uintptr_t>(workspace) % kAlign) return M2RNN_ERR_ALIGN;
+  char *ws = static_cast<char *>(workspace);
+
+  ScanArgs a = base_args(params, lean);
+  a.q = q; a.k = k; a.v = v; a.gate = gate; a.W = W; a.h0 = h0; a.w_r = w_r;
+  a.alpha = params->gate_kind == M2RNN_GATE_PSI ? alpha : nullptr;
+  a.beta = params->gate_kind == M2RNN_GATE_PSI ? beta : nullptr;
+  a.dev_status = dev_status;
+  const bool f32 = params->io_dtype == M2RNN_F32;
+  cudaError_t e = cudaSuccess;
+  if (!ckpt) {
+    // pass 1 of Algorithm 2, thinned: save the state every C steps only
+    ScanArgs f = a;
+    f.y = nullptr; f.hT = nullptr;
+    f.ckpt = reinterpret_cast<float *>(ws + w.ckpt);
+    e = f32 ? launch_fwd_f32(f, s) : launch_fwd_bf16(f, s);
+    if (e != cudaSuccess) return cuda_failed();
+    a.ckpt = f.ckpt;
+  } else {
+    a.ckpt = const_cast<float *>(ckpt);
+  }
+  a.dy = dy; a.d_hT = d_hT; a.dq = dq; a.dk = dk; a.dv = dv; a.dgate = dgate; a.dh0 = dh0;
+  a.dW_part = reinterpret_cast<float *>(ws + w.dW_part);
+  a.dq_part = params->Nq < params->N ? reinterpret_cast<float *>(ws + w.dq_part) : nullptr;
+  a.dk_part = params->Nk < params->N ? reinterpret_cast<float *>(ws + w.dk_part) : nullptr;
+  a.chunk_states = f32 ? reinterpret_cast<float *>(ws + w.chunk_states) : nullptr;
+  const int RS = params->K / a.KC;
+  a.dv_part = RS > 1 ? reinterpret_cast<float *>(ws + w.dv_part) : nullptr;
+  a.dgate_part = RS > 1 ? reinterpret_cast<float *>(ws + w.dgate_part) : nullptr;
+  e = f32 ? launch_bwd_f32(a, s)
+          : (bwd_use_tc(params->B, params->N, params->K, params->V, params->io_dtype) ? launch_bwd_bf16_tc(a, s) : launch_bwd_bf16(a, s));
+  if (e != cudaSuccess) return cuda_failed();
+  e = launch_reduce_dW(a.dW_part, dW, params->B * RS, params->N, params->V, s);
+  if (e != cudaSuccess) return cuda_failed();
+  const size_t BT = tokens_of(params);
+  if (RS > 1) {
+    e = launch_reduce_slabs(a.dv_part, dv, params->io_dtype, RS, BT * params->N * params->V, s);
+    if (e != cudaSuccess) return cuda_failed();
+    e = launch_reduce_slabs(a.dgate_part, dgate, M2RNN_F32, RS, BT * params->N, s);
+    if (e != cudaSuccess) return cuda_failed();
+  }
+  if (a.dq_part) {
+    e = launch_reduce_heads(a.dq_part, dq, params->io_dtype, BT, params->N, params->Nq, params->K, s);
+    if (e != cudaSuccess) return cuda_failed();
+  }
+  if (a.dk_part) {
+    e = launch_reduce_heads(a.dk_part, dk, params->io_dtype, BT, params->N, params->Nk, params->K, s);
+    if (e != cudaSuccess) return cuda_failed();
+  }
+  return M2RNN_OK;
+}
+
 }  // namespace m2rnn
 
 using namespace m2rnn;
@@ -341,8 +424,7 @@ int m2rnn_fwd(const m2rnn_params *params, const void *q, const void *k, const vo
 }
 
 size_t m2rnn_bwd_workspace_bytes(const m2rnn_params *params, int have_ckpt) {
-  if (check_params(params, true) != M2RNN_OK) return 0;
-  return layout(params, have_ckpt != 0).total;
+  return bwd_workspace_bytes(params, have_ckpt != 0, false);
 }
 
 int m2rnn_bwd(const m2rnn_params *params, const void *q, const void *k, const void *v,
@@ -351,77 +433,8 @@ int m2rnn_bwd(const m2rnn_params *params, const void *q, const void *k, const vo
               const float *d_hT, void *dq, void *dk, void *dv, float *dgate, float *dW,
               float *dh0, void *workspace, size_t workspace_bytes, int32_t *dev_status,
               void *stream) {
-  int rc = check_params(params, true);
-  if (rc != M2RNN_OK) return rc;
-  if (!dW) return M2RNN_ERR_NULL;
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (params->B == 0 || params->T == 0 || tokens_of(params) == 0) {
-    // empty scan: the only defined outputs are dW = 0 and dh0 = d_hT (or 0)
-    if (!aligned16(dW) || !aligned16(dh0) || !aligned16(d_hT)) return M2RNN_ERR_ALIGN;
-    cudaError_t e = cudaMemsetAsync(dW, 0, sizeof(float) * params->N * params->V * params->V, s);
-    if (e == cudaSuccess && dh0 && params->B > 0) {
-      const size_t bytes = sizeof(float) * (size_t)params->B * params->N * params->K * params->V;
-      e = d_hT ? cudaMemcpyAsync(dh0, d_hT, bytes, cudaMemcpyDeviceToDevice, s) : cudaMemsetAsync(dh0, 0, bytes, s);
-    }
-    return e == cudaSuccess ? M2RNN_OK : cuda_failed();
-  }
-  if (!q || !k || !v || !gate || !W || !dy || !dq || !dk || !dv || !dgate) return M2RNN_ERR_NULL;
-  if (params->gate_kind == M2RNN_GATE_PSI && (!alpha || !beta)) return M2RNN_ERR_NULL;
-  const void *ptrs[] = {q, k, v, gate, W, h0, w_r, ckpt, dy, d_hT, dq, dk, dv, dgate, dW, dh0};
-  for (const void *p : ptrs)
-    if (!aligned16(p)) return M2RNN_ERR_ALIGN;
-  const Workspace w = layout(params, ckpt != nullptr);
-  if (w.total > 0 && (!workspace || workspace_bytes < w.total)) return M2RNN_ERR_WORKSPACE;
-  if (reinterpret_cast<uintptr_t>(workspace) % kAlign) return M2RNN_ERR_ALIGN;
-  char *ws = static_cast<char *>(workspace);
-
-  ScanArgs a = base_args(params);
-  a.q = q; a.k = k; a.v = v; a.gate = gate; a.W = W; a.h0 = h0; a.w_r = w_r;
-  a.alpha = params->gate_kind == M2RNN_GATE_PSI ? alpha : nullptr;
-  a.beta = params->gate_kind == M2RNN_GATE_PSI ? beta : nullptr;
-  a.dev_status = dev_status;
-  const bool f32 = params->io_dtype == M2RNN_F32;
-  cudaError_t e = cudaSuccess;
-  if (!ckpt) {
-    // pass 1 of Algorithm 2, thinned: save the state every C steps only
-    ScanArgs f = a;
-    f.y = nullptr; f.hT = nullptr;
-    f.ckpt = reinterpret_cast<float *>(ws + w.ckpt);
-    e = f32 ? launch_fwd_f32(f, s) : launch_fwd_bf16(f, s);
-    if (e != cudaSuccess) return cuda_failed();
-    a.ckpt = f.ckpt;
-  } else {
-    a.ckpt = const_cast<float *>(ckpt);
-  }
-  a.dy = dy; a.d_hT = d_hT; a.dq = dq; a.dk = dk; a.dv = dv; a.dgate = dgate; a.dh0 = dh0;
-  a.dW_part = reinterpret_cast<float *>(ws + w.dW_part);
-  a.dq_part = params->Nq < params->N ? reinterpret_cast<float *>(ws + w.dq_part) : nullptr;
-  a.dk_part = params->Nk < params->N ? reinterpret_cast<float *>(ws + w.dk_part) : nullptr;
-  a.chunk_states = f32 ? reinterpret_cast<float *>(ws + w.chunk_states) : nullptr;
-  const int RS = params->K / a.KC;
-  a.dv_part = RS > 1 ? reinterpret_cast<float *>(ws + w.dv_part) : nullptr;
-  a.dgate_part = RS > 1 ? reinterpret_cast<float *>(ws + w.dgate_part) : nullptr;
-  e = f32 ? launch_bwd_f32(a, s)
-          : (bwd_use_tc(params->B, params->N, params->K, params->V, params->io_dtype) ? launch_bwd_bf16_tc(a, s) : launch_bwd_bf16(a, s));
-  if (e != cudaSuccess) return cuda_failed();
-  e = launch_reduce_dW(a.dW_part, dW, params->B * RS, params->N, params->V, s);
-  if (e != cudaSuccess) return cuda_failed();
-  const size_t BT = tokens_of(params);
-  if (RS > 1) {
-    e = launch_reduce_slabs(a.dv_part, dv, params->io_dtype, RS, BT * params->N * params->V, s);
-    if (e != cudaSuccess) return cuda_failed();
-    e = launch_reduce_slabs(a.dgate_part, dgate, M2RNN_F32, RS, BT * params->N, s);
-    if (e != cudaSuccess) return cuda_failed();
-  }
-  if (a.dq_part) {
-    e = launch_reduce_heads(a.dq_part, dq, params->io_dtype, BT, params->N, params->Nq, params->K, s);
-    if (e != cudaSuccess) return cuda_failed();
-  }
-  if (a.dk_part) {
-    e = launch_reduce_heads(a.dk_part, dk, params->io_dtype, BT, params->N, params->Nk, params->K, s);
-    if (e != cudaSuccess) return cuda_failed();
-  }
-  return M2RNN_OK;
+  return bwd_call(params, q, k, v, gate, W, h0, alpha, beta, w_r, ckpt, dy, d_hT, dq, dk, dv, dgate, dW, dh0, workspace, workspace_bytes,
+                  false, dev_status, stream);
 }
 
 int m2rnn_decode_step(const m2rnn_params *params, const void *q, const void *k, const void *v,

@@ -112,8 +112,15 @@ cudaError_t allow_smem(const void *kernel, size_t bytes);   // dynamic shared me
 template <typename... A> cudaError_t allow_smem(void (*kernel)(A...), size_t bytes) {
   return allow_smem(reinterpret_cast<const void *>(kernel), bytes);
 }
-// (tokens: of the batch; they only decide where an fp32 problem is too large for per-slab shares)
-BwdPlan plan_bwd(int B, int N, int K, int V, int io_dtype, size_t tokens = 0);
+// (tokens: of the batch; they only decide where an fp32 problem is too large for per-slab shares.  lean: without
+// such shares, an fp32 problem's groups of rows one after the other)
+BwdPlan plan_bwd(int B, int N, int K, int V, int io_dtype, size_t tokens = 0, bool lean = false);
+// m2rnn_bwd and its workspace query; lean: see plan_bwd
+size_t bwd_workspace_bytes(const m2rnn_params *params, bool have_ckpt, bool lean);
+int bwd_call(const m2rnn_params *params, const void *q, const void *k, const void *v, const float *gate, const void *W,
+             const float *h0, const float *alpha, const float *beta, const void *w_r, const float *ckpt, const void *dy,
+             const float *d_hT, void *dq, void *dk, void *dv, float *dgate, float *dW, float *dh0, void *workspace,
+             size_t workspace_bytes, bool lean, int32_t *dev_status, void *stream);
 int plan_fwd_rows(int B, int N, int K, int V, int io_dtype, size_t tokens = 0);   // state rows per CTA of the forward kernel
 // Which bf16 forward kernel takes a problem: the tcgen05 kernel (scan_fwd_tc.cu) or the mma.sync
 // kernels (scan_fwd_bf16*.cu).  The environment variable M2RNN_FWD_VARIANT = tc | mma | wide

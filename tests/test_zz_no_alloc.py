@@ -77,3 +77,54 @@ def test_matches_workspace_entry_point_twice_in_a_row(oracle, cfgs):
             assert err <= 1e-4 * scale, (cfg.name, name, err, scale)
             # ... and the gradients themselves are right: against the fp64 oracle at the path's tolerance
             assert parity.rel_err(got[name], want[name]) <= parity.TOL[cfg.dtype], (cfg.name, name)
+
+
+# fp32 problems whose groups of rows have more scratch for their shares than the array holds (36.5, 11.0 and 9.7 MiB):
+# B, T, N, K, V, Nq, checkpoints passed, interval
+LEAN = [(2, 512, 8, 64, 64, 8, True, 0), (1, 300, 8, 64, 64, 1, False, 0), (1, 150, 4, 128, 128, 4, True, 40)]
+
+
+def _lean_params(case):
+    B, T, N, K, V, Nq, ck, C = case
+    return binding.Params(B=B, T=T, N=N, Nq=Nq, Nk=N, K=K, V=V, io_dtype=0, gate_kind=1, ckpt_interval=C, dh_clip=0.0)
+
+
+def test_shares_that_do_not_fit_are_not_refused():
+    """Where no device is visible an accepted call ends at the first CUDA call (-6), a refused one before it (-5)."""
+    import os
+    import subprocess
+    import sys
+    from paper_2603_14360_b200 import build
+    build.build()
+    lib = binding._lib()
+    for case in LEAN:
+        assert lib.m2rnn_bwd_workspace_bytes(ctypes.byref(_lean_params(case)), int(case[6])) > binding.STATIC_SCRATCH_BYTES
+    here = os.path.dirname(os.path.abspath(__file__))
+    code = ("import ctypes, sys; sys.path[:0] = [%r, %r]\n"
+            "import test_zz_no_alloc as t\n"
+            "from paper_2603_14360_b200 import binding\n"
+            "fake = ctypes.c_void_p(0x10000)\n"
+            "for case in t.LEAN + [(2, 4096, 32, 128, 128, 1, True, 0)]:\n"
+            "    p = t._lean_params(case)\n"
+            "    print(binding._lib().m2rnn_bwd_static_scratch(ctypes.byref(p), *([fake] * 5), None, None, None, None, fake if case[6] else None,\n"
+            "          fake, None, *([fake] * 5), None, None, None))\n") % (here, os.path.dirname(here))
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, env={**os.environ, "CUDA_VISIBLE_DEVICES": ""}, timeout=300)
+    assert r.stdout.split() == ["-6"] * len(LEAN) + ["-5"], (r.stdout, r.stderr[-2000:])
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("case", LEAN, ids=lambda c: "x".join(map(str, c[:5])))
+def test_groups_one_after_the_other_match_the_workspace_entry_point(case):
+    B, T, N, K, V, Nq, ck, C = case
+    cfg = ScanConfig("lean", B=B, T=T, N=N, K=K, V=V, Nq=Nq, Nk=N, dtype="f32", w_scale=0.5, gate_mean=1.0, seed=35)
+    d = inputs.make_inputs(cfg, backward=True, residual=True, d_hT=True)
+    g = {k: (v.cuda() if isinstance(v, torch.Tensor) else v) for k, v in d.items()}
+    args = [g[x] for x in ("q", "k", "v", "gate", "W", "h0")]
+    kw = dict(w_r=g["w_r"], ckpt_interval=C)
+    ckpt = binding.m2rnn_fwd(*args, save_ckpt=True, **kw)[2] if ck else None
+    ref = binding.m2rnn_bwd(*args, g["dy"], g["d_hT"], ckpt=ckpt, **kw)
+    got = binding.m2rnn_bwd_static_scratch(*args, g["dy"], g["d_hT"], out=_alloc_outputs(g), ckpt=ckpt, **kw)
+    binding.check_device_status()
+    for name, r in ref.items():   # the same terms, their sums over at most 16 groups and 16 units in another order
+        err = (got[name].double() - r.double()).abs().max().item()
+        assert err <= 32 * 2.0 ** -24 * r.abs().max().item(), (name, err)
