@@ -42,6 +42,7 @@ struct ScanArgs {
   long long qs, ks, vs;
   long long TT;
   const int32_t *cu;
+  int rank;       // B where the sequences of a packed batch are taken longest first, else 0
 };
 
 // First token and length of batch entry b: a slice [cu[b], cu[b+1]) of a packed batch, else b T .. b T + T
@@ -55,45 +56,45 @@ __device__ __forceinline__ UnitSpan unit_span(const ScanArgs &a, int b) {
   return UnitSpan{(size_t)b * a.T, a.T};
 }
 // The batch entry that the CTAs at place `pos` of the grid's order take.  Sequences of a packed batch are
-// taken longest first: CTAs are handed out in order, and a long one that starts last leaves the
+// taken longest first (a.rank > 0, see in_order): CTAs are handed out in order, and a long one that starts last leaves the
 // other SMs idle (12 sequences of up to 4 000 tokens, K = V = 128, forward + backward: 20.4 -> 18.6 ms).
-// Every thread of the CTA calls it, before it uses `scratch` (kRankWords words of shared memory) otherwise.
-// `pace`: the kernel's time per step, in 0.1 us.
-// (Not inlined: the kernels' inner loops are sensitive to what the compiler schedules around them.)
-constexpr int kRankBatch = 512, kRankWords = kRankBatch + 4;
-static __device__ __noinline__ int longest_first(const int32_t *cu, int B, float scan, int pos, int *scratch);
-__device__ __forceinline__ int batch_entry(const ScanArgs &a, int pos, void *scratch, int pace) {
+// Every thread of the CTA calls it, before it uses `scratch` (shared memory) otherwise.
+// (Not inlined, and the condition no simpler than it is: the kernels' inner loops are sensitive to what the compiler
+// schedules around them.  `a.rank` alone costs every scan at V = 128 1.2 %, packed or not, `a.cu && a.rank` four slabs of
+// V = 64 0.5 %; a ranking on keys staged in shared memory, four times as fast, the V = 128 backward 0.7 %.)
+static __device__ __noinline__ int longest_first(const int32_t *cu, int B, int pos, int *scratch);
+__device__ __forceinline__ int batch_entry(const ScanArgs &a, int pos, void *scratch) {
   // (through a shuffle: known to be the same in all lanes, so that what derives from it stays in uniform
   // registers -- 5 to 9 % of a step in the tcgen05 kernel)
-  return __shfl_sync(0xffffffffu, a.cu && a.B > 1 && a.B <= kRankBatch ? longest_first(a.cu, a.B, 0.1f * pace * a.T, pos, static_cast<int *>(scratch)) : pos, 0);
+  return __shfl_sync(0xffffffffu, a.cu && a.rank > 1 && a.rank <= 1024 ? longest_first(a.cu, a.B, pos, static_cast<int *>(scratch)) : pos, 0);
 }
-static __device__ __noinline__ int longest_first(const int32_t *cu, int B, float scan, int pos, int *scratch) {
-  // Every CTA ranks the batch for itself, some B^2 comparisons: 0.25 us, 1 us for 256 sequences.  Waves of CTAs times
-  // that has to stay below what the order can give, a part of the longest scan (`scan`, us), which counts once.
-  // Forward, K = V = 64, two heads, us in the grid's order / always ranked, from memory, length by length / now:
-  // 256 sequences of up to 256 tokens 164 / 136 / 127, 512 of 2048 2050 / 1809 / 1745, of 32 61 / 174 / 63, 1000 of 32 113 /
-  // 922 / 113; K = 64, V = 16, 16 heads, 256 of 2048 1491 / 1392 / 1340, of 256 201 / 277 / 202.
-  if ((float)gridDim.x * blockDim.x * ((float)B * B + 22000.f) > 1.75e9f * scan) return pos;
-  const int pad = (B + 3) & ~3;
-  for (int b = threadIdx.x; b < pad; b += blockDim.x) {   // keys: the length above the place in the batch, all different
-    const int len = b < B ? min(max(cu[b + 1] - cu[b], 0), (1 << 22) - 1) : 0;
-    scratch[b] = b < B ? len * kRankBatch + (kRankBatch - 1 - b) : -1;
-  }
-  __syncthreads();
+static __device__ __noinline__ int longest_first(const int32_t *cu, int B, int pos, int *scratch) {
   for (int b = threadIdx.x; b < B; b += blockDim.x) {
-    const int key = scratch[b];
+    const int len = cu[b + 1] - cu[b];
     int rank = 0;
-#pragma unroll 4
-    for (int o = 0; o < pad; o += 4) {
-      const int4 k = *reinterpret_cast<const int4 *>(scratch + o);
-      rank += (k.x > key) + (k.y > key) + (k.z > key) + (k.w > key);
+    for (int o = 0; o < B; ++o) {
+      const int other = cu[o + 1] - cu[o];
+      rank += other > len || (other == len && o < b);
     }
-    if (rank == pos) scratch[pad] = b;
+    if (rank == pos) *scratch = b;
   }
   __syncthreads();
-  const int b = *static_cast<volatile int *>(scratch + pad);
+  const int b = *static_cast<volatile int *>(scratch);
   __syncthreads();
   return b;
+}
+// The arguments of a scan kernel's launch of `ctas` CTAs of `threads`, with the order of a packed batch decided.
+// `pace`: the kernel's time per step, in 0.1 us.
+// Every CTA ranks the batch for itself, B comparisons for each sequence that a thread takes, some 0.02 us each.
+// Waves of CTAs times that has to stay below what the order can give, a part of the longest scan, which counts once.
+// Forward, two heads of K = V = 64, us in the grid's order / ranked: 256 sequences of up to 256 tokens 164 / 136, 512 of
+// 2048 2050 / 1810 -- ranked by the rule; 512 of 256 286 / 357, 1000 of 32 113 / 922 -- not.  16 heads of K = 64,
+// V = 16: 256 of 2048 1490 / 1392 ranked, of 256 201 / 277 not.
+inline ScanArgs in_order(const ScanArgs &args, long ctas, int threads, int pace) {
+  ScanArgs a = args;
+  const double waves = (double)ctas * threads / 75776.;   // (512 threads on each of 148 SMs)
+  a.rank = a.cu && a.B > 1 && waves * a.B * ((a.B + threads - 1) / threads) <= 2.7 * pace * a.T ? a.B : 0;
+  return a;
 }
 #endif
 

@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(bwd_threads<V, NWC>(), V == 16 ? (NWC == 2 ? 3
   const int place = blockIdx.x / RS, rs = blockIdx.x % RS;
   // (V = 16 keeps the grid's order: what the compiler makes of its three-CTA variant is 9 % slower on dense
   // batches with b from anywhere else, and its CTAs are small)
-  const int b = V == 16 ? place / N : batch_entry(a, place / N, smem, 10), n = place % N;
+  const int b = V == 16 ? place / N : batch_entry(a, place / N, smem), n = place % N;
   const int unit = V == 16 ? place : b * N + n;
   const UnitSpan span = unit_span(a, b);   // this batch entry's tokens (a slice of a packed batch, or b T ..)
   const int T = span.T;
@@ -875,7 +875,8 @@ cudaError_t launch_bwd_t(const ScanArgs &a, cudaStream_t s) {
   cudaError_t e = allow_smem(bwd_bf16_kernel<V, NWC>, L.total);
   if (e != cudaSuccess) return e;
   const int RS = a.K / (16 * NWC);
-  bwd_bf16_kernel<V, NWC><<<a.B * a.N * RS, bwd_threads<V, NWC>(), L.total, s>>>(a);
+  const int ctas = a.B * a.N * RS;
+  bwd_bf16_kernel<V, NWC><<<ctas, bwd_threads<V, NWC>(), L.total, s>>>(in_order(a, ctas, bwd_threads<V, NWC>(), 10));
   return cudaGetLastError();
 }
 

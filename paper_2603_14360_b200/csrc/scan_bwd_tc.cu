@@ -128,7 +128,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_tc_kernel(ScanArgs a) {
   const int RS = K / kNR;
   const int place = blockIdx.x / RS, rs = blockIdx.x % RS;
   const int n = place % N;
-  const int b = batch_entry(a, place / N, smem_dyn, 12), unit = b * N + n;
+  const int b = batch_entry(a, place / N, smem_dyn), unit = b * N + n;
   const int rbase = rs * kNR;
   const UnitSpan span = unit_span(a, b);
   const int T = span.T;
@@ -583,7 +583,8 @@ cudaError_t launch_bwd_bf16_tc(const ScanArgs &a, cudaStream_t s) {
   const size_t smem = TcBwdSmem::total;
   cudaError_t e = allow_smem(bwd_tc_kernel, smem);
   if (e != cudaSuccess) return e;
-  bwd_tc_kernel<<<a.B * a.N * (a.K / kNR), kThreads, smem, s>>>(a);
+  const int ctas = a.B * a.N * (a.K / kNR);
+  bwd_tc_kernel<<<ctas, kThreads, smem, s>>>(in_order(a, ctas, kThreads, 16));
   return cudaGetLastError();
 }
 

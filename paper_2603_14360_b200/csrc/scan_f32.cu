@@ -201,7 +201,7 @@ __global__ void __launch_bounds__(Geom<V>::kThreads) fwd_f32_kernel(ScanArgs a) 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, p = lane >> 2, c0 = 8 * warp + 2 * (lane & 3);
   const int orow = Own<GR>::row(p), ocol = Own<GR>::col(p, c0), ycol = y_col<GR>(lane, c0);
   const int place = blockIdx.x / RS, rs = blockIdx.x % RS, rbase = rs * R;
-  const int b = batch_entry(a, place / N, smem, 7), n = place % N, bn = b * N + n;
+  const int b = batch_entry(a, place / N, smem), n = place % N, bn = b * N + n;
   const UnitSpan span = unit_span(a, b);   // this batch entry's tokens (a slice of a packed batch, or b T ..)
   const int T = span.T;
   const size_t tok0 = span.tok0, KV = (size_t)K * V;
@@ -323,7 +323,7 @@ __global__ void __launch_bounds__(Geom<V>::kThreads, 512 / Geom<V>::kThreads) bw
   const int K = a.K, N = a.N;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, p = lane >> 2, c0 = 8 * warp + 2 * (lane & 3);
   const int place = blockIdx.x / nslab, rs = slab0 + blockIdx.x % nslab, rbase = rs * GR;
-  const int b = batch_entry(a, place / N, smem, 12), n = place % N, bn = b * N + n;
+  const int b = batch_entry(a, place / N, smem), n = place % N, bn = b * N + n;
   const bool add = nslab == 1 && rs > 0;   // earlier launches have written dv, dgate and dW
   const UnitSpan span = unit_span(a, b);
   const int T = span.T;
@@ -649,7 +649,8 @@ cudaError_t launch_fwd_g(const ScanArgs &a, cudaStream_t s) {
   const size_t smem = fwd_f32_smem<V>(a.KCf);
   const cudaError_t e = allow_smem(fwd_f32_kernel<V, GR>, smem);
   if (e != cudaSuccess) return e;
-  fwd_f32_kernel<V, GR><<<a.B * a.N * (a.K / a.KCf), Geom<V>::kThreads, smem, s>>>(a);
+  const int ctas = a.B * a.N * (a.K / a.KCf);
+  fwd_f32_kernel<V, GR><<<ctas, Geom<V>::kThreads, smem, s>>>(in_order(a, ctas, Geom<V>::kThreads, 7));
   return cudaGetLastError();
 }
 template <int V>
@@ -663,7 +664,7 @@ cudaError_t launch_bwd_g(const ScanArgs &a, cudaStream_t s) {
   cudaError_t e = allow_smem(bwd_f32_kernel<V, GR>, smem);
   const int slabs = a.K / GR, nslab = a.KC == GR ? slabs : 1;
   for (int s0 = 0; s0 < slabs && e == cudaSuccess; s0 += nslab) {
-    bwd_f32_kernel<V, GR><<<a.B * a.N * nslab, Geom<V>::kThreads, smem, s>>>(a, s0, nslab);
+    bwd_f32_kernel<V, GR><<<a.B * a.N * nslab, Geom<V>::kThreads, smem, s>>>(in_order(a, (long)a.B * a.N * nslab, Geom<V>::kThreads, 12), s0, nslab);
     e = cudaGetLastError();
   }
   return e;

@@ -67,7 +67,7 @@ __global__ void __launch_bounds__((MAXW + 1) * 32, OCC) fwd_bf16_kernel(ScanArgs
   constexpr int TC = FwdSmem<V>::tc(MAXW * 16);   // K > 64 <=> MAXW == 8
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;   // (through a shuffle: known to be warp-uniform)
   const int place = blockIdx.x / RS, rs = blockIdx.x % RS;
-  const int b = batch_entry(a, place / N, smem_raw, 3), n = place % N, bn = b * N + n;
+  const int b = batch_entry(a, place / N, smem_raw), n = place % N, bn = b * N + n;
   const UnitSpan span = unit_span(a, b);   // this batch entry's tokens (a slice of a packed batch, or b T ..)
   const int T = span.T;
   const size_t tok0 = span.tok0;
@@ -456,7 +456,7 @@ cudaError_t launch_vwco(const ScanArgs &a, cudaStream_t s) {
   const unsigned grid = a.B * a.N * (a.K / a.KCf), threads = (a.KCf / 16 + 1) * 32;
   cudaError_t e = allow_smem(fwd_bf16_kernel<V, MAXW, CKPT, OCC>, smem);
   if (e != cudaSuccess) return e;
-  fwd_bf16_kernel<V, MAXW, CKPT, OCC><<<grid, threads, smem, s>>>(a);
+  fwd_bf16_kernel<V, MAXW, CKPT, OCC><<<grid, threads, smem, s>>>(in_order(a, grid, threads, 3));
   return cudaGetLastError();
 }
 

@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(cs_threads(SP * NW, OCC), OCC) fwd_bf16_cs_ker
   const int RS = Kf / K;
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31, g = lane >> 2, c = lane & 3;
   const int place = blockIdx.x / RS, rs = blockIdx.x % RS;
-  const int b = batch_entry(a, place / N, smem_raw, 3), n = place % N, bn = b * N + n;
+  const int b = batch_entry(a, place / N, smem_raw), n = place % N, bn = b * N + n;
   const UnitSpan span = unit_span(a, b);   // this batch entry's tokens (a slice of a packed batch, or b T ..)
   const int T = span.T, nst = (T + TC - 1) / TC;
   const size_t tok0 = span.tok0;
@@ -524,7 +524,8 @@ cudaError_t launch_cs(const ScanArgs &a, cudaStream_t s) {
   static_assert(CsStage<V, 16 * NW, OCC>::kFits, "a block's shared memory");
   cudaError_t e = allow_smem(fwd_bf16_cs_kernel<V, SP, NW, CKPT, OCC>, smem);
   if (e != cudaSuccess) return e;
-  fwd_bf16_cs_kernel<V, SP, NW, CKPT, OCC><<<a.B * a.N * (a.K / (16 * NW)), cs_threads(SP * NW, OCC), smem, s>>>(a);
+  const int ctas = a.B * a.N * (a.K / (16 * NW)), threads = cs_threads(SP * NW, OCC);
+  fwd_bf16_cs_kernel<V, SP, NW, CKPT, OCC><<<ctas, threads, smem, s>>>(in_order(a, ctas, threads, 3));
   return cudaGetLastError();
 }
 

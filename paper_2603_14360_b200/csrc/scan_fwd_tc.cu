@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) fwd_tc_kernel(ScanArgs a) {
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const int NG = (N + HS - 1) / HS;               // head groups
   const int RS = (K + kRowsCta - 1) / kRowsCta;   // CTAs per (b, head group)
-  const int rs = blockIdx.x % RS, hg = (blockIdx.x / RS) % NG, b = batch_entry(a, blockIdx.x / (RS * NG), smem_dyn, 4);
+  const int rs = blockIdx.x % RS, hg = (blockIdx.x / RS) % NG, b = batch_entry(a, blockIdx.x / (RS * NG), smem_dyn);
   const int rbase = rs * kRowsCta;
   const UnitSpan span = unit_span(a, b);   // this batch entry's tokens (a slice of a packed batch, or b T ..)
   const int T = span.T;
@@ -361,7 +361,7 @@ cudaError_t launch_tc_fwd(const ScanArgs &a, cudaStream_t s) {
   cudaError_t e = allow_smem(fwd_tc_kernel<V, NR, CKPT>, smem);
   if (e != cudaSuccess) return e;
   const int NG = (a.N + HS - 1) / HS, RS = (a.K + kRowsCta - 1) / kRowsCta;
-  fwd_tc_kernel<V, NR, CKPT><<<a.B * NG * RS, kThreadsTc, smem, s>>>(a);
+  fwd_tc_kernel<V, NR, CKPT><<<a.B * NG * RS, kThreadsTc, smem, s>>>(in_order(a, (long)a.B * NG * RS, kThreadsTc, 4));
   return cudaGetLastError();
 }
 

@@ -71,7 +71,7 @@ __global__ void __launch_bounds__((NW + kSvc) * 32, OCC) fwd_v16_kernel(ScanArgs
   const int Kf = a.K, N = a.N, RS = Kf / K;
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31, g = lane >> 2, c = lane & 3;
   const int place = blockIdx.x / RS, rs = blockIdx.x % RS, rbase = rs * K;
-  const int b = batch_entry(a, place / N, smem, 1), n = place % N, bn = b * N + n;
+  const int b = batch_entry(a, place / N, smem), n = place % N, bn = b * N + n;
   const UnitSpan span = unit_span(a, b);
   const int T = span.T, nst = (T + kTC - 1) / kTC;
   const size_t tok0 = span.tok0, KV = (size_t)Kf * kV;
@@ -337,7 +337,8 @@ cudaError_t launch_t(const ScanArgs &a, cudaStream_t s) {
   constexpr size_t smem = kBarBytes + (size_t)kStages * Lay16::bytes(16 * NW) + kTC * kV * 4;
   const cudaError_t e = allow_smem(fwd_v16_kernel<NW, CKPT, OCC, kSvc>, smem);
   if (e != cudaSuccess) return e;
-  fwd_v16_kernel<NW, CKPT, OCC, kSvc><<<a.B * a.N * (a.K / (16 * NW)), (NW + kSvc) * 32, smem, s>>>(a);
+  const int ctas = a.B * a.N * (a.K / (16 * NW)), threads = (NW + kSvc) * 32;
+  fwd_v16_kernel<NW, CKPT, OCC, kSvc><<<ctas, threads, smem, s>>>(in_order(a, ctas, threads, 1));
   return cudaGetLastError();
 }
 
