@@ -114,8 +114,12 @@ int m2rnn_bwd_row_slab(const m2rnn_params *params);
 size_t m2rnn_ckpt_bytes(const m2rnn_params *params);
 
 /* Scratch the forward call needs for `params`: 0 unless the library splits the rows of a state
- * over several CTAs (it does when there are few (b,n) units, to fill the GPU), in which case the
- * per-slab shares of y pass through this scratch before a second launch adds them. */
+ * over several CTAs, in which case the per-slab shares of y, (K / rows) x tokens x N x V floats, pass
+ * through this scratch before a second launch adds them.  It splits where there are few (b,n) units, to
+ * fill the GPU; M2RNN_F32 states also where groups of four or eight rows make more warps, and
+ * M2RNN_BF16 states of K > 64, 32 <= V <= 64 into slabs of at most 64 rows -- both for speed only and
+ * up to 4 GiB of shares: m2rnn_fwd also takes those two without a workspace, on whole states and slower
+ * (fp32, 16 units of K = V = 64: 6.0 times; bf16, 192 units of K = 96, V = 64: 2.3 times). */
 size_t m2rnn_fwd_workspace_bytes(const m2rnn_params *params);
 
 /* Forward scan (Algorithm 1; Eq. 1-3).
@@ -125,7 +129,7 @@ size_t m2rnn_fwd_workspace_bytes(const m2rnn_params *params);
  *        ckpt or NULL: ckpt[b,n,c] = H_{c*C}, the state BEFORE step c*C (so ckpt[..,0] = h0),
  *        for m2rnn_bwd.
  *   workspace: device scratch of at least m2rnn_fwd_workspace_bytes(params), 256-byte aligned
- *        (NULL and 0 when that is 0); contents undefined afterwards. */
+ *        (NULL and 0 when that is 0, or to do without: see there); contents undefined afterwards. */
 int m2rnn_fwd(const m2rnn_params *params, const void *q, const void *k, const void *v,
               const float *gate, const void *W, const float *h0, const float *alpha,
               const float *beta, const void *w_r, void *y, float *hT, float *ckpt,

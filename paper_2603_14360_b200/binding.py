@@ -234,7 +234,8 @@ def m2rnn_fwd(q, k, v, gate, W, h0=None, *, gate_kind=GATE_LOGIT, alpha=None, be
               cu_seqlens=None, max_seqlen=None):
     """Forward scan.  Returns (y, hT, ckpt); hT / ckpt are None when not requested.
     ``out`` may hold preallocated ``y`` / ``hT`` / ``ckpt`` tensors to write into; ``workspace``
-    a preallocated uint8 tensor of at least ``m2rnn_fwd_workspace_bytes`` bytes.
+    a preallocated uint8 tensor of at least ``m2rnn_fwd_workspace_bytes`` bytes (an empty one: do without
+    where the library can, at the price of speed).
     q, k, v may be strided views along the token axis (e.g. slices of one fused projection output).
     With ``cu_seqlens`` (int32 [B+1], CUDA) and ``max_seqlen`` the batch is packed: q [tokens,Nq,K],
     k, v, gate [tokens,N], y [tokens,N,V]; states stay [B,N,K,V]."""

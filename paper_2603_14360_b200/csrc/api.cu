@@ -146,18 +146,19 @@ bool fwd_use_tc(int B, int N, int K, int V, int io_dtype) {
   return V == 128 && K % 64 == 0 && (long)(B > 0 ? B : 1) * N * (K / 32) > sm_count();
 }
 
-int plan_fwd_rows(int B, int N, int K, int V, int io_dtype, size_t tokens) {
-  if (io_dtype == M2RNN_F32) return fwd_f32_rows(B, N, K, V, tokens * N * V * sizeof(float));
+int plan_fwd_rows(int B, int N, int K, int V, int io_dtype, size_t tokens, bool lean) {
+  if (io_dtype == M2RNN_F32) return lean ? K : fwd_f32_rows(B, N, K, V, tokens * N * V * sizeof(float));
   if (fwd_use_tc(B, N, K, V, io_dtype)) return fwd_tc_rows_per_cta(B, N, K, V);
   // The smallest slab (a multiple of 16 rows that divides K) that still gives every CTA an SM of its own; with more
   // units than SMs the largest that the column-split kernel has: 32 rows at V = 128 for the sake of
   // registers, 64 below.  Up to 128 rows in one CTA of the one-warp-per-slab kernel only where a K that 48 and
   // 64 do not divide would make V = 32 slabs of 16 rows (440 units, K = 112: 1029 against 1226 us for 1024 steps; K = 96,
-  // V = 64, 192 units: 1682 against 759), or the slabs' shares of y (fp32, added afterwards) take more than 4 GB.
+  // V = 64, 192 units: 1682 against 759), or the slabs' shares of y (fp32, added afterwards) take more than 4 GB or
+  // there is no room for them at all (lean).
   const int kSMs = sm_count();
   const long units = (long)(B > 0 ? B : 1) * N;
   int cap = V > 64 ? 32 : 128;
-  if (V > 16 && V <= 64 && K > 64) {
+  if (V > 16 && V <= 64 && K > 64 && !lean) {
     int kc = 64;
     while (K % kc) kc -= 16;
     if ((V == 64 || kc > 16) && tokens * N * V * sizeof(float) * (K / kc) <= ((size_t)4 << 30)) cap = kc;
@@ -409,7 +410,11 @@ int m2rnn_fwd(const m2rnn_params *params, const void *q, const void *k, const vo
   a.alpha = params->gate_kind == M2RNN_GATE_PSI ? alpha : nullptr;
   a.beta = params->gate_kind == M2RNN_GATE_PSI ? beta : nullptr;
   a.y = y; a.hT = hT; a.ckpt = ckpt; a.dev_status = dev_status;
-  const size_t need = m2rnn_fwd_workspace_bytes(params);
+  size_t need = m2rnn_fwd_workspace_bytes(params);
+  if (need > 0 && !workspace && workspace_bytes == 0) {   // without shares of y, where the kernels can
+    const int rows = plan_fwd_rows(params->B, params->N, params->K, params->V, params->io_dtype, tokens_of(params), true);
+    if (rows == params->K) { a.KCf = rows; need = 0; }
+  }
   if (need > 0) {
     if (!workspace || workspace_bytes < need) return M2RNN_ERR_WORKSPACE;
     if (reinterpret_cast<uintptr_t>(workspace) % kAlign) return M2RNN_ERR_ALIGN;

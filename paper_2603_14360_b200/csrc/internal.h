@@ -122,7 +122,7 @@ int bwd_call(const m2rnn_params *params, const void *q, const void *k, const voi
              const float *h0, const float *alpha, const float *beta, const void *w_r, const float *ckpt, const void *dy,
              const float *d_hT, void *dq, void *dk, void *dv, float *dgate, float *dW, float *dh0, void *workspace,
              size_t workspace_bytes, bool lean, int32_t *dev_status, void *stream);
-int plan_fwd_rows(int B, int N, int K, int V, int io_dtype, size_t tokens = 0);   // state rows per CTA of the forward kernel
+int plan_fwd_rows(int B, int N, int K, int V, int io_dtype, size_t tokens = 0, bool lean = false);   // state rows per CTA of the forward kernel
 // Which bf16 forward kernel takes a problem: the tcgen05 kernel (scan_fwd_tc.cu) or the mma.sync
 // kernels (scan_fwd_bf16*.cu).  The environment variable M2RNN_FWD_VARIANT = tc | mma | wide
 // overrides the choice (benchmarking only).
