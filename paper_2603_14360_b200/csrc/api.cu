@@ -40,25 +40,27 @@ int sm_count() {
   return sms;
 }
 
-namespace {
 // cuCtxGetId through the runtime's driver entry point (no link against libcuda)
+bool current_context(uint64_t *id) {
+  using GetId = CUresult (*)(CUcontext, unsigned long long *);
+  static const GetId get = [] {
+    void *p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPoint("cuCtxGetId", &p, cudaEnableDefault, &q) != cudaSuccess || q != cudaDriverEntryPointSuccess) {
+      (void)cudaGetLastError();
+      p = nullptr;
+    }
+    return reinterpret_cast<GetId>(p);
+  }();
+  unsigned long long n = 0;
+  if (!get || get(nullptr, &n) != CUDA_SUCCESS) return false;   // (null: the current context)
+  *id = n;
+  return true;
+}
+
+namespace {
 struct CudaSmem {
-  bool context(uint64_t *id) const {
-    using GetId = CUresult (*)(CUcontext, unsigned long long *);
-    static const GetId get = [] {
-      void *p = nullptr;
-      cudaDriverEntryPointQueryResult q;
-      if (cudaGetDriverEntryPoint("cuCtxGetId", &p, cudaEnableDefault, &q) != cudaSuccess || q != cudaDriverEntryPointSuccess) {
-        (void)cudaGetLastError();
-        p = nullptr;
-      }
-      return reinterpret_cast<GetId>(p);
-    }();
-    unsigned long long n = 0;
-    if (!get || get(nullptr, &n) != CUDA_SUCCESS) return false;   // (null: the current context)
-    *id = n;
-    return true;
-  }
+  bool context(uint64_t *id) const { return current_context(id); }
   int most(const void *kernel, int *n) const {
     int dev = 0, optin = 0;
     cudaFuncAttributes at;

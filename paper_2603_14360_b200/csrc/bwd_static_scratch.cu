@@ -13,24 +13,30 @@ namespace {
 static __device__ __align__(256) unsigned char g_static_scratch[M2RNN_STATIC_SCRATCH_BYTES];
 
 constexpr int kMaxDevices = 64;
-void *g_scratch_addr[kMaxDevices];  // device address of g_static_scratch, per device; null = not looked up yet
+struct Known { void *addr; uint64_t context; };
+Known g_scratch[kMaxDevices];   // device address of g_static_scratch, per device, and the context it belongs to; null = not looked up yet
 std::mutex g_scratch_mutex;
 
 // In host code `g_static_scratch` only names the symbol; the device address has to be asked for,
-// once per device, with that device current.
+// with that device current: once per device, and again when the device has another context than then (after a
+// reset the array may lie elsewhere).
 int scratch_address(void **out) {
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return M2RNN_ERR_CUDA;
+  uint64_t context = 0;
+  const bool told = m2rnn::current_context(&context);
   std::lock_guard<std::mutex> lock(g_scratch_mutex);
-  if (!g_scratch_addr[dev]) {
+  Known &k = g_scratch[dev];
+  if (!k.addr || !told || k.context != context) {
     void *p = nullptr;
     if (cudaGetSymbolAddress(&p, g_static_scratch) != cudaSuccess || !p) {
       (void)cudaGetLastError();
       return M2RNN_ERR_CUDA;
     }
-    g_scratch_addr[dev] = p;
+    if (!told) (void)m2rnn::current_context(&context);   // (the lookup makes a context current where there was none)
+    k = Known{p, context};
   }
-  *out = g_scratch_addr[dev];
+  *out = k.addr;
   return M2RNN_OK;
 }
 

@@ -109,6 +109,7 @@ struct BwdPlan {
   int C_max;  // largest supported checkpoint interval
 };
 int sm_count();   // SMs of the current device (148 when there is none to ask)
+bool current_context(uint64_t *id);   // the current context's number, unique for the life of the process
 cudaError_t allow_smem(const void *kernel, size_t bytes);   // dynamic shared memory a launch may use
 template <typename... A> cudaError_t allow_smem(void (*kernel)(A...), size_t bytes) {
   return allow_smem(reinterpret_cast<const void *>(kernel), bytes);
