@@ -6,6 +6,7 @@ extension ``_native.so`` that calls it with g++ against torch's headers.
 from __future__ import annotations
 
 import concurrent.futures
+import importlib.metadata
 import os
 import subprocess
 import sys
@@ -16,6 +17,7 @@ CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libm2rnn.so")
 NATIVE = os.path.join(HERE, "_native.so")   # Python extension module: the binding's native half
+NATIVE_FOR = os.path.join(OBJ, "native_for.txt")
 
 SOURCES = ["api.cu", "reduce.cu", "scan_f32.cu", "scan_fwd_bf16.cu", "scan_fwd_bf16_cs.cu", "scan_fwd_v16.cu", "scan_fwd_tc.cu", "scan_bwd_bf16.cu", "scan_bwd_tc.cu", "decode_bf16.cu", "decode_tc_bf16.cu",
            "bwd_static_scratch.cu", "gated_norm.cu", "conv_silu.cu", "selftest.cu"]
@@ -47,10 +49,23 @@ def _compile(src: str, force: bool, verbose: bool) -> str:
     return obj
 
 
-def _build_native(force: bool, verbose: bool) -> None:
+def _native_for() -> str:
+    """What the extension is built against: it calls into torch's C++ libraries, whose interface is a version's own."""
+    return f"torch {importlib.metadata.version('torch')}, Python {sys.version.split()[0]}\n"
+
+
+def _native_is_current() -> bool:
     src = os.path.join(CSRC, "py_native.cpp")
     newest = max(os.path.getmtime(src), os.path.getmtime(os.path.join(ROOT, "include", "m2rnn.h")))
-    if not force and os.path.exists(NATIVE) and os.path.getmtime(NATIVE) >= newest:
+    if not (os.path.exists(NATIVE) and os.path.getmtime(NATIVE) >= newest and os.path.exists(NATIVE_FOR)):
+        return False
+    with open(NATIVE_FOR) as f:
+        return f.read() == _native_for()
+
+
+def _build_native(force: bool, verbose: bool) -> None:
+    src = os.path.join(CSRC, "py_native.cpp")
+    if not force and _native_is_current():
         return
     import sysconfig
     import torch
@@ -67,6 +82,8 @@ def _build_native(force: bool, verbose: bool) -> None:
     if r.returncode:
         raise RuntimeError("g++ failed on py_native.cpp")
     os.replace(tmp, NATIVE)
+    with open(NATIVE_FOR, "w") as f:
+        f.write(_native_for())
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
