@@ -84,3 +84,27 @@ def test_fused_projection_through_conv_into_the_scan(oracle, dtype):
     assert parity.rel_err(y, y_ref) <= tol and parity.rel_err(hT, hT_ref) <= tol
     for name in ("dx", "dw", "dbias"):
         assert parity.rel_err(back[name], back_ref[name]) <= tol, name
+
+
+@pytest.mark.parametrize("with_prev", [False, True])
+def test_fp32_sigmoid_over_its_whole_range(with_prev):
+    """fp32, pre-activations from -100 to 100 and both zeros, element by element: out = pre s(pre) and dx = dout SiLU'(pre).
+
+    Taps (0, 0, 0, 1) make pre = x and dx = dpre.  The sigmoid is r or e r with e = exp(-|x|), r = 1/(1 + e): expf is good to
+    2 ulp, a Newton step leaves r within 2, and the product, the sum 1 + e and out are rounded: 8 ulp = 2^-20 relative,
+    wherever the result is a normal number (below, its spacing 2^-149).  SiLU' = s (1 + x (1 - s)) cancels near its zero at
+    -1.278 and where 1 - s does, so its error is against s (1 + |x| (1 - s)), with 1 - s good to 2^-24 absolute."""
+    x = torch.cat([torch.linspace(-100, 100, 2001), torch.tensor([0.0, -0.0, 1e-30, -1e-30, 87.0, -87.0, 88.5, -88.5, -88.8]),
+                   torch.linspace(-1.3, -1.25, 38)])
+    T = x.numel() // 4
+    x = x[:4 * T].reshape(1, T, 4).contiguous()
+    w = torch.tensor([[0.0, 0.0, 0.0, 1.0]]).repeat(4, 1)
+    dout = torch.full_like(x, 1.0)
+    prev = torch.zeros(1, 3, 4).cuda() if with_prev else None
+    out = binding.m2rnn_conv_silu_fwd(x.cuda(), w.cuda(), None, prev).cpu().double()
+    dx = binding.m2rnn_conv_silu_bwd(x.cuda(), w.cuda(), dout.cuda(), None, prev)["dx"].cpu().double()
+    z = x.double()
+    s, t = torch.sigmoid(z), torch.sigmoid(-z)
+    assert ((out - z * s).abs() <= 2.0 ** -20 * (z * s).abs() + 2.0 ** -148 * (1 + z.abs())).all()
+    bound = 2.0 ** -20 * s * (1 + z.abs() * t) + 2.0 ** -24 * s * z.abs() + 2.0 ** -148 * (1 + z.abs())
+    assert ((dx - s * (1 + z * t)).abs() <= bound).all()
