@@ -138,7 +138,7 @@ bool fwd_use_tc(int B, int N, int K, int V, int io_dtype) {
   if (io_dtype != M2RNN_BF16) return false;
   const char *variant = getenv("M2RNN_FWD_VARIANT");
   if (variant && !strcmp(variant, "tc")) return true;
-  if (variant && (!strcmp(variant, "mma") || !strcmp(variant, "wide"))) return false;
+  if (variant && !strcmp(variant, "mma")) return false;
   // Measured (B200): the round trip of a tcgen05 step (operand store, proxy fence, barrier, eight
   // MMAs at ~30 cycles of issue each, commit, mbarrier, tcgen05.ld) is ~400 cycles before any
   // arithmetic, against ~30 for mma.sync on registers.  It pays only where the register kernels

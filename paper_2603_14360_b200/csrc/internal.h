@@ -125,7 +125,7 @@ int bwd_call(const m2rnn_params *params, const void *q, const void *k, const voi
              size_t workspace_bytes, bool lean, int32_t *dev_status, void *stream);
 int plan_fwd_rows(int B, int N, int K, int V, int io_dtype, size_t tokens = 0, bool lean = false);   // state rows per CTA of the forward kernel
 // Which bf16 forward kernel takes a problem: the tcgen05 kernel (scan_fwd_tc.cu) or the mma.sync
-// kernels (scan_fwd_bf16*.cu).  The environment variable M2RNN_FWD_VARIANT = tc | mma | wide
+// kernels (scan_fwd_bf16*.cu).  The environment variable M2RNN_FWD_VARIANT = tc | mma
 // overrides the choice (benchmarking only).
 bool fwd_use_tc(int B, int N, int K, int V, int io_dtype);
 int fwd_tc_rows_per_cta(int B, int N, int K, int V);                 // scan_fwd_tc.cu: 32 or 64

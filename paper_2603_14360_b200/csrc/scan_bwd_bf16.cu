@@ -885,9 +885,11 @@ cudaError_t launch_bwd_v(const ScanArgs &a, cudaStream_t s) {
   switch (a.KC) {
     case 16: return launch_bwd_t<V, 1>(a, s);
     case 32: return launch_bwd_t<V, 2>(a, s);
-    case 64: return launch_bwd_t<V, 4>(a, s);
-    default: return cudaErrorInvalidValue;
+    case 64:
+      if constexpr (V <= 64) return launch_bwd_t<V, 4>(a, s);   // (the plan gives V = 128 at most 32 rows)
+      break;
   }
+  return cudaErrorInvalidValue;
 }
 
 template <int V>

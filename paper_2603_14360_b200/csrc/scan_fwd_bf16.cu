@@ -1,21 +1,19 @@
-// bf16 tensor-core forward scan (Algorithm 1) for sm_100a.
+// bf16 tensor-core forward scan (Algorithm 1) with one warp per 16 rows, for states that keep more than 64 rows in one CTA:
+// V = 32 and 64, K = 80 to 128 where a split into slabs does not pay or has no room for its shares of y (see plan_fwd_rows).
 //
-// One CTA per (b, n, row slab) -- the K rows of a state are independent recurrences (Eq. 1-2 act
-// row by row), so a state may be split over several CTAs, whose partial readouts a second-stage
-// kernel adds.  Below, K is the slab's row count.  Per CTA: K/16 compute warps, each holding a 16 x V slab of the state in registers
+// One CTA per (b, n).  Per CTA: K/16 compute warps, each holding a 16 x V slab of the state in registers
 // for all T steps (see mma_tile.cuh), plus one service warp.  Per step a compute warp
 //   1. seeds its accumulators with the outer product k_t v_t^T (fp32 FMA),
 //   2. adds H_{t-1} W with V/16 x V/8 mma.sync.m16n8k16 (bf16 operands, fp32 accumulate),
 //   3. applies tanh.approx and the gate, keeping H_t in fp32 and re-packing it to the bf16
 //      A fragments of the next step,
-//   4. forms its partial readout q_t-weighted column sums with shuffles and leaves them in
-//      shared memory.
+//   4. forms its partial readout, q_t-weighted column sums, with one more mma.sync per accumulator tile
+//      and leaves it in shared memory.
 // The service warp runs ahead of and behind the compute warps: it fetches q/k/v/gate for a
 // stage of steps from global memory, converts them to fp32, evaluates the forget gate, and,
 // once a stage is done, adds the warps' readout partials and writes y with 16-byte stores.
 // Stages are handed over with mbarriers; every wait is bounded and reports through dev_status.
 #include <cstdlib>
-#include <cstring>
 
 #include "device_common.cuh"
 #include "internal.h"
@@ -28,43 +26,32 @@ namespace {
 constexpr int kStages = 3;
 constexpr int kBarrierBytes = 64;  // 2 * kStages mbarriers, padded so the stages stay 16-byte aligned
 
+constexpr int kMaxWarps = 8;       // compute warps: 168 registers for each of these and the service warp
+constexpr int TC = 8;              // steps of a stage
+
 template <int V>
 struct FwdSmem {
   // Per stage (floats): q [TC][K], k [TC][K], v [TC][V], f [TC], ypart [TC][NW][V]
-  __host__ __device__ static int stage_floats(int K, int TC) { return TC * (2 * K + V + 1 + (K / 16) * V); }
-  __host__ __device__ static constexpr int tc(int K) { return (V >= 128 || K > 64) ? 8 : 16; }
-  __host__ static size_t bytes(int K) {
-    const int TC = tc(K);
-    size_t b = sizeof(float) * (size_t)kStages * stage_floats(K, TC);
-    if (V > 64) b += (size_t)V * V * 2;  // W fragments
-    return b + kBarrierBytes;
-  }
+  __host__ __device__ static int stage_floats(int K) { return TC * (2 * K + V + 1 + (K / 16) * V); }
+  __host__ static size_t bytes(int K) { return sizeof(float) * (size_t)kStages * stage_floats(K) + kBarrierBytes; }
 };
 
-// MAXW: most compute warps the instantiation is launched with (K <= 16*MAXW).  Registers are
-// granted per 4 warps: up to 4+1 warps leave 255 per thread, 8+1 warps only 168.
 // CKPT: whether checkpoints are written (a compile-time switch keeps the branch out of the hot loop).
-// OCC: CTAs per SM the kernel is compiled for.  With more (b,n) units than SMs, two co-resident
-// CTAs (two chain warps per scheduler) hide each other's latencies; the price is a smaller
-// register budget.
-template <int V, int MAXW, bool CKPT, int OCC>
-__global__ void __launch_bounds__((MAXW + 1) * 32, OCC) fwd_bf16_kernel(ScanArgs a) {
+template <int V, bool CKPT>
+__global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) fwd_bf16_kernel(ScanArgs a) {
   using G = TileGeom<V>;
   constexpr int NT = G::NT, KT = G::KT, SEG = G::SEG;
-  constexpr bool kWInRegs = V <= 64;
-  // The product of a step is split over NSET accumulator sets (k-tile kt adds into set kt % NSET,
+  // The product of a step is split over two accumulator sets (k-tile kt adds into set kt % 2,
   // the sets are summed where they are used): an mma.sync that accumulates onto the previous
   // one's result waits for its whole latency (well over 100 cycles), so KT of them in a row
   // would be most of the step.
-  constexpr int NSET = V == 128 ? 1 : (KT >= 2 ? 2 : 1);
+  constexpr int NSET = 2;
   extern __shared__ __align__(16) unsigned char smem_raw[];
 
   const int Kf = a.K, N = a.N;                       // rows of the whole state
   const int K = a.KCf;                               // rows of this CTA's slab
   const int RS = Kf / K;
   const int NW = K >> 4;
-  constexpr bool kPacked = V <= 64;                  // packed fp32x2 arithmetic (spills at V = 128)
-  constexpr int TC = FwdSmem<V>::tc(MAXW * 16);   // K > 64 <=> MAXW == 8
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;   // (through a shuffle: known to be warp-uniform)
   const int place = blockIdx.x / RS, rs = blockIdx.x % RS;
   const int b = batch_entry(a, place / N, smem_raw), n = place % N, bn = b * N + n;
@@ -72,12 +59,11 @@ __global__ void __launch_bounds__((MAXW + 1) * 32, OCC) fwd_bf16_kernel(ScanArgs
   const int T = span.T;
   const size_t tok0 = span.tok0;
   const int rbase = rs * K;   // first state row of this CTA
-  const int stage_floats = FwdSmem<V>::stage_floats(K, TC);
+  const int stage_floats = FwdSmem<V>::stage_floats(K);
 
   uint64_t *full = reinterpret_cast<uint64_t *>(smem_raw);  // [kStages]
   uint64_t *done = full + kStages;                          // [kStages]
   float *stages = reinterpret_cast<float *>(smem_raw + kBarrierBytes);
-  uint2 *Wf = reinterpret_cast<uint2 *>(stages + (size_t)kStages * stage_floats);  // [KT][NT][32], V > 64 only
 
   if (tid == 0) {
     for (int s = 0; s < kStages; ++s) {
@@ -87,13 +73,6 @@ __global__ void __launch_bounds__((MAXW + 1) * 32, OCC) fwd_bf16_kernel(ScanArgs
     fence_mbar_init();
   }
   const __nv_bfloat16 *Wn = static_cast<const __nv_bfloat16 *>(a.W) + (size_t)n * V * V;
-  if constexpr (!kWInRegs) {
-    for (int x = tid; x < KT * NT * 32; x += blockDim.x) {
-      uint32_t b0, b1;
-      load_w_fragment<V>(Wn, x / (NT * 32), (x / 32) % NT, x & 31, b0, b1);
-      Wf[x] = make_uint2(b0, b1);
-    }
-  }
   __syncthreads();
 
   const int nchunks = (T + TC - 1) / TC;
@@ -109,8 +88,7 @@ __global__ void __launch_bounds__((MAXW + 1) * 32, OCC) fwd_bf16_kernel(ScanArgs
     const __nv_bfloat16 *wr = static_cast<const __nv_bfloat16 *>(a.w_r);
     __nv_bfloat16 *yg = static_cast<__nv_bfloat16 *>(a.y);
 
-    // A stage holds at most 16 x 128 / 8 = 128 (TC = 8, K or V = 128) or 16 x 64 / 8 = 128 rows of
-    // 16 bytes per tensor: 4 per lane.  All loads of a stage are issued before the first use so
+    // A stage holds at most 8 x 128 / 8 = 128 rows of 16 bytes per tensor: 4 per lane.  All loads of a stage are issued before the first use so
     // that one global round trip covers the whole stage.
     constexpr int kPerLane = 4;
     auto fill = [&](int ch) {
@@ -201,13 +179,11 @@ __global__ void __launch_bounds__((MAXW + 1) * 32, OCC) fwd_bf16_kernel(ScanArgs
   const int row0 = 16 * warp + 2 * g;   // memory rows row0, row0+1  <->  MMA rows g, g+8
   const size_t KV = (size_t)Kf * V;
 
-  uint32_t Wr[kWInRegs ? KT : 1][kWInRegs ? NT : 1][2];
-  if constexpr (kWInRegs) {
+  uint32_t Wr[KT][NT][2];
 #pragma unroll
-    for (int kt = 0; kt < KT; ++kt)
+  for (int kt = 0; kt < KT; ++kt)
 #pragma unroll
-      for (int nt = 0; nt < NT; ++nt) load_w_fragment<V>(Wn, kt, nt, lane, Wr[kt][nt][0], Wr[kt][nt][1]);
-  }
+    for (int nt = 0; nt < NT; ++nt) load_w_fragment<V>(Wn, kt, nt, lane, Wr[kt][nt][0], Wr[kt][nt][1]);
 
   // H[nt] = {row g: cols 2nt,2nt+1 of the segment | row g+8: same}
   float H[NT][4];
@@ -243,16 +219,12 @@ __global__ void __launch_bounds__((MAXW + 1) * 32, OCC) fwd_bf16_kernel(ScanArgs
 #pragma unroll
     for (int x = 0; x < SEG / 4; ++x) {
       const float4 v4 = lds128(vrow + 4 * (SEG * c + 4 * x));
-      if constexpr (kPacked) {   // one instruction per two products
-        const float2 k02 = make_float2(kk.x, kk.x), k12 = make_float2(kk.y, kk.y);
-        const float2 a0 = __fmul2_rn(k02, make_float2(v4.x, v4.y)), a1 = __fmul2_rn(k12, make_float2(v4.x, v4.y));
-        const float2 b0 = __fmul2_rn(k02, make_float2(v4.z, v4.w)), b1 = __fmul2_rn(k12, make_float2(v4.z, v4.w));
-        P[0][2 * x][0] = a0.x; P[0][2 * x][1] = a0.y; P[0][2 * x][2] = a1.x; P[0][2 * x][3] = a1.y;
-        P[0][2 * x + 1][0] = b0.x; P[0][2 * x + 1][1] = b0.y; P[0][2 * x + 1][2] = b1.x; P[0][2 * x + 1][3] = b1.y;
-      } else {
-        P[0][2 * x][0] = kk.x * v4.x; P[0][2 * x][1] = kk.x * v4.y; P[0][2 * x][2] = kk.y * v4.x; P[0][2 * x][3] = kk.y * v4.y;
-        P[0][2 * x + 1][0] = kk.x * v4.z; P[0][2 * x + 1][1] = kk.x * v4.w; P[0][2 * x + 1][2] = kk.y * v4.z; P[0][2 * x + 1][3] = kk.y * v4.w;
-      }
+      // (packed fp32 pairs: one instruction per two products)
+      const float2 k02 = make_float2(kk.x, kk.x), k12 = make_float2(kk.y, kk.y);
+      const float2 a0 = __fmul2_rn(k02, make_float2(v4.x, v4.y)), a1 = __fmul2_rn(k12, make_float2(v4.x, v4.y));
+      const float2 b0 = __fmul2_rn(k02, make_float2(v4.z, v4.w)), b1 = __fmul2_rn(k12, make_float2(v4.z, v4.w));
+      P[0][2 * x][0] = a0.x; P[0][2 * x][1] = a0.y; P[0][2 * x][2] = a1.x; P[0][2 * x][3] = a1.y;
+      P[0][2 * x + 1][0] = b0.x; P[0][2 * x + 1][1] = b0.y; P[0][2 * x + 1][2] = b1.x; P[0][2 * x + 1][3] = b1.y;
     }
   };
   // P += A[kt] * W[kt][:]  : one k tile of H W
@@ -260,14 +232,8 @@ __global__ void __launch_bounds__((MAXW + 1) * 32, OCC) fwd_bf16_kernel(ScanArgs
     const int set = kt % NSET;
 #pragma unroll
     for (int nt = 0; nt < NT; ++nt) {
-      if constexpr (kWInRegs) {
-        if (kt >= 1 && kt < NSET) mma_bf16_16816_zero(P[set][nt], Ak, Wr[kt][nt][0], Wr[kt][nt][1]);
-        else mma_bf16_16816(P[set][nt], Ak, Wr[kt][nt][0], Wr[kt][nt][1]);
-      } else {
-        const uint2 w = Wf[(kt * NT + nt) * 32 + lane];
-        if (kt >= 1 && kt < NSET) mma_bf16_16816_zero(P[set][nt], Ak, w.x, w.y);
-        else mma_bf16_16816(P[set][nt], Ak, w.x, w.y);
-      }
+      if (kt == 1) mma_bf16_16816_zero(P[set][nt], Ak, Wr[kt][nt][0], Wr[kt][nt][1]);
+      else mma_bf16_16816(P[set][nt], Ak, Wr[kt][nt][0], Wr[kt][nt][1]);
     }
   };
 
@@ -287,44 +253,26 @@ __global__ void __launch_bounds__((MAXW + 1) * 32, OCC) fwd_bf16_kernel(ScanArgs
   auto step = [&](float (&Pc)[NSET][NT][4], float (&Pn)[NSET][NT][4], float f, uint32_t qrow, uint32_t ydst,
                   uint32_t krow_n, uint32_t vrow_n) {
     seed(Pn, krow_n, vrow_n);
-    const float2 qq = lds64(qrow + 4 * row0);
-    float part[SEG];
-    // packed path: the readout (Eq. 3) on the tensor cores, y^T = q^T H over the slab's 16 rows as
+    // the readout (Eq. 3) on the tensor cores, y^T = q^T H over the slab's 16 rows as
     // one more product per accumulator tile: q is row 0 of an otherwise empty A operand (MMA row m
     // <-> memory row 2m, m + 8 <-> 2m + 1), the packed bf16 fragments of H_t, transposed in
-    // registers, are B.  It replaces the products and the shuffle tree over the rows, which were
-    // half of a V = 16 step's instructions.
+    // registers, are B.
     uint32_t Aq[4] = {0u, 0u, 0u, 0u};
     float Y[NT][4];
-    if constexpr (kPacked) {
-      const float4 q4 = lds128(qrow + 4 * (16 * warp + 4 * c));
-      if (g == 0) { Aq[0] = pack_bf16(q4.x, q4.z); Aq[2] = pack_bf16(q4.y, q4.w); }
-    }
+    const float4 q4 = lds128(qrow + 4 * (16 * warp + 4 * c));
+    if (g == 0) { Aq[0] = pack_bf16(q4.x, q4.z); Aq[2] = pack_bf16(q4.y, q4.w); }
 #pragma unroll
     for (int kt = 0; kt < KT; ++kt) {
 #pragma unroll
       for (int nt = 2 * kt; nt < 2 * kt + 2; ++nt) {
-        if constexpr (kPacked) {
-          float2 hh[2];
+        float2 hh[2];
 #pragma unroll
-          for (int h = 0; h < 2; ++h) {   // the two rows' column pairs, as packed fp32 pairs
-            float2 x = make_float2(Pc[0][nt][2 * h], Pc[0][nt][2 * h + 1]);
-            if constexpr (NSET == 2) x = __fadd2_rn(x, make_float2(Pc[1][nt][2 * h], Pc[1][nt][2 * h + 1]));
-            const float2 z = make_float2(tanh_approx(x.x), tanh_approx(x.y));                                      // Eq. 1
-            const float2 dd = __ffma2_rn(z, make_float2(-1.f, -1.f), make_float2(H[nt][2 * h], H[nt][2 * h + 1]));  // H - Z
-            hh[h] = __ffma2_rn(make_float2(f, f), dd, z);                                                          // Eq. 2
-            H[nt][2 * h] = hh[h].x; H[nt][2 * h + 1] = hh[h].y;
-          }
-        } else {
-#pragma unroll
-          for (int r = 0; r < 4; ++r) {
-            float x = Pc[0][nt][r];
-            if constexpr (NSET == 2) x += Pc[1][nt][r];
-            const float z = tanh_approx(x);                  // Eq. 1
-            H[nt][r] = fmaf(f, H[nt][r] - z, z);             // Eq. 2: f H + (1-f) Z
-          }
-          part[2 * nt] = fmaf(qq.y, H[nt][2], qq.x * H[nt][0]);      // Eq. 3, this thread's two rows
-          part[2 * nt + 1] = fmaf(qq.y, H[nt][3], qq.x * H[nt][1]);
+        for (int h = 0; h < 2; ++h) {   // the two rows' column pairs, as packed fp32 pairs
+          const float2 x = __fadd2_rn(make_float2(Pc[0][nt][2 * h], Pc[0][nt][2 * h + 1]), make_float2(Pc[1][nt][2 * h], Pc[1][nt][2 * h + 1]));
+          const float2 z = make_float2(tanh_approx(x.x), tanh_approx(x.y));                                      // Eq. 1
+          const float2 dd = __ffma2_rn(z, make_float2(-1.f, -1.f), make_float2(H[nt][2 * h], H[nt][2 * h + 1]));  // H - Z
+          hh[h] = __ffma2_rn(make_float2(f, f), dd, z);                                                          // Eq. 2
+          H[nt][2 * h] = hh[h].x; H[nt][2 * h + 1] = hh[h].y;
         }
       }
       uint32_t Ak[4];
@@ -333,27 +281,15 @@ __global__ void __launch_bounds__((MAXW + 1) * 32, OCC) fwd_bf16_kernel(ScanArgs
       Ak[2] = pack_bf16(H[2 * kt + 1][0], H[2 * kt + 1][1]);
       Ak[3] = pack_bf16(H[2 * kt + 1][2], H[2 * kt + 1][3]);
       mma_ktile(Pn, Ak, kt);
-      if constexpr (kPacked) {   // Eq. 3 for accumulator tiles 2 kt and 2 kt + 1
-        mma_bf16_16816_zero(Y[2 * kt], Aq, movmatrix_trans(Ak[0]), movmatrix_trans(Ak[1]));
-        mma_bf16_16816_zero(Y[2 * kt + 1], Aq, movmatrix_trans(Ak[2]), movmatrix_trans(Ak[3]));
-      }
+      // Eq. 3 for accumulator tiles 2 kt and 2 kt + 1
+      mma_bf16_16816_zero(Y[2 * kt], Aq, movmatrix_trans(Ak[0]), movmatrix_trans(Ak[1]));
+      mma_bf16_16816_zero(Y[2 * kt + 1], Aq, movmatrix_trans(Ak[2]), movmatrix_trans(Ak[3]));
     }
-    if constexpr (kPacked) {
-      // row 0 of the products: lanes 0-3 hold the sums over the slab's rows for their SEG columns
-      if (g == 0) {
+    // row 0 of the products: lanes 0-3 hold the sums over the slab's rows for their SEG columns
+    if (g == 0) {
 #pragma unroll
-        for (int x = 0; x < SEG / 4; ++x)
-          sts128(ydst + 4 * (SEG * c + 4 * x), make_float4(Y[2 * x][0], Y[2 * x][1], Y[2 * x + 1][0], Y[2 * x + 1][1]));
-      }
-    } else {
-      reduce_over_rows<SEG>(part, lane);
-      using RO = RowReduceOut<V>;
-      if (RO::owner(lane)) {
-        const uint32_t dst = ydst + 4 * RO::first_col(lane);
-        if constexpr (RO::CNT == 4) sts128(dst, make_float4(part[0], part[1], part[2], part[3]));
-        else if constexpr (RO::CNT == 2) sts64(dst, make_float2(part[0], part[1]));
-        else sts32(dst, part[0]);
-      }
+      for (int x = 0; x < SEG / 4; ++x)
+        sts128(ydst + 4 * (SEG * c + 4 * x), make_float4(Y[2 * x][0], Y[2 * x][1], Y[2 * x + 1][0], Y[2 * x + 1][1]));
     }
   };
 
@@ -450,54 +386,34 @@ __global__ void __launch_bounds__((MAXW + 1) * 32, OCC) fwd_bf16_kernel(ScanArgs
   if (a.hT) store_state(a.hT + bn * KV);
 }
 
-template <int V, int MAXW, bool CKPT, int OCC>
-cudaError_t launch_vwco(const ScanArgs &a, cudaStream_t s) {
+template <int V, bool CKPT>
+cudaError_t launch_vc(const ScanArgs &a, cudaStream_t s) {
   const size_t smem = FwdSmem<V>::bytes(a.KCf);
   const unsigned grid = a.B * a.N * (a.K / a.KCf), threads = (a.KCf / 16 + 1) * 32;
-  cudaError_t e = allow_smem(fwd_bf16_kernel<V, MAXW, CKPT, OCC>, smem);
+  cudaError_t e = allow_smem(fwd_bf16_kernel<V, CKPT>, smem);
   if (e != cudaSuccess) return e;
-  fwd_bf16_kernel<V, MAXW, CKPT, OCC><<<grid, threads, smem, s>>>(in_order(a, grid, threads, 3));
+  fwd_bf16_kernel<V, CKPT><<<grid, threads, smem, s>>>(in_order(a, grid, threads, 3));
   return cudaGetLastError();
 }
-
-template <int V, int MAXW, bool CKPT>
-cudaError_t launch_vwc(const ScanArgs &a, cudaStream_t s) {
-  // two CTAs per SM where there are units to fill them and the slab count leaves the registers
-  if constexpr (MAXW == 4 && V <= 64) {
-    const long ctas = (long)a.B * a.N * (a.K / a.KCf);
-    if (ctas > sm_count()) return launch_vwco<V, MAXW, CKPT, 2>(a, s);
-  }
-  return launch_vwco<V, MAXW, CKPT, 1>(a, s);
-}
-
-template <int V, int MAXW>
-cudaError_t launch_vw(const ScanArgs &a, cudaStream_t s) {
-  return a.ckpt ? launch_vwc<V, MAXW, true>(a, s) : launch_vwc<V, MAXW, false>(a, s);
-}
-
 template <int V>
 cudaError_t launch_v(const ScanArgs &a, cudaStream_t s) {
-  return a.KCf <= 64 ? launch_vw<V, 4>(a, s) : launch_vw<V, 8>(a, s);
+  return a.ckpt ? launch_vc<V, true>(a, s) : launch_vc<V, false>(a, s);
 }
 
 }  // namespace
 
-// The column-split variant (two chain warps per 16-row slab) takes the shapes it supports; the
-// environment variable M2RNN_FWD_VARIANT=wide forces the one-warp-per-slab kernel of this file
-// (benchmarking only).
+// Which forward kernel takes a problem.
 cudaError_t launch_fwd_bf16(const ScanArgs &a, cudaStream_t s) {
   if (fwd_use_tc(a.B, a.N, a.K, a.V, M2RNN_BF16)) return launch_fwd_bf16_tc(a, s);
   if (a.V == 16) return launch_fwd_v16(a, s);
-  const char *variant = getenv("M2RNN_FWD_VARIANT");
   // V = 128, 32 rows per CTA, checkpoints: the tcgen05 kernel's threads hold whole columns and store them with fewer
   // instructions (32 units of K = V = 128, 4096 steps: 1995 -> 1784 us).  Without checkpoints the two take the same time
   // (1723 and 1715) and the column-split kernel's sums keep the order they have with 16 rows, where it is far ahead.
-  if (!variant && a.V == 128 && a.KCf == 32 && a.ckpt) return launch_fwd_bf16_tc(a, s);
-  if (fwd_cs_supported(a) && !(variant && !strcmp(variant, "wide"))) return launch_fwd_bf16_cs(a, s);
+  if (a.V == 128 && a.KCf == 32 && a.ckpt && !getenv("M2RNN_FWD_VARIANT")) return launch_fwd_bf16_tc(a, s);
+  if (fwd_cs_supported(a)) return launch_fwd_bf16_cs(a, s);
   switch (a.V) {
     case 32: return launch_v<32>(a, s);
     case 64: return launch_v<64>(a, s);
-    case 128: return launch_v<128>(a, s);
     default: return cudaErrorInvalidValue;
   }
 }
