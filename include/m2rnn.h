@@ -23,8 +23,9 @@
  *     every state (h0,hT,ckpt,d_hT,dh0,decode state), dgate and dW are fp32.
  *     With M2RNN_BF16 the state x W product runs on tensor cores (bf16 operands, fp32
  *     accumulate) and the state itself stays fp32; with M2RNN_F32 everything is fp32 FMA.
- *   - The library allocates nothing and keeps nothing between calls.  Outputs are
- *     overwritten, never accumulated into.
+ *   - The library allocates nothing and keeps nothing of a call for the next (only constants of the
+ *     device and which of its kernels may use how much shared memory are asked for once).  Outputs
+ *     are overwritten, never accumulated into.
  *   - Calls are asynchronous on `stream` (a cudaStream_t passed as void*; NULL = the
  *     default stream) and never synchronise.  The return value is an m2rnn_status.
  *     Argument errors (every code but M2RNN_ERR_CUDA) are found on the host first: nothing

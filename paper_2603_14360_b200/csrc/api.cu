@@ -145,6 +145,9 @@ bool fwd_use_tc(int B, int N, int K, int V, int io_dtype) {
   // are bound by the legacy tensor path and there are rows to amortise it over: V = 128, 64-row CTAs, and so many of
   // them that 32-row CTAs no longer fit one to an SM (1024 steps of K = V = 128, us: 37 units 442 against 809, 40
   // units 861 against 816; with checkpoints 995 against 926).
+  // Below V = 128 it stays slower at every number of units (1024 steps, us, register kernels / this one): K = V = 64, 128 units
+  // 302 / 448, 192 599 / 694, 256 600 / 696 (with checkpoints 660 / 813), 384 896 / 1375; K = 128, V = 64, 128 units 618 / 741;
+  // K = V = 32, 256 units 169 / 453; K = 64, V = 16, 256 units 137 / 831.
   return V == 128 && K % 64 == 0 && (long)(B > 0 ? B : 1) * N * (K / 32) > sm_count();
 }
 

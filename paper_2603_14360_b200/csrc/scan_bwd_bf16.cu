@@ -283,8 +283,8 @@ __global__ void __launch_bounds__(bwd_threads<V, NWC>(), V == 16 ? (NWC == 2 ? 3
 #pragma unroll
         for (int nt = 0; nt < NT; ++nt) load_w_fragment<V>(Wn, kt, nt, lane, Wr[kt][nt][0], Wr[kt][nt][1]);
     }
-    // (the checkpoint's place walks where four slabs share the issue slots: 8321 -> 8291 us with 256 units of K = V = 64,
-    // 4096 steps; elsewhere that costs what it gives)
+    // (the checkpoint's place walks where four slabs share the issue slots: 256 units of K = V = 64, 2048 steps, 4195 -> 4168 us,
+    // 512 units 8332 -> 8285, 148 units 2099 -> 2086, runs of one form within 0.1 %; elsewhere that costs what it gives)
     constexpr bool kWalkCk = V == 64 && NWC >= 4;
     const float *ck_walk = a.ckpt + ((size_t)unit * a.nchunks + (nch - 1)) * KV;
     for (int j = 0; j < nch; ++j) {

@@ -37,6 +37,8 @@ struct FwdSmem {
 };
 
 // CKPT: whether checkpoints are written (a compile-time switch keeps the branch out of the hot loop).
+// (The launch bound's second argument is needed: without it the compiler takes 20 registers less, and 440 units of K = 112,
+// V = 32 with checkpoints, 1024 steps, 1285 us instead of 1019.)
 template <int V, bool CKPT>
 __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) fwd_bf16_kernel(ScanArgs a) {
   using G = TileGeom<V>;
