@@ -91,13 +91,23 @@ bool bwd_use_tc(int B, int N, int K, int V, int io_dtype) {
   return true;
 }
 
-BwdPlan plan_bwd(int B, int N, int K, int V, int io_dtype, size_t tokens, bool lean) {
+size_t tokens_of(const m2rnn_params *p) { return p->cu_seqlens ? (size_t)p->total_tokens : (size_t)p->B * p->T; }
+
+BwdPlan plan_bwd(const m2rnn_params *p, bool lean, bool have_ckpt) {
+  const int B = p->B, N = p->N, K = p->K, V = p->V;
   BwdPlan pl{};
-  if (io_dtype == M2RNN_F32) {
-    pl.KC = lean ? K : bwd_f32_rows(B, N, K, V, tokens * N * V * sizeof(float)); pl.C = bwd_f32_piece(); pl.C_max = 64;
+  if (p->io_dtype == M2RNN_F32) {
+    pl.KC = lean ? K : bwd_f32_rows(B, N, K, V, p->T > 0 ? tokens_of(p) * N * V * sizeof(float) : 0); pl.C = bwd_f32_piece(); pl.C_max = 64;
     return pl;
   }
-  if (bwd_use_tc(B, N, K, V, io_dtype)) {   // 32-row CTAs, chunks of four steps
+  // V = 16: scan_bwd_v16.cu, except where every slab of 16 rows has an SM to itself: there a slab's step is quicker spread over
+  // the specialised warps of scan_bwd_bf16.cu (1 024 steps, us: 16 slabs 232 against 245, 64 of heads of their own 208 / 232;
+  // 160 slabs 296 / 249).  The latter keeps two chunks on chip, 16 rows of them up to any supported interval.
+  if (V == 16 && (long)(B > 0 ? B : 1) * N * (K / 16) > sm_count()) {
+    const BwdPlan fast = plan_bwd_v16(B, N, p->Nq, p->Nk, K, p->T, p->ckpt_interval, false);
+    return lean ? plan_bwd_v16(B, N, p->Nq, p->Nk, K, p->T, p->ckpt_interval || have_ckpt ? fast.C : 16, true) : fast;
+  }
+  if (bwd_use_tc(B, N, K, V, p->io_dtype)) {   // 32-row CTAs, chunks of four steps
     pl.KC = bwd_tc_rows_per_cta(); pl.C = pl.C_max = bwd_tc_chunk();
     return pl;
   }
@@ -111,26 +121,12 @@ BwdPlan plan_bwd(int B, int N, int K, int V, int io_dtype, size_t tokens, bool l
   for (int cand = 32; cand <= cap; cand *= 2)
     if (K % cand == 0) KC = cand;
   while (KC > 16 && units * (K / KC) < kSMs && units * (K / (KC / 2)) <= kSMs) KC /= 2;
-  // V = 16, whole 64-row states, more units than two CTAs per SM hold (the paper's layer shape: 336
-  // units): 32-row CTAs at three per SM where that needs fewer waves, a 32-row CTA's wave counted
-  // as 0.9 of a 64-row one (measured: the step is latency, not rows; 3.50 -> 3.16 ms at that shape)
-  bool v16_split = false;
-  if (V == 16 && KC == 64 && units > 2L * kSMs) {
-    const long waves64 = (units + 2L * kSMs - 1) / (2L * kSMs), waves32 = (2 * units + 3L * kSMs - 1) / (3L * kSMs);
-    v16_split = 9 * waves32 < 10 * waves64;
-  }
-  if (v16_split) KC = 32;
   pl.KC = KC;
   // Checkpoint interval: as many steps as two chunk buffers fit in shared memory (even, <= 16)
   constexpr size_t kSmemLimit = 227 * 1024;
   int c = 16;
   while (c > 2 && bwd_bf16_smem_bytes(KC, V, c) > kSmemLimit) c -= 2;
-  pl.C_max = c;
-  // V = 16 with more CTAs than SMs (the paper's layer shape: 84 heads): a shorter chunk lets two
-  // (32-row CTAs: three) CTAs share an SM, which saves a wave
-  if (V == 16 && units * (K / KC) > kSMs)
-    while (c > 2 && bwd_bf16_smem_bytes(KC, V, c) > (v16_split ? 72 : 110) * 1024) c -= 2;
-  pl.C = c;
+  pl.C = pl.C_max = c;
   return pl;
 }
 
@@ -197,7 +193,7 @@ int check_params(const m2rnn_params *p, bool need_T) {
   if (p->gate_kind < M2RNN_GATE_VALUE || p->gate_kind > M2RNN_GATE_PSI) return M2RNN_ERR_UNSUPPORTED;
   if (p->K % 16 || p->K < 16 || p->K > 128) return M2RNN_ERR_UNSUPPORTED;
   if (p->V != 16 && p->V != 32 && p->V != 64 && p->V != 128) return M2RNN_ERR_UNSUPPORTED;
-  if (p->ckpt_interval < 0 || p->ckpt_interval > plan_bwd(p->B, p->N, p->K, p->V, p->io_dtype).C_max)
+  if (p->ckpt_interval < 0 || p->ckpt_interval > plan_bwd(p).C_max)
     return M2RNN_ERR_UNSUPPORTED;
   // the bf16 kernels take steps in pairs and checkpoint between pairs
   if (p->io_dtype == M2RNN_BF16 && (p->ckpt_interval & 1)) return M2RNN_ERR_UNSUPPORTED;
@@ -212,11 +208,8 @@ int check_params(const m2rnn_params *p, bool need_T) {
   return M2RNN_OK;
 }
 
-// tokens in the batch
-size_t tokens_of(const m2rnn_params *p) { return p->cu_seqlens ? (size_t)p->total_tokens : (size_t)p->B * p->T; }
-
-int interval_of(const m2rnn_params *p) {
-  return p->ckpt_interval ? p->ckpt_interval : plan_bwd(p->B, p->N, p->K, p->V, p->io_dtype).C;
+int interval_of(const m2rnn_params *p, bool lean = false, bool have_ckpt = true) {
+  return p->ckpt_interval ? p->ckpt_interval : plan_bwd(p, lean, have_ckpt).C;
 }
 
 struct Workspace {
@@ -225,20 +218,22 @@ struct Workspace {
 
 Workspace layout(const m2rnn_params *p, bool have_ckpt, bool lean) {
   Workspace w{};
-  const int C = interval_of(p);
+  const BwdPlan pl = plan_bwd(p, lean, have_ckpt);
+  const int C = interval_of(p, lean, have_ckpt);
   const size_t nch = p->T > 0 ? (size_t)(p->T + C - 1) / C : 0;
   const size_t BN = (size_t)p->B * p->N, KV = (size_t)p->K * p->V;
   size_t off = 0;
   w.ckpt = off;
   if (!have_ckpt) off += align_up(BN * nch * KV * sizeof(float));
-  const int RS = p->K / plan_bwd(p->B, p->N, p->K, p->V, p->io_dtype, tokens_of(p), lean).KC;   // row slabs per state
+  const int RS = p->K / pl.KC;   // row slabs per state
   w.dW_part = off;
   off += align_up(BN * RS * p->V * p->V * sizeof(float));
   const size_t TT = tokens_of(p);
+  const int shares = pl.groups ? pl.groups : p->N;   // of a shared head's dq or dk
   w.dq_part = off;
-  if (p->Nq < p->N) off += align_up(TT * p->N * p->K * sizeof(float));
+  if (p->Nq < shares) off += align_up(TT * shares * p->K * sizeof(float));
   w.dk_part = off;
-  if (p->Nk < p->N) off += align_up(TT * p->N * p->K * sizeof(float));
+  if (p->Nk < shares) off += align_up(TT * shares * p->K * sizeof(float));
   w.chunk_states = off;
   if (p->io_dtype == M2RNN_F32 && C > bwd_f32_piece()) off += align_up(BN * ((C + bwd_f32_piece() - 1) / bwd_f32_piece()) * KV * sizeof(float));
   w.dv_part = off;
@@ -249,13 +244,14 @@ Workspace layout(const m2rnn_params *p, bool have_ckpt, bool lean) {
   return w;
 }
 
-ScanArgs base_args(const m2rnn_params *p, bool lean = false) {
+ScanArgs base_args(const m2rnn_params *p, bool lean = false, bool have_ckpt = true) {
   ScanArgs a{};
   a.B = p->B; a.T = p->T; a.N = p->N; a.Nq = p->Nq; a.Nk = p->Nk; a.K = p->K; a.V = p->V;
   a.gate_kind = p->gate_kind;
-  a.KC = plan_bwd(p->B, p->N, p->K, p->V, p->io_dtype, tokens_of(p), lean).KC;
+  const BwdPlan pl = plan_bwd(p, lean, have_ckpt);
+  a.KC = pl.KC; a.hg = pl.hg; a.groups = pl.groups; a.set = pl.set;
   a.KCf = plan_fwd_rows(p->B, p->N, p->K, p->V, p->io_dtype, tokens_of(p));
-  a.C = interval_of(p);
+  a.C = interval_of(p, lean, have_ckpt);
   a.nchunks = p->T > 0 ? (p->T + a.C - 1) / a.C : 0;
   a.dh_clip = p->dh_clip;
   a.qs = p->q_stride ? p->q_stride : (long long)p->Nq * p->K;
@@ -301,7 +297,7 @@ int bwd_call(const m2rnn_params *params, const void *q, const void *k, const voi
   if (reinterpret_cast<uintptr_t>(workspace) % kAlign) return M2RNN_ERR_ALIGN;
   char *ws = static_cast<char *>(workspace);
 
-  ScanArgs a = base_args(params, lean);
+  ScanArgs a = base_args(params, lean, ckpt != nullptr);
   a.q = q; a.k = k; a.v = v; a.gate = gate; a.W = W; a.h0 = h0; a.w_r = w_r;
   a.alpha = params->gate_kind == M2RNN_GATE_PSI ? alpha : nullptr;
   a.beta = params->gate_kind == M2RNN_GATE_PSI ? beta : nullptr;
@@ -321,13 +317,15 @@ int bwd_call(const m2rnn_params *params, const void *q, const void *k, const voi
   }
   a.dy = dy; a.d_hT = d_hT; a.dq = dq; a.dk = dk; a.dv = dv; a.dgate = dgate; a.dh0 = dh0;
   a.dW_part = reinterpret_cast<float *>(ws + w.dW_part);
-  a.dq_part = params->Nq < params->N ? reinterpret_cast<float *>(ws + w.dq_part) : nullptr;
-  a.dk_part = params->Nk < params->N ? reinterpret_cast<float *>(ws + w.dk_part) : nullptr;
+  const int shares = a.groups ? a.groups : params->N;
+  a.dq_part = params->Nq < shares ? reinterpret_cast<float *>(ws + w.dq_part) : nullptr;
+  a.dk_part = params->Nk < shares ? reinterpret_cast<float *>(ws + w.dk_part) : nullptr;
   a.chunk_states = f32 ? reinterpret_cast<float *>(ws + w.chunk_states) : nullptr;
   const int RS = params->K / a.KC;
   a.dv_part = RS > 1 ? reinterpret_cast<float *>(ws + w.dv_part) : nullptr;
   a.dgate_part = RS > 1 ? reinterpret_cast<float *>(ws + w.dgate_part) : nullptr;
   e = f32 ? launch_bwd_f32(a, s)
+      : a.hg ? launch_bwd_v16(a, s)
           : (bwd_use_tc(params->B, params->N, params->K, params->V, params->io_dtype) ? launch_bwd_bf16_tc(a, s) : launch_bwd_bf16(a, s));
   if (e != cudaSuccess) return cuda_failed();
   e = launch_reduce_dW(a.dW_part, dW, params->B * RS, params->N, params->V, s);
@@ -340,11 +338,11 @@ int bwd_call(const m2rnn_params *params, const void *q, const void *k, const voi
     if (e != cudaSuccess) return cuda_failed();
   }
   if (a.dq_part) {
-    e = launch_reduce_heads(a.dq_part, dq, params->io_dtype, BT, params->N, params->Nq, params->K, s);
+    e = launch_reduce_heads(a.dq_part, dq, params->io_dtype, BT, shares, params->Nq, params->K, s);
     if (e != cudaSuccess) return cuda_failed();
   }
   if (a.dk_part) {
-    e = launch_reduce_heads(a.dk_part, dk, params->io_dtype, BT, params->N, params->Nk, params->K, s);
+    e = launch_reduce_heads(a.dk_part, dk, params->io_dtype, BT, shares, params->Nk, params->K, s);
     if (e != cudaSuccess) return cuda_failed();
   }
   return M2RNN_OK;
@@ -381,7 +379,7 @@ int m2rnn_ckpt_interval(const m2rnn_params *params) {
 int m2rnn_bwd_row_slab(const m2rnn_params *params) {
   int rc = check_params(params, false);
   if (rc != M2RNN_OK) return rc;
-  return plan_bwd(params->B, params->N, params->K, params->V, params->io_dtype, params->T > 0 ? tokens_of(params) : 0).KC;
+  return plan_bwd(params).KC;
 }
 
 size_t m2rnn_ckpt_bytes(const m2rnn_params *params) {

@@ -32,8 +32,8 @@ struct ScanArgs {
   float *dW_part;      // [B*K/KC,N,V,V] per-CTA partial sums of dW
   float *dv_part;      // [K/KC][B,T,N,V] fp32 per-row-slab dv when K/KC > 1, else null
   float *dgate_part;   // [K/KC][B,T,N] fp32 per-row-slab dgate when K/KC > 1, else null
-  float *dq_part;      // [B,T,N,K] fp32 per-head dq when Nq < N, else null
-  float *dk_part;      // [B,T,N,K] fp32 per-head dk when Nk < N, else null
+  float *dq_part;      // [B,T,shares,K] fp32 shares of dq when Nq < N (a share per head; V = 16: per CTA's heads), else null
+  float *dk_part;      // likewise dk, when Nk < N
   float *chunk_states; // fp32 path, C > 16: [B*N, ceil(C/16), K, V] states between the pieces of a chunk
   int32_t *dev_status;
   // token addressing: elements between consecutive tokens of q, k, v (dense: Nq K, Nk K, N V; larger
@@ -42,6 +42,7 @@ struct ScanArgs {
   long long qs, ks, vs;
   long long TT;
   const int32_t *cu;
+  int hg, groups, set;   // backward, V = 16: heads per CTA, CTAs per token's heads (= shares of dq and dk), heads that a CTA's are taken from
   int rank;       // B where the sequences of a packed batch are taken longest first, else 0
 };
 
@@ -107,6 +108,7 @@ struct BwdPlan {
   int KC;     // rows per CTA (fp32 path: 4 or 8, or K for one launch per group of eight)
   int C;      // default checkpoint interval
   int C_max;  // largest supported checkpoint interval
+  int hg, groups, set;   // V = 16 (bf16): see ScanArgs
 };
 int sm_count();   // SMs of the current device (148 when there is none to ask)
 bool current_context(uint64_t *id);   // the current context's number, unique for the life of the process
@@ -114,9 +116,11 @@ cudaError_t allow_smem(const void *kernel, size_t bytes);   // dynamic shared me
 template <typename... A> cudaError_t allow_smem(void (*kernel)(A...), size_t bytes) {
   return allow_smem(reinterpret_cast<const void *>(kernel), bytes);
 }
-// (tokens: of the batch; they only decide where an fp32 problem is too large for per-slab shares.  lean: without
-// such shares, an fp32 problem's groups of rows one after the other)
-BwdPlan plan_bwd(int B, int N, int K, int V, int io_dtype, size_t tokens = 0, bool lean = false);
+// (lean: as little scratch as there can be: an fp32 problem's groups of rows one after the other, without shares of
+// dv and dW; have_ckpt false: the interval is the call's own business)
+BwdPlan plan_bwd(const m2rnn_params *p, bool lean = false, bool have_ckpt = true);
+BwdPlan plan_bwd_v16(int B, int N, int Nq, int Nk, int K, int T, int interval, bool lean);   // scan_bwd_v16.cu: V = 16, bf16
+size_t tokens_of(const m2rnn_params *p);
 // m2rnn_bwd and its workspace query; lean: see plan_bwd
 size_t bwd_workspace_bytes(const m2rnn_params *params, bool have_ckpt, bool lean);
 int bwd_call(const m2rnn_params *params, const void *q, const void *k, const void *v, const float *gate, const void *W,
@@ -145,7 +149,8 @@ cudaError_t launch_fwd_bf16(const ScanArgs &a, cudaStream_t s);     // scan_fwd_
 cudaError_t launch_fwd_v16(const ScanArgs &a, cudaStream_t s);      // scan_fwd_v16.cu: V = 16
 bool fwd_cs_supported(const ScanArgs &a);                            // scan_fwd_bf16_cs.cu
 cudaError_t launch_fwd_bf16_cs(const ScanArgs &a, cudaStream_t s);  // scan_fwd_bf16_cs.cu: two or four warps per 16-row slab
-cudaError_t launch_bwd_bf16(const ScanArgs &a, cudaStream_t s);     // scan_bwd_bf16.cu
+cudaError_t launch_bwd_bf16(const ScanArgs &a, cudaStream_t s);     // scan_bwd_bf16.cu: 32 <= V
+cudaError_t launch_bwd_v16(const ScanArgs &a, cudaStream_t s);      // scan_bwd_v16.cu: V = 16
 // The tcgen05 backward kernel (scan_bwd_tc.cu) takes V = 128; M2RNN_BWD_VARIANT = tc | mma overrides
 // the choice (benchmarking only).
 bool bwd_use_tc(int B, int N, int K, int V, int io_dtype);

@@ -71,6 +71,20 @@ __device__ __forceinline__ void load_w_fragment(const __nv_bfloat16 *__restrict_
   b1 = (uint32_t)w[r2 * V + col] | ((uint32_t)w[r3 * V + col] << 16);
 }
 
+// B fragment (kt, nt) of W^T under the column relabelling of mma_tile.cuh: B[k = j][n = l] = W[l][j].
+template <int V>
+__device__ __forceinline__ void load_wt_fragment(const __nv_bfloat16 *__restrict__ Wn, int kt, int nt, int lane,
+                                                 uint32_t &b0, uint32_t &b1) {
+  using G = TileGeom<V>;
+  const int g = lane >> 2, c = lane & 3;
+  const int l = G::mem_col(8 * nt + g);
+  const int j0 = G::mem_col(16 * kt + 2 * c), j1 = G::mem_col(16 * kt + 2 * c + 1);
+  const int j2 = G::mem_col(16 * kt + 8 + 2 * c), j3 = G::mem_col(16 * kt + 8 + 2 * c + 1);
+  const uint16_t *w = reinterpret_cast<const uint16_t *>(Wn);
+  b0 = (uint32_t)w[l * V + j0] | ((uint32_t)w[l * V + j1] << 16);
+  b1 = (uint32_t)w[l * V + j2] | ((uint32_t)w[l * V + j3] << 16);
+}
+
 // Sum, over the 8 lane groups g of a warp, of per-thread partials p[idx] (idx = 2nt+e, i.e. the
 // thread's SEG memory columns in order), by recursive halving: each round a lane keeps one half
 // of its values and hands the other half to its partner.  Afterwards lane (g,c) holds

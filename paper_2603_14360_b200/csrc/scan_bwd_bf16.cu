@@ -49,20 +49,6 @@ __device__ __forceinline__ float2 unpack_bf16(uint32_t x) {
   return make_float2(__uint_as_float(x << 16), __uint_as_float(x & 0xffff0000u));
 }
 
-// B fragment (kt, nt) of W^T under the column relabelling of mma_tile.cuh: B[k = j][n = l] = W[l][j].
-template <int V>
-__device__ __forceinline__ void load_wt_fragment(const __nv_bfloat16 *__restrict__ Wn, int kt, int nt, int lane,
-                                                 uint32_t &b0, uint32_t &b1) {
-  using G = TileGeom<V>;
-  const int g = lane >> 2, c = lane & 3;
-  const int l = G::mem_col(8 * nt + g);
-  const int j0 = G::mem_col(16 * kt + 2 * c), j1 = G::mem_col(16 * kt + 2 * c + 1);
-  const int j2 = G::mem_col(16 * kt + 8 + 2 * c), j3 = G::mem_col(16 * kt + 8 + 2 * c + 1);
-  const uint16_t *w = reinterpret_cast<const uint16_t *>(Wn);
-  b0 = (uint32_t)w[l * V + j0] | ((uint32_t)w[l * V + j1] << 16);
-  b1 = (uint32_t)w[l * V + j2] | ((uint32_t)w[l * V + j3] << 16);
-}
-
 __device__ __forceinline__ void ldmatrix_x4(uint32_t addr, uint32_t (&r)[4]) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
 }
@@ -125,7 +111,7 @@ template <int V, int NWC>
 __host__ __device__ constexpr int bwd_threads() { return bwd_rebalance<V, NWC>() ? 512 : (2 * NWC + V / 16 + 2) * 32; }
 
 template <int V, int NWC>
-__global__ void __launch_bounds__(bwd_threads<V, NWC>(), V == 16 ? (NWC == 2 ? 3 : 2) : 1) bwd_bf16_kernel(ScanArgs a) {
+__global__ void __launch_bounds__(bwd_threads<V, NWC>(), 1) bwd_bf16_kernel(ScanArgs a) {
   using G = TileGeom<V>;
   constexpr int NT = G::NT, KT = G::KT, SEG = G::SEG;
   constexpr int KC = 16 * NWC, NDW = V / 16;
@@ -142,7 +128,7 @@ __global__ void __launch_bounds__(bwd_threads<V, NWC>(), V == 16 ? (NWC == 2 ? 3
   // Who computes dq = H_t dy and dk = dX v (small MMAs): the dW warps from the tiles, where they have
   // the time (more dW warps than row slabs: sweep64 backward 7.13 -> 5.76 ms, sweep32 2.65 -> 2.43),
   // else the reverse warps from the fragments they hold (with as many slabs as dW warps the dW
-  // warps would set the pace: bptt_bf16 8.37 -> 9.00 ms, the paper's layer shape 3.13 -> 3.41)
+  // warps would set the pace: bptt_bf16 8.37 -> 9.00 ms)
   constexpr bool kDqDw = NDW >= 2 * NWC || (NDW == 1 && NWC == 1), kDkDw = kDqDw;
   extern __shared__ __align__(128) unsigned char smem[];
 
@@ -154,8 +140,7 @@ __global__ void __launch_bounds__(bwd_threads<V, NWC>(), V == 16 ? (NWC == 2 ? 3
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const int g = lane >> 2, c = lane & 3;
   const int place = blockIdx.x / RS, rs = blockIdx.x % RS;
-  // (V = 16 keeps the grid's order: what the compiler makes of its three-CTA variant is 9 % slower on dense
-  // batches with b from anywhere else, and its CTAs are small)
+  // (V = 16 keeps the grid's order: it comes here only where every CTA has an SM to itself)
   const int b = V == 16 ? place / N : batch_entry(a, place / N, smem), n = place % N;
   const int unit = V == 16 ? place : b * N + n;
   const UnitSpan span = unit_span(a, b);   // this batch entry's tokens (a slice of a packed batch, or b T ..)
@@ -884,9 +869,11 @@ template <int V>
 cudaError_t launch_bwd_v(const ScanArgs &a, cudaStream_t s) {
   switch (a.KC) {
     case 16: return launch_bwd_t<V, 1>(a, s);
-    case 32: return launch_bwd_t<V, 2>(a, s);
+    case 32:
+      if constexpr (V > 16) return launch_bwd_t<V, 2>(a, s);    // (V = 16: only single slabs come here)
+      break;
     case 64:
-      if constexpr (V <= 64) return launch_bwd_t<V, 4>(a, s);   // (the plan gives V = 128 at most 32 rows)
+      if constexpr (V == 32 || V == 64) return launch_bwd_t<V, 4>(a, s);   // (the plan gives V = 128 at most 32 rows)
       break;
   }
   return cudaErrorInvalidValue;
