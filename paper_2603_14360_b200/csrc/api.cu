@@ -193,8 +193,7 @@ int check_params(const m2rnn_params *p, bool need_T) {
   if (p->gate_kind < M2RNN_GATE_VALUE || p->gate_kind > M2RNN_GATE_PSI) return M2RNN_ERR_UNSUPPORTED;
   if (p->K % 16 || p->K < 16 || p->K > 128) return M2RNN_ERR_UNSUPPORTED;
   if (p->V != 16 && p->V != 32 && p->V != 64 && p->V != 128) return M2RNN_ERR_UNSUPPORTED;
-  if (p->ckpt_interval < 0 || p->ckpt_interval > plan_bwd(p).C_max)
-    return M2RNN_ERR_UNSUPPORTED;
+  if (p->ckpt_interval < 0 || (p->ckpt_interval > 0 && p->ckpt_interval > plan_bwd(p).C_max)) return M2RNN_ERR_UNSUPPORTED;
   // the bf16 kernels take steps in pairs and checkpoint between pairs
   if (p->io_dtype == M2RNN_BF16 && (p->ckpt_interval & 1)) return M2RNN_ERR_UNSUPPORTED;
   // token strides: at least a token's heads, in 16-byte units
@@ -208,9 +207,7 @@ int check_params(const m2rnn_params *p, bool need_T) {
   return M2RNN_OK;
 }
 
-int interval_of(const m2rnn_params *p, bool lean = false, bool have_ckpt = true) {
-  return p->ckpt_interval ? p->ckpt_interval : plan_bwd(p, lean, have_ckpt).C;
-}
+int interval_of(const m2rnn_params *p) { return p->ckpt_interval ? p->ckpt_interval : plan_bwd(p).C; }
 
 struct Workspace {
   size_t ckpt, dW_part, dq_part, dk_part, chunk_states, dv_part, dgate_part, total;
@@ -219,7 +216,7 @@ struct Workspace {
 Workspace layout(const m2rnn_params *p, bool have_ckpt, bool lean) {
   Workspace w{};
   const BwdPlan pl = plan_bwd(p, lean, have_ckpt);
-  const int C = interval_of(p, lean, have_ckpt);
+  const int C = p->ckpt_interval ? p->ckpt_interval : pl.C;
   const size_t nch = p->T > 0 ? (size_t)(p->T + C - 1) / C : 0;
   const size_t BN = (size_t)p->B * p->N, KV = (size_t)p->K * p->V;
   size_t off = 0;
@@ -244,15 +241,10 @@ Workspace layout(const m2rnn_params *p, bool have_ckpt, bool lean) {
   return w;
 }
 
-ScanArgs base_args(const m2rnn_params *p, bool lean = false, bool have_ckpt = true) {
+ScanArgs base_args(const m2rnn_params *p) {
   ScanArgs a{};
   a.B = p->B; a.T = p->T; a.N = p->N; a.Nq = p->Nq; a.Nk = p->Nk; a.K = p->K; a.V = p->V;
   a.gate_kind = p->gate_kind;
-  const BwdPlan pl = plan_bwd(p, lean, have_ckpt);
-  a.KC = pl.KC; a.hg = pl.hg; a.groups = pl.groups; a.set = pl.set;
-  a.KCf = plan_fwd_rows(p->B, p->N, p->K, p->V, p->io_dtype, tokens_of(p));
-  a.C = interval_of(p, lean, have_ckpt);
-  a.nchunks = p->T > 0 ? (p->T + a.C - 1) / a.C : 0;
   a.dh_clip = p->dh_clip;
   a.qs = p->q_stride ? p->q_stride : (long long)p->Nq * p->K;
   a.ks = p->k_stride ? p->k_stride : (long long)p->Nk * p->K;
@@ -260,6 +252,14 @@ ScanArgs base_args(const m2rnn_params *p, bool lean = false, bool have_ckpt = tr
   a.TT = (long long)tokens_of(p);
   a.cu = p->cu_seqlens;
   return a;
+}
+// (plans only where a call uses them: they are a part of a small call's host time)
+void plan_forward(ScanArgs &a, const m2rnn_params *p) { a.KCf = plan_fwd_rows(p->B, p->N, p->K, p->V, p->io_dtype, tokens_of(p)); }
+void plan_backward(ScanArgs &a, const m2rnn_params *p, bool lean, bool have_ckpt) {
+  const BwdPlan pl = plan_bwd(p, lean, have_ckpt);
+  a.KC = pl.KC; a.hg = pl.hg; a.groups = pl.groups; a.set = pl.set;
+  a.C = p->ckpt_interval ? p->ckpt_interval : pl.C;
+  a.nchunks = p->T > 0 ? (p->T + a.C - 1) / a.C : 0;
 }
 
 }  // namespace
@@ -297,7 +297,8 @@ int bwd_call(const m2rnn_params *params, const void *q, const void *k, const voi
   if (reinterpret_cast<uintptr_t>(workspace) % kAlign) return M2RNN_ERR_ALIGN;
   char *ws = static_cast<char *>(workspace);
 
-  ScanArgs a = base_args(params, lean, ckpt != nullptr);
+  ScanArgs a = base_args(params);
+  plan_backward(a, params, lean, ckpt != nullptr);
   a.q = q; a.k = k; a.v = v; a.gate = gate; a.W = W; a.h0 = h0; a.w_r = w_r;
   a.alpha = params->gate_kind == M2RNN_GATE_PSI ? alpha : nullptr;
   a.beta = params->gate_kind == M2RNN_GATE_PSI ? beta : nullptr;
@@ -307,6 +308,7 @@ int bwd_call(const m2rnn_params *params, const void *q, const void *k, const voi
   if (!ckpt) {
     // pass 1 of Algorithm 2, thinned: save the state every C steps only
     ScanArgs f = a;
+    plan_forward(f, params);
     f.y = nullptr; f.hT = nullptr;
     f.ckpt = reinterpret_cast<float *>(ws + w.ckpt);
     e = f32 ? launch_fwd_f32(f, s) : launch_fwd_bf16(f, s);
@@ -412,6 +414,8 @@ int m2rnn_fwd(const m2rnn_params *params, const void *q, const void *k, const vo
   a.q = q; a.k = k; a.v = v; a.gate = gate; a.W = W; a.h0 = h0; a.w_r = w_r;
   a.alpha = params->gate_kind == M2RNN_GATE_PSI ? alpha : nullptr;
   a.beta = params->gate_kind == M2RNN_GATE_PSI ? beta : nullptr;
+  plan_forward(a, params);
+  if (ckpt) plan_backward(a, params, false, true);      // (the checkpoints' interval)
   a.y = y; a.hT = hT; a.ckpt = ckpt; a.dev_status = dev_status;
   size_t need = m2rnn_fwd_workspace_bytes(params);
   if (need > 0 && !workspace && workspace_bytes == 0) {   // without shares of y, where the kernels can
