@@ -15,6 +15,7 @@
 // repeatable).
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "device_common.cuh"
@@ -30,7 +31,8 @@ constexpr int kConvThreads = kLanes * kSub;
 constexpr int kUFwd = 8, kGFwd = 3;              // forward: rows are fetched in batches of kUFwd steps, kGFwd batches ahead
 constexpr int kOccFwd = 6;
 constexpr int kUBwd = 4, kGBwd = 2;              // backward: in batches of kUBwd steps, kGBwd batches ahead
-constexpr int kOccBwd = 4;                       // CTAs per SM the bf16 backward kernel is compiled for (fp32: as many as fit its registers)
+constexpr int kOccBwd = 4;                       // CTAs per SM the bf16 backward kernel is compiled for
+constexpr int kOccBwdF32 = 2;                    // (fp32: as many as fit its 173 registers)
 
 template <typename T> struct Chunk;             // the channels of one thread
 template <> struct Chunk<float> {
@@ -53,10 +55,8 @@ template <> struct Chunk<__nv_bfloat16> {   // 8 bytes: four channels keep a thr
   }
 };
 
-// sigmoid: through tanh.approx (one special-function instruction, error ~2^-11: below the bf16
-// rounding of the result) on the bf16 path, through expf on the fp32 path
-template <typename T> __device__ __forceinline__ float sigmoid_of(float x);
-template <> __device__ __forceinline__ float sigmoid_of<float>(float x) {
+// sigmoid of the fp32 path
+__device__ __forceinline__ float sigmoid_of(float x) {
   // No branch, one exponential, and the quotient of a number in [1, 2] by Newton's iteration: x -> x + x (1 - d x)
   // squares the relative error of the starting value.  A divide's own path for extreme operands kept the
   // channels of a thread from overlapping: 46 us, 0.7 of it per time step, however small the problem.
@@ -65,17 +65,16 @@ template <> __device__ __forceinline__ float sigmoid_of<float>(float x) {
   r = fmaf(r, fmaf(-d, r, 1.f), r);
   return x >= 0.f ? r : e * r;
 }
-template <> __device__ __forceinline__ float sigmoid_of<__nv_bfloat16>(float x) { return fmaf(0.5f, tanh_approx(0.5f * x), 0.5f); }
 
-// both halves of a pair (the arithmetic below is in packed fp32 pairs: one instruction per two channels)
-template <typename T> __device__ __forceinline__ float2 sigmoid2(float2 x) {
-  if constexpr (sizeof(T) == 2) {
-    const float2 h = __fmul2_rn(x, make_float2(0.5f, 0.5f));
-    return __ffma2_rn(make_float2(tanh_approx(h.x), tanh_approx(h.y)), make_float2(0.5f, 0.5f), make_float2(0.5f, 0.5f));
-  } else {
-    return make_float2(sigmoid_of<T>(x.x), sigmoid_of<T>(x.y));
-  }
-}
+// The arithmetic below is in packed fp32 pairs: one instruction per two channels (of two cycles, as long as two single ones).
+__device__ __forceinline__ float2 sigmoid2(float2 x) { return make_float2(sigmoid_of(x.x), sigmoid_of(x.y)); }
+__device__ __forceinline__ float2 tanh2(float2 x) { return make_float2(tanh_approx(x.x), tanh_approx(x.y)); }
+// On the bf16 path taps and bias are halved when they are loaded, so that the sum is h = pre / 2, and with the sigmoid
+// (1 + tanh h) / 2 through tanh.approx (one special-function instruction, error ~2^-11: below the bf16 rounding of the result)
+//   SiLU(pre) = h + h tanh h,   2 SiLU'(pre) = (1 + tanh h) (1 + h (1 - tanh h)):
+// five packed operations for an output and eight for twice the gradient of pre (whose other half the taps of dx have, and
+// the sums of dw and dbias take at the end), against seven and ten through the sigmoid.
+template <typename T> constexpr float kTapScale = sizeof(T) == 2 ? 0.5f : 1.f;
 template <int CH>
 __device__ __forceinline__ void to_pairs(const float (&v)[CH], float2 (&p)[CH / 2]) {
 #pragma unroll
@@ -116,8 +115,9 @@ __global__ void __launch_bounds__(kConvThreads, kOccFwd) conv_silu_fwd_kernel(in
 #pragma unroll
   for (int e = 0; e < CP; ++e) {
 #pragma unroll
-    for (int s = 0; s < 4; ++s) w2[s][e] = make_float2(to_f32<T>(w[(size_t)(c0 + 2 * e) * 4 + s]), to_f32<T>(w[(size_t)(c0 + 2 * e + 1) * 4 + s]));
-    b2[e] = bias ? make_float2(to_f32<T>(bias[c0 + 2 * e]), to_f32<T>(bias[c0 + 2 * e + 1])) : make_float2(0.f, 0.f);
+    for (int s = 0; s < 4; ++s)
+      w2[s][e] = make_float2(kTapScale<T> * to_f32<T>(w[(size_t)(c0 + 2 * e) * 4 + s]), kTapScale<T> * to_f32<T>(w[(size_t)(c0 + 2 * e + 1) * 4 + s]));
+    b2[e] = bias ? make_float2(kTapScale<T> * to_f32<T>(bias[c0 + 2 * e]), kTapScale<T> * to_f32<T>(bias[c0 + 2 * e + 1])) : make_float2(0.f, 0.f);
   }
   float2 xm3[CP], xm2[CP], xm1[CP];
   {
@@ -162,7 +162,9 @@ __global__ void __launch_bounds__(kConvThreads, kOccFwd) conv_silu_fwd_kernel(in
 #pragma unroll
         for (int e = 0; e < CP; ++e) {
           const float2 pre = __ffma2_rn(w2[3][e], x0[e], __ffma2_rn(w2[2][e], xm1[e], __ffma2_rn(w2[1][e], xm2[e], __ffma2_rn(w2[0][e], xm3[e], b2[e]))));
-          const float2 r = __fmul2_rn(pre, sigmoid2<T>(pre));
+          float2 r;
+          if constexpr (sizeof(T) == 2) r = __ffma2_rn(pre, tanh2(pre), pre);
+          else r = __fmul2_rn(pre, sigmoid2(pre));
           o[2 * e] = r.x; o[2 * e + 1] = r.y;
           xm3[e] = xm2[e]; xm2[e] = xm1[e]; xm1[e] = x0[e];
         }
@@ -177,9 +179,9 @@ __global__ void __launch_bounds__(kConvThreads, kOccFwd) conv_silu_fwd_kernel(in
   cp_async_wait<0>();
 }
 
-// partial sums of a tile: part[tile][5][C] = dw taps 0..3 and dbias
+// partial sums of a tile: part[tile][5][C] = dw taps 0..3 and dbias.  STEPS = 0: runs of `run` steps
 template <typename T, int STEPS>
-__global__ void __launch_bounds__(kConvThreads, sizeof(T) == 2 ? kOccBwd : 1) conv_silu_bwd_kernel(int B, int Tn, int C, const T *__restrict__ x, long long xs,
+__global__ void __launch_bounds__(kConvThreads, sizeof(T) == 2 ? kOccBwd : 1) conv_silu_bwd_kernel(int run, int Tn, int C, const T *__restrict__ x, long long xs,
                                                                      const T *__restrict__ w, const T *__restrict__ bias,
                                                                      const T *__restrict__ prev, const T *__restrict__ dout, long long ds,
                                                                      T *__restrict__ dx, long long dxs, T *__restrict__ dprev,
@@ -189,17 +191,18 @@ __global__ void __launch_bounds__(kConvThreads, sizeof(T) == 2 ? kOccBwd : 1) co
   const int lane = threadIdx.x % kLanes, sub = threadIdx.x / kLanes;
   const int cc = blockIdx.x * kLanes + lane;
   const bool live = cc * CH < C;
-  constexpr int kTile = kSub * STEPS;
-  const int c0 = live ? cc * CH : 0, ntile = (Tn + kTile - 1) / kTile;
-  const int b = blockIdx.y / ntile, t0 = (blockIdx.y % ntile) * kTile + sub * STEPS;
-  const int t1 = max(t0, min(Tn, t0 + STEPS));   // an empty run when the sequence ends before it
+  const int steps = STEPS ? STEPS : run, tile = kSub * steps;
+  const int c0 = live ? cc * CH : 0, ntile = (Tn + tile - 1) / tile;
+  const int b = blockIdx.y / ntile, t0 = (blockIdx.y % ntile) * tile + sub * steps;
+  const int t1 = max(t0, min(Tn, t0 + steps));   // an empty run when the sequence ends before it
   constexpr int CP = CH / 2;            // channel pairs
   float2 w2[4][CP], b2[CP];
 #pragma unroll
   for (int e = 0; e < CP; ++e) {
 #pragma unroll
-    for (int s = 0; s < 4; ++s) w2[s][e] = make_float2(to_f32<T>(w[(size_t)(c0 + 2 * e) * 4 + s]), to_f32<T>(w[(size_t)(c0 + 2 * e + 1) * 4 + s]));
-    b2[e] = bias ? make_float2(to_f32<T>(bias[c0 + 2 * e]), to_f32<T>(bias[c0 + 2 * e + 1])) : make_float2(0.f, 0.f);
+    for (int s = 0; s < 4; ++s)
+      w2[s][e] = make_float2(kTapScale<T> * to_f32<T>(w[(size_t)(c0 + 2 * e) * 4 + s]), kTapScale<T> * to_f32<T>(w[(size_t)(c0 + 2 * e + 1) * 4 + s]));
+    b2[e] = bias ? make_float2(kTapScale<T> * to_f32<T>(bias[c0 + 2 * e]), kTapScale<T> * to_f32<T>(bias[c0 + 2 * e + 1])) : make_float2(0.f, 0.f);
   }
   float2 dw2[4][CP], db2[CP];
 #pragma unroll
@@ -268,9 +271,13 @@ __global__ void __launch_bounds__(kConvThreads, sizeof(T) == 2 ? kOccBwd : 1) co
 #pragma unroll
           for (int e = 0; e < CP; ++e) {
             const float2 pre = __ffma2_rn(w2[3][e], x0[e], __ffma2_rn(w2[2][e], xm1[e], __ffma2_rn(w2[1][e], xm2[e], __ffma2_rn(w2[0][e], xm3[e], b2[e]))));
-            const float2 sg = sigmoid2<T>(pre);
-            // dout * SiLU'(pre),  SiLU'(x) = sg (1 + x (1 - sg))
-            d0[e] = __fmul2_rn(__fmul2_rn(g[e], sg), __ffma2_rn(pre, __ffma2_rn(sg, mone, one), one));
+            if constexpr (sizeof(T) == 2) {       // (pre is h)
+              const float2 th = tanh2(pre);
+              d0[e] = __fmul2_rn(__ffma2_rn(g[e], th, g[e]), __ffma2_rn(pre, __ffma2_rn(th, mone, one), one));
+            } else {       // dout * SiLU'(pre),  SiLU'(x) = sg (1 + x (1 - sg))
+              const float2 sg = sigmoid2(pre);
+              d0[e] = __fmul2_rn(__fmul2_rn(g[e], sg), __ffma2_rn(pre, __ffma2_rn(sg, mone, one), one));
+            }
             if (IN || t < t1) {                                // sums over this run's own steps only
               dw2[0][e] = __ffma2_rn(d0[e], xm3[e], dw2[0][e]); dw2[1][e] = __ffma2_rn(d0[e], xm2[e], dw2[1][e]);
               dw2[2][e] = __ffma2_rn(d0[e], xm1[e], dw2[2][e]); dw2[3][e] = __ffma2_rn(d0[e], x0[e], dw2[3][e]);
@@ -308,8 +315,8 @@ __global__ void __launch_bounds__(kConvThreads, sizeof(T) == 2 ? kOccBwd : 1) co
 #pragma unroll
   for (int e = 0; e < CP; ++e) {
 #pragma unroll
-    for (int s = 0; s < 4; ++s) { dwv[2 * e][s] = dw2[s][e].x; dwv[2 * e + 1][s] = dw2[s][e].y; }
-    dbv[2 * e] = db2[e].x; dbv[2 * e + 1] = db2[e].y;
+    for (int s = 0; s < 4; ++s) { dwv[2 * e][s] = kTapScale<T> * dw2[s][e].x; dwv[2 * e + 1][s] = kTapScale<T> * dw2[s][e].y; }
+    dbv[2 * e] = kTapScale<T> * db2[e].x; dbv[2 * e + 1] = kTapScale<T> * db2[e].y;
   }
   // (dprev of the first tile: the three steps before t = 0 were emitted while t = 0, 1, 2 -- with
   // d3/d2/d1 still zero where they stand for dpre at negative times)
@@ -367,6 +374,24 @@ int steps_per_thread(int B, int T, int C) {
   if (cols * tiles(T, 64) >= 2 * sms) return 64;
   return cols * tiles(T, 16) <= sms ? 16 : 32;
 }
+// Of the backward, where there is enough for runs of 64: the CTAs run in rounds of as many as the SMs hold, and a last round that is
+// half empty costs as much as a full one, so the run is as long as makes them come out even (with its halo and some eight
+// steps' time for its start and its sums).  [8, 2048, 3072] bf16, four CTAs an SM: 2.6 rounds of 64 steps 66.0 us and 3.9 to add
+// the runs' sums, one of 171 steps 62.1 and 2.9; [4, 4096, 1472] 38.9 -> 36.2; fp32 [8, 2048, 1024] 44.8 -> 42.7.  (The
+// forward kernel, six CTAs an SM and nearer to the memory's rate, loses: 38.2 -> 39.5.)
+int bwd_steps(int B, int T, int C, int io_dtype) {
+  const int rule = steps_per_thread(B, T, C);
+  const long cols = (long)B * ((C / 4 + kLanes - 1) / kLanes), slots = (long)sm_count() * (io_dtype == M2RNN_BF16 ? kOccBwd : kOccBwdF32);
+  if (rule < 64 || cols * tiles(T, 64) > 16 * slots) return rule;      // (many rounds: their last does not count)
+  int best = 64;
+  long best_cost = (cols * tiles(T, 64) + slots - 1) / slots * (64 + 3 + 8);
+  for (int n = 1, most = tiles(T, 48); n <= most && (long)B * n <= 65535; ++n) {        // n tiles a sequence
+    const int steps = (T + kSub * n - 1) / (kSub * n);
+    const long cost = (cols * tiles(T, steps) + slots - 1) / slots * (steps + 3 + 8);
+    if (cost < best_cost) { best = steps; best_cost = cost; }
+  }
+  return best;
+}
 dim3 conv_grid(int B, int T, int C, int steps) { return dim3((C / 4 + kLanes - 1) / kLanes, (unsigned)(B * tiles(T, steps))); }
 
 template <typename T, int STEPS>
@@ -377,10 +402,10 @@ void launch_fwd(int B, int Tn, int C, const void *x, long long xs, const void *w
       static_cast<T *>(out), os);
 }
 template <typename T, int STEPS>
-void launch_bwd(int B, int Tn, int C, const void *x, const long long (&st)[3], const void *w, const void *bias, const void *prev,
+void launch_bwd(int B, int Tn, int C, int steps, const void *x, const long long (&st)[3], const void *w, const void *bias, const void *prev,
                 const void *dout, void *dx, void *dprev, float *part, cudaStream_t s) {
-  conv_silu_bwd_kernel<T, STEPS><<<conv_grid(B, Tn, C, STEPS), kConvThreads, 0, s>>>(
-      B, Tn, C, static_cast<const T *>(x), st[0], static_cast<const T *>(w), static_cast<const T *>(bias), static_cast<const T *>(prev),
+  conv_silu_bwd_kernel<T, STEPS><<<conv_grid(B, Tn, C, steps), kConvThreads, 0, s>>>(
+      steps, Tn, C, static_cast<const T *>(x), st[0], static_cast<const T *>(w), static_cast<const T *>(bias), static_cast<const T *>(prev),
       static_cast<const T *>(dout), st[1], static_cast<T *>(dx), st[2], static_cast<T *>(dprev), part);
 }
 
@@ -425,7 +450,8 @@ extern "C" int m2rnn_conv_silu_fwd(int32_t B, int32_t T, int32_t C, int32_t io_d
 
 extern "C" size_t m2rnn_conv_silu_bwd_workspace_bytes(int32_t B, int32_t T, int32_t C) {
   if (B <= 0 || T <= 0 || C <= 0) return 0;
-  return align_up((size_t)B * tiles(T, steps_per_thread(B, T, C)) * 5 * C * sizeof(float));
+  const int most = std::max(tiles(T, bwd_steps(B, T, C, M2RNN_BF16)), tiles(T, bwd_steps(B, T, C, M2RNN_F32)));     // (the type is not known)
+  return align_up((size_t)B * most * 5 * C * sizeof(float));
 }
 
 extern "C" int m2rnn_conv_silu_bwd(int32_t B, int32_t T, int32_t C, int32_t io_dtype, const void *x, int64_t x_stride,
@@ -452,13 +478,13 @@ extern "C" int m2rnn_conv_silu_bwd(int32_t B, int32_t T, int32_t C, int32_t io_d
   if (!workspace || workspace_bytes < need) return M2RNN_ERR_WORKSPACE;
   if (reinterpret_cast<uintptr_t>(workspace) % kAlign) return M2RNN_ERR_ALIGN;
   float *part = static_cast<float *>(workspace);
-  const int steps = steps_per_thread(B, T, C);
-  const auto launch = [&](auto kernel_of) { kernel_of(B, T, C, x, st, w, bias, prev, dout, dx, dprev, part, s); };
+  const int steps = bwd_steps(B, T, C, io_dtype), rule = steps_per_thread(B, T, C);
+  const auto launch = [&](auto kernel_of) { kernel_of(B, T, C, steps, x, st, w, bias, prev, dout, dx, dprev, part, s); };
   const bool bf = io_dtype == M2RNN_BF16;
-  switch (steps) {
+  switch (rule) {
     case 16: launch(bf ? launch_bwd<__nv_bfloat16, 16> : launch_bwd<float, 16>); break;
     case 32: launch(bf ? launch_bwd<__nv_bfloat16, 32> : launch_bwd<float, 32>); break;
-    default: launch(bf ? launch_bwd<__nv_bfloat16, 64> : launch_bwd<float, 64>);
+    default: launch(bf ? launch_bwd<__nv_bfloat16, 0> : launch_bwd<float, 0>);
   }
   if (cudaGetLastError() != cudaSuccess) return M2RNN_ERR_CUDA;
   conv_silu_reduce_kernel<<<(8 * 5 * C + 255) / 256, 256, 0, s>>>(part, B * tiles(T, steps), C, dw, dbias);

@@ -40,6 +40,27 @@ def test_steps_per_thread(oracle, dtype, shape):
     test_forward_backward(oracle, dtype, shape, True)
 
 
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_runs_that_make_rounds_come_out_even(oracle, dtype):
+    """Enough for runs of 64 steps: the backward's runs are of other lengths, neither a multiple of a batch nor of the sequence."""
+    test_forward_backward(oracle, dtype, (3, 2101, 1608), True)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_large_inputs(oracle, dtype):
+    """SiLU and its derivative far out, where the sigmoid is 0 or 1: one tap, so that the products are exact in either type."""
+    d = inputs.make_conv_inputs(2, 40, 64, dtype, seed=17, prev=False)
+    d["w"].zero_(); d["w"][:, 3] = 1.0
+    d["bias"].zero_()
+    d["x"] = (d["x"].float() * 2.0 ** torch.arange(40).sub(10)[None, :, None]).to(d["x"].dtype)
+    g = {k: (None if v is None else v.cuda()) for k, v in d.items()}
+    out, ref = binding.m2rnn_conv_silu_fwd(g["x"], g["w"], g["bias"]), oracle.conv_silu_fwd(F(d["x"]), F(d["w"]), F(d["bias"]))
+    got = binding.m2rnn_conv_silu_bwd(g["x"], g["w"], g["dout"], g["bias"])
+    want = oracle.conv_silu_bwd(F(d["x"]), F(d["w"]), F(d["dout"]), F(d["bias"]))
+    for t in range(40):       # by itself: a large step would hide the others
+        assert parity.rel_err(out[:, t], ref[:, t]) <= parity.TOL[dtype] and parity.rel_err(got["dx"][:, t], want["dx"][:, t]) <= parity.TOL[dtype], t
+
+
 def test_no_bias_and_empty(oracle):
     d = inputs.make_conv_inputs(2, 19, 32, "f32", seed=9, prev=False)
     g = {k: (None if v is None else v.cuda()) for k, v in d.items()}
