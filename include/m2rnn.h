@@ -117,10 +117,10 @@ size_t m2rnn_ckpt_bytes(const m2rnn_params *params);
 /* Scratch the forward call needs for `params`: 0 unless the library splits the rows of a state
  * over several CTAs, in which case the per-slab shares of y, (K / rows) x tokens x N x V floats, pass
  * through this scratch before a second launch adds them.  It splits where there are few (b,n) units, to
- * fill the GPU; M2RNN_F32 states also where groups of four or eight rows make more warps, and
+ * fill the GPU; M2RNN_F32 states also into groups of four rows (V = 16: where groups of four or eight make more warps),
  * M2RNN_BF16 states of K > 64, 32 <= V <= 64 into slabs of at most 64 rows -- both for speed only and
  * up to 4 GiB of shares: m2rnn_fwd also takes those two without a workspace, on whole states and slower
- * (fp32, 16 units of K = V = 64: 6.0 times; bf16, 192 units of K = 96, V = 64: 2.3 times). */
+ * (fp32, 16 units of K = V = 64: 10.6 times; bf16, 192 units of K = 96, V = 64: 2.3 times). */
 size_t m2rnn_fwd_workspace_bytes(const m2rnn_params *params);
 
 /* Forward scan (Algorithm 1; Eq. 1-3).

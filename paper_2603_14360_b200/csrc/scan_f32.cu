@@ -11,7 +11,8 @@
 // step makes the new rows visible.  Sums over l pair even and odd entries (packed fp32x2 FMA).
 // (Until then a CTA held a whole state and read W from shared memory for every product: 1 MB of
 // shared-memory traffic a step and a sixteenth of the SMs at 16 units.  K = V = 64, 16 units, T = 512:
-// forward 3.19 -> 0.37 ms, backward 18.6 -> 0.63 ms.)
+// forward 3.19 -> 0.37 ms, backward 18.6 -> 0.63 ms.  Since then the forward from V = 32 on and the backward of V = 64 have a cut of
+// the product with fewer lanes to a column, below: 0.21 and 0.56 ms.)
 #include "device_common.cuh"
 #include "internal.h"
 
@@ -288,6 +289,264 @@ __global__ void __launch_bounds__(Geom<V>::kThreads) fwd_f32_kernel(ScanArgs a) 
       put<E>(a.hT + bn * KV + (size_t)(rbase + GR * g + orow) * V + ocol, get<E>(H0 + (GR * g + orow) * G::HP + ocol));
 }
 
+// ------------------------------------------------------------------ forward, V >= 32, few rows at a time
+// The same step with the product cut the other way: a warp takes R rows of a group of four and, up to V = 64, all of their
+// columns (V = 128: a quarter), so that up to V = 64 nothing but the warp itself waits for a step.  Lane (q, cg) holds 8 / P of
+// the eight parts of l for CP columns, V CP / P entries of W, 128 registers at V >= 64.  What held the kernel above were
+// the shuffles that add eight lanes' shares of every product (345 us for 512 steps of 16 units, K = V = 64; 218 without
+// them) and the shared memory's bandwidth; here seven eighths of that sum are inside the lane, in the order of the shuffles, so that the
+// two kernels and the decoding step agree bit for bit.
+template <int V>
+struct Wide {
+  static constexpr int CP = V == 32 ? 2 : 4, P = V == 128 ? 4 : 2;      // columns of a lane; lanes that share a column
+  static constexpr int CW = 32 / P * CP, NWR = V / CW;                  // columns of a warp; warps of a row
+  static constexpr int E = CP / P, M = 8 / P, NB = V / 32;              // columns that a lane owns; its parts of l; pieces of a part
+  static constexpr int HP = V + 4;
+  // the l of piece x of part m of lane part q: 4 from 32 x + 4 (q + P m)
+  __device__ static int l_of(int q, int m, int x) { return 32 * x + 4 * (q + P * m); }
+};
+template <int V>
+__device__ __forceinline__ void wide_load_w(const float *__restrict__ W, int q, int c0, float2 (&w)[Wide<V>::M][2 * Wide<V>::NB][Wide<V>::CP]) {
+  using G = Wide<V>;
+#pragma unroll
+  for (int m = 0; m < G::M; ++m)
+#pragma unroll
+    for (int x = 0; x < 2 * G::NB; ++x) {
+      const float *src = W + (size_t)(G::l_of(q, m, x >> 1) + 2 * (x & 1)) * V + c0;
+#pragma unroll
+      for (int e = 0; e < G::CP; ++e) w[m][x][e] = make_float2(src[e], src[V + e]);
+    }
+}
+template <int V>
+__device__ __forceinline__ void wide_load_wt(const float *__restrict__ W, int q, int c0, float2 (&w)[Wide<V>::M][2 * Wide<V>::NB][Wide<V>::CP]) {
+  using G = Wide<V>;
+#pragma unroll
+  for (int m = 0; m < G::M; ++m)
+#pragma unroll
+    for (int x = 0; x < 2 * G::NB; ++x)
+#pragma unroll
+      for (int e = 0; e < G::CP; ++e) w[m][x][e] = *reinterpret_cast<const float2 *>(W + (size_t)(c0 + e) * V + G::l_of(q, m, x >> 1) + 2 * (x & 1));
+}
+// a warp's fragments to shared memory and back: 16 bytes a lane at a time
+template <int V>
+__device__ __forceinline__ void frags_out(float *dst, int lane, const float2 (&w)[Wide<V>::M][2 * Wide<V>::NB][Wide<V>::CP]) {
+  using G = Wide<V>;
+#pragma unroll
+  for (int m = 0; m < G::M; ++m)
+#pragma unroll
+    for (int x = 0; x < 2 * G::NB; ++x)
+#pragma unroll
+      for (int e = 0; e < G::CP; e += 2)
+        *reinterpret_cast<float4 *>(dst + (((m * 2 * G::NB + x) * (G::CP / 2) + e / 2) * 32 + lane) * 4) = make_float4(w[m][x][e].x, w[m][x][e].y, w[m][x][e + 1].x, w[m][x][e + 1].y);
+}
+template <int V>
+__device__ __forceinline__ void frags_in(const float *src, int lane, float2 (&w)[Wide<V>::M][2 * Wide<V>::NB][Wide<V>::CP]) {
+  using G = Wide<V>;
+#pragma unroll
+  for (int m = 0; m < G::M; ++m)
+#pragma unroll
+    for (int x = 0; x < 2 * G::NB; ++x)
+#pragma unroll
+      for (int e = 0; e < G::CP; e += 2) {
+        const float4 t = *reinterpret_cast<const float4 *>(src + (((m * 2 * G::NB + x) * (G::CP / 2) + e / 2) * 32 + lane) * 4);
+        w[m][x][e] = make_float2(t.x, t.y); w[m][x][e + 1] = make_float2(t.z, t.w);
+      }
+}
+// R rows, `pitch` floats apart, times the matrix held in w: o[r][e], column c0 + E q + e of row r
+template <int V, int R>
+__device__ __forceinline__ void wide_product(const float *rows, int pitch, const float2 (&w)[Wide<V>::M][2 * Wide<V>::NB][Wide<V>::CP], int q, int lane,
+                                             float (&o)[R][Wide<V>::E]) {
+  using G = Wide<V>;
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    float u[G::M][G::CP];
+#pragma unroll
+    for (int m = 0; m < G::M; ++m) {
+      float2 acc[G::CP];
+#pragma unroll
+      for (int e = 0; e < G::CP; ++e) acc[e] = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int x = 0; x < G::NB; ++x) {
+        const float4 h = *reinterpret_cast<const float4 *>(rows + r * pitch + G::l_of(q, m, x));
+#pragma unroll
+        for (int e = 0; e < G::CP; ++e) {
+          acc[e] = __ffma2_rn(make_float2(h.x, h.y), w[m][2 * x][e], acc[e]);
+          acc[e] = __ffma2_rn(make_float2(h.z, h.w), w[m][2 * x + 1][e], acc[e]);
+        }
+      }
+#pragma unroll
+      for (int e = 0; e < G::CP; ++e) u[m][e] = acc[e].x + acc[e].y;
+    }
+    // parts p and p ^ 4, then p ^ 2, then p ^ 1: those of a lane are q + P m
+#pragma unroll
+    for (int h = G::M / 2; h >= 1; h >>= 1)
+#pragma unroll
+      for (int m = 0; m < h; ++m)
+#pragma unroll
+        for (int e = 0; e < G::CP; ++e) u[m][e] += u[m + h][e];
+    float t[G::CP];
+#pragma unroll
+    for (int e = 0; e < G::CP; ++e) t[e] = u[0][e];
+#pragma unroll
+    for (int n = G::CP / 2, bit = 16, qb = G::P / 2; qb >= 1; n >>= 1, bit >>= 1, qb >>= 1) {      // (lane bit 16: the higher bit of q)
+      const bool up = lane & bit;
+#pragma unroll
+      for (int e = 0; e < n; ++e) {
+        const float send = up ? t[e] : t[e + n], keep = up ? t[e + n] : t[e];
+        t[e] = keep + __shfl_xor_sync(0xffffffffu, send, bit);
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < G::E; ++e) o[r][e] = t[e];
+  }
+}
+
+// One CTA per (b, n, group of four rows): 4 / R row sets of NWR warps; set i takes rows i, i + 4 / R, ..
+template <int V, int R>
+struct WideFwd {
+  using G = Wide<V>;
+  static constexpr int kSets = 4 / R, kThreads = 32 * G::NWR * kSets;
+  static constexpr int kStage = kSteps * (2 * 4 + V + 1 + 3);      // q, k [16][4], v [16][V], gate [16] (+ alignment)
+  static constexpr int kFloats = 2 * 4 * G::HP + 2 * kStage + 2 * kSteps + kSteps * kSets * V;
+};
+template <int V, int R>
+__global__ void __launch_bounds__(WideFwd<V, R>::kThreads) fwd_f32_wide_kernel(ScanArgs a) {
+  using G = Wide<V>;
+  using WF = WideFwd<V, R>;
+  constexpr int kSets = WF::kSets, E = G::E;
+  extern __shared__ __align__(16) float smem[];
+  const int K = a.K, N = a.N, RS = K / 4;
+  const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), set = warp / G::NWR;
+  const int q = lane / (32 / G::P), c0 = (warp % G::NWR) * G::CW + G::CP * (lane % (32 / G::P)), col = c0 + E * q;
+  const int place = blockIdx.x / RS, rs = blockIdx.x % RS, rbase = rs * 4;
+  const int b = batch_entry(a, place / N, smem), n = place % N, bn = b * N + n;
+  const UnitSpan span = unit_span(a, b);   // this batch entry's tokens (a slice of a packed batch, or b T ..)
+  const int T = span.T;
+  const size_t tok0 = span.tok0, KV = (size_t)K * V;
+  const int hq = n / (N / a.Nq), hk = n / (N / a.Nk);
+
+  float *H0 = smem + set * G::HP, *H1 = H0 + 4 * G::HP;       // this set's rows before and after a step, kSets HP apart
+  float *stages = smem + 8 * G::HP, *fS = stages + 2 * WF::kStage, *yS = fS + 2 * kSteps;      // [16][sets][V] shares of y
+
+  float2 w[G::M][2 * G::NB][G::CP];
+  wide_load_w<V>(static_cast<const float *>(a.W) + (size_t)n * V * V, q, c0, w);
+  const size_t own = (size_t)(rbase + set) * V + col;      // (row i of the set: i kSets V further)
+  float H[R][E];
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const Vec<E> h = a.h0 ? get<E>(a.h0 + bn * KV + own + (size_t)r * kSets * V) : Vec<E>{};
+#pragma unroll
+    for (int e = 0; e < E; ++e) H[r][e] = h.x[e];
+    put<E>(H0 + r * kSets * G::HP + col, h);
+  }
+  auto store_state = [&](float *dst) {
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      Vec<E> h;
+#pragma unroll
+      for (int e = 0; e < E; ++e) h.x[e] = H[r][e];
+      put<E>(dst + own + (size_t)r * kSets * V, h);
+    }
+  };
+  const float al = a.alpha ? a.alpha[n] : 1.f, be = a.beta ? a.beta[n] : 0.f;
+  const float *qg = static_cast<const float *>(a.q), *kg = static_cast<const float *>(a.k);
+  const float *vg = static_cast<const float *>(a.v), *wr = rs == 0 ? static_cast<const float *>(a.w_r) : nullptr;
+  const bool want_y = a.y != nullptr;
+  float *yg = a.y_part ? a.y_part + (size_t)rs * a.TT * N * V : static_cast<float *>(a.y);
+
+  auto stage = [&](int x) { return stages + (x & 1) * WF::kStage; };
+  constexpr int oK = 4 * kSteps, oV = 8 * kSteps, oG = oV + kSteps * V;
+  auto fetch = [&](int ch) {
+    float *st = stage(ch);
+    const int t0 = ch * kSteps, len = min(kSteps, T - t0);
+    const size_t bt = tok0 + t0;
+    if (want_y) stage_rows(st, qg + bt * a.qs + hq * K + rbase, a.qs, len, 4, tid, WF::kThreads);
+    stage_rows(st + oK, kg + bt * a.ks + hk * K + rbase, a.ks, len, 4, tid, WF::kThreads);
+    stage_rows(st + oV, vg + bt * a.vs + n * V, a.vs, len, V, tid, WF::kThreads);
+    if (tid < len) cp4(st + oG + tid, a.gate + (bt + tid) * N + n);
+    cp_commit();
+  };
+  auto gates = [&](int ch) {   // the thread that copied a gate evaluates it
+    if (tid < min(kSteps, T - ch * kSteps)) fS[(ch & 1) * kSteps + tid] = gate_value(a.gate_kind, stage(ch)[oG + tid], al, be, nullptr);
+  };
+  auto row_sync = [&]() {      // the warps of a set have left their columns
+    if constexpr (G::NWR == 1) __syncwarp();
+    else asm volatile("bar.sync %0, %1;" ::"r"(1 + set), "n"(32 * G::NWR) : "memory");
+  };
+  const int nst = (T + kSteps - 1) / kSteps;
+  if (nst > 0) {
+    fetch(0);
+    cp_wait<0>();
+    gates(0);
+  }
+  __syncthreads();
+  int ck_left = 0;
+  float *ck = a.ckpt ? a.ckpt + (size_t)bn * a.nchunks * KV : nullptr;
+  for (int ch = 0; ch < nst; ++ch) {
+    if (ch + 1 < nst) fetch(ch + 1);
+    const float *st = stage(ch), *fs = fS + (ch & 1) * kSteps;
+    const int len = min(kSteps, T - ch * kSteps);
+    for (int s = 0; s < len; ++s) {
+      if (ck) {
+        if (ck_left == 0) { store_state(ck); ck += KV; ck_left = a.C; }
+        --ck_left;
+      }
+      float o[R][E], kk[R], qq[R];
+      const float f = fs[s];
+      const Vec<E> v = get<E>(st + oV + s * V + col);
+#pragma unroll
+      for (int r = 0; r < R; ++r) { kk[r] = st[oK + 4 * s + set + r * kSets]; qq[r] = st[4 * s + set + r * kSets]; }
+      wide_product<V, R>(H0, kSets * G::HP, w, q, lane, o);
+      Vec<E> qh[R];
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        Vec<E> ov, hv, z;
+#pragma unroll
+        for (int e = 0; e < E; ++e) { ov.x[e] = o[r][e]; hv.x[e] = H[r][e]; }
+        const Vec<E> h = update<E>(ov, kk[r], v, f, hv, z);
+        put<E>(H1 + r * kSets * G::HP + col, h);
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+          H[r][e] = h.x[e];
+          qh[r].x[e] = __fmul_rn(qq[r], h.x[e]);
+        }
+      }
+      // (rows 0 and 2, 1 and 3, then both; R = 1: all of that when the stage is done)
+#pragma unroll
+      for (int h = R / 2; h >= 1; h >>= 1)
+#pragma unroll
+        for (int r = 0; r < h; ++r)
+#pragma unroll
+          for (int e = 0; e < E; ++e) qh[r].x[e] += qh[r + h].x[e];
+      put<E>(yS + (s * kSets + set) * V + col, qh[0]);
+      row_sync();
+      float *x = H0; H0 = H1; H1 = x;
+    }
+    if (ch + 1 < nst) { cp_wait<0>(); gates(ch + 1); }
+    __syncthreads();          // the next stage is in, this one's shares of y are
+    // Eq. 3: the sets' shares, in the same order
+    if (want_y)
+      for (int x = tid; x < len * (V / 4); x += WF::kThreads) {
+        const int s = x / (V / 4), j = 4 * (x % (V / 4));
+        float4 y4 = *reinterpret_cast<const float4 *>(yS + s * kSets * V + j);
+        auto add = [](float4 &p, const float4 &r) { p.x += r.x; p.y += r.y; p.z += r.z; p.w += r.w; };
+        if constexpr (kSets == 2) add(y4, *reinterpret_cast<const float4 *>(yS + (s * kSets + 1) * V + j));
+        if constexpr (kSets == 4) {
+          float4 o4 = *reinterpret_cast<const float4 *>(yS + (s * kSets + 1) * V + j);
+          add(y4, *reinterpret_cast<const float4 *>(yS + (s * kSets + 2) * V + j));
+          add(o4, *reinterpret_cast<const float4 *>(yS + (s * kSets + 3) * V + j));
+          add(y4, o4);
+        }
+        float4 w4 = make_float4(0.f, 0.f, 0.f, 0.f), v4 = w4;
+        if (wr) { w4 = *reinterpret_cast<const float4 *>(wr + (size_t)n * V + j); v4 = *reinterpret_cast<const float4 *>(st + oV + s * V + j); }
+        y4.x = fmaf(w4.x, v4.x, y4.x); y4.y = fmaf(w4.y, v4.y, y4.y); y4.z = fmaf(w4.z, v4.z, y4.z); y4.w = fmaf(w4.w, v4.w, y4.w);
+        *reinterpret_cast<float4 *>(yg + ((tok0 + ch * kSteps + s) * N + n) * V + j) = y4;
+      }
+    __syncthreads();          // (the shares' place, and this stage's, are taken again)
+  }
+  if (a.hT) store_state(a.hT + bn * KV);
+}
+
 // ------------------------------------------------------------------ backward (Algorithm 2)
 // One CTA per (b, n, group of eight rows).  Time goes backwards in pieces of up to 16 steps; of a piece
 // the CTA (A) redoes the forward steps, keeping H_{t-1} and Z_t of every step in shared memory,
@@ -299,29 +558,37 @@ __global__ void __launch_bounds__(Geom<V>::kThreads) fwd_f32_kernel(ScanArgs a) 
 // slab0 / nslab: the groups of rows this launch takes.  All of them (nslab = K/8), each leaving its
 // shares of dv, dgate and dW as partials; or one after the other (nslab = 1), the later ones
 // adding to what the earlier ones wrote.
-template <int V, int GR>
+// WIDE (V = 64, groups of four): the products as in the kernel above, a row a warp; the fragments of W and W^T, 128 registers each,
+// lie in shared memory and are taken from there once per piece and direction.
+template <int V, int GR, bool WIDE>
 struct BwdGeom {
   using G = Geom<V>;
+  static constexpr int kThreads = WIDE ? 32 * GR : G::kThreads;
+  static constexpr int kWideFloats = WIDE ? 2 * V * V : 0;
+  static_assert(!WIDE || (V == 64 && GR == 4), "the fragments of a warp that has all columns of a row");
   static constexpr int kTile = GR * G::HP;
   static constexpr int kStage = kSteps * (2 * GR + 2 * V + 1);        // q, k [16][GR], v, dy [16][V], gate [16]
   // dW tiles: 4 x JT elements per thread; with fewer tiles than threads, SP threads share a tile and
   // take every SP-th step
-  static constexpr int JT = V == 128 ? 8 : 4;
-  static constexpr int kTiles = (V / 4) * (V / JT), SP = G::kThreads / kTiles;
-  static constexpr int kFloats = (2 * kSteps + 1) * kTile + 2 * kStage + 4 * kSteps + kSteps * G::kThreads;
+  static constexpr int JT = V == 128 || WIDE ? 8 : 4;
+  static constexpr int kTiles = (V / 4) * (V / JT), SP = kThreads / kTiles;
+  static_assert(SP >= 1, "a tile a thread");
+  static constexpr int kFloats = (2 * kSteps + 1) * kTile + 2 * kStage + 4 * kSteps + kSteps * kThreads + kWideFloats;
   // W and W^T both stay in registers where they fit beside the dW tile; at V = 128 (32 + 32 + 32 of 128
   // registers) each phase reloads its own from L2 once per piece
   static constexpr bool kReload = V == 128;
 };
 
-template <int V, int GR>
-__global__ void __launch_bounds__(Geom<V>::kThreads, 512 / Geom<V>::kThreads) bwd_f32_kernel(ScanArgs a, int slab0, int nslab) {
+template <int V, int GR, bool WIDE>
+__global__ void __launch_bounds__(BwdGeom<V, GR, WIDE>::kThreads, WIDE ? 2 : 512 / Geom<V>::kThreads) bwd_f32_kernel(ScanArgs a, int slab0, int nslab) {
   using G = Geom<V>;
-  using BG = BwdGeom<V, GR>;
-  constexpr int E = GR / 4;
+  using BG = BwdGeom<V, GR, WIDE>;
+  using WG = Wide<64>;      // (of the wide form)
+  constexpr int E = WIDE ? WG::E : GR / 4, kThreads = BG::kThreads;
   extern __shared__ __align__(16) float smem[];
   const int K = a.K, N = a.N;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, p = lane >> 2, c0 = 8 * warp + 2 * (lane & 3);
+  const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+  const int p = WIDE ? lane / (32 / WG::P) : lane >> 2, c0 = WIDE ? WG::CP * (lane % (32 / WG::P)) : 8 * warp + 2 * (lane & 3);
   const int place = blockIdx.x / nslab, rs = slab0 + blockIdx.x % nslab, rbase = rs * GR;
   const int b = batch_entry(a, place / N, smem), n = place % N, bn = b * N + n;
   const bool add = nslab == 1 && rs > 0;   // earlier launches have written dv, dgate and dW
@@ -337,8 +604,15 @@ __global__ void __launch_bounds__(Geom<V>::kThreads, 512 / Geom<V>::kThreads) bw
   float *dfp = dfS + 2 * kSteps;                  // [16][threads] shares of df
 
   const float *Wn = static_cast<const float *>(a.W) + (size_t)n * V * V;
-  float2 w[G::NP][2], wt[BG::kReload ? 1 : G::NP][2];
-  if constexpr (!BG::kReload) {
+  float *wS = dfp + kSteps * kThreads;            // the fragments of W and W^T, 16 bytes a lane at a time
+  float2 w[WIDE ? 1 : G::NP][2], wt[WIDE || BG::kReload ? 1 : G::NP][2];
+  float2 ww[WIDE ? WG::M : 1][2 * WG::NB][WG::CP];
+  if constexpr (WIDE) {
+    wide_load_w<V>(Wn, p, c0, ww);
+    if (warp == 0) frags_out<V>(wS, lane, ww);
+    wide_load_wt<V>(Wn, p, c0, ww);
+    if (warp == 0) frags_out<V>(wS + V * V, lane, ww);
+  } else if constexpr (!BG::kReload) {
     load_w<V>(Wn, p, c0, w);
     load_wt<V>(Wn, p, c0, wt);
   }
@@ -346,7 +620,7 @@ __global__ void __launch_bounds__(Geom<V>::kThreads, 512 / Geom<V>::kThreads) bw
   const float *qg = static_cast<const float *>(a.q), *kg = static_cast<const float *>(a.k);
   const float *vg = static_cast<const float *>(a.v), *wr = static_cast<const float *>(a.w_r);
   const float *dyg = static_cast<const float *>(a.dy);
-  const int orow = Own<GR>::row(p), ocol = Own<GR>::col(p, c0);
+  const int orow = WIDE ? warp : Own<GR>::row(p), ocol = WIDE ? c0 + E * p : Own<GR>::col(p, c0);
   const int own = orow * G::HP + ocol;            // this thread's elements inside a group of rows
   const size_t own_g = (size_t)(rbase + orow) * V + ocol;   // ... inside a state in memory
 
@@ -362,10 +636,10 @@ __global__ void __launch_bounds__(Geom<V>::kThreads, 512 / Geom<V>::kThreads) bw
   auto fetch = [&](int x, Piece pc) {
     float *st = stage(x);
     const size_t bt = tok0 + pc.t0;
-    stage_rows(st, qg + bt * a.qs + hq * K + rbase, a.qs, pc.len, GR, tid, G::kThreads);
-    stage_rows(st + oK, kg + bt * a.ks + hk * K + rbase, a.ks, pc.len, GR, tid, G::kThreads);
-    stage_rows(st + oV, vg + bt * a.vs + n * V, a.vs, pc.len, V, tid, G::kThreads);
-    stage_rows(st + oDY, dyg + (bt * N + n) * V, (long long)N * V, pc.len, V, tid, G::kThreads);
+    stage_rows(st, qg + bt * a.qs + hq * K + rbase, a.qs, pc.len, GR, tid, kThreads);
+    stage_rows(st + oK, kg + bt * a.ks + hk * K + rbase, a.ks, pc.len, GR, tid, kThreads);
+    stage_rows(st + oV, vg + bt * a.vs + n * V, a.vs, pc.len, V, tid, kThreads);
+    stage_rows(st + oDY, dyg + (bt * N + n) * V, (long long)N * V, pc.len, V, tid, kThreads);
     if (tid < pc.len) cp4(st + oG + tid, a.gate + (bt + tid) * N + n);
     cp_commit();
   };
@@ -375,13 +649,33 @@ __global__ void __launch_bounds__(Geom<V>::kThreads, 512 / Geom<V>::kThreads) bw
   float *scratch = a.chunk_states + (size_t)bn * ppc * KV;   // states at the start of a chunk's pieces
 
   Vec<E> C = a.d_hT ? get<E>(a.d_hT + (size_t)bn * KV + own_g) : Vec<E>{};   // carried dL/dH_t
+  // the group's rows at `rows` times W or W^T, this thread's elements of it
+  auto mul = [&](const float *rows, bool transposed) {
+    if constexpr (WIDE) {
+      float t[1][E];
+      Vec<E> o;
+      wide_product<V, 1>(rows + warp * G::HP, 0, ww, p, lane, t);
+#pragma unroll
+      for (int e = 0; e < E; ++e) o.x[e] = t[0][e];
+      return o;
+    } else if constexpr (BG::kReload) {
+      return product<V, GR>(rows, w, p, lane);
+    } else {
+      return transposed ? product<V, GR>(rows, wt, p, lane) : product<V, GR>(rows, w, p, lane);
+    }
+  };
+  // the rows of a step are written (wide: the warp's own is all that its next product needs)
+  auto row_sync = [&]() {
+    if constexpr (WIDE) __syncwarp();
+    else __syncthreads();
+  };
   float2 dW[4][BG::JT / 2];
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
     for (int j = 0; j < BG::JT / 2; ++j) dW[i][j] = make_float2(0.f, 0.f);
   // (a warp's tiles are four by eight, so that its loads of H and dX are one wavefront each)
-  constexpr int WJ = V >= 64 ? 2 : 1;
+  constexpr int WJ = V > 32 ? (BG::JT == 8 ? V / 2 : V) / 32 : 1;
   const int tile = tid % BG::kTiles, tsp = tid / BG::kTiles, tw = tile >> 5;
   const int tl = 4 * (V == 16 ? (tile >> 2) : 4 * (tw / WJ) + (lane >> 3)), tj = 4 * (V == 16 ? (tile & 3) : 8 * (tw % WJ) + (lane & 7));
 
@@ -390,12 +684,12 @@ __global__ void __launch_bounds__(Geom<V>::kThreads, 512 / Geom<V>::kThreads) bw
     const float *st = stage(x), *fs = fS + (x & 1) * kSteps;
     for (int s = 0; s < len; ++s) {
       float *hs = Hc + s * BG::kTile;
-      const Vec<E> o = product<V, GR>(hs, w, p, lane);
+      const Vec<E> o = mul(hs, false);
       Vec<E> z;
       const Vec<E> h = update<E>(o, st[oK + s * GR + orow], get<E>(st + oV + s * V + ocol), fs[s], get<E>(hs + own), z);
       put<E>(hs + BG::kTile + own, h);
       put<E>(Xc + s * BG::kTile + own, z);
-      __syncthreads();
+      row_sync();
     }
   };
 
@@ -407,6 +701,7 @@ __global__ void __launch_bounds__(Geom<V>::kThreads, 512 / Geom<V>::kThreads) bw
     if (np > 1) {   // walk the chunk forward once, leaving the states between its pieces
       if constexpr (BG::kReload) load_w<V>(Wn, p, c0, w);
       __syncthreads();   // the piece before is done with every array
+      if constexpr (WIDE) frags_in<V>(wS, lane, ww);
       Vec<E> h = get<E>(ck);
       for (int i = 0; i + 1 < np; ++i, ++x) {
         const Piece pc = piece(ch, i);
@@ -431,6 +726,7 @@ __global__ void __launch_bounds__(Geom<V>::kThreads, 512 / Geom<V>::kThreads) bw
       gates(x, pc);
       __syncthreads();   // inputs are in; the piece before is done with every array
       put<E>(Hc + own, h0);
+      if constexpr (WIDE) frags_in<V>(wS, lane, ww);
       __syncthreads();
       // the next piece's inputs, unless a pass over its chunk comes first
       fetched = i > 0 || (ch > 0 && a.C <= kSteps);
@@ -440,6 +736,7 @@ __global__ void __launch_bounds__(Geom<V>::kThreads, 512 / Geom<V>::kThreads) bw
       // (B)
       const float *st = stage(x), *fs = fS + (x & 1) * kSteps;
       if constexpr (BG::kReload) load_wt<V>(Wn, p, c0, w);
+      if constexpr (WIDE) frags_in<V>(wS + V * V, lane, ww);
       for (int s = pc.len - 1; s >= 0; --s) {
         const float f = fs[s], q = st[s * GR + orow];
         const Vec<E> dy = get<E>(st + oDY + s * V + ocol), hp = get<E>(Hc + s * BG::kTile + own);
@@ -453,18 +750,17 @@ __global__ void __launch_bounds__(Geom<V>::kThreads, 512 / Geom<V>::kThreads) bw
           df = fmaf(Gv.x[e], hp.x[e] - z.x[e], df);                  // df = sum G (.) (H_{t-1} - Z)
           dX.x[e] = (1.f - f) * Gv.x[e] * (1.f - z.x[e] * z.x[e]);   // through the gate and tanh
         }
-        dfp[s * G::kThreads + tid] = df;
+        dfp[s * kThreads + tid] = df;
         put<E>(xs + own, dX);
-        __syncthreads();
-        Vec<E> o;                                                    // C_{t-1} = f G + dX W^T
-        if constexpr (BG::kReload) o = product<V, GR>(xs, w, p, lane);
-        else o = product<V, GR>(xs, wt, p, lane);
+        row_sync();
+        const Vec<E> o = mul(xs, true);                              // C_{t-1} = f G + dX W^T
 #pragma unroll
         for (int e = 0; e < E; ++e) {
           C.x[e] = fmaf(f, Gv.x[e], o.x[e]);
           if (a.dh_clip > 0.f) C.x[e] = fminf(fmaxf(C.x[e], -a.dh_clip), a.dh_clip);
         }
       }
+      if constexpr (WIDE) __syncthreads();      // all rows of the piece are in
       // (C) dW += H_{t-1}^T dX over the piece's steps and rows
       for (int s = tsp; s < pc.len; s += BG::SP) {
         const float *hs = Hc + s * BG::kTile + tl, *xs = Xc + s * BG::kTile + tj;
@@ -485,7 +781,7 @@ __global__ void __launch_bounds__(Geom<V>::kThreads, 512 / Geom<V>::kThreads) bw
       }
       // dq = H_t dy, dk = dX v: eight lanes per (step, row)
       const size_t bt0 = tok0 + pc.t0;
-      for (int it = tid >> 3; it < pc.len * GR; it += G::kThreads / 8) {
+      for (int it = tid >> 3; it < pc.len * GR; it += kThreads / 8) {
         const int s = it / GR, r = it % GR, e = tid & 7;
         const float *hs = Hc + (s + 1) * BG::kTile + r * G::HP, *xs = Xc + s * BG::kTile + r * G::HP;
         const float *dys = st + oDY + s * V, *vs = st + oV + s * V;
@@ -510,7 +806,7 @@ __global__ void __launch_bounds__(Geom<V>::kThreads, 512 / Geom<V>::kThreads) bw
         }
       }
       // dv = dX^T k over these rows (+ w_r (.) dy from Eq. 3, added with the first group)
-      for (int it = tid; it < pc.len * (V / 4); it += G::kThreads) {
+      for (int it = tid; it < pc.len * (V / 4); it += kThreads) {
         const int s = it / (V / 4), j = 4 * (it % (V / 4));
         float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
@@ -529,10 +825,10 @@ __global__ void __launch_bounds__(Geom<V>::kThreads, 512 / Geom<V>::kThreads) bw
         *dst = o;
       }
       // dgate: a warp sums the threads' shares of a step, then the gate's slope
-      for (int s = warp; s < pc.len; s += G::NW) {
+      for (int s = warp; s < pc.len; s += kThreads / 32) {
         float df = 0.f;
 #pragma unroll
-        for (int i2 = 0; i2 < G::NW; ++i2) df += dfp[s * G::kThreads + 32 * i2 + lane];
+        for (int i2 = 0; i2 < kThreads / 32; ++i2) df += dfp[s * kThreads + 32 * i2 + lane];
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) df += __shfl_xor_sync(0xffffffffu, df, off);
         if (lane == 0) {
@@ -653,25 +949,51 @@ cudaError_t launch_fwd_g(const ScanArgs &a, cudaStream_t s) {
   fwd_f32_kernel<V, GR><<<ctas, Geom<V>::kThreads, smem, s>>>(in_order(a, ctas, Geom<V>::kThreads, 7));
   return cudaGetLastError();
 }
+template <int V, int R>
+cudaError_t launch_fwd_w(const ScanArgs &a, cudaStream_t s) {
+  constexpr size_t smem = sizeof(float) * (size_t)WideFwd<V, R>::kFloats;
+  constexpr int kThreads = WideFwd<V, R>::kThreads;
+  const cudaError_t e = allow_smem(fwd_f32_wide_kernel<V, R>, smem);
+  if (e != cudaSuccess) return e;
+  const int ctas = a.B * a.N * (a.K / 4);
+  fwd_f32_wide_kernel<V, R><<<ctas, kThreads, smem, s>>>(in_order(a, ctas, kThreads, 4));
+  return cudaGetLastError();
+}
 template <int V>
 cudaError_t launch_fwd_v(const ScanArgs &a, cudaStream_t s) {
-  return a.KCf == kRows / 2 ? launch_fwd_g<V, kRows / 2>(a, s) : launch_fwd_g<V, kRows>(a, s);
+  if constexpr (V >= 32) {
+    if (a.KCf == kRows / 2) {
+      // One row a warp while that makes no more than 11 warps an SM, then two, then four: a warp's step is a chain, as long as its rows
+      // are many (256 steps of K = V = 64, us, one / two / four rows: 1 024 rows in all 108 / 118 / 189, 2 048 204 / 185 / 192, 6 144
+      // 538 / 517 / 476; V = 128, two and four: 512 rows 157 / 179, 2 048 585 / 548).
+      const long warps = (long)a.B * a.N * a.K * Wide<V>::NWR, most = 11L * sm_count();
+      if constexpr (V <= 64)
+        if (warps <= most) return launch_fwd_w<V, 1>(a, s);
+      return warps <= 2 * most ? launch_fwd_w<V, 2>(a, s) : launch_fwd_w<V, 4>(a, s);
+    }
+    return launch_fwd_g<V, kRows>(a, s);
+  } else {
+    return a.KCf == kRows / 2 ? launch_fwd_g<V, kRows / 2>(a, s) : launch_fwd_g<V, kRows>(a, s);
+  }
 }
 
-template <int V, int GR>
+template <int V, int GR, bool WIDE>
 cudaError_t launch_bwd_g(const ScanArgs &a, cudaStream_t s) {
-  const size_t smem = sizeof(float) * (size_t)BwdGeom<V, GR>::kFloats;
-  cudaError_t e = allow_smem(bwd_f32_kernel<V, GR>, smem);
+  using BG = BwdGeom<V, GR, WIDE>;
+  const size_t smem = sizeof(float) * (size_t)BG::kFloats;
+  cudaError_t e = allow_smem(bwd_f32_kernel<V, GR, WIDE>, smem);
   const int slabs = a.K / GR, nslab = a.KC == GR ? slabs : 1;
   for (int s0 = 0; s0 < slabs && e == cudaSuccess; s0 += nslab) {
-    bwd_f32_kernel<V, GR><<<a.B * a.N * nslab, Geom<V>::kThreads, smem, s>>>(in_order(a, (long)a.B * a.N * nslab, Geom<V>::kThreads, 12), s0, nslab);
+    bwd_f32_kernel<V, GR, WIDE><<<a.B * a.N * nslab, BG::kThreads, smem, s>>>(in_order(a, (long)a.B * a.N * nslab, BG::kThreads, 12), s0, nslab);
     e = cudaGetLastError();
   }
   return e;
 }
 template <int V>
 cudaError_t launch_bwd_v(const ScanArgs &a, cudaStream_t s) {
-  return a.KC == kRows / 2 ? launch_bwd_g<V, kRows / 2>(a, s) : launch_bwd_g<V, kRows>(a, s);
+  // (wide, 512 steps of K = V = 64, us: 16 units 630 -> 564, 64 units against groups of eight 2 133 -> 1 949, 256 units 3 677 -> 3 793; K = V =
+  // 32, 16 units 306 -> 329)
+  return a.KC == kRows / 2 ? launch_bwd_g<V, kRows / 2, V == 64>(a, s) : launch_bwd_g<V, kRows, false>(a, s);
 }
 
 template <int V>
@@ -686,16 +1008,17 @@ cudaError_t launch_decode_v(const ScanArgs &a, cudaStream_t s) {
 
 }  // namespace
 
-// Rows per CTA.  The step of a warp is a chain of dependent instructions, so a small problem wants as many warps
-// as it can get: groups of four rows while groups of eight would leave an SM fewer than 16 warps (16 units, K = V
-// = 64, T = 512: forward 379 -> 366 us, backward 721 -> 629), else of eight, which need fewer instructions
-// in all.  Forward: whole states where that gives every SM 16 warps -- the groups take turns behind
-// one barrier a step and y needs no shares in memory.  Backward: K stands for one launch per group of
-// eight, each adding to the results of the one before, where the units alone give every SM 64 warps.
-// `share_bytes`: one group's share of y or dv; whole states (one group after the other) too where the
-// shares of all groups would exceed kMaxShares.
+// Rows per CTA.  The step of a warp is a chain of dependent instructions, so a problem wants its rows spread over many warps.
+// Forward, V >= 32: groups of four rows (fwd_f32_wide_kernel), at any number of units (512 steps of K = V = 64, us, against the
+// kernel of eight lanes a column, in groups of four, of eight and whole states: 16 units 370 -> 206, 64 1005 -> 638, 256 1617 -> 1081).
+// V = 16 and the backward: groups of four rows while groups of eight would leave an SM fewer than 16 warps (V = 64: 32), else of eight,
+// which need fewer instructions in all.  Whole states forward (V = 16) where that gives every SM 16 warps -- the groups take turns
+// behind one barrier a step and y needs no shares in memory.  Backward: K stands for one launch per group of eight, each adding to
+// the results of the one before, where the units alone give every SM 64 warps.  `share_bytes`: one group's share of y or dv; whole
+// states (one group after the other) too where the shares of all groups would exceed kMaxShares.
 constexpr size_t kMaxShares = (size_t)4 << 30;
 int fwd_f32_rows(int B, int N, int K, int V, size_t share_bytes) {
+  if (V >= 32) return share_bytes * (K / (kRows / 2)) > kMaxShares ? K : kRows / 2;
   const long warps = (long)(B > 0 ? B : 1) * N * (V / 8), most = 16L * sm_count();   // of whole states
   if (warps >= most || share_bytes * (K / kRows) > kMaxShares) return K;
   return warps * (K / kRows) >= most ? kRows : kRows / 2;
@@ -703,7 +1026,7 @@ int fwd_f32_rows(int B, int N, int K, int V, size_t share_bytes) {
 int bwd_f32_rows(int B, int N, int K, int V, size_t share_bytes) {
   const long warps = (long)(B > 0 ? B : 1) * N * (V / 8), most = 16L * sm_count();
   if (warps >= 4 * most || share_bytes * (K / kRows) > kMaxShares) return K;
-  return warps * (K / kRows) >= most ? kRows : kRows / 2;
+  return warps * (K / kRows) >= (V == 64 ? 2 : 1) * most ? kRows : kRows / 2;
 }
 int bwd_f32_piece() { return kSteps; }
 

@@ -121,3 +121,26 @@ def test_slab_plans_and_pieces(oracle, B, T, N, K, V, ckpt):
     first = {x: g[x][:, 0].contiguous() for x in ("q", "k", "v", "gate")}
     y1 = binding.m2rnn_decode_step(first["q"], first["k"], first["v"], first["gate"], g["W"], state, w_r=g["w_r"])
     assert torch.equal(y1, y[:, 0])
+
+
+# rows a warp of the forward kernel for V >= 32: one, two and four (by the number of units), a ragged last stage, packed sequences
+@pytest.mark.parametrize("B,T,N,K,V", [(2, 35, 4, 48, 32), (3, 18, 20, 48, 32), (5, 17, 24, 64, 32), (1, 33, 2, 64, 64), (3, 20, 13, 64, 64), (5, 17, 20, 64, 64),
+                                       (1, 19, 3, 32, 128), (2, 17, 12, 48, 128)])
+def test_rows_of_a_warp(oracle, B, T, N, K, V):
+    cfg = ScanConfig("rows", B=B, T=T, N=N, K=K, V=V, dtype="f32", w_scale=0.7, seed=950 + T)
+    d = inputs.make_inputs(cfg, residual=True)
+    g = parity.to_dev(d)
+    y, hT, ck = parity.gpu_fwd(cfg, g, save_ckpt=True)
+    y_ref, hT_ref = parity.oracle_fwd(oracle, cfg, d)
+    assert parity.rel_err(y, y_ref) < 1e-4 and parity.rel_err(hT, hT_ref) < 1e-4
+    # bit for bit: whole states one group after the other, and the first step as a decoding step
+    args, kw = [g[x] for x in ("q", "k", "v", "gate", "W", "h0")], dict(w_r=g["w_r"], save_ckpt=True)
+    whole = binding.m2rnn_fwd(*args, workspace=torch.empty(0, dtype=torch.uint8, device="cuda"), **kw)
+    assert all(torch.equal(a, b) for a, b in zip((y, hT, ck), whole))
+    state, first = g["h0"].clone(), {x: g[x][:, 0].contiguous() for x in ("q", "k", "v", "gate")}
+    assert torch.equal(binding.m2rnn_decode_step(first["q"], first["k"], first["v"], first["gate"], g["W"], state, w_r=g["w_r"]), y[:, 0])
+    # the same sequences packed
+    flat = {x: g[x].flatten(0, 1) for x in ("q", "k", "v", "gate")}
+    cu = torch.arange(0, B * T + 1, T, dtype=torch.int32, device="cuda")
+    yp, hp, _ = binding.m2rnn_fwd(flat["q"], flat["k"], flat["v"], flat["gate"], g["W"], g["h0"], w_r=g["w_r"], cu_seqlens=cu, max_seqlen=T)
+    assert torch.equal(yp.unflatten(0, (B, T)), y) and torch.equal(hp, hT)
