@@ -48,6 +48,16 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   return r;
 }
 
+// Products and sums of 16-bit operands in fp32 (sm_100): one instruction, no unpacking.  HA, HB: which half of a, b.
+template <int HA, int HB> __device__ __forceinline__ float fma_bf16(uint32_t a, uint32_t b, float c) {
+  float d;
+  if constexpr (HA == 0 && HB == 0) asm("{.reg .b16 p,q,r,s; mov.b32 {p,q}, %1; mov.b32 {r,s}, %2; fma.rn.f32.bf16 %0, p, r, %3;}" : "=f"(d) : "r"(a), "r"(b), "f"(c));
+  else if constexpr (HA == 0) asm("{.reg .b16 p,q,r,s; mov.b32 {p,q}, %1; mov.b32 {r,s}, %2; fma.rn.f32.bf16 %0, p, s, %3;}" : "=f"(d) : "r"(a), "r"(b), "f"(c));
+  else if constexpr (HB == 0) asm("{.reg .b16 p,q,r,s; mov.b32 {p,q}, %1; mov.b32 {r,s}, %2; fma.rn.f32.bf16 %0, q, r, %3;}" : "=f"(d) : "r"(a), "r"(b), "f"(c));
+  else asm("{.reg .b16 p,q,r,s; mov.b32 {p,q}, %1; mov.b32 {r,s}, %2; fma.rn.f32.bf16 %0, q, s, %3;}" : "=f"(d) : "r"(a), "r"(b), "f"(c));
+  return d;
+}
+
 template <int V>
 struct TileGeom {
   static constexpr int NT = V / 8;    // accumulator tiles per warp

@@ -90,15 +90,6 @@ __device__ __forceinline__ uint32_t transposed(uint32_t x) {   // an 8 x 8 matri
   asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(y) : "r"(x));
   return y;
 }
-// Products and sums of 16-bit operands in fp32 (sm_100): one instruction, no unpacking.  HA, HB: which half of a, b.
-template <int HA, int HB> __device__ __forceinline__ float fma_bf16(uint32_t a, uint32_t b, float c) {
-  float d;
-  if constexpr (HA == 0 && HB == 0) asm("{.reg .b16 p,q,r,s; mov.b32 {p,q}, %1; mov.b32 {r,s}, %2; fma.rn.f32.bf16 %0, p, r, %3;}" : "=f"(d) : "r"(a), "r"(b), "f"(c));
-  else if constexpr (HA == 0) asm("{.reg .b16 p,q,r,s; mov.b32 {p,q}, %1; mov.b32 {r,s}, %2; fma.rn.f32.bf16 %0, p, s, %3;}" : "=f"(d) : "r"(a), "r"(b), "f"(c));
-  else if constexpr (HB == 0) asm("{.reg .b16 p,q,r,s; mov.b32 {p,q}, %1; mov.b32 {r,s}, %2; fma.rn.f32.bf16 %0, q, r, %3;}" : "=f"(d) : "r"(a), "r"(b), "f"(c));
-  else asm("{.reg .b16 p,q,r,s; mov.b32 {p,q}, %1; mov.b32 {r,s}, %2; fma.rn.f32.bf16 %0, q, s, %3;}" : "=f"(d) : "r"(a), "r"(b), "f"(c));
-  return d;
-}
 __device__ __forceinline__ float2 add_f16x2(uint32_t a, float2 c) {          // a + c
   float2 d;
   asm("{.reg .b16 p,q; mov.b32 {p,q}, %2; add.f32.f16 %0, p, %3; add.f32.f16 %1, q, %4;}" : "=f"(d.x), "=f"(d.y) : "r"(a), "f"(c.x), "f"(c.y));

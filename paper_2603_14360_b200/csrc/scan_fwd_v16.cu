@@ -12,7 +12,8 @@
 // Stages of kTC steps are handed over by mbarriers; every wait is bounded and reports through
 // dev_status.
 // (One service warp that fetched and widened a stage when it was free, readout in the chain warps: 84 heads,
-// K = 64, batch 1, 2 and 4 took 120, 161 and 191 ns per step; now 99, 133 and 179.  What counted, in order: the
+// K = 64, batch 1, 2 and 4 took 120, 161 and 191 ns per step; then 99, 133 and 179; now, with seeds straight from bf16
+// (fma.f32.bf16: no unpacking) and half slabs where a CTA has its SM to itself, 94, 126 and 174.  What counted, in order: the
 // service warps' time per stage, which was longer than the chain's; with three CTAs per SM the
 // shared-memory traffic -- k and v as fp32, f per row, cost 10 %.)
 #include "device_common.cuh"
@@ -60,11 +61,12 @@ __device__ __forceinline__ void ldmatrix_x4(uint32_t addr, uint32_t (&r)[4]) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
 }
 
-// NW: slabs (chain warps) of the CTA.  kSvc service warps: four (one per scheduler, two steps of a stage each)
+// NW: slabs of the CTA, a chain warp each, or two of eight rows (HALF).  kSvc service warps: four (one per scheduler, two steps of a stage each)
 // where a CTA has the SM to itself and their latency counts, two (four steps each) where several CTAs
 // share it and their instructions do.
-template <int NW, bool CKPT, int OCC, int kSvc>
-__global__ void __launch_bounds__((NW + kSvc) * 32, OCC) fwd_v16_kernel(ScanArgs a) {
+template <int NW, bool CKPT, int OCC, int kSvc, bool HALF>
+__global__ void __launch_bounds__(((HALF ? 2 : 1) * NW + kSvc) * 32, OCC) fwd_v16_kernel(ScanArgs a) {
+  constexpr int CW = HALF ? 2 * NW : NW, NH = HALF ? 1 : 2;      // chain warps; rows of a thread
   constexpr int K = 16 * NW, kMine = kTC / kSvc, kBlk = 32 / kMine;   // steps of a stage per service warp; stages of a block of gates
   static_assert(kMine * K / 8 <= 32, "a lane stages eight entries of k");
   extern __shared__ __align__(16) unsigned char smem[];
@@ -78,17 +80,17 @@ __global__ void __launch_bounds__((NW + kSvc) * 32, OCC) fwd_v16_kernel(ScanArgs
   uint64_t *full = reinterpret_cast<uint64_t *>(smem), *done = full + kStages;
   const uint32_t st0 = smem_u32(smem) + kBarBytes;
   if (tid == 0) {
-    for (int s = 0; s < kStages; ++s) { mbar_init(&full[s], 33 * kSvc); mbar_init(&done[s], NW); }
+    for (int s = 0; s < kStages; ++s) { mbar_init(&full[s], 33 * kSvc); mbar_init(&done[s], CW); }
     fence_mbar_init();
   }
   __syncthreads();
 
-  if (warp >= NW) {
+  if (warp >= CW) {
     // ------------------------------------------------------------------ service warps
     // Warp sw takes steps sw, sw + kSvc, .. of every stage, for staging and readout alike: it overwrites only q and
     // v that it alone reads (the chain warps are through with a stage when it is done, and write
     // fragments into it only when all service warps have filled it).
-    const int sw = warp - NW;
+    const int sw = warp - CW;
     const int hq = n / (N / a.Nq), hk = n / (N / a.Nk);
     const float al = a.alpha ? a.alpha[n] : 1.f, be = a.beta ? a.beta[n] : 0.f;
     const bool want_y = a.y != nullptr;
@@ -206,7 +208,9 @@ __global__ void __launch_bounds__((NW + kSvc) * 32, OCC) fwd_v16_kernel(ScanArgs
   }
 
   // -------------------------------------------------------------------- chain warps
-  const int row0 = 16 * warp + 2 * g;   // memory rows row0, row0+1  <->  MMA rows g, g+8; columns 4c .. 4c+3
+  // rows of this thread: row0 and row0 + 1 are MMA rows g and g + 8, or (HALF) row0 is MMA row g of a product whose other eight rows are
+  // zero; columns 4c .. 4c+3
+  const int row0 = HALF ? 8 * warp + g : 16 * warp + 2 * g;
   uint32_t Wr[2][2];
 #pragma unroll
   for (int nt = 0; nt < 2; ++nt)
@@ -215,32 +219,34 @@ __global__ void __launch_bounds__((NW + kSvc) * 32, OCC) fwd_v16_kernel(ScanArgs
   const size_t own = (size_t)(rbase + row0) * kV + 4 * c;
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
-    const float4 t4 = a.h0 ? *reinterpret_cast<const float4 *>(a.h0 + bn * KV + own + h * kV) : make_float4(0.f, 0.f, 0.f, 0.f);
+    const float4 t4 = h < NH && a.h0 ? *reinterpret_cast<const float4 *>(a.h0 + bn * KV + own + h * kV) : make_float4(0.f, 0.f, 0.f, 0.f);
     H[0][2 * h] = t4.x; H[0][2 * h + 1] = t4.y; H[1][2 * h] = t4.z; H[1][2 * h + 1] = t4.w;
   }
   auto store_state = [&](float *dst) {
 #pragma unroll
-    for (int h = 0; h < 2; ++h)
+    for (int h = 0; h < NH; ++h)
       *reinterpret_cast<float4 *>(dst + own + h * kV) = make_float4(H[0][2 * h], H[0][2 * h + 1], H[1][2 * h], H[1][2 * h + 1]);
   };
-  // this lane's eight bytes of rows row0 and row0 + 1 in a tile
-  const uint32_t hoff0 = tile16_off(2 * g, c >> 1) + 8u * (c & 1), hoff1 = tile16_off(2 * g + 1, c >> 1) + 8u * (c & 1);
+  // this lane's eight bytes of its rows in a slab's tile
+  const int slab = HALF ? warp >> 1 : warp, trow = HALF ? row0 & 15 : 2 * g;
+  const uint32_t hoff0 = tile16_off(trow, c >> 1) + 8u * (c & 1), hoff1 = tile16_off((trow + 1) & 15, c >> 1) + 8u * (c & 1);
   auto pack = [&](uint32_t (&A)[4]) {
 #pragma unroll
-    for (int nt = 0; nt < 2; ++nt) { A[2 * nt] = pack_bf16(H[nt][0], H[nt][1]); A[2 * nt + 1] = pack_bf16(H[nt][2], H[nt][3]); }
+    for (int nt = 0; nt < 2; ++nt) { A[2 * nt] = pack_bf16(H[nt][0], H[nt][1]); A[2 * nt + 1] = HALF ? 0u : pack_bf16(H[nt][2], H[nt][3]); }
   };
-  // P <- k v^T (the accumulators of a step).  k and v stay bf16 in shared memory: with three CTAs per SM its
-  // bandwidth binds.
+  // P <- k v^T (the accumulators of a step), straight from bf16
   auto seed = [&](float (&P)[2][4], uint32_t kp, uint32_t vp) {
     uint32_t kk, v0, v1;
-    asm volatile("ld.shared.b32 %0, [%1];" : "=r"(kk) : "r"(kp));
+    if constexpr (HALF) { uint16_t x; asm volatile("ld.shared.u16 %0, [%1];" : "=h"(x) : "r"(kp)); kk = x; }
+    else asm volatile("ld.shared.b32 %0, [%1];" : "=r"(kk) : "r"(kp));
     asm volatile("ld.shared.v2.b32 {%0,%1}, [%2];" : "=r"(v0), "=r"(v1) : "r"(vp));
-    const float k0 = __uint_as_float(kk << 16), k1 = __uint_as_float(kk & 0xffff0000u);
-    const float2 va = make_float2(__uint_as_float(v0 << 16), __uint_as_float(v0 & 0xffff0000u)), vb = make_float2(__uint_as_float(v1 << 16), __uint_as_float(v1 & 0xffff0000u));
-    const float2 p00 = __fmul2_rn(make_float2(k0, k0), va), p01 = __fmul2_rn(make_float2(k1, k1), va);
-    const float2 p10 = __fmul2_rn(make_float2(k0, k0), vb), p11 = __fmul2_rn(make_float2(k1, k1), vb);
-    P[0][0] = p00.x; P[0][1] = p00.y; P[0][2] = p01.x; P[0][3] = p01.y;
-    P[1][0] = p10.x; P[1][1] = p10.y; P[1][2] = p11.x; P[1][3] = p11.y;
+#pragma unroll
+    for (int nt = 0; nt < 2; ++nt) {
+      const uint32_t v = nt ? v1 : v0;
+      P[nt][0] = fma_bf16<0, 0>(kk, v, 0.f); P[nt][1] = fma_bf16<0, 1>(kk, v, 0.f);
+      if constexpr (HALF) { P[nt][2] = P[nt][3] = 0.f; }
+      else { P[nt][2] = fma_bf16<1, 0>(kk, v, 0.f); P[nt][3] = fma_bf16<1, 1>(kk, v, 0.f); }
+    }
   };
   // One step.  Pc: H_{t-1} W + k_t v_t^T; Pn: k_{t+1} v_{t+1}^T on entry, that plus H_t W on exit.
   auto step = [&](float (&Pc)[2][4], float (&Pn)[2][4], float f, uint32_t adst) {
@@ -248,7 +254,7 @@ __global__ void __launch_bounds__((NW + kSvc) * 32, OCC) fwd_v16_kernel(ScanArgs
 #pragma unroll
     for (int nt = 0; nt < 2; ++nt)
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
+      for (int h = 0; h < NH; ++h) {
         const float2 z = make_float2(tanh_approx(Pc[nt][2 * h]), tanh_approx(Pc[nt][2 * h + 1]));   // Eq. 1
         const float2 d = __ffma2_rn(z, m1, make_float2(H[nt][2 * h], H[nt][2 * h + 1]));            // H - Z
         const float2 hh = __ffma2_rn(f2, d, z);                                                     // Eq. 2
@@ -259,7 +265,7 @@ __global__ void __launch_bounds__((NW + kSvc) * 32, OCC) fwd_v16_kernel(ScanArgs
     mma_bf16_16816(Pn[0], A, Wr[0][0], Wr[0][1]);
     mma_bf16_16816(Pn[1], A, Wr[1][0], Wr[1][1]);
     asm volatile("st.shared.v2.b32 [%0], {%1,%2};" ::"r"(adst + hoff0), "r"(A[0]), "r"(A[2]) : "memory");
-    asm volatile("st.shared.v2.b32 [%0], {%1,%2};" ::"r"(adst + hoff1), "r"(A[1]), "r"(A[3]) : "memory");
+    if constexpr (!HALF) asm volatile("st.shared.v2.b32 [%0], {%1,%2};" ::"r"(adst + hoff1), "r"(A[1]), "r"(A[3]) : "memory");
   };
 
   float P0[2][4], P1[2][4];
@@ -275,7 +281,7 @@ __global__ void __launch_bounds__((NW + kSvc) * 32, OCC) fwd_v16_kernel(ScanArgs
       ck_left -= steps;
     }
   };
-  const uint32_t ok = Lay16::k(K) + 2u * (uint32_t)row0, ov = Lay16::v(K) + 8u * c, oa = Lay16::a() + 512u * (uint32_t)warp;
+  const uint32_t ok = Lay16::k(K) + 2u * (uint32_t)row0, ov = Lay16::v(K) + 8u * c, oa = Lay16::a() + 512u * (uint32_t)slab;
   constexpr uint32_t dk = 2u * K, dv = 2u * kV, da = 512u * NW;   // per step
   if (T > 0) {
     if (!mbar_wait(&full[0], 0)) { report_timeout(a.dev_status); return; }
@@ -331,14 +337,14 @@ __global__ void __launch_bounds__((NW + kSvc) * 32, OCC) fwd_v16_kernel(ScanArgs
   if (a.hT) store_state(a.hT + bn * KV);
 }
 
-template <int NW, bool CKPT, int OCC>
+template <int NW, bool CKPT, int OCC, bool HALF>
 cudaError_t launch_t(const ScanArgs &a, cudaStream_t s) {
   constexpr int kSvc = OCC > 1 ? 2 : 4;
   constexpr size_t smem = kBarBytes + (size_t)kStages * Lay16::bytes(16 * NW) + kTC * kV * 4;
-  const cudaError_t e = allow_smem(fwd_v16_kernel<NW, CKPT, OCC, kSvc>, smem);
+  const cudaError_t e = allow_smem(fwd_v16_kernel<NW, CKPT, OCC, kSvc, HALF>, smem);
   if (e != cudaSuccess) return e;
-  const int ctas = a.B * a.N * (a.K / (16 * NW)), threads = (NW + kSvc) * 32;
-  fwd_v16_kernel<NW, CKPT, OCC, kSvc><<<ctas, threads, smem, s>>>(in_order(a, ctas, threads, 1));
+  const int ctas = a.B * a.N * (a.K / (16 * NW)), threads = ((HALF ? 2 : 1) * NW + kSvc) * 32;
+  fwd_v16_kernel<NW, CKPT, OCC, kSvc, HALF><<<ctas, threads, smem, s>>>(in_order(a, ctas, threads, 1));
   return cudaGetLastError();
 }
 
@@ -348,10 +354,13 @@ cudaError_t launch_o(const ScanArgs &a, cudaStream_t s) {
   // the paper's layer shape (84 heads x batch 4) then take one wave instead of two
   const long ctas = (long)a.B * a.N * (a.K / (16 * NW)), sms = sm_count();
   if constexpr (NW <= 4) {
-    if (ctas > 2 * sms) return launch_t<NW, CKPT, 3>(a, s);
-    if (ctas > sms) return launch_t<NW, CKPT, 2>(a, s);
+    if (ctas > 2 * sms) return launch_t<NW, CKPT, 3, false>(a, s);
+    if (ctas > sms) return launch_t<NW, CKPT, 2, false>(a, s);
   }
-  return launch_t<NW, CKPT, 1>(a, s);
+  // Alone on an SM, up to four slabs run as twice as many warps of eight rows each: half of a step's MMAs is zeros, but a warp's step
+  // is its chain, and that is shorter by four tanh (1 024 steps, us: 16 heads of K = 64, a slab to an SM 94.9 -> 77.0, 84 heads, four
+  // to an SM 98 -> 94; two CTAs of 168 heads to an SM 129 -> 145).
+  return launch_t<NW, CKPT, 1, (NW <= 4)>(a, s);
 }
 
 }  // namespace

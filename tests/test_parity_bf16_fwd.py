@@ -166,3 +166,18 @@ def test_full_size_forward(oracle, name):
                                           g["W"][n:n + 1].contiguous(), start)
             assert parity.rel_err(yw, y_ref[:, s:e]) < 2e-2, (b, n, s)
             assert parity.rel_err(hw, Hs[:, :, e]) < 2e-2, (b, n, s)
+
+
+@pytest.mark.parametrize("K", [16, 32, 48, 64])
+def test_v16_half_slabs(oracle, K):
+    """V = 16: as many CTAs as have an SM each run warps of eight rows, twice as many units warps of sixteen: the same bits."""
+    cfg = ScanConfig("half", B=2, T=37, N=84, K=K, V=16, Nq=1, Nk=1, gate_mean=1.0, seed=60 + K)
+    d = inputs.make_inputs(cfg, residual=True)
+    g = parity.to_dev(d)
+    args = [g[x] for x in ("q", "k", "v", "gate", "W", "h0")]
+    two = binding.m2rnn_fwd(*args, w_r=g["w_r"], save_ckpt=True, ckpt_interval=8)
+    one = binding.m2rnn_fwd(*(x[:1] if i != 4 else x for i, x in enumerate(args)), w_r=g["w_r"], save_ckpt=True, ckpt_interval=8)
+    binding.check_device_status()
+    assert all(torch.equal(a, b[:1]) for a, b in zip(one, two))
+    y_ref, hT_ref = parity.oracle_fwd(oracle, cfg, d)
+    assert parity.rel_err(two[0], y_ref) <= parity.TOL["bf16"] and parity.rel_err(two[1], hT_ref) <= parity.TOL["bf16"]
