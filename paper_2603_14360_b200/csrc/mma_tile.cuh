@@ -58,6 +58,17 @@ template <int HA, int HB> __device__ __forceinline__ float fma_bf16(uint32_t a, 
   return d;
 }
 
+__device__ __forceinline__ float2 add_f16x2(uint32_t a, float2 c) {          // a + c
+  float2 d;
+  asm("{.reg .b16 p,q; mov.b32 {p,q}, %2; add.f32.f16 %0, p, %3; add.f32.f16 %1, q, %4;}" : "=f"(d.x), "=f"(d.y) : "r"(a), "f"(c.x), "f"(c.y));
+  return d;
+}
+__device__ __forceinline__ float2 square_f16x2(uint32_t a, float c) {        // a^2 + c
+  float2 d;
+  asm("{.reg .b16 p,q; mov.b32 {p,q}, %2; fma.rn.f32.f16 %0, p, p, %3; fma.rn.f32.f16 %1, q, q, %3;}" : "=f"(d.x), "=f"(d.y) : "r"(a), "f"(c));
+  return d;
+}
+
 template <int V>
 struct TileGeom {
   static constexpr int NT = V / 8;    // accumulator tiles per warp

@@ -13,9 +13,10 @@
 //                          dq = H_t dy and dk = dX v are small MMAs on fragments that are in
 //                          registers anyway (H_t is the H_{t-1} tile of the step handled just
 //                          before); dX is also left as a bf16 row-major tile;
-//   dW warps        (V/16) accumulate dW += H_{t-1}^T dX on tensor cores from the two tiles
-//                          (ldmatrix.trans operands), one 16-row slab of dW per warp, off the chain,
-//                          and take dv = dX^T k along as one more row of the same product;
+//   dW warps        (V/16) accumulate dW^T += dX^T H_{t-1} on tensor cores from the two tiles
+//                          (ldmatrix.trans operands), 16 columns of dW per warp, off the chain, and take dv = dX^T k
+//                          along with the same dX fragments (8 fewer MMAs and ldmatrix a step than as one more row of dW:
+//                          256 units of K = V = 64, 1 024 steps, 2 092 -> 2 042 us, K = 64, V = 32 754 -> 724);
 //   loader warp     (1)    stages q, k, v, dy and the gate of coming chunks;
 //   writer warp     (1)    reduces and writes dq, dk, dv, dgate of finished ones.
 //
@@ -124,6 +125,11 @@ __global__ void __launch_bounds__(bwd_threads<V, NWC>(), 1) bwd_bf16_kernel(Scan
   constexpr bool kWalk = !(V == 64 && NWC == 2);
   // packed fp32x2 element-wise arithmetic where it measured faster (elsewhere its register pairs spill)
   constexpr bool kPacked = V <= 32 || (V == 64 && NWC == 4);
+  // Z_t is kept as fp16, negated where the reverse warps take its sums and products straight from the 16-bit values (add.f32.f16,
+  // fma.f32.f16): two instructions an element fewer to unpack, one more each for what packed pairs did at once.  It pays up
+  // to two slabs a CTA (1 024 steps, us, with / without: K = V = 64, 32 units of 16-row CTAs 587 / 605; K = 48, V = 32 615 / 634), not with
+  // four, which are short of issue slots (256 units 2 084 / 2 045; K = 64, V = 32 734 / 724).
+  constexpr bool kMixZ = NWC < 4;
   constexpr int NSET = 1;   // accumulator sets of the state x W product, as in the forward kernel
   // Who computes dq = H_t dy and dk = dX v (small MMAs): the dW warps from the tiles, where they have
   // the time (more dW warps than row slabs: sweep64 backward 7.13 -> 5.76 ms, sweep32 2.65 -> 2.43),
@@ -371,8 +377,8 @@ __global__ void __launch_bounds__(bwd_threads<V, NWC>(), 1) bwd_bf16_kernel(Scan
                 H[nt][r] = fmaf(f, H[nt][r] - z[r], z[r]);
               }
             }
-            zw[2 * u] = pack_f16(z[0], z[1]);
-            zw[2 * u + 1] = pack_f16(z[2], z[3]);
+            zw[2 * u] = kMixZ ? pack_f16(-z[0], -z[1]) : pack_f16(z[0], z[1]);
+            zw[2 * u + 1] = kMixZ ? pack_f16(-z[2], -z[3]) : pack_f16(z[2], z[3]);
           }
           asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(zs + 512u * x), "r"(zw[0]), "r"(zw[1]), "r"(zw[2]), "r"(zw[3]) : "memory");
         }
@@ -506,32 +512,37 @@ __global__ void __launch_bounds__(bwd_threads<V, NWC>(), 1) bwd_bf16_kernel(Scan
 #pragma unroll
           for (int u = 0; u < 2; ++u) {
             const int nt = 2 * x + u;
-            const float2 za = unpack_f16(zw[2 * u]), zb = unpack_f16(zw[2 * u + 1]);
-            const float2 ha = unpack_bf16(hp[nt][0]), hb = unpack_bf16(hp[nt][1]);
-            const float z[4] = {za.x, za.y, zb.x, zb.y}, hprev[4] = {ha.x, ha.y, hb.x, hb.y};
             float dX[4];
-            if constexpr (kPacked) {
-              const float2 dy2 = make_float2(dyv[2 * u], dyv[2 * u + 1]);
 #pragma unroll
-              for (int h = 0; h < 2; ++h) {
-                const float2 z2 = make_float2(z[2 * h], z[2 * h + 1]), hp2 = make_float2(hprev[2 * h], hprev[2 * h + 1]);
+            for (int h = 0; h < 2; ++h) {
+              float2 d2, e2;       // H_{t-1} - Z, Z^2 - 1
+              if constexpr (kMixZ) {
+                d2 = add_f16x2(zw[2 * u + h], unpack_bf16(hp[nt][h]));
+                e2 = square_f16x2(zw[2 * u + h], -1.f);
+              } else {
+                const float2 z2 = unpack_f16(zw[2 * u + h]);
+                d2 = __ffma2_rn(z2, make_float2(-1.f, -1.f), unpack_bf16(hp[nt][h]));
+                e2 = __ffma2_rn(z2, z2, make_float2(-1.f, -1.f));
+              }
+              if constexpr (kPacked) {
+                const float2 dy2 = make_float2(dyv[2 * u], dyv[2 * u + 1]);
                 const float qh = h ? q1 : q0;
                 const float2 G2 = __ffma2_rn(make_float2(qh, qh), dy2, make_float2(Cg[nt][2 * h], Cg[nt][2 * h + 1]));   // G = C + q dy^T
-                df2 = __ffma2_rn(G2, __ffma2_rn(z2, make_float2(-1.f, -1.f), hp2), df2);                                    // df = sum G (.) (H_{t-1} - Z)
-                const float2 x2 = __fmul2_rn(__fmul2_rn(make_float2(-omf, -omf), G2), __ffma2_rn(z2, z2, make_float2(-1.f, -1.f)));   // (1-f) G (1 - Z^2)
-                const float2 c2 = __fmul2_rn(make_float2(f, f), G2);                                                        // gated path into H_{t-1}
+                df2 = __ffma2_rn(G2, d2, df2);                                               // df = sum G (.) (H_{t-1} - Z)
+                const float2 x2 = __fmul2_rn(__fmul2_rn(make_float2(-omf, -omf), G2), e2);   // (1-f) G (1 - Z^2)
+                const float2 c2 = __fmul2_rn(make_float2(f, f), G2);                         // gated path into H_{t-1}
                 dX[2 * h] = x2.x; dX[2 * h + 1] = x2.y;
                 Cg[nt][2 * h] = c2.x; Cg[nt][2 * h + 1] = c2.y;
-              }
-            } else {
+              } else {
+                const float dd[2] = {d2.x, d2.y}, ee[2] = {e2.x, e2.y};
 #pragma unroll
-              for (int r = 0; r < 4; ++r) {
-                const float dyc = dyv[2 * u + (r & 1)];
-                const float qr = (r & 2) ? q1 : q0;
-                const float Gv = fmaf(qr, dyc, Cg[nt][r]);        // G = C + q dy^T
-                df = fmaf(Gv, hprev[r] - z[r], df);               // df = sum G (.) (H_{t-1} - Z)
-                dX[r] = omf * Gv * fmaf(-z[r], z[r], 1.f);        // through the gate and tanh
-                Cg[nt][r] = f * Gv;                               // gated path into H_{t-1}
+                for (int y = 0; y < 2; ++y) {
+                  const int r = 2 * h + y;
+                  const float Gv = fmaf(h ? q1 : q0, dyv[2 * u + y], Cg[nt][r]);     // G = C + q dy^T
+                  df = fmaf(Gv, dd[y], df);                                          // df = sum G (.) (H_{t-1} - Z)
+                  dX[r] = -omf * Gv * ee[y];                                         // through the gate and tanh
+                  Cg[nt][r] = f * Gv;                                                // gated path into H_{t-1}
+                }
               }
             }
             xp[nt][0] = pack_bf16(dX[0], dX[1]);
@@ -623,7 +634,8 @@ __global__ void __launch_bounds__(bwd_threads<V, NWC>(), 1) bwd_bf16_kernel(Scan
 
   if (warp < 2 * NWC + NDW) {
     // ================================================================= dW warps
-    // warp d owns dW rows l in [16d, 16d+16): acc += H_{t-1}[:, l]^T dX, contraction over the CTA's rows
+    // warp d owns dW columns j in [16d, 16d+16): acc += dX[:, j]^T H_{t-1}, contraction over the CTA's rows.  The dX fragments of a
+    // step are read once, for this product and for dv = dX^T k; the tile is free for the reverse warps after that.
     if constexpr (kRebalance) { if constexpr (V == 64) reg_dec<72>(); else reg_dec<104>(); }
     const int d = warp - 2 * NWC;
     float acc[NT][4];
@@ -634,10 +646,9 @@ __global__ void __launch_bounds__(bwd_threads<V, NWC>(), 1) bwd_bf16_kernel(Scan
     // 32 V bytes per kt, added as an immediate): rows of 128 bytes or more keep their chunk swizzle
     // (row & 7 = mr) when 16 rows are added, so the offsets are worked out once.
     constexpr bool kPreOff = kWalk && 2 * V >= 128;
-    uint32_t offA = 0, offDv = 0, offB[NT / 2];
+    uint32_t offA = 0, offB[NT / 2];
     if constexpr (kPreOff) {
       offA = tile_off<V>(mr + 8 * (mi >> 1), 2 * d + (mi & 1));
-      offDv = tile_off<V>(mr + 8 * (mi & 1), 2 * d + (mi >> 1));
 #pragma unroll
       for (int np = 0; np < NT / 2; ++np) offB[np] = tile_off<V>(mr + 8 * (mi & 1), 2 * np + (mi >> 1));
     }
@@ -649,44 +660,40 @@ __global__ void __launch_bounds__(bwd_threads<V, NWC>(), 1) bwd_bf16_kernel(Scan
         const int xb = nstep & 1;
         if (!mbar_wait(&dx_full[xb], (nstep >> 1) & 1)) { report_timeout(a.dev_status); return; }
         const uint32_t ht = state_sa(j, s), xt = sm0 + L.dx + (uint32_t)xb * (KC * V * 2);
-        // dv = dX^T k (Algorithm 2, value-gradient line) rides along as one more row of the product:
-        // an A tile whose row 0 is k and whose other rows are zero; this warp takes columns 16d..16d+15
-        float dvacc[2][4];
-#pragma unroll
-        for (int u = 0; u < 2; ++u) dvacc[u][0] = dvacc[u][1] = dvacc[u][2] = dvacc[u][3] = 0.f;
+        float dvacc[4] = {0.f, 0.f, 0.f, 0.f};     // dv = dX^T k (Algorithm 2, value-gradient line): every column of the product
         const uint32_t kb = slot_sa(j) + 4u * (L.oKB + s * (KC / 2));
+        // A = dX^T: matrices (i 0-7, j 0-7), (i 0-7, j 8-15), (i 8-15, j 0-7), (i 8-15, j 8-15)
+        uint32_t A[NWC][4];
 #pragma unroll
         for (int kt = 0; kt < NWC; ++kt) {
-          // A = H_{t-1}^T: matrices (i 0-7, l 0-7), (i 0-7, l 8-15), (i 8-15, l 0-7), (i 8-15, l 8-15)
-          uint32_t A[4];
-          if constexpr (kPreOff) ldmatrix_x4_trans(ht + offA + (uint32_t)(kt * 32 * V), A[0], A[1], A[2], A[3]);
-          else ldmatrix_x4_trans(ht + tile_off<V>(16 * kt + mr + 8 * (mi >> 1), 2 * d + (mi & 1)), A[0], A[1], A[2], A[3]);
+          if constexpr (kPreOff) ldmatrix_x4_trans(xt + offA + (uint32_t)(kt * 32 * V), A[kt][0], A[kt][1], A[kt][2], A[kt][3]);
+          else ldmatrix_x4_trans(xt + tile_off<V>(16 * kt + mr + 8 * (mi >> 1), 2 * d + (mi & 1)), A[kt][0], A[kt][1], A[kt][2], A[kt][3]);
+        }
+        auto dx_done = [&]() {
+          __syncwarp();
+          if (lane == 0) asm volatile("red.release.cta.shared.add.u32 [%0], 1;" ::"r"(smem_u32(dx_read)) : "memory");
+        };
+        if constexpr (!kDkDw) dx_done();
+#pragma unroll
+        for (int kt = 0; kt < NWC; ++kt) {
 #pragma unroll
           for (int np = 0; np < NT / 2; ++np) {
-            // B = dX: matrices (i 0-7, j-tile 2np), (i 8-15, 2np), (i 0-7, 2np+1), (i 8-15, 2np+1)
+            // B = H_{t-1}: matrices (i 0-7, l-tile 2np), (i 8-15, 2np), (i 0-7, 2np+1), (i 8-15, 2np+1)
             uint32_t b0, b1, b2, b3;
-            if constexpr (kPreOff) ldmatrix_x4_trans(xt + offB[np] + (uint32_t)(kt * 32 * V), b0, b1, b2, b3);
-            else ldmatrix_x4_trans(xt + tile_off<V>(16 * kt + mr + 8 * (mi & 1), 2 * np + (mi >> 1)), b0, b1, b2, b3);
-            mma_bf16_16816(acc[2 * np], A, b0, b1);
-            mma_bf16_16816(acc[2 * np + 1], A, b2, b3);
+            if constexpr (kPreOff) ldmatrix_x4_trans(ht + offB[np] + (uint32_t)(kt * 32 * V), b0, b1, b2, b3);
+            else ldmatrix_x4_trans(ht + tile_off<V>(16 * kt + mr + 8 * (mi & 1), 2 * np + (mi >> 1)), b0, b1, b2, b3);
+            mma_bf16_16816(acc[2 * np], A[kt], b0, b1);
+            mma_bf16_16816(acc[2 * np + 1], A[kt], b2, b3);
           }
+          uint32_t k0, k1;
+          asm volatile("ld.shared.b32 %0, [%1];" : "=r"(k0) : "r"(kb + 4u * (8 * kt + c)));
+          asm volatile("ld.shared.b32 %0, [%1];" : "=r"(k1) : "r"(kb + 4u * (8 * kt + 4 + c)));
+          mma_bf16_16816(dvacc, A[kt], k0, k1);
         }
-#pragma unroll
-        for (int kt = 0; kt < NWC; ++kt) {
-          uint32_t Ak[4] = {0u, 0u, 0u, 0u}, b0, b1, b2, b3;
-          if (g == 0) {
-            asm volatile("ld.shared.b32 %0, [%1];" : "=r"(Ak[0]) : "r"(kb + 4u * (8 * kt + c)));
-            asm volatile("ld.shared.b32 %0, [%1];" : "=r"(Ak[2]) : "r"(kb + 4u * (8 * kt + 4 + c)));
-          }
-          if constexpr (kPreOff) ldmatrix_x4_trans(xt + offDv + (uint32_t)(kt * 32 * V), b0, b1, b2, b3);
-          else ldmatrix_x4_trans(xt + tile_off<V>(16 * kt + mr + 8 * (mi & 1), 2 * d + (mi >> 1)), b0, b1, b2, b3);
-          mma_bf16_16816(dvacc[0], Ak, b0, b1);
-          mma_bf16_16816(dvacc[1], Ak, b2, b3);
-        }
-        if (g == 0) {
-          const uint32_t dst = slot_sa(j) + 4u * (L.oDV + s * V + 16 * d + 2 * c);
-          sts64(dst, make_float2(dvacc[0][0], dvacc[0][1]));
-          sts64(dst + 32u, make_float2(dvacc[1][0], dvacc[1][1]));
+        if (c == 0) {
+          const uint32_t dst = slot_sa(j) + 4u * (L.oDV + s * V + 16 * d + g);
+          sts32(dst, dvacc[0]);
+          sts32(dst + 32u, dvacc[2]);
         }
         // dq = H_t dy and dk = dX v (Algorithm 2, query- and key-gradient lines) for the 16-row
         // slabs this warp takes in turn: A fragments by ldmatrix from the H_t tile (the H_{t-1} tile
@@ -725,18 +732,20 @@ __global__ void __launch_bounds__(bwd_threads<V, NWC>(), 1) bwd_bf16_kernel(Scan
             }
           }
         }
-        __syncwarp();
-        if (lane == 0) asm volatile("red.release.cta.shared.add.u32 [%0], 1;" ::"r"(smem_u32(dx_read)) : "memory");
+        if constexpr (kDkDw) dx_done();
       }
       __syncwarp();
       if (lane == 0) { mbar_arrive(&st_free[j & 1]); mbar_arrive(&out_full[j & (kRing - 1)]); }
     }
     float *dWp = a.dW_part + ((size_t)(b * RS + rs) * N + n) * V * V;   // one partial per CTA, [b][slab][n]
 #pragma unroll
-    for (int nt = 0; nt < NT; ++nt) {
-      *reinterpret_cast<float2 *>(dWp + (size_t)(16 * d + g) * V + 8 * nt + 2 * c) = make_float2(acc[nt][0], acc[nt][1]);
-      *reinterpret_cast<float2 *>(dWp + (size_t)(16 * d + g + 8) * V + 8 * nt + 2 * c) = make_float2(acc[nt][2], acc[nt][3]);
-    }
+    for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {      // row l = 8 nt + 2c + e, columns j = 16 d + g and + 8
+        float *dst = dWp + (size_t)(8 * nt + 2 * c + e) * V + 16 * d + g;
+        dst[0] = acc[nt][e];
+        dst[8] = acc[nt][2 + e];
+      }
     return;
   }
 

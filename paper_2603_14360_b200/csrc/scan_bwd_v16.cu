@@ -90,17 +90,6 @@ __device__ __forceinline__ uint32_t transposed(uint32_t x) {   // an 8 x 8 matri
   asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(y) : "r"(x));
   return y;
 }
-__device__ __forceinline__ float2 add_f16x2(uint32_t a, float2 c) {          // a + c
-  float2 d;
-  asm("{.reg .b16 p,q; mov.b32 {p,q}, %2; add.f32.f16 %0, p, %3; add.f32.f16 %1, q, %4;}" : "=f"(d.x), "=f"(d.y) : "r"(a), "f"(c.x), "f"(c.y));
-  return d;
-}
-__device__ __forceinline__ float2 square_f16x2(uint32_t a, float c) {        // a^2 + c
-  float2 d;
-  asm("{.reg .b16 p,q; mov.b32 {p,q}, %2; fma.rn.f32.f16 %0, p, p, %3; fma.rn.f32.f16 %1, q, q, %3;}" : "=f"(d.x), "=f"(d.y) : "r"(a), "f"(c));
-  return d;
-}
-
 template <int CC, bool CLIP>
 __global__ void __launch_bounds__((kMostSlabs + 2) * 32, 1) bwd_v16_kernel(ScanArgs a) {
   using L = Lay<CC>;
