@@ -70,11 +70,11 @@ struct TcBwdSmem {
   // [2] x { C step blocks (slab + Z), one more slab: the state after the chunk's last step }
   static constexpr uint32_t buf_bytes = kCTc * kStepBytes + kTileBytes, state_bytes = 2u * buf_bytes;
   static constexpr uint32_t oDx = oState + state_bytes, oRing = oDx + 2 * kTileBytes;
-  // words of a ring slot.  In: q, k [C][32] as fp32, f and its slope [C], v and dy [C][128] as the
-  // raw bf16 (a chain thread widens its own element; the helper products take them as pairs).
+  // words of a ring slot.  In: q, k [C][32] and v, dy [C][128] as the raw bf16 (products with an fp32 sum take
+  // them as they are, the helper products as pairs), f and its slope [C].
   // Out: the helpers' shares of dq and dk [C][4][32], dv per row group [C][4][128], one df partial
   // per chain warp [C][16].
-  static constexpr uint32_t oQ = 0, oK = oQ + kCTc * kNR, oF = oK + kCTc * kNR, oDF = oF + 4, oDYB = oDF + 4,
+  static constexpr uint32_t oQ = 0, oK = oQ + kCTc * kNR / 2, oF = oK + kCTc * kNR / 2, oDF = oF + 4, oDYB = oDF + 4,
                             oVB = oDYB + kCTc * kV / 2, oDQ = oVB + kCTc * kV / 2, oDK = oDQ + kCTc * kHelpWarps * kNR,
                             oDV = oDK + kCTc * kHelpWarps * kNR, oDFP = oDV + kCTc * kRowGroups * kV,
                             slot_words = oDFP + kCTc * kChainWarps;
@@ -103,6 +103,7 @@ __device__ __forceinline__ float2 unpack_f16x2(uint32_t x) { return __half22floa
 
 __global__ void __launch_bounds__(kThreads, 1) bwd_tc_kernel(ScanArgs a) {
   using S = TcBwdSmem;
+  constexpr int CT = kCTc;
   constexpr int V = kV;
   const int C = a.C;                 // steps per chunk (<= kCTc, which sizes the buffers)
   extern __shared__ __align__(16) unsigned char smem_dyn[];
@@ -254,9 +255,9 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_tc_kernel(ScanArgs a) {
         if (!mbar_wait(&in_full[it & (kRingTc - 1)], (it / kRingTc) & 1)) { failed = true; break; }
         if (it >= 2 && !mbar_wait(&st_free[it & 1], ((it >> 1) - 1) & 1)) { failed = true; break; }
       }
-      for (int x = 0; x < C; ++x) {
-        const bool rec_on = x < lenR, rev_on = x < lenV;
-        const int sv = lenV - 1 - x;                      // the reverse sweep's step inside its chunk
+      // step x of the chunk's recomputation, step sv of the other's sweep; false: a wait ran out
+      // df: this thread's share of the sweep's step
+      auto step = [&](int x, int sv, bool rec_on, bool rev_on, float &df) -> bool {
         const uint32_t blkR = step_sa(it, x), blkV = step_sa(it - 1, sv);
         // ---- recompute: H_{t-1} -> slab (this step's B operand, and what dW and dq read later)
         if (rec_on) { store_slab(blkR, H); slab_done(rec_slab); ++nrec; }
@@ -266,25 +267,21 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_tc_kernel(ScanArgs a) {
         if (rev_on) {
           const uint4 z0 = *reinterpret_cast<const uint4 *>(base + (blkV - base_sa) + priv);
           const uint32_t zw[kNT / 2] = {z0.x, z0.y, z0.z, z0.w};
-          const float dyj = __uint_as_float((uint32_t)reinterpret_cast<const uint16_t *>(sfV + S::oDYB)[sv * V + j] << 16);
+          const uint32_t dyj = reinterpret_cast<const uint16_t *>(sfV + S::oDYB)[sv * V + j];
           const float f = sfV[S::oF + sv], omf = 1.f - f;
           uint32_t hw[kNT / 2];   // H_{t-1}, this thread's own chunk of the slab it wrote a chunk ago
           asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(hw[0]), "=r"(hw[1]), "=r"(hw[2]), "=r"(hw[3]) : "r"(blkV + own));
-          if (pending && !absorb()) { failed = true; break; }
+          if (pending && !absorb()) return false;
           float dX[kNT];
           float2 df2 = make_float2(0.f, 0.f), dv2 = make_float2(0.f, 0.f);
-          float q8[kNT], k8[kNT];
-#pragma unroll
-          for (int r = 0; r < kNT; r += 4) {
-            *reinterpret_cast<float4 *>(q8 + r) = *reinterpret_cast<const float4 *>(sfV + S::oQ + sv * kNR + i0 + r);
-            *reinterpret_cast<float4 *>(k8 + r) = *reinterpret_cast<const float4 *>(sfV + S::oK + sv * kNR + i0 + r);
-          }
+          const uint4 qw = *reinterpret_cast<const uint4 *>(sfV + S::oQ + (sv * kNR + i0) / 2), kw = *reinterpret_cast<const uint4 *>(sfV + S::oK + (sv * kNR + i0) / 2);
+          const uint32_t q8[kNT / 2] = {qw.x, qw.y, qw.z, qw.w}, k8[kNT / 2] = {kw.x, kw.y, kw.z, kw.w};
 #pragma unroll
           for (int r = 0; r < kNT; r += 2) {
-            const float2 qq = make_float2(q8[r], q8[r + 1]), kk = make_float2(k8[r], k8[r + 1]);
+            const float2 kk = make_float2(__uint_as_float(k8[r / 2] << 16), __uint_as_float(k8[r / 2] & 0xffff0000u));
             const float2 hp = make_float2(__uint_as_float(hw[r / 2] << 16), __uint_as_float(hw[r / 2] & 0xffff0000u));
             const float2 z = unpack_f16x2(zw[r / 2]);
-            const float2 G = __ffma2_rn(qq, make_float2(dyj, dyj), make_float2(Cg[r], Cg[r + 1]));                             // G = C + q dy^T
+            const float2 G = make_float2(fma_bf16<0, 0>(q8[r / 2], dyj, Cg[r]), fma_bf16<1, 0>(q8[r / 2], dyj, Cg[r + 1]));                       // G = C + q dy^T
             df2 = __ffma2_rn(G, __ffma2_rn(z, make_float2(-1.f, -1.f), hp), df2);                                          // df = sum G (.) (H_{t-1} - Z)
             const float2 x2 = __fmul2_rn(__fmul2_rn(make_float2(-omf, -omf), G), __ffma2_rn(z, z, make_float2(-1.f, -1.f)));   // (1-f) G (1 - Z^2)
             const float2 c2 = __fmul2_rn(make_float2(f, f), G);                                                            // gated path into H_{t-1}
@@ -292,12 +289,8 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_tc_kernel(ScanArgs a) {
             dX[r] = x2.x; dX[r + 1] = x2.y;
             Cg[r] = c2.x; Cg[r + 1] = c2.y;
           }
-          // df: summed over the warp here, over the warps by the writer; dv: one share per row group,
-          // added by the writer
-          float df = df2.x + df2.y;
-#pragma unroll
-          for (int off = 16; off > 0; off >>= 1) df += __shfl_xor_sync(0xffffffffu, df, off);
-          if (lane == 0) sfV[S::oDFP + sv * kChainWarps + warp] = df;
+          // dv: one share per row group, added by the writer
+          df = df2.x + df2.y;
           sfV[S::oDV + (sv * kRowGroups + rg) * V + j] = dv2.x + dv2.y;
           // (the buffer is free: the MMA warp issued the previous step's product, whose result was
           // added above, only after the helpers and the dW product were through with it)
@@ -309,19 +302,18 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_tc_kernel(ScanArgs a) {
         }
         // ---- recompute epilogue, while the reverse product is in the tensor core
         if (rec_on) {
-          const float vj = __uint_as_float((uint32_t)reinterpret_cast<const uint16_t *>(sfR + S::oVB)[x * V + j] << 16), f = sfR[S::oF + x];
-          if (!mbar_wait(rec_done, (nrec - 1u) & 1u)) { failed = true; break; }
+          const uint32_t vj = reinterpret_cast<const uint16_t *>(sfR + S::oVB)[x * V + j];
+          const float f = sfR[S::oF + x];
+          if (!mbar_wait(rec_done, (nrec - 1u) & 1u)) return false;
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           float P[kNT];
           tmem_ld(lane_tm + kColP, P);
           uint32_t zw[kNT / 2];
-          float k8[kNT];
-#pragma unroll
-          for (int r = 0; r < kNT; r += 4) *reinterpret_cast<float4 *>(k8 + r) = *reinterpret_cast<const float4 *>(sfR + S::oK + x * kNR + i0 + r);
+          const uint4 kw = *reinterpret_cast<const uint4 *>(sfR + S::oK + (x * kNR + i0) / 2);
+          const uint32_t k8[kNT / 2] = {kw.x, kw.y, kw.z, kw.w};
 #pragma unroll
           for (int r = 0; r < kNT; r += 2) {
-            const float2 kk = make_float2(k8[r], k8[r + 1]);
-            const float2 pre = __ffma2_rn(kk, make_float2(vj, vj), make_float2(P[r], P[r + 1]));
+            const float2 pre = make_float2(fma_bf16<0, 0>(k8[r / 2], vj, P[r]), fma_bf16<1, 0>(k8[r / 2], vj, P[r + 1]));
             const float2 z = make_float2(tanh_approx(pre.x), tanh_approx(pre.y));                            // Eq. 1
             const float2 d = __ffma2_rn(z, make_float2(-1.f, -1.f), make_float2(H[r], H[r + 1]));             // H_{t-1} - Z
             const float2 h = __ffma2_rn(make_float2(f, f), d, z);                                           // Eq. 2
@@ -329,6 +321,43 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_tc_kernel(ScanArgs a) {
             zw[r / 2] = pack_f16x2(z.x, z.y);
           }
           *reinterpret_cast<uint4 *>(base + (blkR - base_sa) + priv) = make_uint4(zw[0], zw[1], zw[2], zw[3]);
+        }
+        return true;
+      };
+      // df is summed over the warp here, over the warps by the writer.  Whole chunks unrolled: their places are constants (32
+      // units of K = V = 128, 1 024 steps: 1 210 -> 1 155 us), and the four steps' sums share their shuffles (-> 1 129;
+      // q, k, v, dy straight from bf16, fma.f32.bf16: -> 1 122).
+      if (lenR == CT && lenV == CT) {
+        float df[CT];
+#pragma unroll
+        for (int x = 0; x < CT; ++x) {
+          df[x] = 0.f;
+          if (!failed) failed = !step(x, CT - 1 - x, true, true, df[x]);
+        }
+        static_assert(CT == 4, "lane bits 16 and 8 pick the step");
+#pragma unroll
+        for (int m = 2, bit = 16; m >= 1; m >>= 1, bit >>= 1) {
+          const bool up = lane & bit;
+#pragma unroll
+          for (int x = 0; x < m; ++x) {
+            const float send = up ? df[x] : df[x + m], keep = up ? df[x + m] : df[x];
+            df[x] = keep + __shfl_xor_sync(0xffffffffu, send, bit);
+          }
+        }
+#pragma unroll
+        for (int off = 4; off > 0; off >>= 1) df[0] += __shfl_xor_sync(0xffffffffu, df[0], off);
+        if ((lane & 7) == 0) sfV[S::oDFP + (CT - 1 - (lane >> 3)) * kChainWarps + warp] = df[0];
+      } else {
+#pragma unroll 1
+        for (int x = 0; x < C && !failed; ++x) {
+          const int sv = lenV - 1 - x;
+          float df = 0.f;
+          failed = !step(x, sv, x < lenR, x < lenV, df);
+          if (x < lenV) {
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) df += __shfl_xor_sync(0xffffffffu, df, off);
+            if (lane == 0) sfV[S::oDFP + sv * kChainWarps + warp] = df;
+          }
         }
       }
       if (failed) break;
@@ -489,8 +518,8 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_tc_kernel(ScanArgs a) {
           const int t = lane >> 2, i = (lane & 3) * 8;
           const uint4 qr = *reinterpret_cast<const uint4 *>(qg + (bt0 + t) * a.qs + (size_t)hq * K + rbase + i);
           const uint4 kr = *reinterpret_cast<const uint4 *>(kg + (bt0 + t) * a.ks + (size_t)hk * K + rbase + i);
-          store8_bf16_as_f32(sf + S::oQ + t * kNR + i, qr);
-          store8_bf16_as_f32(sf + S::oK + t * kNR + i, kr);
+          *reinterpret_cast<uint4 *>(sf + S::oQ + (t * kNR + i) / 2) = qr;
+          *reinterpret_cast<uint4 *>(sf + S::oK + (t * kNR + i) / 2) = kr;
         }
         for (int x = lane; x < 16 * len; x += 32) {
           const int t = x >> 4, i = (x & 15) * 8;
