@@ -130,6 +130,9 @@ __global__ void __launch_bounds__(bwd_threads<V, NWC>(), 1) bwd_bf16_kernel(Scan
   // to two slabs a CTA (1 024 steps, us, with / without: K = V = 64, 32 units of 16-row CTAs 587 / 605; K = 48, V = 32 615 / 634), not with
   // four, which are short of issue slots (256 units 2 084 / 2 045; K = 64, V = 32 734 / 724).
   constexpr bool kMixZ = NWC < 4;
+  // (two steps of a sweep unrolled: 64 units of K = V = 32, 1 024 steps, 309 -> 300 us, 320 of K = 64, V = 32 725 -> 713; elsewhere nothing,
+  // or the registers are not there: K = V = 64, one slab 585 -> 636)
+  constexpr int kUnrollRev = V == 32 && NWC == 4 ? 2 : 1, kUnrollDw = V == 32 || (V == 64 && NWC == 2) ? 2 : 1;
   constexpr int NSET = 1;   // accumulator sets of the state x W product, as in the forward kernel
   // Who computes dq = H_t dy and dk = dX v (small MMAs): the dW warps from the tiles, where they have
   // the time (more dW warps than row slabs: sweep64 backward 7.13 -> 5.76 ms, sweep32 2.65 -> 2.43),
@@ -471,6 +474,7 @@ __global__ void __launch_bounds__(bwd_threads<V, NWC>(), 1) bwd_bf16_kernel(Scan
                     sl + 4u * (L.oDFP + (s * NWC + w) * 32 + lane), sl + 4u * (L.oDQ + s * KC + r0), sl + 4u * (L.oDK + s * KC + r0)};
       };
       Ptrs run = ptrs_at(len - 1);
+#pragma unroll (kUnrollRev)
       for (int s = len - 1; s >= 0; --s, ++nstep) {
         const uint32_t st = kWalk ? run.st : state_sa(j, s);
 #define pF (kWalk ? run.f : sl + 4u * (L.oF + s))
@@ -656,6 +660,7 @@ __global__ void __launch_bounds__(bwd_threads<V, NWC>(), 1) bwd_bf16_kernel(Scan
     for (int j = 0; j < nch; ++j) {
       const int len = chunk_len(j);
       if (!mbar_wait(&st_ready[j & 1], (j >> 1) & 1)) { report_timeout(a.dev_status); return; }
+#pragma unroll (kUnrollDw)
       for (int s = len - 1; s >= 0; --s, ++nstep) {
         const int xb = nstep & 1;
         if (!mbar_wait(&dx_full[xb], (nstep >> 1) & 1)) { report_timeout(a.dev_status); return; }
