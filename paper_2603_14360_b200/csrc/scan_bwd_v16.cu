@@ -53,6 +53,7 @@ struct Lay {
   __host__ __device__ static uint32_t total(int hg, int qb, int kb, int slabs) { return warp(hg, qb, kb, slabs) + (uint32_t)slabs * kWarp; }
 };
 constexpr int kMostSlabs = 10;   // slab warps of a CTA
+constexpr int kRoomWarps = 14;   // warps of an SM with the kernel's registers
 
 __device__ __forceinline__ uint32_t pack_f16(float lo, float hi) {
   uint32_t r;
@@ -90,8 +91,9 @@ __device__ __forceinline__ uint32_t transposed(uint32_t x) {   // an 8 x 8 matri
   asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(y) : "r"(x));
   return y;
 }
+// (bounds for two warps more than a CTA has: 144 registers, which the plan counts with)
 template <int CC, bool CLIP>
-__global__ void __launch_bounds__((kMostSlabs + 2) * 32, 1) bwd_v16_kernel(ScanArgs a) {
+__global__ void __launch_bounds__(kRoomWarps * 32, 1) bwd_v16_kernel(ScanArgs a) {
   using L = Lay<CC>;
   extern __shared__ __align__(128) unsigned char smem[];
   const int K = a.K, N = a.N, C = a.C;
@@ -579,11 +581,11 @@ BwdPlan plan_bwd_v16(int B, int N, int Nq, int Nk, int K, int T, int interval, b
         const long ctas = (long)(B > 0 ? B : 1) * groups * (K / (16 * R));
         const size_t smem = (C <= 8 ? Lay<8>::total(hg, qb, kb, slabs) : Lay<16>::total(hg, qb, kb, slabs)) + 1024;
         constexpr size_t kSm = 228 * 1024;
-        const long by_regs = 65536 / (144 * 32) / (slabs + 2), by_smem = (long)(kSm / smem), room = by_regs < by_smem ? by_regs : by_smem;
+        const long by_regs = kRoomWarps / (slabs + 2), by_smem = (long)(kSm / smem), room = by_regs < by_smem ? by_regs : by_smem;
         if (room < 1 || smem - 1024 > 227 * 1024) continue;
         auto step = [&](long n) {     // of an SM with n CTAs
           const long s = n * slabs;
-          return n ? 155. + 100. * ((s + 3) / 4) + 4. * s + (C <= 8 ? 20. : 0.) + (own_rows && s > 4 ? 12. * (s - 4) / n : 0.) : 0.;
+          return n ? 155. + 100. * ((s + 3) / 4) + 4. * s + (C <= 8 ? 20. : 0.) + (own_rows ? 12. * (s > 4 ? s - 4 : 0) + 4. * (slabs - 1) : 0.) : 0.;
         };
         const long waves = ctas / (sms * room), left = ctas % (sms * room);
         const int RS = K / (16 * R);
