@@ -104,6 +104,7 @@ __global__ void __launch_bounds__(kConvThreads, kOccFwd) conv_silu_fwd_kernel(in
                                                                      const T *__restrict__ w, const T *__restrict__ bias,
                                                                      const T *__restrict__ prev, T *__restrict__ out, long long os) {
   constexpr int CH = Chunk<T>::CH;
+  begin_dependent();
   const int cc = blockIdx.x * kLanes + (threadIdx.x % kLanes), sub = threadIdx.x / kLanes;
   if (cc * CH >= C) return;
   constexpr int kTile = kSub * STEPS;
@@ -187,6 +188,7 @@ __global__ void __launch_bounds__(kConvThreads, sizeof(T) == 2 ? kOccBwd : 1) co
                                                                      T *__restrict__ dx, long long dxs, T *__restrict__ dprev,
                                                                      float *__restrict__ part) {
   constexpr int CH = Chunk<T>::CH;
+  begin_dependent();
   __shared__ float red[kSub - 1][5 * CH][kLanes];    // the sub-tiles' sums, added by sub-tile 0
   const int lane = threadIdx.x % kLanes, sub = threadIdx.x / kLanes;
   const int cc = blockIdx.x * kLanes + lane;
@@ -350,6 +352,7 @@ __global__ void __launch_bounds__(kConvThreads, sizeof(T) == 2 ? kOccBwd : 1) co
 // dw[c][s] = sum over tiles of part[tile][s][c]; dbias[c] likewise from row 4.  Eight lanes share an
 // output: each sums every eighth tile, then a shuffle tree adds the eight (a fixed order).
 __global__ void conv_silu_reduce_kernel(const float *__restrict__ part, int ntiles, int C, float *__restrict__ dw, float *__restrict__ dbias) {
+  begin_dependent();
   const int x = (blockIdx.x * blockDim.x + threadIdx.x) >> 3, r = threadIdx.x & 7;
   const bool live = x < 5 * C;
   const int s = live ? x / C : 0, c = live ? x % C : 0;
@@ -397,14 +400,14 @@ dim3 conv_grid(int B, int T, int C, int steps) { return dim3((C / 4 + kLanes - 1
 template <typename T, int STEPS>
 void launch_fwd(int B, int Tn, int C, const void *x, long long xs, const void *w, const void *bias, const void *prev, void *out, long long os,
                 cudaStream_t s) {
-  conv_silu_fwd_kernel<T, STEPS><<<conv_grid(B, Tn, C, STEPS), kConvThreads, 0, s>>>(
+  (void)launch_early(conv_silu_fwd_kernel<T, STEPS>, conv_grid(B, Tn, C, STEPS), kConvThreads, 0, s,
       B, Tn, C, static_cast<const T *>(x), xs, static_cast<const T *>(w), static_cast<const T *>(bias), static_cast<const T *>(prev),
       static_cast<T *>(out), os);
 }
 template <typename T, int STEPS>
 void launch_bwd(int B, int Tn, int C, int steps, const void *x, const long long (&st)[3], const void *w, const void *bias, const void *prev,
                 const void *dout, void *dx, void *dprev, float *part, cudaStream_t s) {
-  conv_silu_bwd_kernel<T, STEPS><<<conv_grid(B, Tn, C, steps), kConvThreads, 0, s>>>(
+  (void)launch_early(conv_silu_bwd_kernel<T, STEPS>, conv_grid(B, Tn, C, steps), kConvThreads, 0, s,
       steps, Tn, C, static_cast<const T *>(x), st[0], static_cast<const T *>(w), static_cast<const T *>(bias), static_cast<const T *>(prev),
       static_cast<const T *>(dout), st[1], static_cast<T *>(dx), st[2], static_cast<T *>(dprev), part);
 }
@@ -487,6 +490,6 @@ extern "C" int m2rnn_conv_silu_bwd(int32_t B, int32_t T, int32_t C, int32_t io_d
     default: launch(bf ? launch_bwd<__nv_bfloat16, 0> : launch_bwd<float, 0>);
   }
   if (cudaGetLastError() != cudaSuccess) return M2RNN_ERR_CUDA;
-  conv_silu_reduce_kernel<<<(8 * 5 * C + 255) / 256, 256, 0, s>>>(part, B * tiles(T, steps), C, dw, dbias);
+  (void)launch_early(conv_silu_reduce_kernel, (8 * 5 * C + 255) / 256, 256, 0, s, part, B * tiles(T, steps), C, dw, dbias);
   return cudaGetLastError() == cudaSuccess ? M2RNN_OK : M2RNN_ERR_CUDA;
 }

@@ -61,6 +61,7 @@ __global__ void __launch_bounds__(32 * DecCfg<V>::kWarps, 1) decode_bf16_kernel(
   using Cfg = DecCfg<V>;
   constexpr int NT = V / 8, KT = V / 16, SEG = V / 4, NX = V / 16, kStages = Cfg::kStages, kWarps = Cfg::kWarps;
   extern __shared__ __align__(128) unsigned char smem[];
+  begin_dependent();
   const int K = a.K, N = a.N, B = a.B, slabs = K / 16;
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31, g = lane >> 2, c = lane & 3;
   const int dq = N / a.Nq, dk = N / a.Nk;
@@ -232,8 +233,7 @@ cudaError_t launch_decode_v(const ScanArgs &a, cudaStream_t s) {
   const cudaError_t e = allow_smem(decode_bf16_kernel<V>, DecCfg<V>::kSmem);
   if (e != cudaSuccess) return e;
   const long units = (long)a.B * a.N, room = sm_count(), grid = units < room ? units : room, warps = grid * DecCfg<V>::kWarps;
-  decode_bf16_kernel<V><<<(unsigned)grid, 32 * DecCfg<V>::kWarps, DecCfg<V>::kSmem, s>>>(a, (int)(units / warps), (int)(units % warps));
-  return cudaGetLastError();
+  return launch_early(decode_bf16_kernel<V>, (unsigned)grid, 32 * DecCfg<V>::kWarps, DecCfg<V>::kSmem, s, a, (int)(units / warps), (int)(units % warps));
 }
 
 }  // namespace

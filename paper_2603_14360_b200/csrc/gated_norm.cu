@@ -180,6 +180,7 @@ __global__ void __launch_bounds__(kThreads, resident(false, sizeof(T), CPL * R, 
     long tokens, int d, const T *__restrict__ y, const T *__restrict__ g_in, const T *__restrict__ w, float eps, int use_silu,
     T *__restrict__ out, float *__restrict__ rstd) {
   extern __shared__ __align__(16) unsigned char smem[];
+  begin_dependent();
   __shared__ float red[2 * kWarps * R];
   Walk<T, CPL, R, G, 2, FULL> wk(smem, tokens, d);
   const T *const src[2] = {y, g_in};
@@ -238,6 +239,7 @@ __global__ void __launch_bounds__(kThreads, resident(true, sizeof(T), CPL * R, F
     long tokens, int d, const T *__restrict__ y, const T *__restrict__ g_in, const T *__restrict__ w, const float *__restrict__ rstd,
     int use_silu, const T *__restrict__ dout, T *__restrict__ dy, T *__restrict__ dg_in, float *__restrict__ dw_part) {
   extern __shared__ __align__(16) unsigned char smem[];
+  begin_dependent();
   __shared__ float red[2 * kWarps * R];
   Walk<T, CPL, R, G, 3, FULL> wk(smem, tokens, d);
   const T *const src[3] = {y, g_in, dout};
@@ -330,6 +332,7 @@ __global__ void __launch_bounds__(kThreads, resident(true, sizeof(T), CPL * R, F
 // dw[j] = sum over the R per-CTA partials, in a fixed order: 32 interleaved running sums per column (one
 // per warp of the CTA), then their sum in warp order
 __global__ void __launch_bounds__(1024) reduce_partials_kernel(const float *__restrict__ part, float *__restrict__ out, int R, int n) {
+  begin_dependent();
   __shared__ float sm[32][33];
   const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
   const int j = blockIdx.x * 32 + lane;
@@ -417,7 +420,7 @@ cudaError_t launch_fwd(long tokens, int d, const void *y, const void *g, const v
     constexpr int smem = Walk<T, C(), R(), G(), 2, FULL()>::kSmem;
     const cudaError_t e = allow_smem(kern, smem);
     if (e != cudaSuccess) return e;
-    kern<<<sp.grid, kThreads, smem, s>>>(tokens, d, static_cast<const T *>(y), static_cast<const T *>(g), static_cast<const T *>(w), eps, silu_on,
+    (void)launch_early(kern, sp.grid, kThreads, smem, s, tokens, d, static_cast<const T *>(y), static_cast<const T *>(g), static_cast<const T *>(w), eps, silu_on,
                                          static_cast<T *>(out), rstd);
     return cudaGetLastError();
   });
@@ -433,7 +436,7 @@ cudaError_t launch_bwd(long tokens, int d, const void *y, const void *g, const v
     constexpr int smem = Walk<T, C(), R(), G(), 3, FULL()>::kSmem > sums ? Walk<T, C(), R(), G(), 3, FULL()>::kSmem : sums;
     const cudaError_t e = allow_smem(kern, smem);
     if (e != cudaSuccess) return e;
-    kern<<<sp.grid, kThreads, smem, s>>>(tokens, d, static_cast<const T *>(y), static_cast<const T *>(g), static_cast<const T *>(w), rstd, silu_on,
+    (void)launch_early(kern, sp.grid, kThreads, smem, s, tokens, d, static_cast<const T *>(y), static_cast<const T *>(g), static_cast<const T *>(w), rstd, silu_on,
                                          static_cast<const T *>(dout), static_cast<T *>(dy), static_cast<T *>(dg), dw_part);
     return cudaGetLastError();
   });
@@ -484,7 +487,7 @@ int m2rnn_gated_norm_bwd(int64_t tokens, int32_t d, int32_t io_dtype, const void
   cudaError_t e = io_dtype == M2RNN_BF16 ? launch_bwd<__nv_bfloat16>((long)tokens, d, y, g_in, w, rstd, silu_on, dout, dy, dg_in, part, s)
                                          : launch_bwd<float>((long)tokens, d, y, g_in, w, rstd, silu_on, dout, dy, dg_in, part, s);
   if (e != cudaSuccess) { (void)cudaGetLastError(); return M2RNN_ERR_CUDA; }
-  reduce_partials_kernel<<<(d + 31) / 32, 1024, 0, s>>>(part, dw, split_of((long)tokens, d, true, io_dtype).grid, d);
+  (void)launch_early(reduce_partials_kernel, (d + 31) / 32, 1024, 0, s, part, dw, split_of((long)tokens, d, true, io_dtype).grid, d);
   return cudaGetLastError() == cudaSuccess ? M2RNN_OK : M2RNN_ERR_CUDA;
 }
 

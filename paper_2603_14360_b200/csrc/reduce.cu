@@ -8,6 +8,7 @@ namespace {
 
 // dW[n] = sum_b dW_part[b][n]   (Algorithm 2 sums dW over the batch with an atomic add)
 __global__ void reduce_dW_kernel(const float *__restrict__ part, float *__restrict__ dW, int B, size_t NVV) {
+  begin_dependent();
   const size_t x = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (x >= NVV) return;
   float s = 0.f;
@@ -20,6 +21,7 @@ __global__ void reduce_dW_kernel(const float *__restrict__ part, float *__restri
 // multiple of 16), eight heads' loads in flight: HBM-bound (one entry and load after another read 71 MB in 19 us, now 14).
 template <typename TIO>
 __global__ void __launch_bounds__(256) reduce_heads_kernel(const float4 *__restrict__ part, TIO *__restrict__ out, size_t rows, int per, int K4) {
+  begin_dependent();
   const size_t x = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (x >= rows * K4) return;
   const size_t row = x / K4, at = row * per * K4 + x % K4;      // row: (bt, g)
@@ -47,6 +49,7 @@ __global__ void __launch_bounds__(256) reduce_heads_kernel(const float4 *__restr
 // it at 2.2 TB/s: 22 M elements of two slabs 100 us, now 36).
 template <typename TIO>
 __global__ void reduce_slabs_kernel(const float *__restrict__ part, TIO *__restrict__ out, int R, size_t n) {
+  begin_dependent();
   const size_t x = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (x >= n) return;
   float s = 0.f;
@@ -55,6 +58,7 @@ __global__ void reduce_slabs_kernel(const float *__restrict__ part, TIO *__restr
 }
 template <typename TIO>
 __global__ void __launch_bounds__(256) reduce_slabs4_kernel(const float4 *__restrict__ part, TIO *__restrict__ out, int R, size_t n4) {
+  begin_dependent();
   for (size_t x = (size_t)blockIdx.x * blockDim.x + threadIdx.x; x < n4; x += (size_t)gridDim.x * blockDim.x) {
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
     for (int r0 = 0; r0 < R; r0 += 4) {
@@ -82,21 +86,21 @@ cudaError_t launch_reduce_slabs(const float *part, void *out, int io_dtype, int 
     const size_t n4 = n / 4, need = (n4 + 255) / 256, most = (size_t)sm_count() * 32;
     const unsigned grid = (unsigned)(need < most ? need : most);
     const float4 *p = reinterpret_cast<const float4 *>(part);
-    if (io_dtype == M2RNN_F32) reduce_slabs4_kernel<float><<<grid, 256, 0, s>>>(p, static_cast<float *>(out), R, n4);
-    else reduce_slabs4_kernel<__nv_bfloat16><<<grid, 256, 0, s>>>(p, static_cast<__nv_bfloat16 *>(out), R, n4);
+    if (io_dtype == M2RNN_F32) (void)launch_early(reduce_slabs4_kernel<float>, grid, 256, 0, s, p, static_cast<float *>(out), R, n4);
+    else (void)launch_early(reduce_slabs4_kernel<__nv_bfloat16>, grid, 256, 0, s, p, static_cast<__nv_bfloat16 *>(out), R, n4);
     return cudaGetLastError();
   }
   const unsigned grid = (unsigned)((n + 255) / 256);
   if (io_dtype == M2RNN_F32)
-    reduce_slabs_kernel<float><<<grid, 256, 0, s>>>(part, static_cast<float *>(out), R, n);
+    (void)launch_early(reduce_slabs_kernel<float>, grid, 256, 0, s, part, static_cast<float *>(out), R, n);
   else
-    reduce_slabs_kernel<__nv_bfloat16><<<grid, 256, 0, s>>>(part, static_cast<__nv_bfloat16 *>(out), R, n);
+    (void)launch_early(reduce_slabs_kernel<__nv_bfloat16>, grid, 256, 0, s, part, static_cast<__nv_bfloat16 *>(out), R, n);
   return cudaGetLastError();
 }
 
 cudaError_t launch_reduce_dW(const float *dW_part, float *dW, int B, int N, int V, cudaStream_t s) {
   const size_t NVV = (size_t)N * V * V;
-  reduce_dW_kernel<<<(unsigned)((NVV + 255) / 256), 256, 0, s>>>(dW_part, dW, B, NVV);
+  (void)launch_early(reduce_dW_kernel, (unsigned)((NVV + 255) / 256), 256, 0, s, dW_part, dW, B, NVV);
   return cudaGetLastError();
 }
 
@@ -106,8 +110,8 @@ cudaError_t launch_reduce_heads(const float *part, void *out, int io_dtype, size
   const int per = N / Ng, K4 = K / 4;
   const unsigned grid = (unsigned)((rows * K4 + 255) / 256);
   const float4 *p = reinterpret_cast<const float4 *>(part);
-  if (io_dtype == M2RNN_F32) reduce_heads_kernel<float><<<grid, 256, 0, s>>>(p, static_cast<float *>(out), rows, per, K4);
-  else reduce_heads_kernel<__nv_bfloat16><<<grid, 256, 0, s>>>(p, static_cast<__nv_bfloat16 *>(out), rows, per, K4);
+  if (io_dtype == M2RNN_F32) (void)launch_early(reduce_heads_kernel<float>, grid, 256, 0, s, p, static_cast<float *>(out), rows, per, K4);
+  else (void)launch_early(reduce_heads_kernel<__nv_bfloat16>, grid, 256, 0, s, p, static_cast<__nv_bfloat16 *>(out), rows, per, K4);
   return cudaGetLastError();
 }
 
