@@ -10,7 +10,8 @@
 // that keeps its share of the row, its columns' dw sums and the next row on the way (16-byte cp.async
 // into a ring) within two (backward) to four CTAs per SM, whatever the row length.  One partial of dw per
 // persistent CTA, added by a fixed-order second stage.  16 384 rows: of 1 344 features (84 heads x 16)
-// forward 26 us (5.1 TB/s), backward 39 us (5.6 TB/s); of 1 888, 42 and 69 us (6.0 TB/s).  (A warp per row,
+// forward 26 us (5.1 TB/s), backward 39 us (5.6 TB/s); of 1 888, 42 and 69 us (6.0 TB/s).  (Launches apart; one after the
+// other, each started while the one before it ends, the pair of 1 344 takes 65 us and took 70.)  (A warp per row,
 // rows of other lengths than 256 times a power of two walked twice: 31 and 80, 64 and 141 us.  A CTA
 // per row or four rows at a time, a chunk per thread: 31-42 and 60 us, the barriers show.)
 #include <cuda_bf16.h>

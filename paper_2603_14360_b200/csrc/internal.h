@@ -84,13 +84,14 @@ static __device__ __noinline__ int longest_first(const int32_t *cu, int B, int p
   __syncthreads();
   return b;
 }
-// A launch whose set-up overlaps the end of the kernel before it in the stream (programmatic dependent launch): its CTAs may come
-// while that one's last are still running, and wait in begin_dependent, every thread's first statement that is not address
-// arithmetic, until that one is done and its writes are seen.  For the kernels of 5 to 100 us, whose gaps count: a decoding step
-// (B=48, N=84, K=64, V=16, steps back to back) 8.2 -> 6.1 us, conv forward + backward (B=8, T=2048, C=3072) 102.4 -> 101.6, the gated
-// norm's pair (16 384 rows of 1 344) 70 -> 67.5, a prompt of 1 001 tokens through conv, scan and norm (N=84, K=64, V=16) 103.4 -> 100.4.  The scans
-// themselves keep the plain launch: against 0.1 to 30 ms a gap does not count, and their waiting CTAs would take a whole SM's
-// shared memory from other streams' kernels.
+// A launch whose set-up overlaps the end of the kernel before it in the stream (programmatic dependent launch): its CTAs come as
+// that one's last end, and wait in begin_dependent, every thread's first statement that is not address arithmetic, until that one
+// is done and its writes are seen.  For the kernels of 2 to 100 us, whose gaps count: a decoding step (B=48, N=84, K=64, V=16, steps
+// back to back) 8.2 -> 6.0 us, conv forward + backward [8, 2048, 3072] 100.3 -> 93.9, [1, 927, 3920] 20.6 -> 14.9, the gated norm's
+// pair (16 384 rows of 1 344) 70.4 -> 64.6, 1 001 rows 14.4 -> 10.0.  No kernel asks for its dependents before it ends
+// (launch_dependents): waiting CTAs then land where the running ones happen to leave room, not one on each SM, and a grid of one
+// or two rounds is bound by its fullest SM: [1, 927, 3920] 21.4 us so, conv forward in fp32 [1, 2000, 3072] 16.7 against 11.1 (plain
+// 12.4).
 template <typename... P, typename... A>
 inline cudaError_t launch_early(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
   cudaLaunchAttribute at{};
@@ -101,10 +102,7 @@ inline cudaError_t launch_early(void (*kernel)(P...), dim3 grid, dim3 block, siz
   cfg.attrs = &at; cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
-__device__ __forceinline__ void begin_dependent() {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");      // (the next kernel's CTAs may come as room is left)
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-}
+__device__ __forceinline__ void begin_dependent() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // The arguments of a scan kernel's launch of `ctas` CTAs of `threads`, with the order of a packed batch decided.
 // `pace`: the kernel's time per step, in 0.1 us.
 // Every CTA ranks the batch for itself, B comparisons for each sequence that a thread takes, some 0.02 us each.
