@@ -91,7 +91,8 @@ static __device__ __noinline__ int longest_first(const int32_t *cu, int B, int p
 // pair (16 384 rows of 1 344) 70.4 -> 64.6, 1 001 rows 14.4 -> 10.0.  No kernel asks for its dependents before it ends
 // (launch_dependents): waiting CTAs then land where the running ones happen to leave room, not one on each SM, and a grid of one
 // or two rounds is bound by its fullest SM: [1, 927, 3920] 21.4 us so, conv forward in fp32 [1, 2000, 3072] 16.7 against 11.1 (plain
-// 12.4).
+// 12.4).  Of the scans those of short steps take it: 1 001 tokens through conv, scan and norm (N=84, K=64, V=16) 99.7 -> 98.0, one
+// sequence of 433 tokens forward + backward (30 heads of K=V=32) 196.5 -> 192.2; the V = 128 kernels on the tensor memory gain nothing.
 template <typename... P, typename... A>
 inline cudaError_t launch_early(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
   cudaLaunchAttribute at{};

@@ -140,6 +140,7 @@ __global__ void __launch_bounds__(bwd_threads<V, NWC>(), 1) bwd_bf16_kernel(Scan
   // warps would set the pace: bptt_bf16 8.37 -> 9.00 ms)
   constexpr bool kDqDw = NDW >= 2 * NWC || (NDW == 1 && NWC == 1), kDkDw = kDqDw;
   extern __shared__ __align__(128) unsigned char smem[];
+  begin_dependent();
 
   const int K = a.K, N = a.N, C = a.C;
   const int RS = K / KC;
@@ -875,8 +876,7 @@ cudaError_t launch_bwd_t(const ScanArgs &a, cudaStream_t s) {
   if (e != cudaSuccess) return e;
   const int RS = a.K / (16 * NWC);
   const int ctas = a.B * a.N * RS;
-  bwd_bf16_kernel<V, NWC><<<ctas, bwd_threads<V, NWC>(), L.total, s>>>(in_order(a, ctas, bwd_threads<V, NWC>(), 10));
-  return cudaGetLastError();
+  return launch_early(bwd_bf16_kernel<V, NWC>, ctas, bwd_threads<V, NWC>(), L.total, s, in_order(a, ctas, bwd_threads<V, NWC>(), 10));
 }
 
 template <int V>

@@ -96,6 +96,7 @@ template <int CC, bool CLIP>
 __global__ void __launch_bounds__(kRoomWarps * 32, 1) bwd_v16_kernel(ScanArgs a) {
   using L = Lay<CC>;
   extern __shared__ __align__(128) unsigned char smem[];
+  begin_dependent();
   const int K = a.K, N = a.N, C = a.C;
   const int R = a.KC / 16, RS = K / a.KC, hg = a.hg;
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31, g = lane >> 2, c = lane & 3;
@@ -553,8 +554,7 @@ cudaError_t launch_t(const ScanArgs &a, cudaStream_t s) {
   const cudaError_t e = allow_smem(bwd_v16_kernel<CC, CLIP>, smem);
   if (e != cudaSuccess) return e;
   const int ctas = a.B * a.groups * (a.K / a.KC), threads = (a.hg * R + 2) * 32;
-  bwd_v16_kernel<CC, CLIP><<<ctas, threads, smem, s>>>(in_order(a, ctas, threads, 2));
-  return cudaGetLastError();
+  return launch_early(bwd_v16_kernel<CC, CLIP>, ctas, threads, smem, s, in_order(a, ctas, threads, 2));
 }
 
 }  // namespace

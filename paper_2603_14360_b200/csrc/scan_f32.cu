@@ -198,6 +198,7 @@ __global__ void __launch_bounds__(Geom<V>::kThreads) fwd_f32_kernel(ScanArgs a) 
   constexpr int E = GR / 4;
   constexpr int kTile = GR * G::HP;
   extern __shared__ __align__(16) float smem[];
+  begin_dependent();
   const int K = a.K, N = a.N, R = a.KCf, RS = K / R, ng = R / GR;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, p = lane >> 2, c0 = 8 * warp + 2 * (lane & 3);
   const int orow = Own<GR>::row(p), ocol = Own<GR>::col(p, c0), ycol = y_col<GR>(lane, c0);
@@ -415,6 +416,7 @@ __global__ void __launch_bounds__(WideFwd<V, R>::kThreads) fwd_f32_wide_kernel(S
   using WF = WideFwd<V, R>;
   constexpr int kSets = WF::kSets, E = G::E;
   extern __shared__ __align__(16) float smem[];
+  begin_dependent();
   const int K = a.K, N = a.N, RS = K / 4;
   const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), set = warp / G::NWR;
   const int q = lane / (32 / G::P), c0 = (warp % G::NWR) * G::CW + G::CP * (lane % (32 / G::P)), col = c0 + E * q;
@@ -586,6 +588,7 @@ __global__ void __launch_bounds__(BwdGeom<V, GR, WIDE>::kThreads, WIDE ? 2 : 512
   using WG = Wide<64>;      // (of the wide form)
   constexpr int E = WIDE ? WG::E : GR / 4, kThreads = BG::kThreads;
   extern __shared__ __align__(16) float smem[];
+  begin_dependent();
   const int K = a.K, N = a.N;
   const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
   const int p = WIDE ? lane / (32 / WG::P) : lane >> 2, c0 = WIDE ? WG::CP * (lane % (32 / WG::P)) : 8 * warp + 2 * (lane & 3);
@@ -887,6 +890,7 @@ __global__ void __launch_bounds__(Geom<V>::kThreads, DecGeom<V>::kOcc) decode_f3
   using G = Geom<V>;
   constexpr int kStage = DecGeom<V>::kStage;
   extern __shared__ __align__(16) float smem[];
+  begin_dependent();
   const int K = a.K, N = a.N, B = a.B, ng = K / kRows;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, p = lane >> 2, c0 = 8 * warp + 2 * (lane & 3), ycol = y_col<kRows>(lane, c0);
   const size_t KV = (size_t)K * V;
@@ -946,8 +950,7 @@ cudaError_t launch_fwd_g(const ScanArgs &a, cudaStream_t s) {
   const cudaError_t e = allow_smem(fwd_f32_kernel<V, GR>, smem);
   if (e != cudaSuccess) return e;
   const int ctas = a.B * a.N * (a.K / a.KCf);
-  fwd_f32_kernel<V, GR><<<ctas, Geom<V>::kThreads, smem, s>>>(in_order(a, ctas, Geom<V>::kThreads, 7));
-  return cudaGetLastError();
+  return launch_early(fwd_f32_kernel<V, GR>, ctas, Geom<V>::kThreads, smem, s, in_order(a, ctas, Geom<V>::kThreads, 7));
 }
 template <int V, int R>
 cudaError_t launch_fwd_w(const ScanArgs &a, cudaStream_t s) {
@@ -956,8 +959,7 @@ cudaError_t launch_fwd_w(const ScanArgs &a, cudaStream_t s) {
   const cudaError_t e = allow_smem(fwd_f32_wide_kernel<V, R>, smem);
   if (e != cudaSuccess) return e;
   const int ctas = a.B * a.N * (a.K / 4);
-  fwd_f32_wide_kernel<V, R><<<ctas, kThreads, smem, s>>>(in_order(a, ctas, kThreads, 4));
-  return cudaGetLastError();
+  return launch_early(fwd_f32_wide_kernel<V, R>, ctas, kThreads, smem, s, in_order(a, ctas, kThreads, 4));
 }
 template <int V>
 cudaError_t launch_fwd_v(const ScanArgs &a, cudaStream_t s) {
@@ -984,8 +986,7 @@ cudaError_t launch_bwd_g(const ScanArgs &a, cudaStream_t s) {
   cudaError_t e = allow_smem(bwd_f32_kernel<V, GR, WIDE>, smem);
   const int slabs = a.K / GR, nslab = a.KC == GR ? slabs : 1;
   for (int s0 = 0; s0 < slabs && e == cudaSuccess; s0 += nslab) {
-    bwd_f32_kernel<V, GR, WIDE><<<a.B * a.N * nslab, BG::kThreads, smem, s>>>(in_order(a, (long)a.B * a.N * nslab, BG::kThreads, 12), s0, nslab);
-    e = cudaGetLastError();
+    e = launch_early(bwd_f32_kernel<V, GR, WIDE>, a.B * a.N * nslab, BG::kThreads, smem, s, in_order(a, (long)a.B * a.N * nslab, BG::kThreads, 12), s0, nslab);
   }
   return e;
 }
@@ -1002,8 +1003,7 @@ cudaError_t launch_decode_v(const ScanArgs &a, cudaStream_t s) {
   const cudaError_t e = allow_smem(decode_f32_kernel<V>, smem);
   if (e != cudaSuccess) return e;
   const long units = (long)a.B * a.N, room = (long)sm_count() * DecGeom<V>::kOcc;
-  decode_f32_kernel<V><<<(unsigned)(units < room ? units : room), Geom<V>::kThreads, smem, s>>>(a);
-  return cudaGetLastError();
+  return launch_early(decode_f32_kernel<V>, (unsigned)(units < room ? units : room), Geom<V>::kThreads, smem, s, a);
 }
 
 }  // namespace

@@ -118,6 +118,7 @@ __global__ void __launch_bounds__(cs_threads(SP * NW, OCC), OCC) fwd_bf16_cs_ker
   static_assert(kMine * K / 8 <= 32, "a lane stages eight entries of k");
   static_assert(kMine % 2 == 0, "the readout of one slab takes two steps at a time");
   extern __shared__ __align__(128) unsigned char smem_raw[];
+  begin_dependent();
 
   const int Kf = a.K, N = a.N;            // rows of the whole state
   const int RS = Kf / K;
@@ -525,8 +526,7 @@ cudaError_t launch_cs(const ScanArgs &a, cudaStream_t s) {
   cudaError_t e = allow_smem(fwd_bf16_cs_kernel<V, SP, NW, CKPT, OCC>, smem);
   if (e != cudaSuccess) return e;
   const int ctas = a.B * a.N * (a.K / (16 * NW)), threads = cs_threads(SP * NW, OCC);
-  fwd_bf16_cs_kernel<V, SP, NW, CKPT, OCC><<<ctas, threads, smem, s>>>(in_order(a, ctas, threads, 3));
-  return cudaGetLastError();
+  return launch_early(fwd_bf16_cs_kernel<V, SP, NW, CKPT, OCC>, ctas, threads, smem, s, in_order(a, ctas, threads, 3));
 }
 
 template <int V, int SP, int NW, bool CKPT>

@@ -70,6 +70,7 @@ __global__ void __launch_bounds__(((HALF ? 2 : 1) * NW + kSvc) * 32, OCC) fwd_v1
   constexpr int K = 16 * NW, kMine = kTC / kSvc, kBlk = 32 / kMine;   // steps of a stage per service warp; stages of a block of gates
   static_assert(kMine * K / 8 <= 32, "a lane stages eight entries of k");
   extern __shared__ __align__(16) unsigned char smem[];
+  begin_dependent();
   const int Kf = a.K, N = a.N, RS = Kf / K;
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31, g = lane >> 2, c = lane & 3;
   const int place = blockIdx.x / RS, rs = blockIdx.x % RS, rbase = rs * K;
@@ -344,8 +345,7 @@ cudaError_t launch_t(const ScanArgs &a, cudaStream_t s) {
   const cudaError_t e = allow_smem(fwd_v16_kernel<NW, CKPT, OCC, kSvc, HALF>, smem);
   if (e != cudaSuccess) return e;
   const int ctas = a.B * a.N * (a.K / (16 * NW)), threads = ((HALF ? 2 : 1) * NW + kSvc) * 32;
-  fwd_v16_kernel<NW, CKPT, OCC, kSvc, HALF><<<ctas, threads, smem, s>>>(in_order(a, ctas, threads, 1));
-  return cudaGetLastError();
+  return launch_early(fwd_v16_kernel<NW, CKPT, OCC, kSvc, HALF>, ctas, threads, smem, s, in_order(a, ctas, threads, 1));
 }
 
 template <int NW, bool CKPT>

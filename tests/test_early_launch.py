@@ -1,4 +1,4 @@
-"""Kernels whose launch overlaps the end of the one before (conv, gated norm, decoding step, the sums of partials): a chain in which
+"""Kernels whose launch overlaps the end of the one before (conv, gated norm, decoding step, scans, the sums of partials): a chain in which
 each call reads what the one before wrote gives the same bits with the device idle before each call, back to back, behind a copy and
 another stream's event, and replayed from a CUDA graph."""
 import pytest
@@ -41,6 +41,14 @@ def test_chain_of_dependent_calls(B, T, N, V):
             stop()
             s2 = binding.m2rnn_decode_step(q, k, s1, gate, g["W"], state)
             stop()
+            for to in (torch.bfloat16, torch.float32):
+                a = [t.to(to) for t in (g["q"], g["k"], y.view(B, T, N, V))] + [g["gate"], g["W"].to(to), state]
+                stop()
+                z, hT, ck = binding.m2rnn_fwd(*a, save_ckpt=True)
+                stop()
+                gr = binding.m2rnn_bwd(*a, z, hT, ckpt=ck)
+                stop()
+                res += [z, hT, *gr.values()]
             move(x, d["dx"])
             res += [c, y, rstd, *n.values(), *(t for t in d.values() if t is not None), s1, s2]
         stop()
