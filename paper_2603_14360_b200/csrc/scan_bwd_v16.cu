@@ -18,7 +18,7 @@
 // some 165 instructions of a slab warp, 57 of them on the FMA pipe, whose packed fp32 pairs take two cycles like two single ones:
 // products and sums of 16-bit operands are taken without unpacking instead (fma.f32.bf16, add.f32.f16, one cycle each).
 // Backward of that shape, 1 024 steps: 796 us with four kinds of warps that handed states over through shared memory, two waves,
-// and a share of dq and dk per head; 484 now.  Tried and slower: states of a chunk in registers (eight steps unrolled twice:
+// and a share of dq and dk per head; 465 now.  Tried and slower: states of a chunk in registers (eight steps unrolled twice:
 // the instruction cache), fp32 copies of k, v, q, dy (shared-memory bandwidth), stmatrix and ldmatrix for the transposition.
 #include <cuda_fp16.h>
 
