@@ -184,6 +184,13 @@ int cuda_failed() {
 
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
+// The longest checkpoint interval, by a plan that has not seen the caller's: that one is still to be checked.
+int longest_interval(const m2rnn_params *p) {
+  m2rnn_params unset = *p;
+  unset.ckpt_interval = 0;
+  return plan_bwd(&unset).C_max;
+}
+
 int check_params(const m2rnn_params *p, bool need_T) {
   if (!p) return M2RNN_ERR_NULL;
   if (p->B < 0 || p->N <= 0 || p->K <= 0 || p->V <= 0 || (need_T && p->T < 0)) return M2RNN_ERR_SHAPE;
@@ -193,7 +200,7 @@ int check_params(const m2rnn_params *p, bool need_T) {
   if (p->gate_kind < M2RNN_GATE_VALUE || p->gate_kind > M2RNN_GATE_PSI) return M2RNN_ERR_UNSUPPORTED;
   if (p->K % 16 || p->K < 16 || p->K > 128) return M2RNN_ERR_UNSUPPORTED;
   if (p->V != 16 && p->V != 32 && p->V != 64 && p->V != 128) return M2RNN_ERR_UNSUPPORTED;
-  if (p->ckpt_interval < 0 || (p->ckpt_interval > 0 && p->ckpt_interval > plan_bwd(p).C_max)) return M2RNN_ERR_UNSUPPORTED;
+  if (p->ckpt_interval < 0 || (p->ckpt_interval > 0 && p->ckpt_interval > longest_interval(p))) return M2RNN_ERR_UNSUPPORTED;
   // the bf16 kernels take steps in pairs and checkpoint between pairs
   if (p->io_dtype == M2RNN_BF16 && (p->ckpt_interval & 1)) return M2RNN_ERR_UNSUPPORTED;
   // token strides: at least a token's heads, in 16-byte units

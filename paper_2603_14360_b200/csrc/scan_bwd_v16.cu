@@ -574,10 +574,11 @@ BwdPlan plan_bwd_v16(int B, int N, int Nq, int Nk, int K, int T, int interval, b
   const int set = std::gcd(Nq < N ? N / Nq : N, Nk < N ? N / Nk : N);
   const bool own_rows = Nq == N || Nk == N;
   double best_cost = 0.;
-  for (int C = interval ? interval : 8; C <= (interval ? interval : 16); C += 8)
+  const int choices[2] = {interval ? interval : 8, 16};
+  for (int x = 0; x < (interval ? 1 : 2); ++x)
     for (int R = 1; R <= K / 16 && R <= kMostSlabs; ++R)
       for (int hg = 1; K / 16 % R == 0 && hg * R <= kMostSlabs && hg <= set; ++hg) {
-        const int groups = N / set * ((set + hg - 1) / hg), slabs = hg * R, qb = Nq < N ? R : slabs, kb = Nk < N ? R : slabs;
+        const int C = choices[x], groups = N / set * ((set + hg - 1) / hg), slabs = hg * R, qb = Nq < N ? R : slabs, kb = Nk < N ? R : slabs;
         const long ctas = (long)(B > 0 ? B : 1) * groups * (K / (16 * R));
         const size_t smem = (C <= 8 ? Lay<8>::total(hg, qb, kb, slabs) : Lay<16>::total(hg, qb, kb, slabs)) + 1024;
         constexpr size_t kSm = 228 * 1024;
@@ -594,7 +595,7 @@ BwdPlan plan_bwd_v16(int B, int N, int Nq, int Nk, int K, int T, int interval, b
         const bool better = !best.KC || (lean ? 16 * R > best.KC || (16 * R == best.KC && hg > best.hg) : cost < best_cost);
         if (!better) continue;
         best_cost = cost;
-        best.KC = 16 * R; best.C = interval ? interval : C; best.hg = hg; best.groups = groups; best.set = set;
+        best.KC = 16 * R; best.C = C; best.hg = hg; best.groups = groups; best.set = set;
       }
   best.C_max = 16;
   return best;

@@ -3,6 +3,8 @@ the header declares, and rejects bad arguments before launching anything."""
 import ctypes
 import os
 import re
+import subprocess
+import sys
 
 import pytest
 
@@ -148,6 +150,25 @@ def test_plans_for_small_states_with_many_units(lib):
     # a caller may still ask for a longer chunk, up to what one CTA's shared memory holds
     assert lib.m2rnn_ckpt_interval(ctypes.byref(_p(B=4, N=84, Nq=1, Nk=1, K=64, V=16, T=64, ckpt_interval=12))) == 12
     assert lib.m2rnn_ckpt_interval(ctypes.byref(_p(B=4, N=84, Nq=1, Nk=1, K=64, V=16, T=64, ckpt_interval=18))) == -3
+
+
+def test_every_unsupported_interval_is_refused(lib):
+    """Intervals up to the largest int, at shapes of every backward kernel: refused by every call, at once (in a process of its own,
+    so that a call that does not come back is an error and not a hang)."""
+    shapes = [dict(B=4, N=84, Nq=1, Nk=1, K=64, V=16), dict(B=1, N=4, Nq=1, Nk=1, K=64, V=16), dict(B=2, N=96, Nq=96, Nk=96, K=16, V=16),
+              dict(K=64, V=32), dict(K=64, V=64), dict(K=128, V=128), dict(K=48, V=128), dict(K=64, V=16, io_dtype=0), dict(K=64, V=128, io_dtype=0)]
+    code = ("import ctypes, sys; sys.path[:0] = [%r, %r]\n"
+            "from test_abi import _fwd, _p, binding\n"
+            "lib = binding._lib()\n"
+            "for s in %r:\n"
+            "    for c in (66, 1000, 2 ** 31 - 16, 2 ** 31 - 9, 2 ** 31 - 8, 2 ** 31 - 2, 2 ** 31 - 1, -1, -2 ** 31):\n"
+            "        p = _p(**s, ckpt_interval=c)\n"
+            "        r = ctypes.byref(p)\n"
+            "        assert (_fwd(lib, p), lib.m2rnn_ckpt_interval(r), lib.m2rnn_bwd_row_slab(r)) == (-3, -3, -3), (s, c)\n"
+            "        assert not (lib.m2rnn_ckpt_bytes(r) or lib.m2rnn_fwd_workspace_bytes(r) or lib.m2rnn_bwd_workspace_bytes(r, 0)), (s, c)\n"
+            "print('refused')\n") % (os.path.dirname(os.path.abspath(__file__)), ROOT, shapes)
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=120)
+    assert r.stdout == "refused\n", r.stderr[-2000:]
 
 
 def test_gated_norm_rejects_bad_arguments(lib):
