@@ -73,8 +73,9 @@ typedef struct {
   int32_t K, V;          /* state is K x V per (b,n); the transition matrix is V x V          */
   int32_t io_dtype;      /* m2rnn_dtype                                                       */
   int32_t gate_kind;     /* m2rnn_gate_kind                                                   */
-  int32_t ckpt_interval; /* steps between saved states; 0 = library default for (K,V,dtype);
-                            at most m2rnn_ckpt_interval's bound, and even for M2RNN_BF16        */
+  int32_t ckpt_interval; /* steps between saved states; 0 = library default, which depends on B, N, Nq, Nk,
+                            K, V, io_dtype and the device's SM count, but not on T.  M2RNN_BF16: even and at
+                            most 16 (less where a kernel keeps less on chip); M2RNN_F32: at most 64 */
   float dh_clip;         /* <= 0: off.  Else the state gradient carried to the previous step is
                             clamped elementwise to [-dh_clip, dh_clip] after every reverse step
                             (section "Gradient Clipping"; the paper gives no threshold or form) */
@@ -108,10 +109,12 @@ int m2rnn_ckpt_interval(const m2rnn_params *params);
 /* Rows of a state that one CTA of the backward kernel takes for `params` (a divisor of K); <= 0
  * is an m2rnn_status.  The K rows of a state are independent recurrences (Eq. 1-2 act row by row),
  * so the backward pass may split them over K/rows CTAs; when it does, dv and dgate (sums over all
- * rows) are finished by two extra reduction launches. */
+ * rows) are finished by two extra reduction launches.  (M2RNN_BF16 with V = 16 splits by T too; M2RNN_F32 by the tokens.) */
 int m2rnn_bwd_row_slab(const m2rnn_params *params);
 
-/* Bytes of the checkpoint tensor [B,N,ceil(T/C),K,V] (fp32). */
+/* Bytes of the checkpoint tensor [B,N,ceil(T/C),K,V] (fp32).  They never fall as T grows, so a buffer for
+ * the longest sequence does for every shorter one of the same sizes.  Another B or another number of heads may
+ * come with another C: ask again, or set ckpt_interval. */
 size_t m2rnn_ckpt_bytes(const m2rnn_params *params);
 
 /* Scratch the forward call needs for `params`: 0 unless the library splits the rows of a state
@@ -137,7 +140,8 @@ int m2rnn_fwd(const m2rnn_params *params, const void *q, const void *k, const vo
               void *workspace, size_t workspace_bytes, int32_t *dev_status, void *stream);
 
 /* Scratch the backward call needs for `params`; `have_ckpt` != 0 if the caller will pass the
- * checkpoints written by m2rnn_fwd (otherwise the workspace also holds them). */
+ * checkpoints written by m2rnn_fwd (otherwise the workspace also holds them).  It never falls as T grows, but
+ * for M2RNN_F32 where the row groups' shares of dv would pass 4 GiB: the groups then take turns, without shares. */
 size_t m2rnn_bwd_workspace_bytes(const m2rnn_params *params, int have_ckpt);
 
 /* Backward through time (Algorithm 2, with the state gradient carried across steps:

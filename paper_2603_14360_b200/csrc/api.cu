@@ -97,7 +97,7 @@ BwdPlan plan_bwd(const m2rnn_params *p, bool lean, bool have_ckpt) {
   const int B = p->B, N = p->N, K = p->K, V = p->V;
   BwdPlan pl{};
   if (p->io_dtype == M2RNN_F32) {
-    pl.KC = lean ? K : bwd_f32_rows(B, N, K, V, p->T > 0 ? tokens_of(p) * N * V * sizeof(float) : 0); pl.C = bwd_f32_piece(); pl.C_max = 64;
+    pl.KC = lean ? K : bwd_f32_rows(B, N, K, V, p->T > 0 ? tokens_of(p) * N * V * sizeof(float) : 0); pl.C = pl.interval = bwd_f32_piece(); pl.C_max = 64;
     return pl;
   }
   // V = 16: scan_bwd_v16.cu, except where every slab of 16 rows has an SM to itself: there a slab's step is quicker spread over
@@ -105,10 +105,10 @@ BwdPlan plan_bwd(const m2rnn_params *p, bool lean, bool have_ckpt) {
   // 160 slabs 296 / 249).  The latter keeps two chunks on chip, 16 rows of them up to any supported interval.
   if (V == 16 && (long)(B > 0 ? B : 1) * N * (K / 16) > sm_count()) {
     const BwdPlan fast = plan_bwd_v16(B, N, p->Nq, p->Nk, K, p->T, p->ckpt_interval, false);
-    return lean ? plan_bwd_v16(B, N, p->Nq, p->Nk, K, p->T, p->ckpt_interval || have_ckpt ? fast.C : 16, true) : fast;
+    return lean ? plan_bwd_v16(B, N, p->Nq, p->Nk, K, p->T, p->ckpt_interval || have_ckpt ? fast.interval : 16, true) : fast;
   }
   if (bwd_use_tc(B, N, K, V, p->io_dtype)) {   // 32-row CTAs, chunks of four steps
-    pl.KC = bwd_tc_rows_per_cta(); pl.C = pl.C_max = bwd_tc_chunk();
+    pl.KC = bwd_tc_rows_per_cta(); pl.C = pl.interval = pl.C_max = bwd_tc_chunk();
     return pl;
   }
   // Rows per CTA: the largest slab that still spreads the problem over the SMs (rows are independent
@@ -126,7 +126,7 @@ BwdPlan plan_bwd(const m2rnn_params *p, bool lean, bool have_ckpt) {
   constexpr size_t kSmemLimit = 227 * 1024;
   int c = 16;
   while (c > 2 && bwd_bf16_smem_bytes(KC, V, c) > kSmemLimit) c -= 2;
-  pl.C = pl.C_max = c;
+  pl.C = pl.interval = pl.C_max = c;
   return pl;
 }
 
@@ -214,7 +214,7 @@ int check_params(const m2rnn_params *p, bool need_T) {
   return M2RNN_OK;
 }
 
-int interval_of(const m2rnn_params *p) { return p->ckpt_interval ? p->ckpt_interval : plan_bwd(p).C; }
+int interval_of(const m2rnn_params *p) { return p->ckpt_interval ? p->ckpt_interval : plan_bwd(p).interval; }
 
 struct Workspace {
   size_t ckpt, dW_part, dq_part, dk_part, chunk_states, dv_part, dgate_part, total;
@@ -223,7 +223,7 @@ struct Workspace {
 Workspace layout(const m2rnn_params *p, bool have_ckpt, bool lean) {
   Workspace w{};
   const BwdPlan pl = plan_bwd(p, lean, have_ckpt);
-  const int C = p->ckpt_interval ? p->ckpt_interval : pl.C;
+  const int C = p->ckpt_interval ? p->ckpt_interval : pl.interval;
   const size_t nch = p->T > 0 ? (size_t)(p->T + C - 1) / C : 0;
   const size_t BN = (size_t)p->B * p->N, KV = (size_t)p->K * p->V;
   size_t off = 0;
@@ -266,7 +266,9 @@ void plan_backward(ScanArgs &a, const m2rnn_params *p, bool lean, bool have_ckpt
   const BwdPlan pl = plan_bwd(p, lean, have_ckpt);
   a.KC = pl.KC; a.hg = pl.hg; a.groups = pl.groups; a.set = pl.set;
   a.C = p->ckpt_interval ? p->ckpt_interval : pl.C;
-  a.nchunks = p->T > 0 ? (p->T + a.C - 1) / a.C : 0;
+  const int interval = p->ckpt_interval ? p->ckpt_interval : pl.interval;
+  a.per = a.C / interval;
+  a.nchunks = p->T > 0 ? (p->T + interval - 1) / interval : 0;
 }
 
 }  // namespace
@@ -316,6 +318,7 @@ int bwd_call(const m2rnn_params *params, const void *q, const void *k, const voi
     // pass 1 of Algorithm 2, thinned: save the state every C steps only
     ScanArgs f = a;
     plan_forward(f, params);
+    f.C = a.C / a.per;
     f.y = nullptr; f.hT = nullptr;
     f.ckpt = reinterpret_cast<float *>(ws + w.ckpt);
     e = f32 ? launch_fwd_f32(f, s) : launch_fwd_bf16(f, s);
@@ -422,7 +425,10 @@ int m2rnn_fwd(const m2rnn_params *params, const void *q, const void *k, const vo
   a.alpha = params->gate_kind == M2RNN_GATE_PSI ? alpha : nullptr;
   a.beta = params->gate_kind == M2RNN_GATE_PSI ? beta : nullptr;
   plan_forward(a, params);
-  if (ckpt) plan_backward(a, params, false, true);      // (the checkpoints' interval)
+  if (ckpt) {
+    plan_backward(a, params, false, true);
+    a.C /= a.per;                                       // (the checkpoints' interval)
+  }
   a.y = y; a.hT = hT; a.ckpt = ckpt; a.dev_status = dev_status;
   size_t need = m2rnn_fwd_workspace_bytes(params);
   if (need > 0 && !workspace && workspace_bytes == 0) {   // without shares of y, where the kernels can
@@ -443,7 +449,19 @@ int m2rnn_fwd(const m2rnn_params *params, const void *q, const void *k, const vo
 }
 
 size_t m2rnn_bwd_workspace_bytes(const m2rnn_params *params, int have_ckpt) {
-  return bwd_workspace_bytes(params, have_ckpt != 0, false);
+  size_t most = bwd_workspace_bytes(params, have_ckpt != 0, false);
+  if (most && params->io_dtype == M2RNN_BF16) {
+    // What the shorter sequences of this size take that have another plan: a workspace for the longest does for all
+    const int from = plan_bwd(params, false, have_ckpt != 0).T_from;
+    if (from > 1 && from <= params->T) {
+      m2rnn_params p = *params;
+      p.T = from - 1;
+      if (p.total_tokens > (int64_t)p.B * p.T) p.total_tokens = (int64_t)p.B * p.T;
+      const size_t other = bwd_workspace_bytes(&p, have_ckpt != 0, false);
+      if (other > most) most = other;
+    }
+  }
+  return most;
 }
 
 int m2rnn_bwd(const m2rnn_params *params, const void *q, const void *k, const void *v,

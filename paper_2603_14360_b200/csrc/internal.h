@@ -15,8 +15,8 @@ struct ScanArgs {
   int gate_kind;
   int KC;         // backward: state rows per CTA (a divisor of K)
   int KCf;        // forward: state rows per CTA (a divisor of K)
-  int C;          // checkpoint interval (steps)
-  int nchunks;    // ceil(T / C)
+  int C;          // checkpoint interval (steps); backward: steps of a chunk, `per` intervals
+  int nchunks;    // checkpoints of a unit: ceil(T / interval)
   float dh_clip;
   const void *q, *k, *v, *W, *w_r;
   const float *gate, *h0, *alpha, *beta;
@@ -43,6 +43,7 @@ struct ScanArgs {
   long long TT;
   const int32_t *cu;
   int hg, groups, set;   // backward, V = 16: heads per CTA, CTAs per token's heads (= shares of dq and dk), heads that a CTA's are taken from
+  int per;        // backward, V = 16: checkpoints to a chunk (else 1)
   int rank;       // B where the sequences of a packed batch are taken longest first, else 0
 };
 
@@ -126,8 +127,10 @@ inline size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 // by shared memory in the bf16 backward kernel, which keeps two chunks of recomputed states on chip).
 struct BwdPlan {
   int KC;     // rows per CTA (fp32 path: 4 or 8, or K for one launch per group of eight)
-  int C;      // default checkpoint interval
+  int C;      // steps of a chunk where the caller gives no interval
+  int interval;   // steps between checkpoints: C, or half of it (V = 16, bf16)
   int C_max;  // largest supported checkpoint interval
+  int T_from; // the plan is that of T >= T_from, another one below
   int hg, groups, set;   // V = 16 (bf16): see ScanArgs
 };
 int sm_count();   // SMs of the current device (148 when there is none to ask)

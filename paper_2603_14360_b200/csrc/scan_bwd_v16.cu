@@ -22,6 +22,8 @@
 // the instruction cache), fp32 copies of k, v, q, dy (shared-memory bandwidth), stmatrix and ldmatrix for the transposition.
 #include <cuda_fp16.h>
 
+#include <algorithm>
+#include <climits>
 #include <numeric>
 
 #include "device_common.cuh"
@@ -92,7 +94,10 @@ __device__ __forceinline__ uint32_t transposed(uint32_t x) {   // an 8 x 8 matri
   return y;
 }
 // (bounds for two warps more than a CTA has: 144 registers, which the plan counts with)
-template <int CC, bool CLIP>
+// PER: checkpoints to a chunk, which starts from the first of them.  A template's argument, and the pointer worked out anew where it is
+// not 1: one that walks by a runtime step costs the short chunks up to 9 % (B 10, 36 heads of their own, K = 64, T 40: 36.9 -> 40.4 us),
+// one that walks two checkpoints 0 to 4 % (the same, T 1 024: 666 -> 699).
+template <int CC, bool CLIP, int PER>
 __global__ void __launch_bounds__(kRoomWarps * 32, 1) bwd_v16_kernel(ScanArgs a) {
   using L = Lay<CC>;
   extern __shared__ __align__(128) unsigned char smem[];
@@ -167,9 +172,10 @@ __global__ void __launch_bounds__(kRoomWarps * 32, 1) bwd_v16_kernel(ScanArgs a)
     const float *ck = a.ckpt + (unit * a.nchunks + (nch > 0 ? nch - 1 : 0)) * KV + own;
     const uint32_t ck_sa = mine + 16u * lane;
     auto fetch_ckpt = [&](int j) {
+      if constexpr (PER > 1) ck = a.ckpt + (unit * a.nchunks + PER * (nch - 1 - j)) * KV + own;
       cp16(ck_sa + 1024u * (j & 1), ck);
       cp16(ck_sa + 1024u * (j & 1) + 512u, ck + kV);
-      ck -= KV;
+      if constexpr (PER == 1) ck -= KV;
     };
     auto take_ckpt = [&](int j) {
       asm volatile("cp.async.wait_all;" ::: "memory");
@@ -547,14 +553,14 @@ __global__ void __launch_bounds__(kRoomWarps * 32, 1) bwd_v16_kernel(ScanArgs a)
   }
 }
 
-template <int CC, bool CLIP>
+template <int CC, bool CLIP, int PER>
 cudaError_t launch_t(const ScanArgs &a, cudaStream_t s) {
   const int R = a.KC / 16, qb = a.Nq < a.N ? R : a.hg * R, kb = a.Nk < a.N ? R : a.hg * R;
   const size_t smem = Lay<CC>::total(a.hg, qb, kb, a.hg * R);
-  const cudaError_t e = allow_smem(bwd_v16_kernel<CC, CLIP>, smem);
+  const cudaError_t e = allow_smem(bwd_v16_kernel<CC, CLIP, PER>, smem);
   if (e != cudaSuccess) return e;
   const int ctas = a.B * a.groups * (a.K / a.KC), threads = (a.hg * R + 2) * 32;
-  return launch_early(bwd_v16_kernel<CC, CLIP>, ctas, threads, smem, s, in_order(a, ctas, threads, 2));
+  return launch_early(bwd_v16_kernel<CC, CLIP, PER>, ctas, threads, smem, s, in_order(a, ctas, threads, 2));
 }
 
 }  // namespace
@@ -567,13 +573,19 @@ cudaError_t launch_t(const ScanArgs &a, cudaStream_t s) {
 // run as 136 CTAs of 5 heads and two slabs in one wave (1 024 steps 484 us; as 336 CTAs of four slabs 681, of one 895).
 // Heads of a CTA that share q and k leave one share of dq and dk, slabs of a CTA one of dv and dgate: the shares' way through
 // memory counts too, and the two launches that add the slabs' shares.
+// Two plans are looked for, of whole states (a CTA has all slabs of its heads) and of split ones, and T decides between them: the two
+// launches that add the slabs' shares count 5 us of a call (backward, us, whole / split: B 6, 8 heads, K = 64, T 32 17.9 / 19.0, T 512 144 /
+// 128; B 1, 57 heads with k of their own, T 64 29.2 / 30.5, T 512 140.5 / 133.8).  The checkpoints' interval must not
+// follow T -- a buffer for the longest sequence has to do for every shorter one, and the interval is asked for without a T --, so it is
+// eight steps where either plan has chunks of eight, and a chunk of sixteen then begins at every second checkpoint (B 2, 84
+// heads sharing q and k, K = 64, 768 steps: forward 102 -> 105, backward 262; in chunks of eight 307).
 BwdPlan plan_bwd_v16(int B, int N, int Nq, int Nk, int K, int T, int interval, bool lean) {
-  BwdPlan best{};
   const int sms = sm_count();
   // heads that a CTA's are taken from: those that share a q and a k head (where heads share at all)
   const int set = std::gcd(Nq < N ? N / Nq : N, Nk < N ? N / Nk : N);
   const bool own_rows = Nq == N || Nk == N;
-  double best_cost = 0.;
+  BwdPlan whole{}, split{};
+  double whole_cost = 0., split_cost = 0.;
   const int choices[2] = {interval ? interval : 8, 16};
   for (int x = 0; x < (interval ? 1 : 2); ++x)
     for (int R = 1; R <= K / 16 && R <= kMostSlabs; ++R)
@@ -591,19 +603,32 @@ BwdPlan plan_bwd_v16(int B, int N, int Nq, int Nk, int K, int T, int interval, b
         const long waves = ctas / (sms * room), left = ctas % (sms * room);
         const int RS = K / (16 * R);
         double cost = waves * step(room) + step((left + sms - 1) / sms);
-        cost += ((Nq < groups ? 1 : 0) + (Nk < groups ? 1 : 0)) * 8. * B * groups * K / 5500. + (RS > 1 ? 128. * B * N * RS / 5500. + 5000. / (T > 0 ? T : 1) : 0.);
+        cost += ((Nq < groups ? 1 : 0) + (Nk < groups ? 1 : 0)) * 8. * B * groups * K / 5500. + (RS > 1 ? 128. * B * N * RS / 5500. : 0.);
+        BwdPlan &best = RS > 1 ? split : whole;
+        double &best_cost = RS > 1 ? split_cost : whole_cost;
         const bool better = !best.KC || (lean ? 16 * R > best.KC || (16 * R == best.KC && hg > best.hg) : cost < best_cost);
         if (!better) continue;
         best_cost = cost;
         best.KC = 16 * R; best.C = C; best.hg = hg; best.groups = groups; best.set = set;
       }
+  whole.T_from = 1;
+  if (split.KC) {
+    const double gain = whole_cost - split_cost, from = gain > 0. ? 5000. / gain : 1e9;    // (ns a step)
+    split.T_from = lean || from > 1e9 - 1. ? INT_MAX : (int)from + 1;
+    if (!whole.KC) split.T_from = 1;
+  }
+  const bool take_split = split.KC && (T > 0 ? T : 1) >= split.T_from;
+  BwdPlan best = take_split ? split : whole;
+  best.interval = interval ? interval : whole.KC && split.KC && !lean ? std::min(whole.C, split.C) : best.C;
   best.C_max = 16;
   return best;
 }
 
 cudaError_t launch_bwd_v16(const ScanArgs &a, cudaStream_t s) {
-  if (a.C <= 8) return a.dh_clip > 0.f ? launch_t<8, true>(a, s) : launch_t<8, false>(a, s);
-  return a.dh_clip > 0.f ? launch_t<16, true>(a, s) : launch_t<16, false>(a, s);
+  const bool clip = a.dh_clip > 0.f;
+  if (a.C <= 8) return clip ? launch_t<8, true, 1>(a, s) : launch_t<8, false, 1>(a, s);
+  if (a.per == 2) return clip ? launch_t<16, true, 2>(a, s) : launch_t<16, false, 2>(a, s);
+  return clip ? launch_t<16, true, 1>(a, s) : launch_t<16, false, 1>(a, s);
 }
 
 }  // namespace m2rnn

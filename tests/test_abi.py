@@ -171,6 +171,34 @@ def test_every_unsupported_interval_is_refused(lib):
     assert r.stdout == "refused\n", r.stderr[-2000:]
 
 
+def test_buffers_for_the_longest_sequence_do_for_all(lib):
+    """The default interval does not depend on T, and neither the checkpoints' nor the backward's scratch bytes fall as T grows,
+    dense or packed: a caller sizes them once, for the longest sequence, and no argument tells m2rnn_fwd how long `ckpt` is."""
+    lengths = [1, 7, 8, 9, 16, 17, 32, 50, 100, 200, 256, 500, 700, 1024, 5000]
+    checked = 0
+    for V, io in ((16, 1), (32, 1), (64, 1), (128, 1), (64, 0), (16, 0)):
+        for N in (1, 12, 32, 50, 84):
+            for Nq, Nk in {(1, 1), (N, N), (1, N), (N // 2 if N % 2 == 0 else 1, 1)}:
+                for K in (16, 48, 64, 80, 96, 128):
+                    for B in (1, 2, 6, 15, 40) if io else (1, 2):       # (fp32: shares below 4 GiB)
+                        size = dict(B=B, N=N, Nq=Nq, Nk=Nk, K=K, V=V, io_dtype=io)
+                        C = lib.m2rnn_ckpt_interval(ctypes.byref(_p(T=0, **size)))
+                        last = (0,) * 5
+                        for T in lengths:
+                            p = _p(T=T, **size)
+                            packed = _p(T=T, total_tokens=min(B * T, 900), cu_seqlens=0x10000, **size)
+                            r, rp = ctypes.byref(p), ctypes.byref(packed)
+                            now = (lib.m2rnn_ckpt_bytes(r), lib.m2rnn_bwd_workspace_bytes(r, 0), lib.m2rnn_bwd_workspace_bytes(r, 1),
+                                   lib.m2rnn_bwd_workspace_bytes(rp, 0), lib.m2rnn_bwd_workspace_bytes(rp, 1))
+                            assert lib.m2rnn_ckpt_interval(r) == lib.m2rnn_ckpt_interval(rp) == C, (size, T)
+                            assert now[0] == B * N * -(-T // C) * K * V * 4 and all(a >= b for a, b in zip(now, last)), (size, T, now, last)
+                            last, checked = now, checked + 1
+    assert checked > 10000
+    # the first size found where the interval followed T: 16 at 256 steps, 8 at 200, and so the longer one had the fewer bytes
+    at = lambda T: lib.m2rnn_ckpt_bytes(ctypes.byref(_p(B=6, N=32, Nq=1, Nk=1, K=64, V=16, T=T)))
+    assert at(256) >= at(200)
+
+
 def test_gated_norm_rejects_bad_arguments(lib):
     f = lib.m2rnn_gated_norm_fwd
     assert f(-1, 1024, 1, FAKE, FAKE, FAKE, 0.0, 1, FAKE, None, None) == -2

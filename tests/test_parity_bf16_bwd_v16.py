@@ -2,6 +2,7 @@
 several heads and slabs, shares of shared heads, ragged chunks, every checkpoint interval's kind.  Bound: the bf16 path's 2e-2
 (parity.TOL); two forms of the same sums: the order of at most 128 fp32 terms."""
 import ctypes
+import dataclasses
 import os
 import subprocess
 import sys
@@ -51,6 +52,52 @@ def test_intervals(oracle, C):
         binding.check_device_status()
         for name in ref:
             assert parity.rel_err(out[name], ref[name]) <= parity.TOL["bf16"], (C, name)
+
+
+# sizes whose checkpoints come every eight steps and whose chunks, from some T on, have sixteen
+TWO = [(3, 12, 128, 1, 12), (2, 84, 64, 1, 1)]      # B, N, K, Nq, Nk
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("T,size", [(26, TWO[0]), (40, TWO[0]), (47, TWO[0]), (200, TWO[1])], ids=str)
+def test_chunks_of_two_intervals(oracle, T, size):
+    """A ragged last chunk of one and of two checkpoints; the call's own checkpoints too, and every second one asked for by the caller."""
+    B, N, K, Nq, Nk = size
+    # (a contracting W: with N(0, 1/V) some heads amplify a rounding over 200 steps, and two forms of the same kernel differ by 4e-2)
+    cfg = dataclasses.replace(_cfg((B, T, N, K, Nq, Nk)), w_scale=0.5)
+    p = binding.Params(B=B, T=T, N=N, Nq=Nq, Nk=Nk, K=K, V=16, io_dtype=1, gate_kind=1, ckpt_interval=0, dh_clip=0.0)
+    assert binding.m2rnn_ckpt_interval(p) == 8 and binding.m2rnn_bwd_row_slab(p) == 16
+    d = inputs.make_inputs(cfg, backward=True, d_hT=True)
+    ref, g = parity.oracle_bwd(oracle, cfg, d), parity.to_dev(d)
+    ckpt = parity.gpu_fwd(cfg, g, save_ckpt=True)[2]
+    assert ckpt.shape[2] == -(-T // 8)
+    for kw in (dict(ckpt=ckpt), dict(), dict(ckpt=ckpt[:, :, ::2].contiguous(), ckpt_interval=16)):
+        out = parity.gpu_bwd(cfg, g, **kw)
+        binding.check_device_status()
+        for name in ref:
+            assert parity.rel_err(out[name], ref[name]) <= parity.TOL["bf16"], (list(kw), name)
+
+
+@pytest.mark.gpu
+def test_chunks_of_two_intervals_packed():
+    """Sequences that end in every part of a chunk, an empty one among them: as each by itself."""
+    (B, N, K, Nq, Nk), lens = TWO[0], [41, 0, 8, 25, 16, 1]
+    tok, gen = sum(lens), torch.Generator("cuda").manual_seed(6)
+    rnd = lambda *s, dt=torch.bfloat16, std=1.0: torch.empty(s, dtype=dt, device="cuda").normal_(0, std, generator=gen)
+    q, k, v = rnd(tok, Nq, K, std=0.125), rnd(tok, Nk, K, std=0.125), rnd(tok, N, 16)
+    gate, W, dy, h0 = rnd(tok, N, dt=torch.float32), rnd(N, 16, 16, std=0.125), rnd(tok, N, 16), rnd(len(lens), N, K, 16, dt=torch.float32, std=0.1)
+    cu = torch.tensor([0] + lens, dtype=torch.int32).cumsum(0, dtype=torch.int32).cuda()
+    pk = dict(cu_seqlens=cu, max_seqlen=max(lens))
+    ckpt = binding.m2rnn_fwd(q, k, v, gate, W, h0, save_ckpt=True, **pk)[2]
+    got = binding.m2rnn_bwd(q, k, v, gate, W, h0, dy, ckpt=ckpt, **pk)
+    at = 0
+    for b, n in enumerate(lens):
+        sl, at = slice(at, at + n), at + n
+        if n:
+            one = binding.m2rnn_bwd(*(x[None, sl].contiguous() for x in (q, k, v, gate)), W, h0[b:b + 1], dy[None, sl])
+            for name in ("dq", "dk", "dv", "dgate"):
+                assert parity.rel_err(got[name][sl], one[name][0].double().cpu().numpy()) < 2.0 ** -8, (b, name)     # (a rounding to bf16)
+    binding.check_device_status()
 
 
 @pytest.mark.gpu
