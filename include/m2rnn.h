@@ -122,8 +122,9 @@ size_t m2rnn_ckpt_bytes(const m2rnn_params *params);
  * through this scratch before a second launch adds them.  It splits where there are few (b,n) units, to
  * fill the GPU; M2RNN_F32 states also into groups of four rows (V = 16: where groups of four or eight make more warps),
  * M2RNN_BF16 states of K > 64, 32 <= V <= 64 into slabs of at most 64 rows -- both for speed only and
- * up to 4 GiB of shares: m2rnn_fwd also takes those two without a workspace, on whole states and slower
- * (fp32, 16 units of K = V = 64: 10.6 times; bf16, 192 units of K = 96, V = 64: 2.3 times). */
+ * up to 4 GiB of shares (M2RNN_F32 with few units: 8), beyond which M2RNN_F32 takes groups of eight rows or whole
+ * states: m2rnn_fwd also takes those two without a workspace, on whole states and slower
+ * (fp32, 16 units of K = V = 64: 10.6 times, 2 048 units 1.2 times; bf16, 192 units of K = 96, V = 64: 2.3 times). */
 size_t m2rnn_fwd_workspace_bytes(const m2rnn_params *params);
 
 /* Forward scan (Algorithm 1; Eq. 1-3).

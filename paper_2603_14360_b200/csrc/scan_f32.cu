@@ -1009,8 +1009,13 @@ cudaError_t launch_decode_v(const ScanArgs &a, cudaStream_t s) {
 }  // namespace
 
 // Rows per CTA.  The step of a warp is a chain of dependent instructions, so a problem wants its rows spread over many warps.
-// Forward, V >= 32: groups of four rows (fwd_f32_wide_kernel), at any number of units (512 steps of K = V = 64, us, against the
-// kernel of eight lanes a column, in groups of four, of eight and whole states: 16 units 370 -> 206, 64 1005 -> 638, 256 1617 -> 1081).
+// Forward, V >= 32: groups of four rows (fwd_f32_wide_kernel), at any number of units that their shares of y leave room for.  256
+// steps, us, groups of four / of eight / whole states: K = V = 64, 16 units 106 / 194 / 1 097, 128 625 / 836 / 1 098, 512 2 137 / 3 183 / 3 153, 2 048
+// 8 443 / 12 486 / 10 372; K = V = 32, 2 048 units 1 631 / 2 422 / 2 002; K = V = 128, 16 units 548 / 759 / 4 539, 256 7 355 / 10 580 / 9 073.  The shares
+// are memory bought for that 18 to 50 %, 4 GiB of the GPU's 180 at most.  Where groups of four would need more, groups of eight while
+// the units alone leave an SM fewer than 16 warps and their shares fit (four sequences of 32 768 tokens, ten heads of K = V = 64, ms: 34 by
+// groups of four in 5 GiB, 46 in 2.5, whole states 139); whole states beyond.  Where groups of eight would leave an SM fewer than 16 warps
+// it is groups of four up to 8 GiB (one of 70 000, 16 heads: 27 against 51 and 298).
 // V = 16 and the backward: groups of four rows while groups of eight would leave an SM fewer than 16 warps (V = 64: 32), else of eight,
 // which need fewer instructions in all.  Whole states forward (V = 16) where that gives every SM 16 warps -- the groups take turns
 // behind one barrier a step and y needs no shares in memory.  Backward: K stands for one launch per group of eight, each adding to
@@ -1018,8 +1023,8 @@ cudaError_t launch_decode_v(const ScanArgs &a, cudaStream_t s) {
 // states (one group after the other) too where the shares of all groups would exceed kMaxShares.
 constexpr size_t kMaxShares = (size_t)4 << 30;
 int fwd_f32_rows(int B, int N, int K, int V, size_t share_bytes) {
-  if (V >= 32) return share_bytes * (K / (kRows / 2)) > kMaxShares ? K : kRows / 2;
   const long warps = (long)(B > 0 ? B : 1) * N * (V / 8), most = 16L * sm_count();   // of whole states
+  if (V >= 32 && share_bytes * (K / (kRows / 2)) <= kMaxShares) return kRows / 2;
   if (warps >= most || share_bytes * (K / kRows) > kMaxShares) return K;
   return warps * (K / kRows) >= most ? kRows : kRows / 2;
 }

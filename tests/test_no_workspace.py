@@ -56,3 +56,36 @@ def test_whole_states_without_a_workspace(oracle, case):
     assert parity.rel_err(whole[0], y_ref) <= parity.TOL[dtype] and parity.rel_err(whole[1], hT_ref) <= parity.TOL[dtype]
     if dtype == "f32":      # the same sums in the same order, however a state is split
         assert all(torch.equal(a, b) for a, b in zip(split, whole))
+
+
+# B, T, N, K, V, shares of y: where groups of four rows would need more than 4 GiB.  As groups of four while groups of eight would leave
+# an SM idle, as groups of eight, on whole states (where those make 16 warps an SM, or eight do not fit either)
+LARGE = [(1, 65537, 16, 64, 64, 16), (1, 131072, 16, 64, 64, 16), (4, 32768, 10, 64, 64, 8), (4, 8193, 16, 128, 64, 16), (4, 16384, 16, 128, 64, 16),
+         (4, 8192, 16, 128, 128, 16), (4, 16384, 20, 128, 32, 16), (1, 131073, 16, 64, 64, 1), (8, 2049, 64, 64, 64, 1), (8, 2048, 64, 64, 64, 16)]
+
+
+@pytest.mark.parametrize("case", LARGE, ids=lambda c: "x".join(map(str, c)))
+def test_rows_of_large_fp32_problems(case):
+    B, T, N, K, V, shares = case
+    p = binding.Params(B=B, T=T, N=N, Nq=N, Nk=N, K=K, V=V, io_dtype=0, gate_kind=1, ckpt_interval=0, dh_clip=0.0)
+    assert binding.m2rnn_fwd_workspace_bytes(p) == (shares * B * T * N * V * 4 if shares > 1 else 0)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("case", [LARGE[0], LARGE[2], LARGE[5], LARGE[6]], ids=lambda c: "x".join(map(str, c)))
+def test_large_fp32_problems_match_whole_states(case):
+    """States: bit for bit, however they are split; y too in groups of four rows.  Groups of eight add their two fours first: two orders
+    of K / 4 terms each, which differ by at most 2 (K / 4) 2^-24 of the sum of |q_r H_r|, and |H| <= 1 (a mean of tanh and an h0 below 1)."""
+    B, T, N, K, V, shares = case
+    gen = torch.Generator("cuda").manual_seed(8)
+    rnd = lambda *s, std=1.0: torch.empty(s, device="cuda").normal_(0, std, generator=gen)
+    q, k, v = rnd(B, T, 1, K, std=K ** -0.5), rnd(B, T, 1, K, std=K ** -0.5), rnd(B, T, N, V)
+    args = [q, k, v, rnd(B, T, N) + 1.0, rnd(N, V, V, std=0.5 * V ** -0.5), rnd(B, N, K, V, std=0.1)]
+    split = binding.m2rnn_fwd(*args)
+    whole = binding.m2rnn_fwd(*args, workspace=torch.empty(0, dtype=torch.uint8, device="cuda"))
+    binding.check_device_status()
+    assert torch.equal(split[1], whole[1]) and args[5].abs().max() < 1
+    if shares == K // 4:
+        assert torch.equal(split[0], whole[0])
+    else:
+        assert ((split[0] - whole[0]).abs().amax(-1) <= K / 2 * 2.0 ** -24 * q.abs().sum(-1)).all()
