@@ -388,8 +388,13 @@ int bwd_steps(int B, int T, int C, int io_dtype) {
   if (rule < 64 || cols * tiles(T, 64) > 16 * slots) return rule;      // (many rounds: their last does not count)
   int best = 64;
   long best_cost = (cols * tiles(T, 64) + slots - 1) / slots * (64 + 3 + 8);
-  for (int n = 1, most = tiles(T, 48); n <= most && (long)B * n <= 65535; ++n) {        // n tiles a sequence
-    const int steps = (T + kSub * n - 1) / (kSub * n);
+  // Of the runs that take `rounds` rounds the shortest costs least: as many tiles a sequence as fill them.  (No more than 22 to look at:
+  // up to 16 rounds of runs of 64, and runs no shorter than 48.)
+  const long most = std::min<long>(tiles(T, 48), 65535 / B);
+  for (long rounds = 1, n = 0; n < most; ++rounds) {
+    n = std::min(most, rounds * slots / cols);
+    if (n < 1) continue;
+    const int steps = (int)((T + kSub * n - 1) / (kSub * n));
     const long cost = (cols * tiles(T, steps) + slots - 1) / slots * (steps + 3 + 8);
     if (cost < best_cost) { best = steps; best_cost = cost; }
   }

@@ -1,10 +1,13 @@
 """Host-side checks of the C ABI that need no GPU: the library loads, exports every symbol
 the header declares, and rejects bad arguments before launching anything."""
 import ctypes
+import math
 import os
+import random
 import re
 import subprocess
 import sys
+import timeit
 
 import pytest
 
@@ -150,6 +153,31 @@ def test_plans_for_small_states_with_many_units(lib):
     # a caller may still ask for a longer chunk, up to what one CTA's shared memory holds
     assert lib.m2rnn_ckpt_interval(ctypes.byref(_p(B=4, N=84, Nq=1, Nk=1, K=64, V=16, T=64, ckpt_interval=12))) == 12
     assert lib.m2rnn_ckpt_interval(ctypes.byref(_p(B=4, N=84, Nq=1, Nk=1, K=64, V=16, T=64, ckpt_interval=18))) == -3
+
+
+def _conv_bwd_tiles(B, T, C, per_sm, sms=148):
+    """Tiles a sequence of the conv's backward, by trying every length of a run."""
+    tiles = lambda steps: -(-T // (4 * steps))
+    cols, slots = B * -(-(C // 4) // 32), sms * per_sm
+    if cols * tiles(64) < 2 * sms:
+        return tiles(16 if cols * tiles(16) <= sms else 32)
+    if cols * tiles(64) > 16 * slots:
+        return tiles(64)
+    cost = lambda steps: -(-cols * tiles(steps) // slots) * (steps + 11)
+    runs = [64] + [-(-T // (4 * n)) for n in range(1, min(tiles(48), 65535 // B) + 1)]
+    return tiles(min(runs, key=cost))
+
+
+def test_conv_backward_runs(lib):
+    """The scratch of the conv's backward (five sums a channel and tile, for the type that takes more of them) is that of the best run
+    over all lengths, and finding it is not a search over all of them: the query of a long sequence takes microseconds."""
+    rng = random.Random(3)
+    sizes = [(1, 1000000, 128), (1, 65536, 256), (8, 2048, 3072), (1, 70000, 8), (3, 20000, 8192), (65535, 300, 8), (30000, 600, 8)]
+    sizes += [(rng.randint(1, 64), int(math.exp(rng.uniform(1, 12))), 8 * int(math.exp(rng.uniform(0, 7)))) for _ in range(150)]
+    for B, T, C in sizes:
+        most = max(_conv_bwd_tiles(B, T, C, 4), _conv_bwd_tiles(B, T, C, 2))
+        assert lib.m2rnn_conv_silu_bwd_workspace_bytes(B, T, C) == -(-B * most * 5 * C * 4 // 256) * 256, (B, T, C)
+    assert min(timeit.repeat(lambda: lib.m2rnn_conv_silu_bwd_workspace_bytes(1, 1000000, 128), number=100, repeat=10)) < 100 * 20e-6
 
 
 def test_every_unsupported_interval_is_refused(lib):
