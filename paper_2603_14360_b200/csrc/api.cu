@@ -4,6 +4,7 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <atomic>
 #include <cstdlib>
 #include <cstring>
@@ -220,9 +221,8 @@ struct Workspace {
   size_t ckpt, dW_part, dq_part, dk_part, chunk_states, dv_part, dgate_part, total;
 };
 
-Workspace layout(const m2rnn_params *p, bool have_ckpt, bool lean) {
+Workspace layout(const m2rnn_params *p, const BwdPlan &pl, bool have_ckpt) {
   Workspace w{};
-  const BwdPlan pl = plan_bwd(p, lean, have_ckpt);
   const int C = p->ckpt_interval ? p->ckpt_interval : pl.interval;
   const size_t nch = p->T > 0 ? (size_t)(p->T + C - 1) / C : 0;
   const size_t BN = (size_t)p->B * p->N, KV = (size_t)p->K * p->V;
@@ -262,8 +262,7 @@ ScanArgs base_args(const m2rnn_params *p) {
 }
 // (plans only where a call uses them: they are a part of a small call's host time)
 void plan_forward(ScanArgs &a, const m2rnn_params *p) { a.KCf = plan_fwd_rows(p->B, p->N, p->K, p->V, p->io_dtype, tokens_of(p)); }
-void plan_backward(ScanArgs &a, const m2rnn_params *p, bool lean, bool have_ckpt) {
-  const BwdPlan pl = plan_bwd(p, lean, have_ckpt);
+void plan_backward(ScanArgs &a, const m2rnn_params *p, const BwdPlan &pl) {
   a.KC = pl.KC; a.hg = pl.hg; a.groups = pl.groups; a.set = pl.set;
   a.C = p->ckpt_interval ? p->ckpt_interval : pl.C;
   const int interval = p->ckpt_interval ? p->ckpt_interval : pl.interval;
@@ -275,7 +274,7 @@ void plan_backward(ScanArgs &a, const m2rnn_params *p, bool lean, bool have_ckpt
 
 size_t bwd_workspace_bytes(const m2rnn_params *params, bool have_ckpt, bool lean) {
   if (check_params(params, true) != M2RNN_OK) return 0;
-  return layout(params, have_ckpt, lean).total;
+  return layout(params, plan_bwd(params, lean, have_ckpt), have_ckpt).total;
 }
 
 int bwd_call(const m2rnn_params *params, const void *q, const void *k, const void *v, const float *gate, const void *W,
@@ -301,13 +300,14 @@ int bwd_call(const m2rnn_params *params, const void *q, const void *k, const voi
   const void *ptrs[] = {q, k, v, gate, W, h0, w_r, ckpt, dy, d_hT, dq, dk, dv, dgate, dW, dh0};
   for (const void *p : ptrs)
     if (!aligned16(p)) return M2RNN_ERR_ALIGN;
-  const Workspace w = layout(params, ckpt != nullptr, lean);
+  const BwdPlan pl = plan_bwd(params, lean, ckpt != nullptr);
+  const Workspace w = layout(params, pl, ckpt != nullptr);
   if (w.total > 0 && (!workspace || workspace_bytes < w.total)) return M2RNN_ERR_WORKSPACE;
   if (reinterpret_cast<uintptr_t>(workspace) % kAlign) return M2RNN_ERR_ALIGN;
   char *ws = static_cast<char *>(workspace);
 
   ScanArgs a = base_args(params);
-  plan_backward(a, params, lean, ckpt != nullptr);
+  plan_backward(a, params, pl);
   a.q = q; a.k = k; a.v = v; a.gate = gate; a.W = W; a.h0 = h0; a.w_r = w_r;
   a.alpha = params->gate_kind == M2RNN_GATE_PSI ? alpha : nullptr;
   a.beta = params->gate_kind == M2RNN_GATE_PSI ? beta : nullptr;
@@ -426,7 +426,7 @@ int m2rnn_fwd(const m2rnn_params *params, const void *q, const void *k, const vo
   a.beta = params->gate_kind == M2RNN_GATE_PSI ? beta : nullptr;
   plan_forward(a, params);
   if (ckpt) {
-    plan_backward(a, params, false, true);
+    plan_backward(a, params, plan_bwd(params));
     a.C /= a.per;                                       // (the checkpoints' interval)
   }
   a.y = y; a.hT = hT; a.ckpt = ckpt; a.dev_status = dev_status;
@@ -449,17 +449,15 @@ int m2rnn_fwd(const m2rnn_params *params, const void *q, const void *k, const vo
 }
 
 size_t m2rnn_bwd_workspace_bytes(const m2rnn_params *params, int have_ckpt) {
-  size_t most = bwd_workspace_bytes(params, have_ckpt != 0, false);
-  if (most && params->io_dtype == M2RNN_BF16) {
+  if (check_params(params, true) != M2RNN_OK) return 0;
+  const BwdPlan pl = plan_bwd(params, false, have_ckpt != 0);
+  size_t most = layout(params, pl, have_ckpt != 0).total;
+  if (pl.T_from > 1 && pl.T_from <= params->T) {
     // What the shorter sequences of this size take that have another plan: a workspace for the longest does for all
-    const int from = plan_bwd(params, false, have_ckpt != 0).T_from;
-    if (from > 1 && from <= params->T) {
-      m2rnn_params p = *params;
-      p.T = from - 1;
-      if (p.total_tokens > (int64_t)p.B * p.T) p.total_tokens = (int64_t)p.B * p.T;
-      const size_t other = bwd_workspace_bytes(&p, have_ckpt != 0, false);
-      if (other > most) most = other;
-    }
+    m2rnn_params p = *params;
+    p.T = pl.T_from - 1;
+    if (p.total_tokens > (int64_t)p.B * p.T) p.total_tokens = (int64_t)p.B * p.T;
+    most = std::max(most, layout(&p, plan_bwd(&p, false, have_ckpt != 0), have_ckpt != 0).total);
   }
   return most;
 }
