@@ -270,7 +270,11 @@ PyObject *py_fwd(PyObject *, PyObject *const *a, Py_ssize_t n) {
   Tensor hT, ckpt, ws;
   if (const Tensor *t = opt_tensor(a[14], "hT")) hT = *t;
   else if (truth(a[12])) hT = empty({p.B, p.N, p.K, p.V}, ScalarType::Float, dev);
-  if (const Tensor *t = opt_tensor(a[15], "ckpt")) ckpt = *t;
+  if (const Tensor *t = opt_tensor(a[15], "ckpt")) {
+    ckpt = *t;
+    if (!ckpt.is_cuda()) fail(PyExc_ValueError, "ckpt must be a CUDA tensor");
+    if (ckpt.nbytes() < m2rnn_ckpt_bytes(&p)) fail(PyExc_ValueError, "ckpt: smaller than m2rnn_ckpt_bytes");   // (the call itself cannot tell)
+  }
   else if (truth(a[10])) {
     const int C = interval(p);
     ckpt = empty({p.B, p.N, (p.T + C - 1) / C, p.K, p.V}, ScalarType::Float, dev);

@@ -74,3 +74,16 @@ def test_conv_refuses_a_cpu_tensor(fake, bwd, arg):
             binding.m2rnn_conv_silu_bwd(a["x"], a["w"], a["dout"], a["bias"], a["prev"])
         else:
             binding.m2rnn_conv_silu_fwd(a["x"], a["w"], a["bias"], a["prev"])
+
+
+@pytest.mark.parametrize("T,interval,steps", [(256, 0, 200), (200, 8, 192), (9, 2, 8)])
+def test_scan_refuses_a_checkpoint_tensor_that_is_too_small(fake, T, interval, steps):
+    """The library is not told how long `ckpt` is: 6 sequences of 32 heads, whose checkpoints come every eight steps unless asked otherwise."""
+    B, N, K, V, f32 = 6, 32, 64, 16, torch.float32
+    q, k, v, W = fake(B, T, 1, K), fake(B, T, 1, K), fake(B, T, N, V), fake(N, V, V)
+    out = dict(y=fake(B, T, N, V), hT=fake(B, N, K, V, dtype=f32), ckpt=fake(B, N, steps // (interval or 8), K, V, dtype=f32))
+    with pytest.raises(ValueError, match="^ckpt: smaller"):
+        binding.m2rnn_fwd(q, k, v, fake(B, T, N, dtype=f32), W, save_ckpt=True, ckpt_interval=interval, out=out)
+    out["ckpt"] = fake(B, N, T, K, V, dtype=f32, device="cpu")
+    with pytest.raises(ValueError, match="^ckpt must be a CUDA tensor"):
+        binding.m2rnn_fwd(q, k, v, fake(B, T, N, dtype=f32), W, save_ckpt=True, ckpt_interval=interval, out=out)
