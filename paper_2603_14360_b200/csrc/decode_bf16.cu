@@ -52,10 +52,6 @@ __device__ __forceinline__ void a_fragment(const float (&H)[NT][4], int kt, uint
   }
 }
 
-__device__ __forceinline__ void cp16(uint32_t dst_sa, const float *src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst_sa), "l"(src) : "memory");
-}
-
 template <int V>
 __global__ void __launch_bounds__(32 * DecCfg<V>::kWarps, 1) decode_bf16_kernel(ScanArgs a, int per, int extra) {
   using Cfg = DecCfg<V>;

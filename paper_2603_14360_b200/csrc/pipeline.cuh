@@ -89,6 +89,15 @@ __device__ __forceinline__ void sts32(uint32_t addr, float v) {
   asm volatile("st.shared.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
 }
 
+// asynchronous copy of 16 bytes from global to shared memory
+__device__ __forceinline__ void cp16(uint32_t dst_sa, const void *src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst_sa), "l"(src) : "memory");
+}
+// arrives at the barrier once this thread's copies so far have landed (counted among the barrier's arrivals)
+__device__ __forceinline__ void cp_arrive(uint64_t *bar) {
+  asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+
 // 8 bf16 (one 16-byte load) widened to 8 floats in shared memory
 __device__ __forceinline__ void store8_bf16_as_f32(float *dst, const uint4 raw) {
   float4 lo, hi;

@@ -24,8 +24,6 @@
 // buffers).  Hand-over is by mbarriers; every wait is bounded and reports through dev_status.
 // Sums over rows that span CTAs (dv, dgate, dW) and over batch (dW) or shared heads (dq, dk) are
 // finished by fixed-order second-stage kernels.
-#include <cuda_fp16.h>
-
 #include "device_common.cuh"
 #include "internal.h"
 #include "mma_tile.cuh"
@@ -37,22 +35,6 @@ namespace {
 
 constexpr int kRing = 4;         // chunk slots of staged inputs / outputs in flight
 constexpr int kBarBytes = 256;   // room for the mbarriers below
-
-__device__ __forceinline__ uint32_t pack_f16(float lo, float hi) {
-  uint32_t r;
-  asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
-  return r;
-}
-__device__ __forceinline__ float2 unpack_f16(uint32_t x) {
-  return __half22float2(*reinterpret_cast<const __half2 *>(&x));
-}
-__device__ __forceinline__ float2 unpack_bf16(uint32_t x) {
-  return make_float2(__uint_as_float(x << 16), __uint_as_float(x & 0xffff0000u));
-}
-
-__device__ __forceinline__ void ldmatrix_x4(uint32_t addr, uint32_t (&r)[4]) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
-}
 
 // Register re-balancing between warpgroups (4 aligned warps): the kernel is compiled for an even
 // split (128 per thread here), then the chain warps take registers that the dW and service warps

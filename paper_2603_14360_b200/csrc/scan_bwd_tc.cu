@@ -35,8 +35,6 @@
 // product read the other.  Hand-over is by mbarriers; every wait is bounded and reports through
 // dev_status; a common exit frees the tensor memory.  Row-slab sums (dv, dgate, dW) are finished
 // by the second-stage kernels.
-#include <cuda_fp16.h>
-
 #include "device_common.cuh"
 #include "internal.h"
 #include "mma_tile.cuh"
@@ -94,12 +92,6 @@ __device__ __forceinline__ uint32_t slab_off(int i, int l) {
 __device__ __forceinline__ void ldmatrix_x4_trans(uint32_t addr, uint32_t (&r)[4]) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
 }
-__device__ __forceinline__ uint32_t pack_f16x2(float lo, float hi) {
-  uint32_t r;
-  asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
-  return r;
-}
-__device__ __forceinline__ float2 unpack_f16x2(uint32_t x) { return __half22float2(*reinterpret_cast<const __half2 *>(&x)); }
 
 __global__ void __launch_bounds__(kThreads, 1) bwd_tc_kernel(ScanArgs a) {
   using S = TcBwdSmem;
@@ -280,7 +272,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_tc_kernel(ScanArgs a) {
           for (int r = 0; r < kNT; r += 2) {
             const float2 kk = make_float2(__uint_as_float(k8[r / 2] << 16), __uint_as_float(k8[r / 2] & 0xffff0000u));
             const float2 hp = make_float2(__uint_as_float(hw[r / 2] << 16), __uint_as_float(hw[r / 2] & 0xffff0000u));
-            const float2 z = unpack_f16x2(zw[r / 2]);
+            const float2 z = unpack_f16(zw[r / 2]);
             const float2 G = make_float2(fma_bf16<0, 0>(q8[r / 2], dyj, Cg[r]), fma_bf16<1, 0>(q8[r / 2], dyj, Cg[r + 1]));                       // G = C + q dy^T
             df2 = __ffma2_rn(G, __ffma2_rn(z, make_float2(-1.f, -1.f), hp), df2);                                          // df = sum G (.) (H_{t-1} - Z)
             const float2 x2 = __fmul2_rn(__fmul2_rn(make_float2(-omf, -omf), G), __ffma2_rn(z, z, make_float2(-1.f, -1.f)));   // (1-f) G (1 - Z^2)
@@ -318,7 +310,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_tc_kernel(ScanArgs a) {
             const float2 d = __ffma2_rn(z, make_float2(-1.f, -1.f), make_float2(H[r], H[r + 1]));             // H_{t-1} - Z
             const float2 h = __ffma2_rn(make_float2(f, f), d, z);                                           // Eq. 2
             H[r] = h.x; H[r + 1] = h.y;
-            zw[r / 2] = pack_f16x2(z.x, z.y);
+            zw[r / 2] = pack_f16(z.x, z.y);
           }
           *reinterpret_cast<uint4 *>(base + (blkR - base_sa) + priv) = make_uint4(zw[0], zw[1], zw[2], zw[3]);
         }

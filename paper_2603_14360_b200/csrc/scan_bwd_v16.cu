@@ -20,8 +20,6 @@
 // Backward of that shape, 1 024 steps: 796 us with four kinds of warps that handed states over through shared memory, two waves,
 // and a share of dq and dk per head; 465 now.  Tried and slower: states of a chunk in registers (eight steps unrolled twice:
 // the instruction cache), fp32 copies of k, v, q, dy (shared-memory bandwidth), stmatrix and ldmatrix for the transposition.
-#include <cuda_fp16.h>
-
 #include <algorithm>
 #include <climits>
 #include <numeric>
@@ -57,13 +55,6 @@ struct Lay {
 constexpr int kMostSlabs = 10;   // slab warps of a CTA
 constexpr int kRoomWarps = 14;   // warps of an SM with the kernel's registers
 
-__device__ __forceinline__ uint32_t pack_f16(float lo, float hi) {
-  uint32_t r;
-  asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
-  return r;
-}
-__device__ __forceinline__ float2 unpack_f16(uint32_t x) { return __half22float2(*reinterpret_cast<const __half2 *>(&x)); }
-__device__ __forceinline__ float2 unpack_bf16(uint32_t x) { return make_float2(__uint_as_float(x << 16), __uint_as_float(x & 0xffff0000u)); }
 __device__ __forceinline__ uint32_t ldsu32(uint32_t addr) {
   uint32_t x;
   asm volatile("ld.shared.b32 %0, [%1];" : "=r"(x) : "r"(addr));
@@ -81,12 +72,6 @@ __device__ __forceinline__ uint4 get128(uint32_t addr) {
 }
 __device__ __forceinline__ void put128(uint32_t addr, const uint4 x) {
   asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(x.x), "r"(x.y), "r"(x.z), "r"(x.w) : "memory");
-}
-__device__ __forceinline__ void cp16(uint32_t dst_sa, const void *src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst_sa), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_arrive(uint64_t *bar) {
-  asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 __device__ __forceinline__ uint32_t transposed(uint32_t x) {   // an 8 x 8 matrix, two entries of a row a thread
   uint32_t y;

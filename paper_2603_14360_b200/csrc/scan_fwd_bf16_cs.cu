@@ -81,10 +81,6 @@ __host__ __device__ constexpr int cs_threads(int chain_warps, int occ) { return 
 // registers a thread can have
 __host__ __device__ constexpr int cs_regs(int chain_warps, int occ) { return 65536 / (occ * cs_threads(chain_warps, occ)); }
 
-// asynchronous copy of 16 bytes from global to shared memory
-__device__ __forceinline__ void cp16(uint32_t dst_sa, const void *src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst_sa), "l"(src) : "memory");
-}
 __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N> __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 __device__ __forceinline__ void lds_b128(uint32_t addr, uint32_t (&r)[4]) {

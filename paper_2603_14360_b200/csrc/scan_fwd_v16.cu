@@ -44,22 +44,10 @@ __device__ __forceinline__ float lds_bf16(uint32_t addr) {
   asm volatile("ld.shared.u16 %0, [%1];" : "=h"(x) : "r"(addr));
   return __uint_as_float((uint32_t)x << 16);
 }
-// asynchronous copy of 16 bytes from global to shared memory
-__device__ __forceinline__ void cp16(uint32_t dst_sa, const void *src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst_sa), "l"(src) : "memory");
-}
-// arrives at the barrier once this thread's copies so far have landed (counted among the barrier's arrivals)
-__device__ __forceinline__ void cp_arrive(uint64_t *bar) {
-  asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
 
 // byte offset of eight-column chunk `chunk` of row `row` of a slab's H_t tile, [16 rows][16 columns] bf16:
 // chunks swapped in every other group of four rows, so that the eight rows of an ldmatrix cover all banks
 __device__ __forceinline__ uint32_t tile16_off(int row, int chunk) { return (uint32_t)(row * 32 + ((chunk ^ ((row >> 2) & 1)) << 4)); }
-
-__device__ __forceinline__ void ldmatrix_x4(uint32_t addr, uint32_t (&r)[4]) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
-}
 
 // NW: slabs of the CTA, a chain warp each, or two of eight rows (HALF).  kSvc service warps: four (one per scheduler, two steps of a stage each)
 // where a CTA has the SM to itself and their latency counts, two (four steps each) where several CTAs
