@@ -105,7 +105,8 @@ BwdPlan plan_bwd(const m2rnn_params *p, bool lean, bool have_ckpt) {
   // the specialised warps of scan_bwd_bf16.cu (1 024 steps, us: 16 slabs 232 against 245, 64 of heads of their own 208 / 232;
   // 160 slabs 296 / 249).  The latter keeps two chunks on chip, 16 rows of them up to any supported interval.
   if (V == 16 && (long)(B > 0 ? B : 1) * N * (K / 16) > sm_count()) {
-    const BwdPlan fast = plan_bwd_v16(B, N, p->Nq, p->Nk, K, p->T, p->ckpt_interval, false);
+    BwdPlan fast = plan_bwd_v16(B, N, p->Nq, p->Nk, K, p->T, p->ckpt_interval, false);
+    if (!have_ckpt && !p->ckpt_interval) fast.interval = fast.C;      // (the call's own checkpoints: a chunk's first is enough)
     return lean ? plan_bwd_v16(B, N, p->Nq, p->Nk, K, p->T, p->ckpt_interval || have_ckpt ? fast.interval : 16, true) : fast;
   }
   if (bwd_use_tc(B, N, K, V, p->io_dtype)) {   // 32-row CTAs, chunks of four steps

@@ -79,6 +79,12 @@ def test_chunks_of_two_intervals(oracle, T, size):
 
 
 @pytest.mark.gpu
+def test_chunks_of_two_intervals_clipped(oracle):
+    B, N, K, Nq, Nk = TWO[0]
+    parity.check_bwd(oracle, ScanConfig("clip", B=B, T=40, N=N, K=K, V=16, Nq=Nq, Nk=Nk, dist="saturating", gate_mean=1.0, seed=9), dh_clip=0.5)
+
+
+@pytest.mark.gpu
 def test_chunks_of_two_intervals_packed():
     """Sequences that end in every part of a chunk, an empty one among them: as each by itself."""
     (B, N, K, Nq, Nk), lens = TWO[0], [41, 0, 8, 25, 16, 1]
@@ -131,6 +137,22 @@ def test_packed_slices_match_the_sequences_one_by_one(oracle):
         dW, at = dW + one["dW"], at + n
     binding.check_device_status()
     assert parity.rel_err(got["dW"], dW.double().cpu().numpy()) < 1e-5
+
+
+def test_limited_scratch_holds_the_calls_own_checkpoints():
+    """Nothing asks for checkpoints every eight steps where the call makes its own and its chunks have sixteen: 7.0 to 7.9 MiB, and 2.3 to
+    3.4 more with twice as many (-6: accepted, and no device)."""
+    code = ("import ctypes, sys; sys.path[:0] = [%r]\n"
+            "from paper_2603_14360_b200 import build, binding as b\n"
+            "build.build()\n"
+            "f = ctypes.c_void_p(0x10000)\n"
+            "for B, T, N, Nq in ((6, 100, 8, 1), (6, 144, 8, 4), (2, 256, 12, 6)):\n"
+            "    p = b.Params(B=B, T=T, N=N, Nq=Nq, Nk=1, K=128, V=16, io_dtype=1, gate_kind=1, ckpt_interval=0, dh_clip=0.0)\n"
+            "    print(b._lib().m2rnn_ckpt_interval(ctypes.byref(p)),\n"
+            "          b._lib().m2rnn_bwd_static_scratch(ctypes.byref(p), *([f] * 5), None, None, None, None, None, f, None, *([f] * 5), None, None, None))\n"
+            ) % os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, env={**os.environ, "CUDA_VISIBLE_DEVICES": ""}, timeout=300)
+    assert r.stdout.split() == ["8", "-6"] * 3, (r.stdout, r.stderr[-2000:])
 
 
 def test_scratch_where_it_is_limited():
