@@ -11,8 +11,9 @@
 // The code a warp runs once is kept short: the first pass through an instruction comes from the L2
 // (the slab loop unrolled by four cost a small batch 4 us, 64-bit divisions another 1.5).
 // A CTA that takes eight slabs at a time behind barriers, two stages ahead, spends 1.9 us of latency on
-// them whatever their size.  The paper's layer (N = 84, K = 64, V = 16) at batch 48: 25.6 -> 6.0 us (8.2 without the early launch), at
-// batch 400: 200 -> 50 us (5.5 TB/s).
+// them whatever their size.  The paper's layer (N = 84, K = 64, V = 16) at batch 48: 25.6 -> 8.2 us, 6.0
+// where steps follow one another on a stream (the early launch hides the gap between them; a step after which the GPU is waited for,
+// host and all, 17.2 -> 16.1); at batch 400: 200 -> 50 us (5.5 TB/s).
 #include "device_common.cuh"
 #include "internal.h"
 #include "mma_tile.cuh"

@@ -16,7 +16,8 @@
 //   dW warps        (V/16) accumulate dW^T += dX^T H_{t-1} on tensor cores from the two tiles
 //                          (ldmatrix.trans operands), 16 columns of dW per warp, off the chain, and take dv = dX^T k
 //                          along with the same dX fragments (8 fewer MMAs and ldmatrix a step than as one more row of dW:
-//                          256 units of K = V = 64, 1 024 steps, 2 092 -> 2 042 us, K = 64, V = 32 754 -> 724);
+//                          256 units of K = V = 64, 1 024 steps, 2 092 -> 2 042 us; 320 of K = 64, V = 32, 512 steps, 754 -> 724;
+//                          64 of K = V = 64, two slabs a CTA, lose 0.6 %: 8 192 steps 5 351 -> 5 386);
 //   loader warp     (1)    stages q, k, v, dy and the gate of coming chunks;
 //   writer warp     (1)    reduces and writes dq, dk, dv, dgate of finished ones.
 //

@@ -14,11 +14,11 @@
 // Hand-over is by mbarriers between these two and the slab warps only; every wait is bounded and reports through dev_status.
 //
 // What bounds it: instruction issue, and with it how many slab warps the busiest scheduler has (three on the paper's layer
-// shape: 84 heads, K = 64, batch 4, one wave of ten slabs an SM, 454 ns a step; a warp with a scheduler to itself 240).  A step is
+// shape: 84 heads, K = 64, batch 4, one wave of ten slabs an SM, 442 ns a step; a warp with a scheduler to itself 240).  A step is
 // some 165 instructions of a slab warp, 57 of them on the FMA pipe, whose packed fp32 pairs take two cycles like two single ones:
 // products and sums of 16-bit operands are taken without unpacking instead (fma.f32.bf16, add.f32.f16, one cycle each).
-// Backward of that shape, 1 024 steps: 796 us with four kinds of warps that handed states over through shared memory, two waves,
-// and a share of dq and dk per head; 465 now.  Tried and slower: states of a chunk in registers (eight steps unrolled twice:
+// Backward call of that shape, 1 024 steps: 799 us with four kinds of warps that handed states over through shared memory, two waves,
+// and a share of dq and dk per head; 473 now, 452 of them this kernel.  Tried and slower: states of a chunk in registers (eight steps unrolled twice:
 // the instruction cache), fp32 copies of k, v, q, dy (shared-memory bandwidth), stmatrix and ldmatrix for the transposition.
 #include <algorithm>
 #include <climits>
@@ -555,12 +555,13 @@ cudaError_t launch_t(const ScanArgs &a, cudaStream_t s) {
 // A step costs what its busiest scheduler's slab warps cost (ns; one CTA with the SM to itself, 2 048 steps): one slab 239, four
 // 259, six 355, eight 382, ten 424, with chunks of 16 steps some 20 less; where heads do not share q and k the service warps have
 // a head's rows for each slab: eight 494.  Fewer CTAs than SMs want small ones, more want ten slabs each: 336 units of K = 64
-// run as 136 CTAs of 5 heads and two slabs in one wave (1 024 steps 484 us; as 336 CTAs of four slabs 681, of one 895).
+// run as 136 CTAs of 5 heads and two slabs in one wave (1 024 steps 452 us; 336 CTAs of four slabs 644, 1 344 of one slab 687).
 // Heads of a CTA that share q and k leave one share of dq and dk, slabs of a CTA one of dv and dgate: the shares' way through
 // memory counts too, and the two launches that add the slabs' shares.
 // Two plans are looked for, of whole states (a CTA has all slabs of its heads) and of split ones, and T decides between them: the two
-// launches that add the slabs' shares count 5 us of a call (backward, us, whole / split: B 6, 8 heads, K = 64, T 32 17.9 / 19.0, T 512 144 /
-// 128; B 1, 57 heads with k of their own, T 64 29.2 / 30.5, T 512 140.5 / 133.8).  The checkpoints' interval must not
+// launches that add the slabs' shares count 5 us of a call.  That keeps the short calls whole and is late for some (backward, us, whole /
+// split: B 6, 8 heads, K = 64, T 32 17.9 / 19.0, 128 42.8 / 40.1, 512 144 / 128, split from 322 on; B 1, 57 heads with k of their own, T 64
+// 29.2 / 30.5, 256 76.1 / 74.4, 512 140.5 / 133.8, split from 341 on).  The checkpoints' interval must not
 // follow T -- a buffer for the longest sequence has to do for every shorter one, and the interval is asked for without a T --, so it is
 // eight steps where either plan has chunks of eight, and a chunk of sixteen then begins at every second checkpoint (B 2, 84
 // heads sharing q and k, K = 64, 768 steps: forward 102 -> 105, backward 262; in chunks of eight 307).
